@@ -221,3 +221,55 @@ def tolerance(case):
         return dict(rel=1e-3, max=2e-3)
     # an fp16 output is rounded to 2.1e-4 (2-norm); with the fp16 rounding of (q - z) * Delta 2.9e-4 against fp64
     return dict(rel=1e-3, max=8e-3)
+
+
+def _dequantized(qweight, scales, zeros, N, K, bits=4):
+    """(q - z) * Delta in fp64 [N][K], from the packed arrays (layout: include/awq_b200.h)."""
+    if bits == 3:
+        u = qweight.view(torch.int32).view(-1, 3)
+        last = ((u[:, 0] >> 3) & 0x11111111) | ((u[:, 1] >> 2) & 0x22222222) | ((u[:, 2] >> 1) & 0x44444444)
+        words = torch.cat([u & 0x77777777, last[:, None]], dim=1).contiguous()
+    else:
+        words = qweight.view(torch.int32)
+    # a word's byte b holds column {0, 2, 1, 3}[b] of its four, rows g (low nibble) and g + 8 (high)
+    b = words.view(torch.uint8).view(N // 16, K // 64, 8, 4, 4, 4)[..., [0, 2, 1, 3]]       # band, tile, g, t, j, column
+    q = torch.stack([b & 15, b >> 4], dim=1).permute(0, 1, 3, 2, 5, 4, 6).reshape(N, K)     # band, h, g, tile, j, t, column
+    stored = scales.shape[1]
+    z = zeros.view(N // 32, stored, 2, 8)
+    z = torch.stack([z & 15, z >> 4], dim=0).permute(1, 3, 0, 4, 2).reshape(N, stored, 1)   # pair, band, h, g, group
+    d = scales.permute(0, 2, 1).reshape(N, stored, 1)
+    return ((q.view(N, stored, -1).double() - z.double()) * d.double()).view(N, K)
+
+
+def _quantized(W, s, group, top=15.0):
+    """(q - z) * Delta in fp64 by the quantizer's definition: fp32 w' and quotients, Delta kept in fp16."""
+    w = (W.float() * s).view(W.shape[0], -1, group)
+    mn, mx = w.amin(dim=2, keepdim=True), w.amax(dim=2, keepdim=True)
+    d = ((mx - mn) / torch.full_like(mn, top)).half()
+    d = torch.where(torch.isfinite(d) & (d != 0), d, torch.ones_like(d)).float()
+    z = torch.round(-mn / d).clamp(0.0, top)
+    q = (torch.round(w / d) + z).clamp(0.0, top)
+    return ((q - z).double() * d.double()).view(W.shape)
+
+
+def exact(case, seed):
+    """What `run` returns, in 64 bits, from the inputs that `prepare` makes; None where only packed arrays come back."""
+    kind = case["kind"]
+    if kind in ("quantize", "clip"):
+        return None
+    state = prepare(case, seed)
+    if kind == "layer":
+        return [(x.double() * inv_s.double()) @ _dequantized(*m[:3], m[3], K).t() for x, inv_s, mats, K, _ in state["calls"] for m in mats]
+    if kind != "alpha":
+        packed = (state["qweight"], state["scales"], state["zeros"], case["N"], case["K"])
+        return state["x"].double() @ _dequantized(*packed, bits=3 if kind == "int3" else 4).t()
+    W, X, stat = state["W"], state["X"], state["stat"]
+    target = X.double() @ W.double().t()
+    losses = []
+    for alpha in state["alphas"]:
+        # the statistic is positive and finite here; alpha is an fp32 argument, s an fp32 array
+        a32 = torch.tensor(alpha, dtype=torch.float32).double().item()
+        s = stat.sqrt() if alpha == 0.5 else (stat.double() ** a32).float()
+        y = (X.float() / s).half().double() @ _quantized(W, s, case["group"]).t()
+        losses.append(float((y - target).square().mean()))
+    return (losses, None)
