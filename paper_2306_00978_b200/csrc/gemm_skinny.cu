@@ -28,8 +28,10 @@
 // zero points (global loads, two iterations ahead) 80 us; those parameters by tensor-map copies into
 // shared memory, one box per unit, 75 us (an iteration no longer ends on a load that left two
 // iterations earlier but whose register is moved one iteration earlier); a second issuing thread
-// 65 us (one thread issued a product per ~105 cycles, 850 per stage; alone on the SM it issues one
-// per ~80); dequantizer warps that own every second stage instead of half of every stage 63 us.
+// 65 us; dequantizer warps that own every second stage instead of half of every stage 63 us; issuing
+// warps that run their loop converged (elect_one in tcgen05.cuh) 46 us - until then a thread issued a
+// product per ~105 cycles and its wait-and-issue chain was the longest one in the block (64 us at 32
+// tokens against 48 us with no products issued at all).
 // A deeper ring of packed weights (10 stages instead of 6) and fewer commits (two per turn of the
 // ring instead of one per stage) changed nothing by themselves.  What is left is the issue rate of
 // the four schedulers: a dequantizer warp spends about 100 instructions on 8 packed words (13 per
@@ -137,111 +139,122 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
 
     if (warp == 0) {
         // ------------------------------------------------------------ weight copies
-        if (lane == 0) {
-            uint32_t stage = 0, phase = 0;
-            unsigned int issued = 0, par_issued = 0;
-            bool ok = true;
-            for (int u = u0; u < u1 && ok; ++u) {
-                const int c = chunk_of(u), slab = u - c * nslabs;
-                const int kb0 = c * CK, nt = tiles_of(c);
-                // the unit's scales and zero points: boxes of 8 bands (4 band pairs) x the chunk's groups
-                const uint32_t pb = (uint32_t)(u - u0) & 1u, puse = ((uint32_t)(u - u0) >> 1) & 1u;
-                if (!mbar_wait(par_empty(pb), puse ^ 1u, ctl)) { ok = false; break; }
+        const bool lead = elect_one();
+        uint32_t stage = 0, phase = 0;
+        unsigned int issued = 0, par_issued = 0;
+        bool ok = true;
+        for (int u = u0; u < u1 && ok; ++u) {
+            const int c = chunk_of(u), slab = u - c * nslabs;
+            const int kb0 = c * CK, nt = tiles_of(c);
+            // the unit's scales and zero points: boxes of 8 bands (4 band pairs) x the chunk's groups
+            const uint32_t pb = (uint32_t)(u - u0) & 1u, puse = ((uint32_t)(u - u0) >> 1) & 1u;
+            if (!mbar_wait_warp(par_empty(pb), puse ^ 1u, ctl)) { ok = false; break; }
+            if (lead) {
                 mbar_arrive_expect_tx(par_full(pb), par_bytes);
                 tma_load_2d(par_base + pb * (uint32_t)kSkParBytes, &sc_map, (kb0 / KPG) * 16, slab * 8, par_full(pb));
                 tma_load_2d(par_base + pb * (uint32_t)kSkParBytes + z_in_par, &z_map, (kb0 / KPG) * 16, slab * 4, par_full(pb));
-                ++par_issued;
-                for (int j = 0; j < nt; j += 2) {
-                    if (!mbar_wait(raw_empty(stage), phase ^ 1u, ctl)) { ok = false; break; }
+            }
+            __syncwarp();
+            ++par_issued;
+            for (int j = 0; j < nt; j += 2) {
+                if (!mbar_wait_warp(raw_empty(stage), phase ^ 1u, ctl)) { ok = false; break; }
+                if (lead) {
                     mbar_arrive_expect_tx(raw_full(stage), kSkStageBytes);
                     // 8 bands x 2 k-blocks (256 words) at (word kb * 128 of the band's run, first band)
                     tma_load_2d(w_base + stage * kSkStageBytes, &w_map, (kb0 + j) * 128, slab * 8, raw_full(stage));
-                    ++issued;
-                    if (++stage == R) { stage = 0; phase ^= 1u; }
                 }
+                __syncwarp();
+                ++issued;
+                if (++stage == R) { stage = 0; phase ^= 1u; }
             }
-            if (!ok) {
-                // giving up: let the copies already issued land before the block exits
-                const unsigned int pending = issued < (unsigned)R ? issued : (unsigned)R;
-                uint32_t st = stage, ph = phase;
-                for (unsigned int i = 0; i < pending; ++i) {
-                    if (st == 0) { st = R - 1; ph ^= 1u; } else { --st; }
-                    const unsigned long long t0 = global_ns();
-                    while (!mbar_try_wait(raw_full(st), ph) && global_ns() - t0 < drain_limit_ns(ctl)) {}
-                }
-                for (unsigned int i = 0; i < 2u && i < par_issued; ++i) {
-                    const unsigned int k = par_issued - 1u - i;          // the k-th parameter copy: buffer k & 1, use k >> 1
-                    const unsigned long long t0 = global_ns();
-                    while (!mbar_try_wait(par_full(k & 1u), (k >> 1) & 1u) && global_ns() - t0 < drain_limit_ns(ctl)) {}
-                }
+        }
+        if (!ok) {
+            // giving up: let the copies already issued land before the block exits
+            const unsigned int pending = issued < (unsigned)R ? issued : (unsigned)R;
+            uint32_t st = stage, ph = phase;
+            for (unsigned int i = 0; i < pending; ++i) {
+                if (st == 0) { st = R - 1; ph ^= 1u; } else { --st; }
+                const unsigned long long t0 = global_ns();
+                while (!mbar_try_wait(raw_full(st), ph) && global_ns() - t0 < drain_limit_ns(ctl)) {}
+            }
+            for (unsigned int i = 0; i < 2u && i < par_issued; ++i) {
+                const unsigned int k = par_issued - 1u - i;              // the k-th parameter copy: buffer k & 1, use k >> 1
+                const unsigned long long t0 = global_ns();
+                while (!mbar_try_wait(par_full(k & 1u), (k >> 1) & 1u) && global_ns() - t0 < drain_limit_ns(ctl)) {}
             }
         }
     } else if (warp == 2) {
         // ------------------------------------------------------------ x copies, one slice per chunk
-        if (lane == 0) {
-            asm volatile("griddepcontrol.wait;" ::: "memory");
-            int cur = -1;
-            uint32_t n = 0;
-            for (int u = u0; u < u1; ++u) {
-                const int c = chunk_of(u);
-                if (c == cur) continue;
-                // the products that read the previous slice have completed
-                if (n > 0 && !mbar_wait_relaxed(x_empty, (n - 1u) & 1u, ctl)) break;
-                const int nt = tiles_of(c);
+        const bool lead = elect_one();
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        int cur = -1;
+        uint32_t n = 0;
+        for (int u = u0; u < u1; ++u) {
+            const int c = chunk_of(u);
+            if (c == cur) continue;
+            // the products that read the previous slice have completed
+            if (n > 0 && !__all_sync(0xFFFFFFFFu, mbar_wait_relaxed(x_empty, (n - 1u) & 1u, ctl))) break;
+            const int nt = tiles_of(c);
+            if (lead) {
                 mbar_arrive_expect_tx(x_full, (uint32_t)(nt * BN * 128));
                 for (int kb = 0; kb < nt; ++kb)
                     tma_load_2d(x_base + (uint32_t)(kb * BN * 128), &x_map, (c * CK + kb) * kBK, 0, x_full);
-                cur = c;
-                ++n;
             }
-            if (s_abort && n > 0) {
-                // giving up: the last slice's copies must have landed before the block exits
-                const unsigned long long t0 = global_ns();
-                while (!mbar_try_wait(x_full, (n - 1u) & 1u) && global_ns() - t0 < drain_limit_ns(ctl)) {}
-            }
+            __syncwarp();
+            cur = c;
+            ++n;
+        }
+        if (s_abort && n > 0) {
+            // giving up: the last slice's copies must have landed before the block exits
+            const unsigned long long t0 = global_ns();
+            while (!mbar_try_wait(x_full, (n - 1u) & 1u) && global_ns() - t0 < drain_limit_ns(ctl)) {}
         }
     } else if (warp == 1 || warp == 3) {
         // ------------------------------------------------------------ products
-        // Two issuing threads: a thread cannot issue these small products faster than one per
-        // ~50 - 100 cycles, which alone would cap the kernel below the HBM rate.  Thread h takes
-        // k-block h of every stage into an accumulator of its own; the epilogue adds the two.
-        if (lane == 0) {
-            constexpr uint32_t idesc = instr_desc(BN);
-            const int h = warp >> 1;
-            uint32_t stage = 0, phase = 0, xn = 0;
-            int local = 0, cur = -1;
-            bool ok = true;
-            for (int u = u0; u < u1 && ok; ++u, ++local) {
-                const int c = chunk_of(u);
-                const int nt = tiles_of(c);
-                if (c != cur) {
-                    if (!mbar_wait(x_full, xn & 1u, ctl)) break;
-                    ++xn;
-                    cur = c;
-                }
-                const int b = local & 1;
-                const uint32_t use = (uint32_t)(local >> 1) & 1u;
-                if (!mbar_wait(acc_empty(b), use ^ 1u, ctl)) break;
+        // Two issuing warps: warp h takes k-block h of every stage into an accumulator of its own; the
+        // epilogue adds the two.
+        const bool lead = elect_one();
+        constexpr uint32_t idesc = instr_desc(BN);
+        const int h = warp >> 1;
+        uint32_t stage = 0, phase = 0, xn = 0;
+        int local = 0, cur = -1;
+        bool ok = true;
+        for (int u = u0; u < u1 && ok; ++u, ++local) {
+            const int c = chunk_of(u);
+            const int nt = tiles_of(c);
+            if (c != cur) {
+                if (!mbar_wait_warp(x_full, xn & 1u, ctl)) break;
+                ++xn;
+                cur = c;
+            }
+            const int b = local & 1;
+            const uint32_t use = (uint32_t)(local >> 1) & 1u;
+            if (!mbar_wait_warp(acc_empty(b), use ^ 1u, ctl)) break;
+            tc_fence_after();
+            const uint32_t d_tmem = tmem_base + (uint32_t)((2 * b + h) * BN);
+            uint64_t bdesc = smem_desc_sw128(x_base + (uint32_t)(h * BN * 128));
+            for (int j = 0; j < nt; j += 2) {
+                if (!mbar_wait_warp(a_full(stage), phase, ctl)) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)((2 * b + h) * BN);
-                uint64_t bdesc = smem_desc_sw128(x_base + (uint32_t)(h * BN * 128));
-                for (int j = 0; j < nt; j += 2) {
-                    if (!mbar_wait(a_full(stage), phase, ctl)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t a_tmem = tmem_base + (uint32_t)(A0 + stage * 64 + 32 * h);
+                const uint32_t a_tmem = tmem_base + (uint32_t)(A0 + stage * 64 + 32 * h);
+                if (lead) {
 #pragma unroll
                     for (int k = 0; k < kBK / 16; ++k)           // A: +8 columns, B: +32 bytes per K = 16 step
                         umma_f16_a_tmem(d_tmem, a_tmem + (uint32_t)(8 * k), bdesc + (uint64_t)(2 * k), idesc,
                                         (j != 0 || k != 0) ? 1u : 0u);
                     if (stage % GS == GS - 1) umma_commit(a_empty(stage / GS));
-                    bdesc += (uint64_t)((2 * BN * 128) >> 4);   // two k-blocks further in the slice of x
-                    if (++stage == S) { stage = 0; phase ^= 1u; }
                 }
-                if (!ok) break;
+                __syncwarp();
+                bdesc += (uint64_t)((2 * BN * 128) >> 4);       // two k-blocks further in the slice of x
+                if (++stage == S) { stage = 0; phase ^= 1u; }
+            }
+            if (!ok) break;
+            if (lead) {
                 umma_commit(acc_full(b));
                 // the slice of x may be replaced once the products of its last unit have completed
                 if (u + 1 < u1 && chunk_of(u + 1) != c) umma_commit(x_empty);
             }
+            __syncwarp();
         }
     } else if (warp >= 8) {
         // ------------------------------------------------------------ dequantizers

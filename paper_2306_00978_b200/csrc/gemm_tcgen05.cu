@@ -118,67 +118,72 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer
-        if (lane == 0) {
-            uint32_t stage = 0, phase = 0;
-            unsigned int issued = 0;
-            bool ok = true;
-            for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x) {
-                const int tile = item / splits, sp = item - tile * splits;
-                const int slab = tile / m_tiles, mt = tile % m_tiles;
-                const int kb1 = kb_begin(sp + 1);
-                for (int kb = kb_begin(sp); kb < kb1; ++kb) {
-                    if (!mbar_wait(empty(stage), phase ^ 1u, ctl)) { ok = false; break; }
+        const bool lead = elect_one();
+        uint32_t stage = 0, phase = 0;
+        unsigned int issued = 0;
+        bool ok = true;
+        for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x) {
+            const int tile = item / splits, sp = item - tile * splits;
+            const int slab = tile / m_tiles, mt = tile % m_tiles;
+            const int kb1 = kb_begin(sp + 1);
+            for (int kb = kb_begin(sp); kb < kb1; ++kb) {
+                if (!mbar_wait_warp(empty(stage), phase ^ 1u, ctl)) { ok = false; break; }
+                if (lead) {
                     const uint32_t bar = raw_full(stage);
                     mbar_arrive_expect_tx(bar, Cfg::kTxBytes);
                     tma_load_2d(x_addr(stage), &x_map, kb * kBK, mt * BN, bar);
                     // weights: box of 8 bands x 512 bytes (128 words) at (k-block, first band)
                     tma_load_2d(x_addr(stage) + Cfg::kXTileBytes, &w_map, kb * 128, slab * 8, bar);
-                    ++issued;
-                    if (++stage == S) { stage = 0; phase ^= 1u; }
                 }
+                __syncwarp();
+                ++issued;
+                if (++stage == S) { stage = 0; phase ^= 1u; }
             }
-            if (!ok) {
-                // giving up: let the copies already issued land before the block exits
-                const unsigned int pending = issued < (unsigned)S ? issued : (unsigned)S;
-                uint32_t st = stage, ph = phase;
-                for (unsigned int i = 0; i < pending; ++i) {
-                    if (st == 0) { st = S - 1; ph ^= 1u; } else { --st; }
-                    const unsigned long long t0 = global_ns();
-                    while (!mbar_try_wait(raw_full(st), ph) && global_ns() - t0 < 100000000ull) {}
-                }
+        }
+        if (!ok) {
+            // giving up: let the copies already issued land before the block exits
+            const unsigned int pending = issued < (unsigned)S ? issued : (unsigned)S;
+            uint32_t st = stage, ph = phase;
+            for (unsigned int i = 0; i < pending; ++i) {
+                if (st == 0) { st = S - 1; ph ^= 1u; } else { --st; }
+                const unsigned long long t0 = global_ns();
+                while (!mbar_try_wait(raw_full(st), ph) && global_ns() - t0 < 100000000ull) {}
             }
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t idesc = instr_desc(BN);
-            uint32_t stage = 0, phase = 0;
-            int local = 0;
-            bool ok = true;
-            for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x, ++local) {
-                const int sp = item % splits;
-                const int kb0 = kb_begin(sp), kb1 = kb_begin(sp + 1);
-                const int b = local % NACC;
-                const uint32_t use = (uint32_t)(local / NACC) & 1u;
-                if (!mbar_wait(acc_empty(b), use ^ 1u, ctl)) { ok = false; break; }
+        const bool lead = elect_one();
+        constexpr uint32_t idesc = instr_desc(BN);
+        uint32_t stage = 0, phase = 0;
+        int local = 0;
+        bool ok = true;
+        for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x, ++local) {
+            const int sp = item % splits;
+            const int kb0 = kb_begin(sp), kb1 = kb_begin(sp + 1);
+            const int b = local % NACC;
+            const uint32_t use = (uint32_t)(local / NACC) & 1u;
+            if (!mbar_wait_warp(acc_empty(b), use ^ 1u, ctl)) { ok = false; break; }
+            tc_fence_after();
+            const uint32_t d_tmem = tmem_base + (uint32_t)(b * BN);
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (!mbar_wait_warp(raw_full(stage), phase, ctl) || !mbar_wait_warp(a_full(stage), phase, ctl)) {
+                    ok = false; break;
+                }
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(b * BN);
-                for (int kb = kb0; kb < kb1; ++kb) {
-                    if (!mbar_wait(raw_full(stage), phase, ctl) || !mbar_wait(a_full(stage), phase, ctl)) {
-                        ok = false; break;
-                    }
-                    tc_fence_after();
-                    const uint32_t a_tmem = tmem_base + (uint32_t)(Cfg::kAColumn0 + stage * 32);
-                    const uint64_t bdesc = smem_desc_sw128(x_addr(stage));
+                const uint32_t a_tmem = tmem_base + (uint32_t)(Cfg::kAColumn0 + stage * 32);
+                const uint64_t bdesc = smem_desc_sw128(x_addr(stage));
+                if (lead) {
 #pragma unroll
-                    for (int k = 0; k < kBK / 16; ++k)       // A: +8 columns, B: +32 bytes per K = 16 step
+                    for (int k = 0; k < kBK / 16; ++k)           // A: +8 columns, B: +32 bytes per K = 16 step
                         umma_f16_a_tmem(d_tmem, a_tmem + (uint32_t)(8 * k), bdesc + (uint64_t)(2 * k), idesc,
                                         (kb != kb0 || k != 0) ? 1u : 0u);
                     umma_commit(empty(stage));
-                    if (++stage == S) { stage = 0; phase ^= 1u; }
                 }
-                if (ok) umma_commit(acc_full(b));
+                __syncwarp();
+                if (++stage == S) { stage = 0; phase ^= 1u; }
             }
+            if (ok && lead) umma_commit(acc_full(b));
+            __syncwarp();
         }
     } else if (warp >= 8) {
         // -------------------------------------------------------------- dequantizers

@@ -8,7 +8,9 @@
 // 128 x 256 x 16 MMA per 128 cycles) set the pace at ~770 cycles per k-block.  In a pair each
 // block stages only its half of the tokens (the tensor cores of both SMs read both halves), and
 // a stage covers K = 128, so the polls and commits are paid once per eight MMAs: ~1120 cycles per
-// stage against the pipe's 1024.
+// stage against the pipe's 1024.  (Both figures with the issuing loop inside `if (lane == 0)`; converged
+// loops with one elected lane, see tcgen05.cuh, took 13824 -> 5120 at 2048 tokens from 210 to 204 us and
+// 4096 -> 11008 at 8192 tokens from 597 to 587 us.)
 //
 // Block r of a pair (r = rank in the cluster) owns
 //   - A: output channels 128 r .. 128 r + 127 of the 256-channel slab, dequantized by its own
@@ -209,16 +211,17 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer
-        if (lane == 0) {
-            const uint32_t leader_x_full0 = map_to_rank(x_full(0), 0);
-            uint32_t stage = 0, phase = 0;
-            unsigned int issued = 0;
-            bool ok = true;
-            while (ok && pieces.next(tile, k0, k1)) {
-                const int slab = (tile / m_tiles) * 2 + (int)rank;          // 128-channel slab of this block
-                const int tok0 = (tile % m_tiles) * kPairTokens + (int)rank * kHalfTokens;
-                for (int ks = k0; ks < k1; ++ks) {
-                    if (!mbar_wait(empty(stage), phase ^ 1u, ctl)) { ok = false; break; }
+        const bool lead = elect_one();
+        const uint32_t leader_x_full0 = map_to_rank(x_full(0), 0);
+        uint32_t stage = 0, phase = 0;
+        unsigned int issued = 0;
+        bool ok = true;
+        while (ok && pieces.next(tile, k0, k1)) {
+            const int slab = (tile / m_tiles) * 2 + (int)rank;              // 128-channel slab of this block
+            const int tok0 = (tile % m_tiles) * kPairTokens + (int)rank * kHalfTokens;
+            for (int ks = k0; ks < k1; ++ks) {
+                if (!mbar_wait_warp(empty(stage), phase ^ 1u, ctl)) { ok = false; break; }
+                if (lead) {
                     if (rank == 0) mbar_arrive_expect_tx(x_full(stage), 2u * Cfg::kXTileBytes);
                     const uint32_t xbar = leader_x_full0 + 8u * stage;
                     tma_load_2d_pair(x_addr(stage), &x_map, ks * kStageK, tok0, xbar);
@@ -227,26 +230,28 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                     mbar_arrive_expect_tx(bar, (uint32_t)Cfg::kWBytes);
                     // weights: box of 8 bands x 1 KB (256 words: two k-tiles) at (stage, first band)
                     tma_load_2d(x_addr(stage) + Cfg::kXTileBytes, &w_map, ks * 256, slab * 8, bar);
-                    ++issued;
-                    if (++stage == S) { stage = 0; phase ^= 1u; }
                 }
+                __syncwarp();
+                ++issued;
+                if (++stage == S) { stage = 0; phase ^= 1u; }
             }
-            if (!ok) {
-                // giving up: let the copies already issued land before the block exits
-                const unsigned int pending = issued < (unsigned)S ? issued : (unsigned)S;
-                uint32_t st = stage, ph = phase;
-                for (unsigned int i = 0; i < pending; ++i) {
-                    if (st == 0) { st = S - 1; ph ^= 1u; } else { --st; }
-                    const unsigned long long t0 = global_ns();
-                    while (!mbar_try_wait(w_full(st), ph) && global_ns() - t0 < 100000000ull) {}
-                }
-                const unsigned long long t1 = global_ns();          // and the x halves (counted on the leader)
-                while (global_ns() - t1 < 1000000ull) __nanosleep(1000);
+        }
+        if (!ok) {
+            // giving up: let the copies already issued land before the block exits
+            const unsigned int pending = issued < (unsigned)S ? issued : (unsigned)S;
+            uint32_t st = stage, ph = phase;
+            for (unsigned int i = 0; i < pending; ++i) {
+                if (st == 0) { st = S - 1; ph ^= 1u; } else { --st; }
+                const unsigned long long t0 = global_ns();
+                while (!mbar_try_wait(w_full(st), ph) && global_ns() - t0 < 100000000ull) {}
             }
+            const unsigned long long t1 = global_ns();              // and the x halves (counted on the leader)
+            while (global_ns() - t1 < 1000000ull) __nanosleep(1000);
         }
     } else if (warp == 1) {
         // ------------------------------------------------- MMA issuer (leader block only)
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
+            const bool lead = elect_one();
             constexpr uint32_t idesc = instr_desc_pair();
             const uint32_t peer_acc_full = map_to_rank(acc_full, 1);
             const uint32_t peer_empty0 = map_to_rank(empty(0), 1);
@@ -254,30 +259,34 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
             int local = 0;
             bool ok = true;
             for (; ok && pieces.next(tile, k0, k1); ++local) {
-                if (!mbar_wait(acc_empty, ((uint32_t)local & 1u) ^ 1u, ctl)) { ok = false; break; }
+                if (!mbar_wait_warp(acc_empty, ((uint32_t)local & 1u) ^ 1u, ctl)) { ok = false; break; }
                 tc_fence_after();
                 for (int ks = k0; ks < k1; ++ks) {
                     // both barriers are normally complete already: poll them together
                     const bool xr = mbar_try_wait(x_full(stage), phase), ar = mbar_try_wait(a_full(stage), phase);
-                    if (!(xr && ar) &&
-                        (!mbar_wait(x_full(stage), phase, ctl) || !mbar_wait(a_full(stage), phase, ctl))) {
+                    if (!__all_sync(0xFFFFFFFFu, xr && ar) &&
+                        (!mbar_wait_warp(x_full(stage), phase, ctl) || !mbar_wait_warp(a_full(stage), phase, ctl))) {
                         ok = false; break;
                     }
                     tc_fence_after();
                     const uint32_t a_tmem = tmem_base + (uint32_t)(Cfg::kAColumn0 + stage * Cfg::kAColsPerStage);
                     const uint64_t bdesc = smem_desc_sw128(x_addr(stage));
+                    if (lead) {
 #pragma unroll
-                    for (int k = 0; k < kStageK / 16; ++k) {
-                        // A: 8 columns per K = 16; B: 32 bytes per K = 16 inside a 64-wide half, halves 16 KB apart
-                        const uint64_t boff = (uint64_t)(((k >> 2) * Cfg::kXHalfBytes + (k & 3) * 32) >> 4);
-                        umma_pair_f16_a_tmem(tmem_base, a_tmem + (uint32_t)(8 * k), bdesc + boff, idesc,
-                                             (ks > k0 || k > 0) ? 1u : 0u);
+                        for (int k = 0; k < kStageK / 16; ++k) {
+                            // A: 8 columns per K = 16; B: 32 bytes per K = 16 inside a 64-wide half, halves 16 KB apart
+                            const uint64_t boff = (uint64_t)(((k >> 2) * Cfg::kXHalfBytes + (k & 3) * 32) >> 4);
+                            umma_pair_f16_a_tmem(tmem_base, a_tmem + (uint32_t)(8 * k), bdesc + boff, idesc,
+                                                 (ks > k0 || k > 0) ? 1u : 0u);
+                        }
+                        umma_pair_commit(empty(stage));
+                        umma_pair_commit(peer_empty0 + 8u * stage);
                     }
-                    umma_pair_commit(empty(stage));
-                    umma_pair_commit(peer_empty0 + 8u * stage);
+                    __syncwarp();
                     if (++stage == S) { stage = 0; phase ^= 1u; }
                 }
-                if (ok) { umma_pair_commit(acc_full); umma_pair_commit(peer_acc_full); }
+                if (ok && lead) { umma_pair_commit(acc_full); umma_pair_commit(peer_acc_full); }
+                __syncwarp();
             }
         }
     } else if (warp >= 8 && warp < 16) {

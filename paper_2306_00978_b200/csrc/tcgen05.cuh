@@ -12,6 +12,20 @@ namespace awq {
 constexpr int kBK = 64;   // k-block: 64 input channels = one 128-byte swizzle row of fp16
 
 // ------------------------------------------------------------------ small PTX wrappers
+// One lane of a converged warp, chosen the same way every time.  The warps that issue copies and products
+// run their whole loop converged - every lane polls the barriers and forms the operands - and only the
+// instruction itself is predicated on this lane: descriptors and addresses then stay in uniform
+// registers.  With the loop inside `if (lane == 0)` every product first moved its operands there, and one
+// thread issued a product per ~80 - 105 cycles (8192 -> 28672 at 32 tokens 64 -> 50 us).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p) :: "memory");
+    return p != 0;
+}
+// the bounded wait of a converged warp: true only if no lane gave up
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, const WaitCtl& ctl) {
+    return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, ctl));
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
