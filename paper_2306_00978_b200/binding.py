@@ -190,6 +190,14 @@ def ensure_workspace(nbytes: int) -> None:
     _workspace[dev] = buf
 
 
+def _workspace_for_multi(M: int, mats, K: int, group: int) -> None:
+    """What the calls need one by one, and what all of them in one launch can use (M <= 64).  While a
+    stream is capturing nothing is registered for the latter: the call then runs one by one."""
+    ensure_workspace(max(workspace_bytes(M, m[3], K, group) for m in mats))
+    if M <= 64 and len(mats) > 1 and not torch.cuda.is_current_stream_capturing():
+        ensure_workspace(workspace_bytes(M, sum(m[3] for m in mats), K, group))
+
+
 def workspace_bytes(M: int, N: int, K: int, group: int) -> int:
     return int(lib().awq_workspace_bytes(M, N, K, group))
 
@@ -222,8 +230,8 @@ def linear_multi(x: torch.Tensor, mats, K: int, group: int, outs=None):
         raise AwqError("x must be [M][K]")
     if outs is None:
         outs = [torch.empty((M, m[3]), dtype=torch.float16, device=x.device) for m in mats]
-    if M <= 16:
-        ensure_workspace(max(workspace_bytes(M, m[3], K, group) for m in mats))
+    if M <= 64:
+        _workspace_for_multi(M, mats, K, group)
     arr = (_Problem * len(mats))()
     for k, ((qw, sc, zp, N), y) in enumerate(zip(mats, outs)):
         arr[k] = _Problem(_dev(qw, torch.uint8, "qweight"), _dev(sc, torch.float16, "scales"),
@@ -247,7 +255,7 @@ def linear_multi_scaled(x: torch.Tensor, inv_s: torch.Tensor, mats, K: int, grou
         outs = [torch.empty((M, m[3]), dtype=torch.float16, device=x.device) for m in mats]
     if x_scratch is None and lib().awq_linear_scaled_needs_scratch(M, sum(m[3] for m in mats), K, int(group)):
         x_scratch = torch.empty_like(x)
-    ensure_workspace(max(workspace_bytes(M, m[3], K, group) for m in mats))
+    _workspace_for_multi(M, mats, K, group)
     arr = (_Problem * len(mats))()
     for k, ((qw, sc, zp, N), y) in enumerate(zip(mats, outs)):
         arr[k] = _Problem(_dev(qw, torch.uint8, "qweight"), _dev(sc, torch.float16, "scales"),

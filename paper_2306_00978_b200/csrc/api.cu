@@ -165,10 +165,7 @@ int awq_search_clip(const void* W, const float* act_mean_abs, float alpha, int g
                                         ratios, n_ratios, clip_ratio, N, K, (cudaStream_t)stream));
 }
 
-// Where the chunked matrix-vector kernel beats the tensor-core kernels (measured, us, chunked against
-// tensor-core: at 16 tokens 10.9 / 13.5 on 4096 -> 4096, 17.4 / 25.9 on 4096 -> 11008, 20.9 / 26.2 on
-// 11008 -> 4096, 45 / 98 on 8192 -> 28672; at 24 tokens 14.0 / 13.9, 23.2 / 26.1, 27.4 / 26.2, 60.7 / 98;
-// at 32 tokens 17.6 / 13.8, 28.4 / 25.8, 33.4 / 26.4, 79 / 81).
+// Where the chunked matrix-vector kernel beats the band kernel, up to 8 tokens.
 // With one token fragment its time does not depend on M (32 us on the 70B shapes for 1 .. 8 tokens),
 // while the band kernel's grows with the tokens that travel through its stages.  Chunked / band, us:
 //   8192 -> 28672   3 tokens 31.3 / 34.5   5: 31.9 / 38.9   8: 32.5 / 49.1
@@ -183,9 +180,17 @@ static bool mid_kernel_preferred(int M, int N, int K) {
     const long long nk = (long long)N * K;
     if (M < 2) return false;
     if (M == 2) return K >= 12288 && nk >= (1LL << 26);   // 13824 -> 5120: 13.6 / 14.2 us, 28672 -> 8192: 32.3 / 33.5 us
-    if (M <= 8) return K > 4096 && nk >= (M <= 4 ? (1LL << 26) : (1LL << 25));
-    if (M <= 16) return true;
-    return M <= 24 && nk >= (1LL << 25);
+    return M <= 8 && K > 4096 && nk >= (M <= 4 ? (1LL << 26) : (1LL << 25));
+}
+
+// Where the chunked tensor-core kernel runs: 9 .. 64 tokens, and below where the output rows are too few
+// for the band kernel.  Measured, us, against what ran there before: the chunked matrix-vector kernel with
+// more than one token fragment (4096 -> 4096 / 4096 -> 11008 / 11008 -> 4096 / 8192 -> 28672 at 16 tokens
+// 7.1 / 12.7 / 12.8 / 37.9 against 7.7 / 13.3 / 14.7 / 39.1, at 24 tokens 8.2 / 15.1 / 15.2 / 43.9 against
+// 9.7 / 16.8 / 18.3 / 52.0), and the split-K kernel (1024 -> 1024 at 4 / 8 tokens 4.5 / 4.5 against 7.9 /
+// 10.0, 2048 -> 1536 5.3 / 5.2 against 7.9 / 10.2).
+static bool skinny_kernel_preferred(int M, int total_n, int K, int group, int sms) {
+    return M <= 64 && (M > 8 || !gemv_uses_band_kernel(M, total_n, sms)) && gemm_skinny_applies(M, total_n, K, group);
 }
 
 static int resolve_path(int M, int K, int path) {
@@ -204,16 +209,14 @@ size_t awq_workspace_bytes(int M, int N, int K, int group) {
         sms = 160;                           // no device to ask: an upper bound for this GPU family
     }
     size_t gemm = gemm_workspace_bytes(M, N, sms);
-    const size_t mid = (M <= 32 && gemv_mid_applies(M, N, K, group, sms)) ? gemv_mid_workspace_bytes(M, N, K) : 0;
-    if (M > 8 && mid > gemm) gemm = mid;
-    if (M > 8 && gemm_skinny_applies(M, N, K, group)) {
-        const size_t skinny = gemm_skinny_workspace_bytes(M, N, K, group, sms);
-        if (skinny > gemm) gemm = skinny;
-    }
+    const size_t mid = (M <= 8 && gemv_mid_applies(M, N, K, group, sms)) ? gemv_mid_workspace_bytes(M, N, K) : 0;
+    const size_t skinny = skinny_kernel_preferred(M, N, K, group, sms) ? gemm_skinny_workspace_bytes(M, N, K, group, sms) : 0;
+    if (skinny > gemm) gemm = skinny;
     if (M > 16) return gemm;
-    const size_t gemv = gemv_workspace_bytes(M);   // required by the split-K matrix-vector kernel
-    if (M <= 8) return gemv > mid ? gemv : mid;    // awq_linear never takes the tensor-core kernel here
-    return gemv > gemm ? gemv : gemm;
+    size_t gemv = gemv_workspace_bytes(M);         // required by the split-K matrix-vector kernel
+    if (M > 8) return gemv > gemm ? gemv : gemm;
+    if (mid > gemv) gemv = mid;                    // awq_linear takes no prefill kernel here
+    return gemv > skinny ? gemv : skinny;
 }
 
 int awq_set_workspace(void* dev_ptr, size_t bytes) {
@@ -253,17 +256,16 @@ int awq_linear_path(const void* x, const void* qweight, const void* scales, cons
     }
     DeviceState* d;
     if (int rc = device_state(&d)) return rc;
-    if (automatic && mid_kernel_preferred(M, N, K) && gemv_mid_applies(M, N, K, group, d->sms)) {
+    if (automatic && skinny_kernel_preferred(M, N, K, group, d->sms)) {
+        const size_t need = gemm_skinny_workspace_bytes(M, N, K, group, d->sms);
+        std::lock_guard<std::mutex> lock(g_mutex);
+        if (d->workspace_bytes >= need) path = AWQ_PATH_GEMM_SKINNY;
+    }
+    if (automatic && path == AWQ_PATH_GEMV && mid_kernel_preferred(M, N, K) && gemv_mid_applies(M, N, K, group, d->sms)) {
         std::lock_guard<std::mutex> lock(g_mutex);
         if (d->workspace_bytes >= gemv_mid_workspace_bytes(M, N, K)) path = AWQ_PATH_GEMV_MID;
     }
-    if (automatic && path == AWQ_PATH_GEMM && M > 16 && M <= 64 && gemm_skinny_applies(M, N, K, group)) {
-        // 17 .. 64 tokens: the chunked tensor-core kernel (measured against the prefill kernels at 32
-        // and 64 tokens: 10.1 / 13.7 and 11.1 / 16.1 us on 4096 -> 4096, 20.7 / 26.2 and 20.8 / 31.4 us
-        // on 4096 -> 11008, 66.5 / 80.9 and 73.5 / 81.2 us on 8192 -> 28672)
-        std::lock_guard<std::mutex> lock(g_mutex);
-        if (d->workspace_bytes >= gemm_skinny_workspace_bytes(M, N, K, group, d->sms)) path = AWQ_PATH_GEMM_SKINNY;
-    }
+    if (path == AWQ_PATH_GEMV_MID && M > 8 && gemm_skinny_applies(M, N, K, group)) path = AWQ_PATH_GEMM_SKINNY;
     if (path == AWQ_PATH_GEMV_MID) {
         if (!gemv_mid_applies(M, N, K, group, d->sms)) return AWQ_ERR_BAD_SHAPE;
         void* ws = nullptr;
@@ -276,13 +278,15 @@ int awq_linear_path(const void* x, const void* qweight, const void* scales, cons
                                          take_packed_written(d), (cudaStream_t)stream));
     }
     if (path == AWQ_PATH_GEMM_SKINNY) {
+        const size_t need = gemm_skinny_workspace_bytes(M, N, K, group, d->sms);
         void* ws = nullptr;
         {
             std::lock_guard<std::mutex> lock(g_mutex);
-            if (d->workspace_bytes < gemm_skinny_workspace_bytes(M, N, K, group, d->sms)) return AWQ_ERR_NO_WORKSPACE;
+            if (d->workspace_bytes < need) return AWQ_ERR_NO_WORKSPACE;
             ws = d->workspace;
         }
-        return note_cuda(launch_gemm_skinny(x, qweight, scales, zeros, y, M, N, K, group, ws, d->status_word,
+        const GemvMatrix one = {qweight, scales, zeros, y, N};
+        return note_cuda(launch_gemm_skinny(x, &one, 1, M, K, group, nullptr, ws, d->status_word,
                                             d->sms, take_packed_written(d), (cudaStream_t)stream));
     }
     const bool tensor_path = path == AWQ_PATH_GEMM || path == AWQ_PATH_GEMM_1SM;
@@ -363,6 +367,24 @@ int awq_static_scratch_fill(int value, void* stream) {
     return note_cuda(cudaMemsetAsync(scratch, value & 0xFF, kCounterBytes, (cudaStream_t)stream));
 }
 
+// All matrices in one launch of the chunked tensor-core kernel, if the workspace holds their partial sums.
+static int linear_multi_skinny(DeviceState* d, const void* x, const float* inv_s, const AwqLinearProblem* problems,
+                               int count, int total_n, int M, int K, int group, void* stream, bool* launched) {
+    const size_t need = gemm_skinny_workspace_bytes(M, total_n, K, group, d->sms);
+    void* ws = nullptr;
+    {
+        std::lock_guard<std::mutex> lock(g_mutex);
+        if (d->workspace_bytes < need) return AWQ_OK;
+        ws = d->workspace;
+    }
+    GemvMatrix mats[kMaxMulti];
+    for (int i = 0; i < count; ++i)
+        mats[i] = GemvMatrix{problems[i].qweight, problems[i].scales, problems[i].zeros, problems[i].y, problems[i].N};
+    *launched = true;
+    return note_cuda(launch_gemm_skinny(x, mats, count, M, K, group, inv_s, ws, d->status_word, d->sms,
+                                        take_packed_written(d), (cudaStream_t)stream));
+}
+
 int awq_linear_multi(const void* x, const AwqLinearProblem* problems, int count,
                      int M, int K, int group, void* stream) {
     if (!problems || !x) return AWQ_ERR_NULL_POINTER;
@@ -388,6 +410,11 @@ int awq_linear_multi(const void* x, const AwqLinearProblem* problems, int count,
                                  problems[i].N};
         return note_cuda(launch_gemv_band(x, mats, count, M, K, group, d->status_word, d->sms,
                                           take_packed_written(d), (cudaStream_t)stream));
+    }
+    if (skinny_kernel_preferred(M, total_n, K, group, d->sms)) {
+        bool launched = false;
+        const int rc = linear_multi_skinny(d, x, nullptr, problems, count, total_n, M, K, group, stream, &launched);
+        if (rc != AWQ_OK || launched) return rc;
     }
     // otherwise one call per matrix, as awq_linear would run it
     for (int i = 0; i < count; ++i) {
@@ -445,8 +472,13 @@ int awq_linear_multi_scaled(const void* x, const float* inv_s, void* x_scratch, 
         return note_cuda(launch_gemv_band(x, mats, count, M, K, group, d->status_word, d->sms,
                                           take_packed_written(d), (cudaStream_t)stream, inv_s));
     }
-    // no kernel to fold it into: scale first (one more launch), then the plain calls
     if (!x_scratch) return AWQ_ERR_NULL_POINTER;
+    if (skinny_kernel_preferred(M, total_n, K, group, d->sms)) {
+        bool launched = false;
+        const int rc = linear_multi_skinny(d, x, inv_s, problems, count, total_n, M, K, group, stream, &launched);
+        if (rc != AWQ_OK || launched) return rc;
+    }
+    // no kernel to fold it into: scale first (one more launch), then the plain calls
     if (int rc = note_cuda(launch_multiply_by_inverse(x, inv_s, x_scratch, M, K, (cudaStream_t)stream))) return rc;
     return awq_linear_multi(x_scratch, problems, count, M, K, group, stream);
 }

@@ -118,9 +118,12 @@ cudaError_t launch_chunk_reduce(const float* partial, void* y, int chunks, size_
 // 17 .. 64 tokens on the tensor cores (gemm_skinny.cu): units of one 128-channel slab x one chunk of
 // K, the chunk's slice of x resident in shared memory, partial sums per chunk in the workspace
 bool gemm_skinny_applies(int M, int N, int K, int group);
+// `count` matrices (1..kMaxMulti) sharing x, K and the group size in one launch (N: the sum of theirs);
+// inv_s: nullptr, or the inverse channel scales (fp32 [K], device), multiplied into x on the way.
+// Up to 32 tokens q - z enters the products as an integer and Delta is applied in fp32; above, fp16 (q - z) * Delta does.
 size_t gemm_skinny_workspace_bytes(int M, int N, int K, int group, int sms);
-cudaError_t launch_gemm_skinny(const void* x, const void* qweight, const void* scales, const void* zeros, void* y,
-                               int M, int N, int K, int group, void* workspace, unsigned int* status_word, int sms,
+cudaError_t launch_gemm_skinny(const void* x, const GemvMatrix* mats, int count, int M, int K, int group,
+                               const float* inv_s, void* workspace, unsigned int* status_word, int sms,
                                bool serialize, cudaStream_t st);
 
 // scale search (search.cu)

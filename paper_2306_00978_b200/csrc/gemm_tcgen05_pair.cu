@@ -336,12 +336,12 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                     uint32_t v[16];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        constexpr uint32_t kMagic = 0x64006400u, kSixteenth = 0x2C002C00u;
+                        constexpr uint32_t kSixteenth = 0x2C002C00u;
                         const uint32_t w = wds[j], w8 = w >> 8;
-                        v[4 * j + 0] = hmul2_u32(hsub2_u32((w & 0x000F000Fu) | kMagic, zlo), d_up);
-                        v[4 * j + 1] = hmul2_u32(hsub2_u32((w8 & 0x000F000Fu) | kMagic, zlo), d_up);
-                        v[4 * j + 2] = hmul2_u32(hfma2_u32((w & 0x00F000F0u) | kMagic, kSixteenth, zhi), d_lo);
-                        v[4 * j + 3] = hmul2_u32(hfma2_u32((w8 & 0x00F000F0u) | kMagic, kSixteenth, zhi), d_lo);
+                        v[4 * j + 0] = hmul2_u32(hsub2_u32(code_pair(w, kLowCodes), zlo), d_up);
+                        v[4 * j + 1] = hmul2_u32(hsub2_u32(code_pair(w8, kLowCodes), zlo), d_up);
+                        v[4 * j + 2] = hmul2_u32(hfma2_u32(code_pair(w, kHighCodes), kSixteenth, zhi), d_lo);
+                        v[4 * j + 3] = hmul2_u32(hfma2_u32(code_pair(w8, kHighCodes), kSixteenth, zhi), d_lo);
                     }
                     tmem_st_16x32cols(taddr_band + stage * (uint32_t)Cfg::kAColsPerStage + 32u * h, v);
                 }

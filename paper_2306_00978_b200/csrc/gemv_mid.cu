@@ -1,5 +1,5 @@
-// The layer for a medium number of tokens (9 .. 32), Sec. 4.2's fused dequantize + product where
-// it is still a bandwidth problem (4 M FLOP per weight byte against a ridge of about 280).
+// The layer for 2 .. 8 tokens on long rows (Sec. 4.2's fused dequantize + product, a bandwidth
+// problem: 4 M FLOP per weight byte against a ridge of about 280).
 //
 // The tensor-memory kernels pay about 9 us per launch (allocation, first copies, split-K hand-over,
 // store drain) and re-read x for every 128-channel tile; the band matrix-vector kernel keeps its
@@ -31,8 +31,8 @@
 //     every block slows to 25.3 us (the memory system gives this access pattern about 4.7 TB/s), the
 //     four crossing blocks still end at 29 us, and the reduce kernel's dependent loads cost 2 us;
 //   * the next chunk's slice of x fetched at the start into a second buffer: 31.0 -> 30.1 us here,
-//     but 42.8 -> 47.3 us on 28672 -> 8192 at 16 tokens (a fifth of the blocks cross there and
-//     start later), 0.2 - 0.6 us slower on the 7B shapes.
+//     but slower on 28672 -> 8192 (a fifth of the blocks cross there and start later) and 0.2 - 0.6 us
+//     slower on the 7B shapes.
 // Stages of 32 KB (4 k-tiles per band) instead of 16 KB: 31.7 -> 31.0 us.
 #include "tcgen05.cuh"
 
@@ -63,7 +63,7 @@ __device__ __forceinline__ void mid_mma(float (&c)[4], uint32_t a0, uint32_t a1,
 }
 
 struct MidLayout {
-    int mtok;            // M rounded up to a multiple of 8 (whole B fragments)
+    int mtok;            // tokens of a B fragment
     int x_off, x_row;    // x slice [mtok][x_row bytes]
     int xg_off;          // fp32 [groups of the chunk][mtok]: 2^-24 times the sums of x
     int par_off;         // two buffers of a unit's parameters: scales [16 bands][groups][16] fp16, then
@@ -72,9 +72,9 @@ struct MidLayout {
     int bar_off, total;
 };
 
-inline MidLayout mid_layout(int M, int group, int chunk_tiles = kMidChunkTiles) {
+inline MidLayout mid_layout(int group, int chunk_tiles = kMidChunkTiles) {
     MidLayout l;
-    l.mtok = ((M + 7) / 8) * 8;
+    l.mtok = 8;
     const int groups = chunk_tiles * 64 / group;
     l.x_off = kMidStages * kMidStageBytes;
     l.x_row = chunk_tiles * 128 + 32;
@@ -87,8 +87,8 @@ inline MidLayout mid_layout(int M, int group, int chunk_tiles = kMidChunkTiles) 
     return l;
 }
 
-// MT = 8-token B fragments per product (tokens rounded up to 8 MT); CT = k-tiles per chunk.
-template <int G, int MT, int CT>
+// CT = k-tiles per chunk; one B fragment of 8 tokens (absent ones are zero).
+template <int G, int CT>
 __global__ void __launch_bounds__(kMidThreads, 1)
 gemv_mid_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap sc_map,
                 const __grid_constant__ CUtensorMap z_map, const __half* __restrict__ x,
@@ -98,7 +98,7 @@ gemv_mid_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant
     __shared__ unsigned int s_abort;
     constexpr int TPG = G / 64;                          // k-tiles per group
     constexpr int GPC = CT / TPG;                        // groups per chunk
-    constexpr int S = kMidStages;
+    constexpr int S = kMidStages, MT = 1;
     const uint32_t sbase = smem_u32(smem);
     // barriers: full[s] at 8s, empty[s] at 64 + 8s, par_full[b] at 128 + 8b, par_empty[b] at 160 + 8b
     const uint32_t bars = sbase + (uint32_t)lay.bar_off;
@@ -184,27 +184,12 @@ gemv_mid_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant
             // of x over each group and token, times 2^-24 (the products carry that factor)
             cur_chunk = c;
             named_barrier_sync(1, kMidMathWarps * 32);              // everybody is done with the old slice
-            // From three token fragments on, all of a thread's loads leave before its first store (one
-            // after the other they are a chain of latencies: 8192 -> 28672 at 24 tokens 55.8 -> 52.3 us;
-            // with one or two fragments a thread has two or four loads, and the registers of a batch
-            // cost the main loop more than the chain: 40.0 -> 41.0 us at 16 tokens).
-            constexpr int FB = MT >= 3 ? 8 : 1;
             const int pieces_per_row = nt * 8, total = lay.mtok * pieces_per_row;
-            for (int i0 = threadIdx.x; i0 < total; i0 += FB * kMidMathWarps * 32) {
-                uint4 v[FB];
-#pragma unroll
-                for (int q = 0; q < FB; ++q) {
-                    const int i = i0 + q * kMidMathWarps * 32;
-                    const int m = i / pieces_per_row, p = i - m * pieces_per_row;
-                    v[q] = make_uint4(0u, 0u, 0u, 0u);
-                    if (i < total && m < M) v[q] = __ldg(reinterpret_cast<const uint4*>(x + (size_t)m * K + (size_t)kt0 * 64) + p);
-                }
-#pragma unroll
-                for (int q = 0; q < FB; ++q) {
-                    const int i = i0 + q * kMidMathWarps * 32;
-                    const int m = i / pieces_per_row, p = i - m * pieces_per_row;
-                    if (i < total) *reinterpret_cast<uint4*>(xs + m * lay.x_row + p * 16) = v[q];
-                }
+            for (int i = threadIdx.x; i < total; i += kMidMathWarps * 32) {
+                const int m = i / pieces_per_row, p = i - m * pieces_per_row;
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if (m < M) v = __ldg(reinterpret_cast<const uint4*>(x + (size_t)m * K + (size_t)kt0 * 64) + p);
+                *reinterpret_cast<uint4*>(xs + m * lay.x_row + p * 16) = v;
             }
             named_barrier_sync(1, kMidMathWarps * 32);
             const int ngr = nt / TPG;
@@ -336,9 +321,8 @@ gemv_mid_reduce_kernel(const float* __restrict__ partial, __half* __restrict__ y
 // k-tiles per chunk for a problem: 16, or 8 where the units (chunks x groups of 16 bands) then fill
 // the blocks' equal shares much better (the slowest block sets the time).  Halving the chunk doubles
 // the partial sums (M / 32 of the weight bytes at 8 k-tiles, written and read back) and the per-unit
-// work (x slice, scales, filling the ring), so the gain has to be large.  Measured at 16 tokens:
-// 4096 -> 4096 10.4 -> 7.9 us and 11008 -> 4096 18.7 -> 16.9 us (shares 0.43 -> 0.86 and
-// 0.59 -> 0.79 full), but 28672 -> 8192 43.7 -> 51.6 us (0.87 -> 0.93; 33.9 -> 39.5 us at 4 tokens).
+// work (x slice, scales, filling the ring), so the gain has to be large: 11008 -> 4096 is a
+// case for 8 (shares 0.59 -> 0.79 full), 28672 -> 8192 is not (0.87 -> 0.93; 33.9 -> 39.5 us at 4 tokens).
 static int mid_chunk_tiles(int N, int K, int sms) {
     const int nbg = (N / 16 + kMidMathWarps - 1) / kMidMathWarps;
     auto efficiency = [&](int ct) {
@@ -355,8 +339,8 @@ size_t gemv_mid_workspace_bytes(int M, int N, int K) {
 }
 bool gemv_mid_applies(int M, int N, int K, int group, int sms) {
     (void)N; (void)sms;
-    if (M < 1 || M > 32 || K > 65536) return false;
-    return mid_layout(M, group).total <= kMidSmem && encode_fn() != nullptr;
+    if (M < 1 || M > 8 || K > 65536) return false;
+    return mid_layout(group).total <= kMidSmem && encode_fn() != nullptr;
 }
 
 cudaError_t launch_gemv_mid(const void* x, const void* qweight, const void* scales, const void* zeros, void* y,
@@ -365,7 +349,7 @@ cudaError_t launch_gemv_mid(const void* x, const void* qweight, const void* scal
     EncodeTiledFn enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
     const int ct = mid_chunk_tiles(N, K, sms);
-    const MidLayout lay = mid_layout(M, group, ct);
+    const MidLayout lay = mid_layout(group, ct);
     const int ng = K / group, gpc = ct * 64 / group;
     const cuuint32_t estr[2] = {1, 1};
     CUtensorMap wmap, scmap, zmap;
@@ -417,35 +401,26 @@ cudaError_t launch_gemv_mid(const void* x, const void* qweight, const void* scal
     cfg.attrs = attr;
     cfg.numAttrs = serialize ? 0 : 1;
     cudaError_t e;
-#define AWQ_MID_LAUNCH2(GG, MTT)                                                                    \
-    do {                                                                                            \
-        if (ct == 16) AWQ_MID_LAUNCH(GG, MTT, 16); else AWQ_MID_LAUNCH(GG, MTT, 8);                 \
-    } while (0)
-#define AWQ_MID_LAUNCH(GG, MTT, CTT)                                                                \
+#define AWQ_MID_LAUNCH(GG, CTT)                                                                     \
     do {                                                                                            \
         static bool done[64] = {};                                                                  \
         int dev = 0;                                                                                \
         e = cudaGetDevice(&dev);                                                                    \
         if (e != cudaSuccess) return e;                                                             \
         if (!done[dev & 63]) {                                                                      \
-            e = cudaFuncSetAttribute(gemv_mid_kernel<GG, MTT, CTT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMidSmem); \
+            e = cudaFuncSetAttribute(gemv_mid_kernel<GG, CTT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMidSmem); \
             if (e != cudaSuccess) return e;                                                         \
             done[dev & 63] = true;                                                                  \
         }                                                                                           \
-        e = cudaLaunchKernelEx(&cfg, gemv_mid_kernel<GG, MTT, CTT>, wmap, scmap, zmap,                   \
+        e = cudaLaunchKernelEx(&cfg, gemv_mid_kernel<GG, CTT>, wmap, scmap, zmap,                   \
                                reinterpret_cast<const __half*>(x), partial, M, N, K, lay, starts, status_word); \
         if (e != cudaSuccess) return e;                                                             \
     } while (0)
-#define AWQ_MID_PICK(GG)                                                                            \
-    do {                                                                                            \
-        if (lay.mtok <= 8) AWQ_MID_LAUNCH2(GG, 1);                                                  \
-        else if (lay.mtok <= 16) AWQ_MID_LAUNCH2(GG, 2);                                            \
-        else if (lay.mtok <= 24) AWQ_MID_LAUNCH2(GG, 3);                                            \
-        else AWQ_MID_LAUNCH2(GG, 4);                                                                \
-    } while (0)
-    if (group == 128) AWQ_MID_PICK(128); else AWQ_MID_PICK(64);
-#undef AWQ_MID_PICK
-#undef AWQ_MID_LAUNCH2
+    if (group == 128) {
+        if (ct == 16) AWQ_MID_LAUNCH(128, 16); else AWQ_MID_LAUNCH(128, 8);
+    } else {
+        if (ct == 16) AWQ_MID_LAUNCH(64, 16); else AWQ_MID_LAUNCH(64, 8);
+    }
 #undef AWQ_MID_LAUNCH
     count_launch();
     e = launch_chunk_reduce(partial, y, chunks, (size_t)M * N, st);

@@ -1,0 +1,71 @@
+"""The chunked tensor-core kernel (awq_linear with 9 .. 64 tokens, and fewer where the output rows are few):
+token tiles, groups, ragged chunks and several matrices in one launch, against the fp64 oracle."""
+import numpy as np
+import pytest
+
+from oracle import awq_oracle as orc
+from paper_2306_00978_b200 import synth
+from tests.util import Case, assert_parity, oracle_packed_to_cuda, to_cuda
+
+pytestmark = pytest.mark.gpu
+
+
+def unrounded_bound(x, W):
+    """Up to 32 tokens nothing is rounded before the output: the products (q - z) * x are exact in the
+    tensor core, their sums, the multiplications by Delta and the sums over groups and chunks are fp32.
+    At most K + 64 roundings of 2^-24 act on partial results bounded by sum |W||x|; the fp16 output adds
+    2^-11 of the value (or 2^-25 in its subnormal range)."""
+    a = np.abs(x.astype(np.float64)) @ np.abs(W).T
+    ref = x.astype(np.float64) @ W.T
+    return ref, 2.0 ** -11 * np.abs(ref) + 2.0 ** -25 + (x.shape[1] + 64) * 2.0 ** -24 * a
+
+
+@pytest.mark.parametrize("N,K,M,G", [
+    (128, 128, 1, 64), (128, 128, 9, 128),        # one slab, half a stage; few rows: also below 9 tokens
+    (256, 384, 16, 128),                           # last stage of the chunk holds one pair of k-blocks
+    (384, 2176, 17, 64),                           # past one chunk of 16 groups, 32-token tile
+    (1152, 4224, 32, 128),                         # several chunks, the last one short
+    (128, 9088, 8, 128),                           # one slab, many chunks
+    (19072, 640, 12, 64),                          # more units than blocks, ranges that cross chunks
+    (2048, 5120, 31, 256),                         # a group stored per 128 columns
+    (512, 1152, 33, 64), (1280, 3200, 64, 128),    # 64-token tile
+])
+def test_linear(N, K, M, G):
+    from paper_2306_00978_b200 import binding
+    case = Case(7000 + N + K + M + G, N, K, M, G, 0.5)
+    packed = oracle_packed_to_cuda(case)
+    y = binding.linear(to_cuda(case.x), *packed, N, K, G)
+    again = binding.linear(to_cuda(case.x), *packed, N, K, G)
+    binding.poll_status()
+    y = y.cpu().numpy()
+    assert np.array_equal(y.view(np.uint16), again.cpu().numpy().view(np.uint16))
+    if M <= 32:
+        ref, bound = unrounded_bound(case.x, orc.dequantize(case.codes, case.zeros, case.scales, G))
+        assert (np.abs(y.astype(np.float64) - ref) <= bound).all()
+    else:
+        assert_parity(y, case.y_ref(), f"N={N} K={K} M={M} G={G}")
+
+
+@pytest.mark.parametrize("widths,K,M,G", [
+    ((256, 128, 384), 1408, 10, 128),              # three matrices, slabs end to end
+    ((1024, 1024), 4096, 32, 64),
+    ((512, 128, 128, 896), 2688, 48, 128),
+])
+def test_several_matrices_and_the_folded_scale(widths, K, M, G):
+    """One launch (and the kernel that adds the chunks) serves all matrices; the scaled call gives bit for
+    bit what the plain one gives on x' = fp16(x * inv_s)."""
+    from paper_2306_00978_b200 import binding
+    cases = [Case(8100 + i, n, K, M, G, 0.5) for i, n in enumerate(widths)]
+    mats = [(*oracle_packed_to_cuda(c), c.N) for c in cases]
+    x_raw = synth.activations(8199, M, K)
+    inv_s = (np.float32(1.0) / cases[0].s).astype(np.float32)
+    x = (x_raw.astype(np.float32) * inv_s[None, :]).astype(np.float16)
+    plain = binding.linear_multi(to_cuda(x), mats, K, G)
+    n0 = binding.launch_count()
+    scaled = binding.linear_multi_scaled(to_cuda(x_raw), to_cuda(inv_s), mats, K, G)
+    assert binding.launch_count() - n0 == 2
+    binding.poll_status()
+    for c, y, ys in zip(cases, plain, scaled):
+        ref = orc.linear(x, orc.dequantize(c.codes, c.zeros, c.scales, G))
+        assert_parity(y.cpu().numpy(), ref, f"N={c.N} of {widths}")
+        assert np.array_equal(y.cpu().numpy().view(np.uint16), ys.cpu().numpy().view(np.uint16))
