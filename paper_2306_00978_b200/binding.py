@@ -35,6 +35,7 @@ class _Problem(ctypes.Structure):
                 ("y", ctypes.c_void_p), ("N", ctypes.c_int)]
 
 _lib = None
+_native = None                 # csrc/native_calls.cpp, connected to the library when that is loaded
 _workspace: dict = {}          # device index -> torch tensor registered with the library
 
 
@@ -44,7 +45,7 @@ class AwqError(RuntimeError):
 
 def lib() -> ctypes.CDLL:
     """Loads the library on first use; raises if it is missing (no CPU or eager fallback)."""
-    global _lib
+    global _lib, _native
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -83,7 +84,13 @@ def lib() -> ctypes.CDLL:
     L.awq_last_cuda_error.restype, L.awq_last_cuda_error.argtypes = ctypes.c_char_p, []
     L.awq_layout_version.restype, L.awq_layout_version.argtypes = i, []
     L.awq_launch_count.restype, L.awq_launch_count.argtypes = ctypes.c_ulonglong, []
-    _lib = L
+    try:
+        from . import _native as native
+    except ImportError as e:
+        raise AwqError(f"_native.so cannot be loaded ({e}): build it with `python -m paper_2306_00978_b200.build`") from e
+    native.connect(*(ctypes.cast(f, ctypes.c_void_p).value for f in (L.awq_workspace_bytes, L.awq_linear_path, L.awq_linear_int3)),
+                   _workspace, _check)
+    _native, _lib = native, L
     return L
 
 
@@ -206,6 +213,10 @@ def linear(x: torch.Tensor, qweight: torch.Tensor, scales: torch.Tensor, zeros: 
            N: int, K: int, group: int, out: Optional[torch.Tensor] = None,
            path: int = PATH_AUTO) -> torch.Tensor:
     """awq_linear / awq_linear_path: y = x . dequant(Wq)^T, x fp16 [M][K] already divided by s."""
+    if _native is not None:                                   # the ordinary call; None: something is out of the ordinary
+        y = _native.linear(x, qweight, scales, zeros, N, K, group, out, path)
+        if y is not None:
+            return y
     M = x.shape[0]
     if x.shape[1] != K:
         raise AwqError("x must be [M][K]")
@@ -286,6 +297,10 @@ def linear_int3(x: torch.Tensor, qweight3: torch.Tensor, scales: torch.Tensor, z
                 scratch: Optional[torch.Tensor] = None) -> torch.Tensor:
     """awq_linear_int3: the layer on the 3-bit storage (`scratch`, N*K/2 bytes, is allocated here
     when the shape needs the expansion and none is given)."""
+    if _native is not None and scratch is None:
+        y = _native.linear_int3(x, qweight3, scales, zeros, N, K, group, out)
+        if y is not None:
+            return y
     M = x.shape[0]
     y = out if out is not None else torch.empty((M, N), dtype=torch.float16, device=x.device)
     ensure_workspace(workspace_bytes(M, N, K, group))
