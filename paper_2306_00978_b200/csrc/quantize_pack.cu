@@ -286,73 +286,166 @@ quantize_pack_tile_kernel(const __half* __restrict__ W, const float* __restrict_
 // error is written to clip[n][group].  The choice decides integer codes downstream, so the error
 // is defined operation by operation: dequant = (q - z) * Delta (one fp32 multiply), e = dequant -
 // w', err += e * e in fp32 over ascending k (no contraction), a NaN error counts as +inf.
-// grid = (ceil(K / 2048), N), block = 256: one row's chunk of w' in shared memory; a thread takes
-// one (group, ratio) pair at a time and walks the group's elements in order.
-constexpr int kClipChunk = 2048;
+// grid = (K / G, N / 64), block = 128: one group of columns of 64 rows.  Its w' stay in shared memory, and
+// a thread takes one (row, two ratios) item at a time and walks the group's elements
+// in order, both ratios in one packed fp32 instruction each (multiply, add and fused multiply-add on two
+// floats round each half as the scalar ones do).  As in the quantizer the quotient's rounded value comes
+// from w' * (1 / Delta) by one fused multiply-add, and the largest distance of a product from its integer
+// decides per (row, ratio) whether that was safe; if not (about 0.05 % of them) the item is redone with
+// the division.  Arithmetic bounds it: 6 packed instructions, two moves and 5 min / max per element and
+// ratio pair, ~4.9 us per ratio on 4096 -> 4096 and ~15 us for the rest.  4096 -> 4096 with 20 ratios 306 us
+// with a scalar division per element and ratio (a row's 2048 columns per 256 threads); packed with the
+// pairs (w', w') kept in shared memory, 11 warps per SM, 153 us; w' kept once, 20 warps, 117 us; with four
+// times four elements unrolled 112 us (192 or 256 threads: 119, 113 us).
+constexpr int kClipRows = 64, kClipThreads = 128;
 struct ClipGrid {
     float r[kMaxClipRatios];
     int n;
 };
 
-template <int G>
-__global__ void __launch_bounds__(256)
-clip_search_kernel(const __half* __restrict__ W, const float* __restrict__ a, float alpha, int mode,
-                   const ClipGrid ratios, float top, float* __restrict__ clip, int N, int K) {
-    constexpr int kGroups = kClipChunk / G;
-    __shared__ float w_sm[kClipChunk];
-    __shared__ float mn_sm[kGroups], mx_sm[kGroups];
-    __shared__ float err_sm[kGroups * kMaxClipRatios];
-    const int n = blockIdx.y, k0 = blockIdx.x * kClipChunk;
-    const int cols = min(kClipChunk, K - k0);              // a multiple of 128: whole groups
-    const int ngr = cols / G;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 d; asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi)); return d;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c)); return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 d; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+    f32x2 d; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d;
+}
 
-    for (int i = threadIdx.x; i < cols; i += 256) {
-        const float sk = channel_scale_one(mode == kAlphaZero ? 1.0f : a[k0 + i], alpha, mode);
-        w_sm[i] = __fmul_rn(__half2float(W[(size_t)n * K + k0 + i]), sk);          // Eq. 3
+// the error of one (row, ratio) as it is defined; wg = its w'
+template <int G>
+__device__ __noinline__ float clip_error_by_division(const float* wg, float d, float z, float top) {
+    float err = 0.0f;
+    for (int k = 0; k < G; ++k) {
+        const float w = wg[k];
+        const float q = fminf(fmaxf(__fadd_rn(rintf(__fdiv_rn(w, d)), z), 0.0f), top);
+        const float e = __fsub_rn(__fmul_rn(__fsub_rn(q, z), d), w);
+        err = __fadd_rn(err, __fmul_rn(e, e));
     }
+    return err;
+}
+
+template <int G>
+struct ClipSmem {
+    static constexpr int kRowFloats = G + 4;                // 16 bytes more, so that rows start on different banks
+    float w[kClipRows * kRowFloats];
+    float err[kClipRows * (kMaxClipRatios + 1)];
+    float2 mm[kClipRows];
+    float s[G];
+};
+
+template <int G>
+__global__ void __launch_bounds__(kClipThreads)
+clip_search_kernel(const __half* __restrict__ W, const float* __restrict__ a, float alpha, int mode,
+                   const __grid_constant__ ClipGrid ratios, float top, float* __restrict__ clip, int N, int K,
+                   bool aligned) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ClipSmem<G>& sm = *reinterpret_cast<ClipSmem<G>*>(smem_raw);
+    constexpr int kPieces = G / 8, kRowFloats = ClipSmem<G>::kRowFloats;
+    const int n0 = blockIdx.y * kClipRows, k0 = blockIdx.x * G;
+    const int tid = threadIdx.x;
+
+    for (int i = tid; i < G; i += kClipThreads) sm.s[i] = channel_scale_one(mode == kAlphaZero ? 1.0f : a[k0 + i], alpha, mode);
     __syncthreads();
-    for (int gi = warp; gi < ngr; gi += 8) {
-        float mn = INFINITY, mx = -INFINITY;
+    // w' = w * s (Eq. 3), eight columns of a row per thread; the row's min / max over its kPieces lanes
+#pragma unroll 4
+    for (int i = tid; i < kClipRows * kPieces; i += kClipThreads) {
+        const int row = i / kPieces, p = i % kPieces;
+        const __half* src = W + (size_t)(n0 + row) * K + k0 + p * 8;
+        __half h[8];
+        if (aligned) {
+            *reinterpret_cast<uint4*>(h) = __ldg(reinterpret_cast<const uint4*>(src));
+        } else {
 #pragma unroll
-        for (int e = 0; e < G / 32; ++e) {
-            const float w = w_sm[gi * G + e * 32 + lane];
-            mn = fminf(mn, w);
-            mx = fmaxf(mx, w);
+            for (int e = 0; e < 8; ++e) h[e] = src[e];
         }
+        float mn = INFINITY, mx = -INFINITY;
+        float* dst = sm.w + row * kRowFloats + p * 8;
+        float wv[8];
 #pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) {
+        for (int e = 0; e < 8; ++e) {
+            wv[e] = __fmul_rn(__half2float(h[e]), sm.s[p * 8 + e]);
+            mn = fminf(mn, wv[e]);
+            mx = fmaxf(mx, wv[e]);
+        }
+        *reinterpret_cast<float4*>(dst) = make_float4(wv[0], wv[1], wv[2], wv[3]);
+        *reinterpret_cast<float4*>(dst + 4) = make_float4(wv[4], wv[5], wv[6], wv[7]);
+#pragma unroll
+        for (int off = kPieces / 2; off >= 1; off >>= 1) {
             mn = fminf(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, off));
             mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
         }
-        if (lane == 0) { mn_sm[gi] = mn; mx_sm[gi] = mx; }
+        if (p == 0) sm.mm[row] = make_float2(mn, mx);
     }
     __syncthreads();
-    const int nr = ratios.n;
-    for (int item = threadIdx.x; item < ngr * nr; item += 256) {
-        const int gi = item / nr, i = item - gi * nr;
-        const float r = ratios.r[i];
-        __half d16;
-        float d, z;
-        group_params(__fmul_rn(mn_sm[gi], r), __fmul_rn(mx_sm[gi], r), top, d16, d, z);
-        const float* wg = w_sm + gi * G;
-        float err = 0.0f;
-#pragma unroll 4
-        for (int k = 0; k < G; ++k) {
-            const float w = wg[k];
-            const float q = fminf(fmaxf(__fadd_rn(rintf(__fdiv_rn(w, d)), z), 0.0f), top);
-            const float e = __fsub_rn(__fmul_rn(__fsub_rn(q, z), d), w);
-            err = __fadd_rn(err, __fmul_rn(e, e));
+    const int nr = ratios.n, np = (nr + 1) / 2;
+    for (int item = tid; item < kClipRows * np; item += kClipThreads) {
+        const int row = item / np, i0 = 2 * (item - row * np), i1 = min(i0 + 1, nr - 1);
+        const float2 mm = sm.mm[row];
+        float d[2], z[2], rd[2], thr[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const float r = ratios.r[j ? i1 : i0];
+            __half d16;
+            group_params(__fmul_rn(mm.x, r), __fmul_rn(mm.y, r), top, d16, d[j], z[j]);
+            rd[j] = __frcp_rn(d[j]);
+            // |w rd - fl(w / d)| <= 2^-23 |w / d| (1 / d and the quotient are rounded once each); the distance
+            // itself is off by at most 2^-26, the threshold by 2^-25
+            const float tmax = __fmul_rn(fmaxf(fabsf(mm.x), fabsf(mm.y)), rd[j]);
+            thr[j] = tmax < 1024.0f ? 0.5f - fmaf(tmax, 1.25e-7f, 6e-8f) : -1.0f;
         }
-        err_sm[gi * kMaxClipRatios + i] = (err != err) ? INFINITY : err;
+        const f32x2 rd2 = pack2(rd[0], rd[1]), d2 = pack2(d[0], d[1]), big = pack2(12582912.0f, 12582912.0f);
+        const float lo0 = z[0] - top, lo1 = z[1] - top, hi0 = z[0], hi1 = z[1];
+        const float* wg = sm.w + row * kRowFloats;
+        f32x2 err = pack2(0.0f, 0.0f);
+        float dm0 = 0.0f, dm1 = 0.0f;
+#pragma unroll 4
+        for (int k = 0; k < G; k += 4) {
+            const float4 w4 = *reinterpret_cast<const float4*>(wg + k);
+            const float we[4] = {w4.x, w4.y, w4.z, w4.w};
+            float da[4], db[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const f32x2 w = pack2(we[e], we[e]);
+                const f32x2 u = fma2(w, rd2, big);               // rounded to an integer in the sum
+                const f32x2 nr2 = sub2(big, u);                  // minus that integer
+                unpack2(fma2(w, rd2, nr2), da[e], db[e]);        // its distance from the product
+                float q0, q1;
+                unpack2(nr2, q0, q1);
+                q0 = fminf(fmaxf(q0, lo0), hi0);                 // z - q
+                q1 = fminf(fmaxf(q1, lo1), hi1);
+                const f32x2 dif = add2(mul2(pack2(q0, q1), d2), w);      // minus the difference: its square is the same
+                err = add2(err, mul2(dif, dif));
+            }
+            dm0 = max3(max3(dm0, fabsf(da[0]), fabsf(da[1])), fabsf(da[2]), fabsf(da[3]));
+            dm1 = max3(max3(dm1, fabsf(db[0]), fabsf(db[1])), fabsf(db[2]), fabsf(db[3]));
+        }
+        float e0, e1;
+        unpack2(err, e0, e1);
+        if (!(dm0 < thr[0])) e0 = clip_error_by_division<G>(wg, d[0], z[0], top);
+        if (!(dm1 < thr[1])) e1 = clip_error_by_division<G>(wg, d[1], z[1], top);
+        float* out = sm.err + row * (kMaxClipRatios + 1);
+        out[i0] = (e0 != e0) ? INFINITY : e0;
+        if (i1 > i0) out[i1] = (e1 != e1) ? INFINITY : e1;
     }
     __syncthreads();
-    if ((int)threadIdx.x < ngr) {
-        const float* e = err_sm + threadIdx.x * kMaxClipRatios;
+    if (tid < kClipRows) {
+        const float* e = sm.err + tid * (kMaxClipRatios + 1);
         int best = 0;
         for (int i = 1; i < nr; ++i)
             if (e[i] < e[best]) best = i;
-        clip[(size_t)n * (K / G) + k0 / G + threadIdx.x] = ratios.r[best];
+        clip[(size_t)(n0 + tid) * (K / G) + blockIdx.x] = ratios.r[best];
     }
 }
 
@@ -422,21 +515,35 @@ cudaError_t launch_quantize_pack(const __half* W, const float* a, float alpha, i
     return cudaGetLastError();
 }
 
+template <int G>
+static cudaError_t launch_clip(const __half* W, const float* a, float alpha, int mode, const ClipGrid& ratios, float top,
+                               float* clip, int N, int K, bool aligned, cudaStream_t st) {
+    static bool done[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (!done[dev & 63]) {
+        e = cudaFuncSetAttribute(clip_search_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClipSmem<G>));
+        if (e != cudaSuccess) return e;
+        done[dev & 63] = true;
+    }
+    clip_search_kernel<G><<<dim3(K / G, N / kClipRows), kClipThreads, sizeof(ClipSmem<G>), st>>>(
+        W, a, alpha, mode, ratios, top, clip, N, K, aligned);
+    count_launch();
+    return cudaGetLastError();
+}
+
 cudaError_t launch_clip_search(const __half* W, const float* a, float alpha, int group, int bits,
                                const float* ratios, int n_ratios, float* clip, int N, int K,
                                cudaStream_t st) {
     ClipGrid grid_r;
     grid_r.n = n_ratios;
     for (int i = 0; i < kMaxClipRatios; ++i) grid_r.r[i] = i < n_ratios ? ratios[i] : 1.0f;
-    const dim3 grid((K + kClipChunk - 1) / kClipChunk, N);
     const int mode = (int)alpha_mode(alpha);
     const float top = (float)((1 << bits) - 1);
-    if (group == 128)
-        clip_search_kernel<128><<<grid, 256, 0, st>>>(W, a, alpha, mode, grid_r, top, clip, N, K);
-    else
-        clip_search_kernel<64><<<grid, 256, 0, st>>>(W, a, alpha, mode, grid_r, top, clip, N, K);
-    count_launch();
-    return cudaGetLastError();
+    const bool aligned = (reinterpret_cast<uintptr_t>(W) & 15u) == 0;   // rows are multiples of 256 bytes
+    return group == 128 ? launch_clip<128>(W, a, alpha, mode, grid_r, top, clip, N, K, aligned, st)
+                        : launch_clip<64>(W, a, alpha, mode, grid_r, top, clip, N, K, aligned, st);
 }
 
 cudaError_t launch_unpack(const uint32_t* qweight, const __half* scales, const uint8_t* zeros,

@@ -118,3 +118,26 @@ def test_symmetric_quantizer_bit_exact_and_layer_parity(N, K, G, bits, clipped):
             y = binding.linear(to_cuda(x), *got, N, K, G)
             binding.poll_status()
             assert_parity(y.cpu().numpy(), orc.linear(x, Wdq), f"symmetric N={N} K={K} M={M}")
+
+
+@pytest.mark.parametrize("n_ratios", [1, 2, 3, 31, 32])
+def test_clip_search_ratio_counts_special_weights_and_alignment(n_ratios):
+    """Odd and even ratio lists (the kernel takes ratios in pairs), weights on the ties of the grid (the
+    quotient decides, not the product), zero, huge and infinite groups, and W at an address that only 2-byte
+    elements allow: the same ratios as the oracle's, bit for bit."""
+    import torch
+    from paper_2306_00978_b200 import binding
+    N, K, G = 128, 384, 128
+    rng = np.random.default_rng(n_ratios)
+    W = (rng.integers(-16, 17, size=(N, K)) * 0.5 / 16).astype(np.float16)      # many quotients at k + 1/2
+    W[3, :128] = 0.0
+    W[4, 128:256] = 6.0e4
+    W[5, 5] = np.inf
+    W[6, 300] = -6.0e4
+    ratios = [float(r) for r in np.linspace(1.0, 0.3, n_ratios).astype(np.float32)]
+    want = orc.search_clip(W, np.ones(K, np.float32), G, ratios, bits=4)
+    for offset in (0, 1):
+        buf = torch.zeros(N * K + 8, dtype=torch.float16, device="cuda")
+        buf[offset:offset + N * K] = to_cuda(W).reshape(-1)
+        got = binding.search_clip(buf[offset:offset + N * K].view(N, K), None, 0.0, G, ratios, bits=4)
+        assert np.array_equal(got.cpu().numpy().view(np.uint32), want.view(np.uint32)), offset
