@@ -293,14 +293,16 @@ quantize_pack_tile_kernel(const __half* __restrict__ W, const float* __restrict_
 // from w' * (1 / Delta) by one fused multiply-add, and the largest distance of a product from its integer
 // decides per (row, ratio) whether that was safe; if not (about 0.05 % of them) the item is redone with
 // the division.  Arithmetic bounds it: 6 packed instructions, two moves and 5 min / max per element and
-// ratio pair, ~4.9 us per ratio on 4096 -> 4096 and ~15 us for the rest.  4096 -> 4096 with 20 ratios 306 us
+// ratio pair, ~5.6 us per ratio on 4096 -> 4096 and ~15 us for the rest.  4096 -> 4096 with 20 ratios 306 us
 // with a scalar division per element and ratio (a row's 2048 columns per 256 threads); packed with the
 // pairs (w', w') kept in shared memory, 11 warps per SM, 153 us; w' kept once, 20 warps, 117 us; with four
-// times four elements unrolled 112 us (192 or 256 threads: 119, 113 us).
+// times four elements unrolled 112 us (192 or 256 threads: 119, 113 us); with the products kept from
+// contraction (mul2) 126 us.
 constexpr int kClipRows = 64, kClipThreads = 128;
 struct ClipGrid {
     float r[kMaxClipRatios];
     int n;
+    float minus_zero;                                       // -0.0f, see mul2
 };
 
 typedef unsigned long long f32x2;
@@ -313,9 +315,10 @@ __device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
 __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
     f32x2 d; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c)); return d;
 }
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-    f32x2 d; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d;
-}
+// The rounded product, as a * b + (-0.0) with the zero in a kernel argument: the assembler contracts
+// mul.rn.f32x2 with an add.rn.f32x2 behind it into one fused instruction (unlike the scalar forms with
+// explicit rounding), which the errors here must not be.
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b, f32x2 minus_zero) { return fma2(a, b, minus_zero); }
 __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
     f32x2 d; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d;
 }
@@ -406,6 +409,7 @@ clip_search_kernel(const __half* __restrict__ W, const float* __restrict__ a, fl
             thr[j] = tmax < 1024.0f ? 0.5f - fmaf(tmax, 1.25e-7f, 6e-8f) : -1.0f;
         }
         const f32x2 rd2 = pack2(rd[0], rd[1]), d2 = pack2(d[0], d[1]), big = pack2(12582912.0f, 12582912.0f);
+        const f32x2 mz = pack2(ratios.minus_zero, ratios.minus_zero);
         const float lo0 = z[0] - top, lo1 = z[1] - top, hi0 = z[0], hi1 = z[1];
         const float* wg = sm.w + row * kRowFloats;
         f32x2 err = pack2(0.0f, 0.0f);
@@ -425,8 +429,8 @@ clip_search_kernel(const __half* __restrict__ W, const float* __restrict__ a, fl
                 unpack2(nr2, q0, q1);
                 q0 = fminf(fmaxf(q0, lo0), hi0);                 // z - q
                 q1 = fminf(fmaxf(q1, lo1), hi1);
-                const f32x2 dif = add2(mul2(pack2(q0, q1), d2), w);      // minus the difference: its square is the same
-                err = add2(err, mul2(dif, dif));
+                const f32x2 dif = add2(mul2(pack2(q0, q1), d2, mz), w);  // minus the difference: its square is the same
+                err = add2(err, mul2(dif, dif, mz));
             }
             dm0 = max3(max3(dm0, fabsf(da[0]), fabsf(da[1])), fabsf(da[2]), fabsf(da[3]));
             dm1 = max3(max3(dm1, fabsf(db[0]), fabsf(db[1])), fabsf(db[2]), fabsf(db[3]));
@@ -538,6 +542,7 @@ cudaError_t launch_clip_search(const __half* W, const float* a, float alpha, int
                                cudaStream_t st) {
     ClipGrid grid_r;
     grid_r.n = n_ratios;
+    grid_r.minus_zero = -0.0f;
     for (int i = 0; i < kMaxClipRatios; ++i) grid_r.r[i] = i < n_ratios ? ratios[i] : 1.0f;
     const int mode = (int)alpha_mode(alpha);
     const float top = (float)((1 << bits) - 1);

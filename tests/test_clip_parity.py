@@ -141,3 +141,17 @@ def test_clip_search_ratio_counts_special_weights_and_alignment(n_ratios):
         buf[offset:offset + N * K] = to_cuda(W).reshape(-1)
         got = binding.search_clip(buf[offset:offset + N * K].view(N, K), None, 0.0, G, ratios, bits=4)
         assert np.array_equal(got.cpu().numpy().view(np.uint32), want.view(np.uint32)), offset
+
+
+def test_clip_search_errors_are_not_contracted():
+    """err += e * e is a multiplication and an addition, each rounded.  Of 2^20 seeded groups these two are
+    the ones where a fused multiply-add in its place moves the least error to another ratio."""
+    import torch
+    from paper_2306_00978_b200 import binding
+    rows = (np.random.default_rng(2026).standard_normal((1 << 20, 64)) * 0.02).astype(np.float16)[[51450, 699600]]
+    W = np.tile(np.concatenate([rows, rows[::-1]], axis=1), (64, 1))                       # [128][128]: both orders
+    a = np.tile((np.random.default_rng(7).random(64) + 0.5).astype(np.float32), 2)
+    ratios = [float(r) for r in np.linspace(1.0, 0.5, 32).astype(np.float32)]
+    want = orc.search_clip(W, a, 64, ratios, bits=3)
+    got = binding.search_clip(to_cuda(W), to_cuda(a), 1.0, 64, ratios, bits=3)
+    assert np.array_equal(got.cpu().numpy().view(np.uint32), want.view(np.uint32))
