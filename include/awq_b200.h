@@ -78,9 +78,8 @@ typedef enum AwqPath {
     AWQ_PATH_GEMV = 1,          /* fused dequant matrix-vector kernel, M <= 16: band kernel when
                                    M <= 8 and N/16 is not much below the SM count, else split-K */
     AWQ_PATH_GEMM = 2,          /* tcgen05 tensor-core kernel, any M >= 1: pairs of SMs
-                                   (cta_group::2, 256 channels x 256 tokens per tile) when N is a
-                                   multiple of 256 and M > 128 (M > 64 from N = 8192, M >= 32 from
-                                   N = 16384), else one SM per tile */
+                                   (cta_group::2, 256 channels x 64 .. 256 tokens per tile) when
+                                   M > 64 (M >= 32 from N = 16384), else one SM per tile */
     AWQ_PATH_GEMV_SPLITK = 3,   /* the split-K matrix-vector kernel, M <= 16 */
     AWQ_PATH_GEMM_1SM = 4,      /* the tensor-core kernel with one SM per tile, any M >= 1 */
     AWQ_PATH_GEMV_MID = 5,      /* M <= 8: the chunked matrix-vector kernel: work units of 16 bands
@@ -337,9 +336,9 @@ int awq_search_alpha(const void* W, const float* act_mean_abs, const void* X, in
  *    splits, fp32 partial sums added in split order by whichever SM finishes a tile last), which
  *    keeps all SMs busy when N / 128 is below the SM count;
  *  - the SM-pair prefill kernel (see AWQ_PATH_GEMM) cuts the tiles' K loops into equal ranges over
- *    all SM pairs (stream-K) and sums split tiles in a fixed order; without a workspace whole tiles
- *    go round-robin (same result up to fp32 summation order, slower when the tile count is not a
- *    multiple of the pair count).
+ *    all SM pairs (stream-K) where that pays and sums split tiles in a fixed order; without a workspace whole
+ *    tiles go round-robin (same result up to fp32 summation order, slower when the tile count is not
+ *    a multiple of the pair count).
  * awq_set_workspace: registers caller-owned device memory for the current device; the first
  * 4096 bytes are cleared with a synchronous cudaMemset.  Pass (NULL, 0) to unregister.
  * The memory must stay valid until it is unregistered or replaced. */

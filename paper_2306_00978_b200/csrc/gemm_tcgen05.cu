@@ -474,9 +474,9 @@ cudaError_t launch_gemm(const void* x, const void* qweight, const void* scales, 
     if (e != cudaSuccess) return e;
     CUtensorMap map, wmap;
     if (path_pair_allowed && gemm_pair_applies(M, N)) {
-        if (!make_x_map(&map, 128) || !make_w_map(&wmap, 256)) return cudaErrorInvalidValue;
+        if (!make_w_map(&wmap, 256)) return cudaErrorInvalidValue;
         bool launched = false;
-        e = launch_gemm_pair(map, wmap, ymap, scales, zeros, M, N, K, group, workspace, workspace_bytes,
+        e = launch_gemm_pair(x, wmap, ymap, scales, zeros, M, N, K, group, workspace, workspace_bytes,
                              status_word, sms, st, &launched);
         if (e != cudaSuccess || launched) return e;
     }
@@ -495,8 +495,8 @@ cudaError_t launch_gemm(const void* x, const void* qweight, const void* scales, 
 }
 
 size_t gemm_workspace_bytes(int M, int N, int sms) {
+    if (M > 128 && N % 256 != 0) return 0;       // (stream-K is used here too if the caller's workspace happens to suffice)
     if (gemm_pair_applies(M, N)) return gemm_pair_workspace_bytes(sms);
-    if (M > 128) return 0;
     // split-K of the one-SM kernel: the most it can use for this M and N (any K)
     const int bn = M > 64 ? 128 : M > 32 ? 64 : 32;
     const int tiles = N / 128;

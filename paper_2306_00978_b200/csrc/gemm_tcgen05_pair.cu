@@ -1,27 +1,29 @@
 // Prefill path of the layer for large token counts (Sec. 4.2: fused dequantize + matrix-matrix
 // product): the dataflow of gemm_tcgen05.cu, run by PAIRS of thread blocks (a cluster of two SMs)
-// that issue one tcgen05.mma.cta_group::2 of M = 256 output channels x N = 256 tokens.
+// that issue one tcgen05.mma.cta_group::2 of M = 256 output channels x N = 64 .. 256 tokens.
 //
 // Why pairs, and why 128-channel stages.  With one block per 128 x 256 tile every 64-wide k-block
-// moves 72 KB through shared memory and costs the single MMA-issuing thread two barrier polls,
-// four MMAs and a commit; measured, that thread (not the tensor pipe, which sustains one
-// 128 x 256 x 16 MMA per 128 cycles) set the pace at ~770 cycles per k-block.  In a pair each
-// block stages only its half of the tokens (the tensor cores of both SMs read both halves), and
-// a stage covers K = 128, so the polls and commits are paid once per eight MMAs: ~1120 cycles per
-// stage against the pipe's 1024.  (Both figures with the issuing loop inside `if (lane == 0)`; converged
-// loops with one elected lane, see tcgen05.cuh, took 13824 -> 5120 at 2048 tokens from 210 to 204 us and
-// 4096 -> 11008 at 8192 tokens from 597 to 587 us.)
+// moves 72 KB through shared memory and costs the MMA-issuing warp two barrier polls, four MMAs and a
+// commit: it, not the tensor pipe (one 128 x 256 x 16 MMA per 128 cycles), set the pace.  In a pair
+// each block stages only its half of the tokens (the tensor cores of both SMs read both halves), and
+// a stage covers K = 128, so the polls and commits are paid once per eight MMAs.
+// Tiles are 64, 128, 192 or 256 tokens wide (choose_tile).  At 256 a stage takes ~1070 cycles against the
+// pipe's 1024.  Narrower tiles are bound by the dequantizers (~620 cycles a stage, whatever the
+// width up to 128: the conversion's instructions and the tensor-memory stores) once nothing waits: sixteen
+// dequantizer warps, and a ring of up to eight stages in shared memory behind the four whose A is in tensor
+// memory (128 tokens, one tile per pair, 108 stages: 55 us with four stages, 42 us with eight; 256 tokens gain
+// nothing from a fifth).
 //
 // Block r of a pair (r = rank in the cluster) owns
 //   - A: output channels 128 r .. 128 r + 127 of the 256-channel slab, dequantized by its own
-//        warps 8-15 into its own tensor memory (64 columns per stage),
-//   - B: tokens 128 r .. 128 r + 127 of the 256-token tile in its own shared memory (two 64-wide
-//        128-byte-swizzled halves per stage),
-//   - D: the fp32 accumulator rows of its 128 channels x all 256 tokens in its own tensor memory,
-//        drained by its own epilogue warps (4-7: tokens 0..127, 16-19: tokens 128..255).
+//        warps into its own tensor memory (64 columns per stage),
+//   - B: its half of the tile's tokens in its own shared memory (two 64-wide 128-byte-swizzled
+//        halves per stage),
+//   - D: the fp32 accumulator rows of its 128 channels x all tokens in its own tensor memory (two of them
+//        up to 128 tokens), drained by its own epilogue warps (half of the tokens each four).
 // Only the leader (rank 0) issues MMAs.  Barriers that the leader's MMA thread waits on live in the
 // leader's shared memory: x_full (both blocks' x copies complete their bytes there), a_full (16
-// dequantizer warps, 8 of them arriving remotely), acc_empty (16 epilogue warps).  The MMA
+// dequantizer warps, 8 of each block), acc_empty (16 epilogue warps).  The MMA
 // thread's tcgen05.commit arrives on "empty" and "acc_full" of BOTH blocks.
 //
 // Tile balance: with a workspace, and when whole tiles would leave pairs idle for long, the tiles'
@@ -37,23 +39,29 @@ namespace awq {
 
 namespace {
 
-constexpr int kPairThreads = 640;                // warps: 0 copy, 1 MMA, 4-7 and 16-19 epilogue, 8-15 dequant
-constexpr int kPairTokens = 256;                 // tokens per tile (N of the MMA)
-constexpr int kHalfTokens = 128;                 // tokens staged by each block
-
 constexpr int kStageK = 128;                     // input channels per pipeline stage (two k-tiles)
 
-struct PairCfg {
-    static constexpr int kXHalfBytes = kHalfTokens * kBK * 2;                // 16 KB: one 64-wide swizzled half
-    static constexpr int kXTileBytes = 2 * kXHalfBytes;                      // 128 tokens x 128 channels
+// BN = tokens per tile (N of the MMA); each block stages half of them
+template <int BN> struct PairCfg {
+    // 256 tokens: a stage's products take 1024 cycles, eight dequantizer warps (one per band) keep up; with
+    // fewer tokens sixteen, every second stage each, so that a warp's chain of latencies spans two stages
+    static constexpr int kDequantWarps = BN >= 256 ? 8 : 16;
+    static constexpr int kEpilogueWarp1 = 8 + kDequantWarps;                 // first warp of the second epilogue half
+    static constexpr int kThreads = (kEpilogueWarp1 + 4) * 32;               // warps: 0 copy, 1 MMA, 4-7 epilogue, 8.. dequant, 4 epilogue
+    static constexpr int kHalf = BN / 2;                                     // tokens staged by each block, and per epilogue half
+    static constexpr int kXHalfBytes = kHalf * kBK * 2;                      // one 64-wide swizzled half
+    static constexpr int kXTileBytes = 2 * kXHalfBytes;                      // BN / 2 tokens x 128 channels
     static constexpr int kWBytes = 2 * kTileBytes;                           // 8 bands x 2 k-tiles x 512 bytes
-    static constexpr int kStageBytes = kXTileBytes + kWBytes;                // 40 KB
+    static constexpr int kStageBytes = kXTileBytes + kWBytes;                // 40 KB at 256 tokens
     static constexpr int kOutBytes = 8 * 2 * 2048;                           // 8 epilogue warps x 2 staging blocks
-    static constexpr int kStages = 4;
-    static constexpr int kAColumn0 = kPairTokens;                            // tensor memory: accumulator, then A
+    static constexpr int kStages = BN >= 256 ? 4 : BN >= 192 ? 6 : 8;        // what shared memory holds
+    static constexpr int kSlots = 4;                                         // stages whose A is in tensor memory
+    static constexpr uint32_t kNumAcc = BN <= 128 ? 2 : 1;                   // accumulators in tensor memory
+    static constexpr int kAColumn0 = 256;                                    // tensor memory: accumulators, then A
     static constexpr int kAColsPerStage = 64;                                // 8 columns per K = 16
-    static constexpr int kTmemCols = 512;                                    // 256 + 4 x 64
+    static constexpr int kTmemCols = 512;                                    // 256 + kSlots x 64
     static constexpr int kSmemBytes = kStages * kStageBytes + kOutBytes + 1024 /*align*/ + 512 /*barriers*/;
+    static constexpr int kPartialFloats = 256 * BN;                          // one pair's fp32 accumulator
 };
 
 // ---------------------------------------------------------------- cluster-scope PTX wrappers
@@ -102,8 +110,8 @@ __device__ __forceinline__ void umma_pair_commit(uint32_t cluster_bar) {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                  ::"r"(cluster_bar) : "memory");
 }
-__host__ __device__ constexpr uint32_t instr_desc_pair() {     // D fp32, A/B fp16 K-major, M = 256, N = 256
-    return (1u << 4) | ((uint32_t)(kPairTokens >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+__host__ __device__ constexpr uint32_t instr_desc_pair(int bn) {     // D fp32, A/B fp16 K-major, M = 256, N = bn
+    return (1u << 4) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
 }
 
 // Work of one pair: a sequence of pieces (tile, stages k0 .. k1-1 of the tile's K / 128).
@@ -142,18 +150,17 @@ __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
     return v;
 }
 
-constexpr int kPartialFloats = 256 * kPairTokens;    // one pair's fp32 accumulator (256 KB)
-
 // ------------------------------------------------------------------------- the kernel
-template <int G>
-__global__ void __launch_bounds__(kPairThreads, 1)
+template <int G, int BN>
+__global__ void __launch_bounds__(PairCfg<BN>::kThreads, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap w_map,
                  const __grid_constant__ CUtensorMap y_map,
                  const __half* __restrict__ scales, const unsigned char* __restrict__ zeros,
                  int M, int N, int K, unsigned int* status_word,
                  float* partials, unsigned int* flags) {
-    using Cfg = PairCfg;
-    constexpr int S = Cfg::kStages;
+    using Cfg = PairCfg<BN>;
+    constexpr int S = Cfg::kStages, SL = Cfg::kSlots;
+    constexpr uint32_t NACC = Cfg::kNumAcc;
     constexpr int GPS = kStageK / G;                 // quantization groups per stage: 1 or 2
     extern __shared__ unsigned char smem_dyn[];
     __shared__ unsigned int s_abort;
@@ -162,22 +169,22 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     const uint32_t dyn = smem_u32(smem_dyn);
     const uint32_t base = (dyn + 1023u) & ~1023u;                    // 1024-byte aligned stage ring
     unsigned char* base_ptr = smem_dyn + (base - dyn);
-    // stage layout: [x, k-half 0 (128 tokens x 64) | x, k-half 1 | packed weights (8 bands x 1 KB)]
+    // stage layout: [x, k-half 0 (BN / 2 tokens x 64) | x, k-half 1 | packed weights (8 bands x 1 KB)]
     auto x_addr = [&](int s) { return base + (uint32_t)s * Cfg::kStageBytes; };
     auto w_ptr = [&](int s) { return base_ptr + (size_t)s * Cfg::kStageBytes + Cfg::kXTileBytes; };
     const uint32_t out_base = base + (uint32_t)S * Cfg::kStageBytes;
     const uint32_t bars = out_base + (uint32_t)Cfg::kOutBytes;
     auto w_full = [&](int s) { return bars + 8u * (uint32_t)s; };               // own weights landed
     auto x_full = [&](int s) { return bars + 8u * (uint32_t)(S + s); };         // leader: both blocks' x landed
-    auto a_full = [&](int s) { return bars + 8u * (uint32_t)(2 * S + s); };     // leader: both blocks' A stored
-    auto empty = [&](int s) { return bars + 8u * (uint32_t)(3 * S + s); };      // stage free again
-    const uint32_t acc_full = bars + 8u * (uint32_t)(4 * S);                    // accumulator complete
-    const uint32_t acc_empty = bars + 8u * (uint32_t)(4 * S + 1);               // leader: accumulator drained
+    auto empty = [&](int s) { return bars + 8u * (uint32_t)(2 * S + s); };      // stage free again: its products are done
+    auto a_full = [&](int s) { return bars + 8u * (uint32_t)(3 * S + s); };     // leader: both blocks' A stored (per slot)
+    auto acc_full = [&](uint32_t b) { return bars + 8u * ((uint32_t)(3 * S + SL) + b); };        // accumulator complete
+    auto acc_empty = [&](uint32_t b) { return bars + 8u * ((uint32_t)(3 * S + SL + 2) + b); };   // leader: accumulator drained
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
-    const int m_tiles = (M + kPairTokens - 1) / kPairTokens;
-    const int total_tiles = (N / 256) * m_tiles;
+    const int m_tiles = (M + BN - 1) / BN;
+    const int total_tiles = ((N + 255) / 256) * m_tiles;     // an odd last slab of 128 channels pairs with an absent one
     const int cluster = (int)cluster_id_x(), num_clusters = (int)num_clusters_x();
     const int nks = K / kStageK;                     // stages per tile
     const long long total_stages = (long long)total_tiles * nks;
@@ -191,10 +198,10 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     if (threadIdx.x == 0) {
         s_abort = 0u;
         for (int s = 0; s < S; ++s) {
-            mbar_init(w_full(s), 1); mbar_init(x_full(s), 1); mbar_init(a_full(s), 16); mbar_init(empty(s), 1);
+            mbar_init(w_full(s), 1); mbar_init(x_full(s), 1); mbar_init(empty(s), 1);
         }
-        mbar_init(acc_full, 1);
-        mbar_init(acc_empty, 16);
+        for (int s = 0; s < SL; ++s) mbar_init(a_full(s), 16);
+        for (uint32_t b = 0; b < NACC; ++b) { mbar_init(acc_full(b), 1); mbar_init(acc_empty(b), 16); }
         mbar_fence_init();
     }
     if (warp == 1) {
@@ -218,7 +225,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         bool ok = true;
         while (ok && pieces.next(tile, k0, k1)) {
             const int slab = (tile / m_tiles) * 2 + (int)rank;              // 128-channel slab of this block
-            const int tok0 = (tile % m_tiles) * kPairTokens + (int)rank * kHalfTokens;
+            const int tok0 = (tile % m_tiles) * BN + (int)rank * Cfg::kHalf;
             for (int ks = k0; ks < k1; ++ks) {
                 if (!mbar_wait_warp(empty(stage), phase ^ 1u, ctl)) { ok = false; break; }
                 if (lead) {
@@ -252,31 +259,31 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         // ------------------------------------------------- MMA issuer (leader block only)
         if (rank == 0) {
             const bool lead = elect_one();
-            constexpr uint32_t idesc = instr_desc_pair();
-            const uint32_t peer_acc_full = map_to_rank(acc_full, 1);
+            constexpr uint32_t idesc = instr_desc_pair(BN);
+            const uint32_t peer_acc_full0 = map_to_rank(acc_full(0), 1);
             const uint32_t peer_empty0 = map_to_rank(empty(0), 1);
-            uint32_t stage = 0, phase = 0;
-            int local = 0;
+            uint32_t stage = 0, phase = 0, slot = 0, slot_phase = 0, acc = 0, acc_phase = 0;
             bool ok = true;
-            for (; ok && pieces.next(tile, k0, k1); ++local) {
-                if (!mbar_wait_warp(acc_empty, ((uint32_t)local & 1u) ^ 1u, ctl)) { ok = false; break; }
+            while (ok && pieces.next(tile, k0, k1)) {
+                if (!mbar_wait_warp(acc_empty(acc), acc_phase ^ 1u, ctl)) { ok = false; break; }
                 tc_fence_after();
+                const uint32_t d_tmem = tmem_base + acc * (uint32_t)BN;
                 for (int ks = k0; ks < k1; ++ks) {
                     // both barriers are normally complete already: poll them together
-                    const bool xr = mbar_try_wait(x_full(stage), phase), ar = mbar_try_wait(a_full(stage), phase);
+                    const bool xr = mbar_try_wait(x_full(stage), phase), ar = mbar_try_wait(a_full(slot), slot_phase);
                     if (!__all_sync(0xFFFFFFFFu, xr && ar) &&
-                        (!mbar_wait_warp(x_full(stage), phase, ctl) || !mbar_wait_warp(a_full(stage), phase, ctl))) {
+                        (!mbar_wait_warp(x_full(stage), phase, ctl) || !mbar_wait_warp(a_full(slot), slot_phase, ctl))) {
                         ok = false; break;
                     }
                     tc_fence_after();
-                    const uint32_t a_tmem = tmem_base + (uint32_t)(Cfg::kAColumn0 + stage * Cfg::kAColsPerStage);
+                    const uint32_t a_tmem = tmem_base + (uint32_t)(Cfg::kAColumn0 + slot * Cfg::kAColsPerStage);
                     const uint64_t bdesc = smem_desc_sw128(x_addr(stage));
                     if (lead) {
 #pragma unroll
                         for (int k = 0; k < kStageK / 16; ++k) {
-                            // A: 8 columns per K = 16; B: 32 bytes per K = 16 inside a 64-wide half, halves 16 KB apart
+                            // A: 8 columns per K = 16; B: 32 bytes per K = 16 inside a 64-wide half
                             const uint64_t boff = (uint64_t)(((k >> 2) * Cfg::kXHalfBytes + (k & 3) * 32) >> 4);
-                            umma_pair_f16_a_tmem(tmem_base, a_tmem + (uint32_t)(8 * k), bdesc + boff, idesc,
+                            umma_pair_f16_a_tmem(d_tmem, a_tmem + (uint32_t)(8 * k), bdesc + boff, idesc,
                                                  (ks > k0 || k > 0) ? 1u : 0u);
                         }
                         umma_pair_commit(empty(stage));
@@ -284,46 +291,55 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                     }
                     __syncwarp();
                     if (++stage == S) { stage = 0; phase ^= 1u; }
+                    if (++slot == SL) { slot = 0; slot_phase ^= 1u; }
                 }
-                if (ok && lead) { umma_pair_commit(acc_full); umma_pair_commit(peer_acc_full); }
+                if (ok && lead) { umma_pair_commit(acc_full(acc)); umma_pair_commit(peer_acc_full0 + 8u * acc); }
                 __syncwarp();
+                if (++acc == NACC) { acc = 0; acc_phase ^= 1u; }
             }
         }
-    } else if (warp >= 8 && warp < 16) {
+    } else if (warp >= 8 && warp < Cfg::kEpilogueWarp1) {
         // -------------------------------------------------------------- dequantizers
-        // one warp per 16-row band of this block's 128 channels, two k-tiles per stage; see
-        // gemm_tcgen05.cu for the piece <-> register layout
-        const int wi = warp - 8, quad = wi & 3, hsel = wi >> 2;
+        // a warp takes a 16-row band of this block's 128 channels, two k-tiles per stage - every stage, or
+        // every STEPth of those of all its pieces end to end; see gemm_tcgen05.cu for the piece <-> register layout
+        constexpr int STEP = Cfg::kDequantWarps / 8;
+        const int wi = warp - 8, quad = wi & 3, hsel = (wi >> 2) & 1;
         const int band = 2 * quad + hsel;
         const int g = lane >> 2;
-        const int ng = K / G;
+        const int ng = K / G, bands = N / 16;
         const uint32_t taddr_band = tmem_base + ((uint32_t)(quad * 32 + hsel * 16) << 16) + (uint32_t)Cfg::kAColumn0;
         const uint32_t leader_a_full0 = map_to_rank(a_full(0), 0);
-        uint32_t stage = 0, phase = 0;
+        int first = wi >> 3;                             // this warp's first stage inside the next piece
+        uint32_t stage = (uint32_t)first, phase = 0, slot = (uint32_t)first;
+        // the slot's previous use was kSlots stages ago: its products are done when that stage is empty
+        uint32_t old = (uint32_t)(first + S - SL), old_phase = 1u;     // (both below S: first <= 1, and 0 where S = SL)
+        static_assert(S > SL || STEP == 1, "stage index of the slot's previous use");
         bool ok = true;
         while (ok && pieces.next(tile, k0, k1)) {
-            const int slab = (tile / m_tiles) * 2 + (int)rank;
+            // (an absent slab's warps read the last band's parameters for rows that nobody keeps)
+            const int gband = min(((tile / m_tiles) * 2 + (int)rank) * 8 + band, bands - 1);
             // this lane's rows' parameters: scales [band][group][16], zero bytes [band pair][group][16]
-            const unsigned short* sc_g = reinterpret_cast<const unsigned short*>(scales) +
-                                         (size_t)(slab * 8 + band) * ng * 16 + g;
-            const unsigned char* z_g = zeros + (size_t)(slab * 4 + (band >> 1)) * ng * 16 + (band & 1) * 8 + g;
-            // parameters of the current stage's groups and of the next stage's (fetched one stage ahead)
+            const unsigned short* sc_g = reinterpret_cast<const unsigned short*>(scales) + (size_t)gband * ng * 16 + g;
+            const unsigned char* z_g = zeros + (size_t)(gband >> 1) * ng * 16 + (gband & 1) * 8 + g;
+            // parameters of the current stage's groups and of this warp's next stage's (fetched one ahead)
             uint32_t du[GPS], dl[GPS], zb[GPS], du1[GPS], dl1[GPS], zb1[GPS];
 #pragma unroll
             for (int q = 0; q < GPS; ++q) {
-                const int g0 = k0 * GPS + q;
+                const int g0 = min((k0 + first) * GPS + q, ng - 1);
                 du1[q] = __ldg(sc_g + g0 * 16); dl1[q] = __ldg(sc_g + g0 * 16 + 8); zb1[q] = __ldg(z_g + g0 * 16);
             }
-            for (int ks = k0; ks < k1; ++ks) {
+            int ks = k0 + first;
+            for (; ks < k1; ks += STEP) {
 #pragma unroll
                 for (int q = 0; q < GPS; ++q) {
                     du[q] = du1[q]; dl[q] = dl1[q]; zb[q] = zb1[q];
-                    const int gn = min((ks + 1) * GPS + q, ng - 1);
+                    const int gn = min((ks + STEP) * GPS + q, ng - 1);
                     du1[q] = __ldg(sc_g + gn * 16); dl1[q] = __ldg(sc_g + gn * 16 + 8); zb1[q] = __ldg(z_g + gn * 16);
                 }
-                ok = mbar_wait(w_full(stage), phase, ctl);
+                ok = mbar_wait(w_full(stage), phase, ctl) && mbar_wait(empty(old), old_phase, ctl);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
+                tc_fence_after();
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {                     // the stage's two 64-wide k-tiles
                     const int q = GPS == 2 ? h : 0;
@@ -343,27 +359,32 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                         v[4 * j + 2] = hmul2_u32(hfma2_u32(code_pair(w, kHighCodes), kSixteenth, zhi), d_lo);
                         v[4 * j + 3] = hmul2_u32(hfma2_u32(code_pair(w8, kHighCodes), kSixteenth, zhi), d_lo);
                     }
-                    tmem_st_16x32cols(taddr_band + stage * (uint32_t)Cfg::kAColsPerStage + 32u * h, v);
+                    tmem_st_16x32cols(taddr_band + slot * (uint32_t)Cfg::kAColsPerStage + 32u * h, v);
                 }
                 tmem_st_wait();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(leader_a_full0 + 8u * stage);
-                if (++stage == S) { stage = 0; phase ^= 1u; }
+                if (lane == 0) mbar_arrive_cluster(leader_a_full0 + 8u * slot);
+                stage += STEP;
+                if (stage >= (uint32_t)S) { stage -= S; phase ^= 1u; }
+                old += STEP;
+                if (old >= (uint32_t)S) { old -= S; old_phase ^= 1u; }
+                slot = (slot + STEP) % SL;
             }
+            first = ks - k1;                             // where this warp's stages resume
         }
     } else if (warp >= 4) {
         // ------------------------------------------------------------------ epilogue
-        // warps 4-7 drain token columns 0..127 of the accumulator, warps 16-19 columns 128..255
+        // warps 4-7 drain the first half of the accumulator's token columns, the last four warps the second
         const int quad = warp & 3;                     // TMEM lanes 32*quad .. +31
-        const int half = warp >= 16 ? 1 : 0;
-        const uint32_t leader_acc_empty = map_to_rank(acc_empty, 0);
+        const int half = warp >= Cfg::kEpilogueWarp1 ? 1 : 0;
+        const uint32_t leader_acc_empty0 = map_to_rank(acc_empty(0), 0);
         // this warp's part of a pair's fp32 partial tile: [rank][warp][chunk][register][lane]
-        const size_t part_off = (size_t)((((int)rank * 8 + half * 4 + quad) * 4) * 1024 + lane);
-        int local = 0;
+        const size_t part_off = (size_t)((((int)rank * 8 + half * 4 + quad) * (Cfg::kHalf / 32)) * 1024 + lane);
+        uint32_t acc = 0, acc_phase = 0;
         int obuf = 0;
         bool ok = true;
-        for (; ok && pieces.next(tile, k0, k1); ++local) {
+        while (ok && pieces.next(tile, k0, k1)) {
             const int slab = (tile / m_tiles) * 2 + (int)rank, mt = tile % m_tiles;
             // A piece that does not start the tile is a contribution: its fp32 sums go to this pair's
             // slot of the workspace.  A piece that starts the tile but does not end it waits for the
@@ -393,51 +414,55 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                     __nanosleep(64);
                 }
             }
+            constexpr bool kPrefetch = Cfg::kDequantWarps == 8;     // (with sixteen there are too few registers)
             float p[32];
-            const float* src0 = partials + (size_t)(cluster + 1) * kPartialFloats + part_off;
-            if (n_contrib > 0 && ok) {
+            const float* src0 = partials + (size_t)(cluster + 1) * Cfg::kPartialFloats + part_off;
+            if (kPrefetch && n_contrib > 0 && ok) {
 #pragma unroll
                 for (int i = 0; i < 32; ++i) p[i] = __ldcg(src0 + i * 32);
             }
-            ok = ok && mbar_wait(acc_full, (uint32_t)local & 1u, ctl);
+            ok = ok && mbar_wait(acc_full(acc), acc_phase, ctl);
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
             tc_fence_after();
             const int n0 = slab * 128 + quad * 32;
-            const int m0 = mt * kPairTokens + half * kHalfTokens;
-            const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * kHalfTokens);
+            const int m0 = mt * BN + half * Cfg::kHalf;
+            const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + acc * (uint32_t)BN + (uint32_t)(half * Cfg::kHalf);
 #pragma unroll 1
-            for (int c = 0; c < kHalfTokens; c += 32) {
+            for (int c = 0; c < Cfg::kHalf; c += 32) {
                 uint32_t r[32];
                 tmem_ld_32cols(taddr + (uint32_t)c, r);
                 tmem_ld_wait();
-                if (c + 32 >= kHalfTokens) {
+                if (c + 32 >= Cfg::kHalf) {
                     // the accumulator is in registers: the MMA thread may start the next piece
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive_cluster(leader_acc_empty);
+                    if (lane == 0) mbar_arrive_cluster(leader_acc_empty0 + 8u * acc);
                 }
                 if (contributes) {
-                    float* dst = partials + (size_t)cluster * kPartialFloats + part_off + (size_t)c * 32;
+                    float* dst = partials + (size_t)cluster * Cfg::kPartialFloats + part_off + (size_t)c * 32;
 #pragma unroll
                     for (int i = 0; i < 32; ++i) __stcg(dst + i * 32, __uint_as_float(r[i]));
                     continue;
                 }
                 if (n_contrib > 0) {
+                    if (kPrefetch) {
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) + p[i]);
-                    for (int j = 1; j < n_contrib; ++j) {
-                        const float* src = partials + (size_t)(cluster + 1 + j) * kPartialFloats + part_off + (size_t)c * 32;
+                        for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) + p[i]);
+                    }
+                    for (int j = kPrefetch ? 1 : 0; j < n_contrib; ++j) {
+                        const float* src = src0 + (size_t)j * Cfg::kPartialFloats + (size_t)c * 32;
 #pragma unroll
                         for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) + __ldcg(src + i * 32));
                     }
-                    if (c + 32 < kHalfTokens) {                     // the next chunk of the first contribution
+                    if (kPrefetch && c + 32 < Cfg::kHalf) {         // the next chunk of the first contribution
 #pragma unroll
                         for (int i = 0; i < 32; ++i) p[i] = __ldcg(src0 + (size_t)(c + 32) * 32 + i * 32);
                     }
                 }
                 // stage the 32 x 32 block as [token][channel] fp16 and hand it to the copy engine
-                // (rows past M are clipped by the tensor map)
+                // (rows past M are clipped by the tensor map; blocks that lie outside y are left out)
+                if (n0 >= N || m0 + c >= M) continue;
                 if (lane == 0) bulk_wait_read_1();                  // the store that last used this buffer
                 __syncwarp();
                 const uint32_t tb = out_base + (uint32_t)(((half * 4 + quad) * 2 + obuf) * 2048);
@@ -464,6 +489,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 for (int j = 0; j < n_contrib; ++j)
                     if (atomicAdd(flags + cluster + 1 + j, 1u) == 31u) atomicExch(flags + cluster + 1 + j, 0u);
             }
+            if (++acc == NACC) { acc = 0; acc_phase ^= 1u; }
         }
         if (lane == 0) bulk_wait_all();                             // all of y written before exit
     }
@@ -481,7 +507,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
 
 // ------------------------------------------------------------------------------ host
 // pairs that can be resident at once on the current device (0 if the query fails); cached
-template <int G>
+template <int G, int BN>
 int resident_pairs(int sms, cudaError_t* err) {
     static bool done[64] = {};
     static int pairs[64] = {};
@@ -489,20 +515,20 @@ int resident_pairs(int sms, cudaError_t* err) {
     cudaGetDevice(&dev);
     *err = cudaSuccess;
     if (!done[dev & 63]) {
-        *err = cudaFuncSetAttribute(gemm_pair_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    PairCfg::kSmemBytes);
+        *err = cudaFuncSetAttribute(gemm_pair_kernel<G, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    PairCfg<BN>::kSmemBytes);
         if (*err != cudaSuccess) return 0;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.gridDim = dim3((unsigned)(sms & ~1));
-        cfg.blockDim = dim3(kPairThreads);
-        cfg.dynamicSmemBytes = PairCfg::kSmemBytes;
+        cfg.blockDim = dim3(PairCfg<BN>::kThreads);
+        cfg.dynamicSmemBytes = PairCfg<BN>::kSmemBytes;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, gemm_pair_kernel<G>, &cfg) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveClusters(&n, gemm_pair_kernel<G, BN>, &cfg) != cudaSuccess) {
             (void)cudaGetLastError();
             n = 0;
         }
@@ -512,30 +538,23 @@ int resident_pairs(int sms, cudaError_t* err) {
     return pairs[dev & 63];
 }
 
-template <int G>
+template <int G, int BN>
 cudaError_t launch_pair(const CUtensorMap& xmap, const CUtensorMap& wmap, const CUtensorMap& ymap,
-                        const void* scales, const void* zeros, int M, int N, int K,
+                        const void* scales, const void* zeros, int M, int N, int K, bool streamk,
                         void* workspace, size_t workspace_bytes,
                         unsigned int* status_word, int sms, cudaStream_t st, bool* launched) {
-    using Cfg = PairCfg;
+    using Cfg = PairCfg<BN>;
     cudaError_t e;
-    const int resident = resident_pairs<G>(sms, &e);
+    const int resident = resident_pairs<G, BN>(sms, &e);
     if (e != cudaSuccess) return e;
     // pairs that cannot all be resident at once would leave SMs idle (and a tile's owner waiting)
     if (resident * 2 < sms - 4) { *launched = false; return cudaSuccess; }
-    const long long tiles = (long long)(N / 256) * ((M + kPairTokens - 1) / kPairTokens);
+    const long long tiles = (long long)((N + 255) / 256) * ((M + BN - 1) / BN);
     const long long stages = tiles * (K / kStageK);
-    // Stream-K needs one fp32 tile per pair behind the counters at the head of the workspace.  It
-    // costs every pair two more accumulator drains and a pass over a partial tile (about 10 us),
-    // so it is used only when whole tiles would leave the pairs idle for longer than that: the
-    // idle time of the last round-robin wave, in stages (~0.8 us each) per pair.  Launches of
-    // more than about 0.3 ms run into the power limit, where idle pairs let the busy ones clock
-    // higher and an even split gains nothing (measured: 5 % slower): those keep whole tiles.
-    const long long waves = (tiles + resident - 1) / resident;
-    const long long idle_stages = (waves * resident - tiles) * (K / kStageK) / resident;
-    const bool streamk = workspace != nullptr && idle_stages > 25 && stages / resident < 400 &&
-                         workspace_bytes >= kCounterBytes + (size_t)resident * kPartialFloats * sizeof(float) &&
-                         (size_t)resident * sizeof(unsigned int) <= kCounterBytes;
+    // Stream-K needs one fp32 tile per pair behind the counters at the head of the workspace.
+    streamk = streamk && workspace != nullptr &&
+              workspace_bytes >= kCounterBytes + (size_t)resident * Cfg::kPartialFloats * sizeof(float) &&
+              (size_t)resident * sizeof(unsigned int) <= kCounterBytes;
     long long want = tiles;
     if (streamk && stages / 4 > want) want = stages / 4;          // at least four stages per pair
     const int clusters = (int)(want < resident ? want : resident);
@@ -544,7 +563,7 @@ cudaError_t launch_pair(const CUtensorMap& xmap, const CUtensorMap& wmap, const 
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3((unsigned)(2 * clusters));
-    cfg.blockDim = dim3(kPairThreads);
+    cfg.blockDim = dim3(Cfg::kThreads);
     cfg.dynamicSmemBytes = Cfg::kSmemBytes;
     cfg.stream = st;
     cfg.attrs = attr;
@@ -552,7 +571,7 @@ cudaError_t launch_pair(const CUtensorMap& xmap, const CUtensorMap& wmap, const 
     float* partials = streamk ? reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + kCounterBytes)
                               : nullptr;
     unsigned int* flags = static_cast<unsigned int*>(workspace);
-    e = cudaLaunchKernelEx(&cfg, gemm_pair_kernel<G>, xmap, wmap, ymap, reinterpret_cast<const __half*>(scales),
+    e = cudaLaunchKernelEx(&cfg, gemm_pair_kernel<G, BN>, xmap, wmap, ymap, reinterpret_cast<const __half*>(scales),
                            reinterpret_cast<const unsigned char*>(zeros), M, N, K, status_word, partials, flags);
     if (e != cudaSuccess) return e;
     count_launch();
@@ -560,33 +579,79 @@ cudaError_t launch_pair(const CUtensorMap& xmap, const CUtensorMap& wmap, const 
     return cudaGetLastError();
 }
 
+// Tokens per tile, and whether to cut the tiles' K loops into equal ranges (stream-K).  A launch takes `start`
+// us plus `stage` us per 128 input channels of each wave of tiles (both measured with one tile per pair, on
+// 4096 -> 4096 and 13824 -> 5120: 17.4 / 17.2 / 21.9 / 26.8 and 42.8 / 42.2 / 54.8 / 69.2 us with 64 / 128 /
+// 192 / 256 tokens); stream-K replaces the last wave by an even share but costs its pairs two more
+// drains and a pass over a partial tile (8.5 us at 64 tokens, 10 us at 256; at 128 and 192, with
+// sixteen dequantizer warps too few registers are left to fetch those sums in one go, 16 us and more: not
+// offered).  With all pairs busy a stage of any size takes up to 1.3 times as long, so the estimates
+// rank, they do not predict.  256 tokens are kept unless another tile promises 4 % (they move the
+// fewest bytes per product), and launches beyond about 0.3 ms, which run into the power limit, keep
+// whole tiles: idle pairs let the busy ones clock higher (an even split measured 5 % slower there).
+// 4096 -> 4096 at 333 tokens: 26.6 us with 256 tokens per tile (32 tiles for 74 pairs), 18.7 us with 128;
+// 5120 -> 13824 at 100 tokens 34 -> 24.6 us; 13824 -> 5120 at 2048 tokens 205 us (256, stream-K), 202 us (192).
+struct PairChoice { int bn; bool streamk; };
+PairChoice choose_tile(int M, int N, int K, int pairs, bool streamk_possible) {
+    static const struct { int bn; double start, stage, streamk; } kTiles[] = {
+        {256, 9.0, 0.557, 10.0}, {192, 8.5, 0.425, 0.0}, {128, 7.0, 0.325, 0.0}, {64, 6.6, 0.330, 8.5}};
+    PairChoice best = {256, false};
+    double best_cost = 1e30;
+    const long long nks = K / kStageK;
+    for (const auto& t : kTiles) {
+        const long long tiles = (long long)((N + 255) / 256) * ((M + t.bn - 1) / t.bn);
+        const long long waves = (tiles + pairs - 1) / pairs;
+        const double bias = t.bn == 256 ? 1.0 : 1.04;
+        const double plain = bias * (t.start + (double)(waves * nks) * t.stage);
+        if (plain < best_cost) { best_cost = plain; best = {t.bn, false}; }
+        const long long share = (tiles * nks + pairs - 1) / pairs;
+        const double even = bias * (t.start + (double)share * t.stage + t.streamk);
+        if (t.streamk > 0.0 && streamk_possible && (double)share * t.stage < 225.0 && even < best_cost) {
+            best_cost = even;
+            best = {t.bn, true};
+        }
+    }
+    return best;
+}
+
 }  // namespace
 
-// Above 128 tokens always; below, where the one-SM kernel's 128-channel tiles re-read x too often:
-// measured at M = 96 .. 128, 27.6 against 42 us on 4096 -> 11008; at M = 32 .. 128, 77 .. 84 against
-// 98 .. 117 us on 8192 -> 28672; but 26.5 against 13 .. 19 us on 4096 -> 4096 (few tiles: the
-// one-SM kernel with split-K wins).
-bool gemm_pair_applies(int M, int N) {
-    if (N % 256 != 0) return false;
-    return M > 128 || (M > 64 && N >= 8192) || (M >= 32 && N >= 16384);
-}
+// Above 64 tokens always; below, on wide matrices when the chunked kernel does not serve the call.
+bool gemm_pair_applies(int M, int N) { return M > 64 || (M >= 32 && N >= 16384); }
 
 // workspace with which the pair kernel balances its tiles over all SM pairs (stream-K)
 size_t gemm_pair_workspace_bytes(int sms) {
-    return kCounterBytes + (size_t)(sms / 2) * kPartialFloats * sizeof(float);
+    return kCounterBytes + (size_t)(sms / 2) * PairCfg<256>::kPartialFloats * sizeof(float);
 }
 
 // Launches the pair kernel if this device can keep (nearly) all its SMs busy with pairs;
 // otherwise *launched is false and the caller uses the single-block kernel.
-cudaError_t launch_gemm_pair(const CUtensorMap& xmap128, const CUtensorMap& wmap, const CUtensorMap& ymap,
+cudaError_t launch_gemm_pair(const void* x, const CUtensorMap& wmap, const CUtensorMap& ymap,
                              const void* scales, const void* zeros, int M, int N, int K, int group,
                              void* workspace, size_t workspace_bytes,
                              unsigned int* status_word, int sms, cudaStream_t st, bool* launched) {
-    if (group == 128)
-        return launch_pair<128>(xmap128, wmap, ymap, scales, zeros, M, N, K, workspace, workspace_bytes,
-                                status_word, sms, st, launched);
-    return launch_pair<64>(xmap128, wmap, ymap, scales, zeros, M, N, K, workspace, workspace_bytes,
-                           status_word, sms, st, launched);
+    const PairChoice c = choose_tile(M, N, K, sms / 2, workspace != nullptr);
+    CUtensorMap xmap;
+    {
+        // x as [M][K] fp16 in boxes of half a tile's tokens x one k-block, 128-byte swizzle
+        const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)M};
+        const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
+        const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)(c.bn / 2)}, estr[2] = {1, 1};
+        if (encode_fn()(&xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(x), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+#define AWQ_PAIR_CASE(GG, BNN)                                                                                     \
+    return launch_pair<GG, BNN>(xmap, wmap, ymap, scales, zeros, M, N, K, c.streamk, workspace, workspace_bytes,  \
+                                status_word, sms, st, launched)
+    if (group == 128) {
+        switch (c.bn) { case 64: AWQ_PAIR_CASE(128, 64); case 128: AWQ_PAIR_CASE(128, 128);
+                        case 192: AWQ_PAIR_CASE(128, 192); default: AWQ_PAIR_CASE(128, 256); }
+    }
+    switch (c.bn) { case 64: AWQ_PAIR_CASE(64, 64); case 128: AWQ_PAIR_CASE(64, 128);
+                    case 192: AWQ_PAIR_CASE(64, 192); default: AWQ_PAIR_CASE(64, 256); }
+#undef AWQ_PAIR_CASE
 }
 
 }  // namespace awq
