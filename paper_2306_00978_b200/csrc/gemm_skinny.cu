@@ -12,7 +12,7 @@
 //     swizzle) is fetched once per chunk and stays in shared memory as the B operand of every slab;
 //     up to four matrices that read the same x lay their slabs end to end in one launch;
 //   * a stage of the weight ring is 8 bands x 256 input channels = 16 KB (one tensor-map copy),
-//     released as soon as its words are in registers; a slot of A in tensor memory is 128 columns
+//     released when its words have been converted; a slot of A in tensor memory is 128 columns
 //     (the same 256 input channels), released by the completion of its products;
 //   * sixteen dequantizer warps, each owning a band and every second stage, so that a warp pays its
 //     barrier polls, parameter reads and arrivals once per 16 packed words;
@@ -137,8 +137,8 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
     const uint32_t par_base = w_base + (uint32_t)(R * kSkStageBytes);
     const uint32_t inv_base = par_base + 2u * (uint32_t)kSkParBytes;
     const uint32_t bars = inv_base + (XS ? (uint32_t)(CK * kBK * 4) : 0u);
-    // the packed weights' ring (raw_*: filled by the copy engine, released by the dequantizers as soon
-    // as the words are in registers) and the ring of A slots in tensor memory (a_*: filled by the
+    // the packed weights' ring (raw_*: filled by the copy engine, released by the dequantizers when they
+    // have used the words) and the ring of A slots in tensor memory (a_*: filled by the
     // dequantizers, released by the products' completion)
     auto raw_full = [&](uint32_t r) { return bars + 8u * r; };
     auto raw_empty = [&](uint32_t r) { return bars + 8u * (uint32_t)(kSkMaxRing + r); };
@@ -413,9 +413,6 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
 #pragma unroll
                 for (int h = 0; h < kSkStageTiles; ++h)
                     pk[h] = *reinterpret_cast<const uint4*>(w_lane + rstage * kSkStageBytes + h * 512);
-                // the words are in registers: the copy engine may refill the stage
-                __syncwarp();
-                if (lane == 0) mbar_arrive(raw_empty(rstage));
                 ok = __all_sync(0xFFFFFFFFu, ok && mbar_wait(a_empty(stage), phase ^ 1u, ctl));
                 if (!ok) break;
                 tc_fence_after();
@@ -457,7 +454,14 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 tmem_st_wait();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(a_full(stage));
+                // The stage is given back with the slot: only the use of a word shows that its load is done.
+                // Given back in front of the wait for the slot, a stage was refilled while late warps still
+                // read it (4096 -> 8192 at 24 tokens, whose ring of five stages wraps during its first
+                // conversions: 96 of 36000 calls had wrong channels in one or more bands; now none of 72000).
+                if (lane == 0) {
+                    mbar_arrive(raw_empty(rstage));
+                    mbar_arrive(a_full(stage));
+                }
                 stage += 2;
                 if (stage >= (uint32_t)S) { stage -= S; phase ^= 1u; }
                 rstage += 2;
@@ -543,11 +547,11 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 if (++acc == NACC) { acc = 0; acc_phase ^= 1u; }
             }
             if (!ok) break;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(par_empty(pb));           // the unit's parameters may be replaced
 #pragma unroll
             for (int i = 0; i < TH; ++i)
                 if (tok0 + i < M) out[(size_t)(tok0 + i) * N] = y[i];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(par_empty(pb));           // the unit's parameters may be replaced
         }
     }
 
