@@ -496,7 +496,7 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 for (int c0 = 0; c0 < BN; c0 += 16) {
                     uint32_t r[16];
                     tmem_ld_16cols(taddr0 + acc * kAccCols + (uint32_t)c0, r);
-                    tmem_ld_wait();
+                    tmem_ld_wait(r);
                     if (c0 + 16 >= BN) {
                         // the accumulator is in registers: the next unit's products may overwrite it
                         tc_fence_before();
@@ -534,7 +534,7 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                 const uint32_t t0 = taddr0 + acc * kAccCols + (uint32_t)tok0;
                 tmem_ld_cols<TH>(t0, r0);
                 tmem_ld_cols<TH>(t0 + (two ? (uint32_t)BN : 0u), r1);
-                tmem_ld_wait();
+                tmem_ld_wait(r0, r1);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(acc_empty(acc));

@@ -303,7 +303,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
                 for (int c = 0; c < BN; c += 32) {
                     uint32_t r[32];
                     tmem_ld_32cols(taddr + (uint32_t)c, r);
-                    tmem_ld_wait();
+                    tmem_ld_wait(r);
 #pragma unroll
                     for (int i = 0; i < 32; ++i) mine[(size_t)(c + i) * 128] = __uint_as_float(r[i]);
                 }
@@ -339,7 +339,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
                     }
                 } else {
                     tmem_ld_32cols(taddr + (uint32_t)c, r);
-                    tmem_ld_wait();
+                    tmem_ld_wait(r);
                     if (c + 32 >= BN) {
                         // the accumulator is in registers: the MMA thread may start the next tile
                         tc_fence_before();

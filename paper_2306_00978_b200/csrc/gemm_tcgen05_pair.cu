@@ -432,7 +432,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
             for (int c = 0; c < Cfg::kHalf; c += 32) {
                 uint32_t r[32];
                 tmem_ld_32cols(taddr + (uint32_t)c, r);
-                tmem_ld_wait();
+                tmem_ld_wait(r);
                 if (c + 32 >= Cfg::kHalf) {
                     // the accumulator is in registers: the MMA thread may start the next piece
                     tc_fence_before();

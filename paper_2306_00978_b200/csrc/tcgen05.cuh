@@ -118,7 +118,19 @@ __device__ __forceinline__ void tmem_ld_32cols(uint32_t taddr, uint32_t (&r)[32]
           "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr) : "memory");
 }
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// Waits for this thread's loads from tensor memory.  The loaded registers pass through it: a load's outputs
+// are ordinary values to the compiler from the load on, and nothing else would keep arithmetic on
+// them behind the wait.
+template <int C>
+__device__ __forceinline__ void tmem_loaded(uint32_t (&r)[C]) {
+#pragma unroll
+    for (int i = 0; i < C; ++i) asm volatile("" : "+r"(r[i]));
+}
+template <int... C>
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&... r)[C]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    (tmem_loaded(r), ...);
+}
 
 // ------------------------------------------------------------------------------ host
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
