@@ -572,19 +572,20 @@ struct SkOutputs {
     int end[kMaxMulti];                              // first channel of the next matrix
 };
 __global__ void __launch_bounds__(256)
-skinny_reduce_kernel(const float* __restrict__ partial, const __grid_constant__ SkOutputs out, int chunks, int M, int N) {
+skinny_reduce_kernel(const float* partial, const __grid_constant__ SkOutputs out, int chunks, int M, int N) {
     // launched with programmatic stream serialization behind the kernel above: it may be resident
-    // before that kernel has finished, and lets the launch behind it start its own weight copies
+    // before that kernel has finished (so the sums, written during its lifetime, are no read-only data: they
+    // are read through L2), and lets the launch behind it start its own weight copies
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int n = (int)(blockIdx.x * blockDim.x + threadIdx.x) * 4, m = blockIdx.y;
     if (n >= N) return;
     const size_t mn = (size_t)M * N;
     const float* p = partial + (size_t)m * N + n;
-    float4 s = *reinterpret_cast<const float4*>(p);
+    float4 s = __ldcg(reinterpret_cast<const float4*>(p));
 #pragma unroll 4
     for (int c = 1; c < chunks; ++c) {
-        const float4 v = *reinterpret_cast<const float4*>(p + (size_t)c * mn);
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(p + (size_t)c * mn));
         s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
     }
     const __half2 lo = __floats2half2_rn(s.x, s.y), hi = __floats2half2_rn(s.z, s.w);

@@ -297,16 +297,17 @@ gemv_mid_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant
 
 // y[m][n] = fp16(sum over the chunks, ascending, of partial[c][m][n]): four outputs per thread.
 __global__ void __launch_bounds__(256)
-gemv_mid_reduce_kernel(const float* __restrict__ partial, __half* __restrict__ y, int chunks, size_t mn) {
+gemv_mid_reduce_kernel(const float* partial, __half* __restrict__ y, int chunks, size_t mn) {
     // launched with programmatic stream serialization behind the kernel above: it may be resident
-    // before that kernel has finished, and lets the launch behind it start its own weight copies
+    // before that kernel has finished (so the sums, written during its lifetime, are no read-only data: they
+    // are read through L2), and lets the launch behind it start its own weight copies
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (i >= mn) return;
-    float4 s = *reinterpret_cast<const float4*>(partial + i);
+    float4 s = __ldcg(reinterpret_cast<const float4*>(partial + i));
     for (int c = 1; c < chunks; ++c) {
-        const float4 v = *reinterpret_cast<const float4*>(partial + (size_t)c * mn + i);
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(partial + (size_t)c * mn + i));
         s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
     }
     const __half2 lo = __floats2half2_rn(s.x, s.y), hi = __floats2half2_rn(s.z, s.w);
