@@ -321,13 +321,15 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_const
                             const uint32_t d_tmem = tmem_base + acc * kAccCols;
                             products(d_tmem, q * KPG, (q + 1) * KPG, true);
                             if (j + (q + 1) * KPG < nt) products(d_tmem + (uint32_t)BN, (q + 1) * KPG, (q + 2) * KPG, true);
+                            // The slot of A before the last pair's sums: what the epilogue waits for comes last,
+                            // so that no arrival is outstanding when the block exits.
+                            if (q + 2 >= GPS || j + (q + 2) * KPG >= nt) umma_commit(a_empty(stage));
                             umma_commit(acc_full(acc));
                         }
                         __syncwarp();
                         if (++acc == NACC) { acc = 0; acc_phase ^= 1u; }
                     }
                     if (!ok) break;
-                    if (lead) umma_commit(a_empty(stage));
                 } else if (lead) {
                     products(tmem_base + acc * kAccCols, 0, kSkStageTiles, j == 0);
                     umma_commit(a_empty(stage));
