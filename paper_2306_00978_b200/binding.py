@@ -184,12 +184,19 @@ def search_clip(W: torch.Tensor, act_mean_abs: Optional[torch.Tensor], alpha: fl
 
 
 def ensure_workspace(nbytes: int) -> None:
-    """Registers (growing if needed) a torch-allocated scratch buffer for the current device."""
+    """Registers (growing if needed) a torch-allocated scratch buffer for the current device.
+
+    While the current stream is capturing nothing can be allocated, and nothing is: the call then does
+    what the library does with the workspace at hand, which is another kernel (other last bits), or the
+    error for a missing workspace where there is none.  One call of the same sizes before the capture makes
+    the captured call the one that runs outside."""
     if nbytes <= 0:
         return
     dev = torch.cuda.current_device()
     cur = _workspace.get(dev)
     if cur is not None and cur.numel() >= nbytes:
+        return
+    if torch.cuda.is_current_stream_capturing():
         return
     torch.cuda.synchronize()
     buf = torch.empty(max(nbytes, 1 << 22), dtype=torch.uint8, device=f"cuda:{dev}")
@@ -198,10 +205,9 @@ def ensure_workspace(nbytes: int) -> None:
 
 
 def _workspace_for_multi(M: int, mats, K: int, group: int) -> None:
-    """What the calls need one by one, and what all of them in one launch can use (M <= 64).  While a
-    stream is capturing nothing is registered for the latter: the call then runs one by one."""
+    """What the calls need one by one, and what all of them in one launch can use (M <= 64)."""
     ensure_workspace(max(workspace_bytes(M, m[3], K, group) for m in mats))
-    if M <= 64 and len(mats) > 1 and not torch.cuda.is_current_stream_capturing():
+    if M <= 64 and len(mats) > 1:
         ensure_workspace(workspace_bytes(M, sum(m[3] for m in mats), K, group))
 
 

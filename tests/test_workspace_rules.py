@@ -1,0 +1,75 @@
+"""The binding's workspace: what a stream capture may and may not do, and that a call's result does not depend
+on which calls came before it."""
+import numpy as np
+import pytest
+
+from tests.util import Case, assert_parity, oracle_packed_to_cuda, to_cuda
+
+
+def test_nothing_is_registered_while_capturing(monkeypatch):
+    import torch
+    from paper_2306_00978_b200 import binding
+
+    def not_now(*a, **k):
+        raise AssertionError("allocated, registered or synchronized while capturing")
+    monkeypatch.setattr(binding, "_workspace", {})
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: True)
+    monkeypatch.setattr(torch.cuda, "synchronize", not_now)
+    monkeypatch.setattr(torch, "empty", not_now)
+    binding.ensure_workspace(1 << 20)
+    assert not binding._workspace
+
+
+class _NoWorkspace:
+    """Nothing registered inside, what was registered is registered again afterwards."""
+
+    def __enter__(self):
+        import torch
+        from paper_2306_00978_b200 import binding
+        torch.cuda.synchronize()
+        self.dev = torch.cuda.current_device()
+        self.saved = binding._workspace.pop(self.dev, None)
+        assert binding.lib().awq_set_workspace(None, 0) == 0
+
+    def __exit__(self, *exc):
+        import torch
+        from paper_2306_00978_b200 import binding
+        torch.cuda.synchronize()
+        binding._workspace.pop(self.dev, None)
+        assert binding.lib().awq_set_workspace(None, 0) == 0
+        if self.saved is not None:
+            assert binding.lib().awq_set_workspace(self.saved.data_ptr(), self.saved.numel()) == 0
+            binding._workspace[self.dev] = self.saved
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M", [32, 48, 200])
+def test_several_matrices_in_a_capture(M):
+    """linear_multi in a capture: without a call before it the kernels that need no workspace, after one the
+    bits of the call outside."""
+    import torch
+    from paper_2306_00978_b200 import binding
+    K, G = 1408, 128
+    cases = [Case(9300 + i, n, K, M, G, 0.5) for i, n in enumerate((384, 256))]
+    mats = [(*oracle_packed_to_cuda(c), c.N) for c in cases]
+    x = to_cuda(cases[0].x)
+    outs = [torch.zeros((M, c.N), dtype=torch.float16, device="cuda") for c in cases]
+
+    def captured():
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            binding.linear_multi(x, mats, K, G, outs=outs)
+        graph.replay()
+        binding.poll_status()
+        return [y.clone() for y in outs]
+
+    with _NoWorkspace():
+        binding.poll_status()
+        for y, c in zip(captured(), cases):
+            assert not binding._workspace
+            c.x = cases[0].x
+            assert_parity(y.cpu().numpy(), c.y_ref(), f"captured without a workspace, M={M}, N={c.N}")
+        eager = binding.linear_multi(x, mats, K, G)
+        for y, want in zip(captured(), eager):
+            assert torch.equal(y, want)
