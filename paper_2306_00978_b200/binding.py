@@ -247,8 +247,7 @@ def linear_multi(x: torch.Tensor, mats, K: int, group: int, outs=None):
         raise AwqError("x must be [M][K]")
     if outs is None:
         outs = [torch.empty((M, m[3]), dtype=torch.float16, device=x.device) for m in mats]
-    if M <= 64:
-        _workspace_for_multi(M, mats, K, group)
+    _workspace_for_multi(M, mats, K, group)
     arr = (_Problem * len(mats))()
     for k, ((qw, sc, zp, N), y) in enumerate(zip(mats, outs)):
         arr[k] = _Problem(_dev(qw, torch.uint8, "qweight"), _dev(sc, torch.float16, "scales"),

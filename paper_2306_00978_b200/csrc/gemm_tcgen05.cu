@@ -495,10 +495,9 @@ cudaError_t launch_gemm(const void* x, const void* qweight, const void* scales, 
 }
 
 size_t gemm_workspace_bytes(int M, int N, int sms) {
-    if (M > 128 && N % 256 != 0) return 0;       // (stream-K is used here too if the caller's workspace happens to suffice)
     if (gemm_pair_applies(M, N)) return gemm_pair_workspace_bytes(sms);
     // split-K of the one-SM kernel: the most it can use for this M and N (any K)
-    const int bn = M > 64 ? 128 : M > 32 ? 64 : 32;
+    const int bn = M > 32 ? 64 : 32;
     const int tiles = N / 128;
     if (tiles * 4 > kMaxSlabs) return 0;
     return kCounterBytes + (size_t)tiles * kMaxSplits * 128 * bn * sizeof(float);

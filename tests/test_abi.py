@@ -44,7 +44,9 @@ def test_sizes_and_layout_version(lib):
     assert lib.awq_workspace_bytes(12, 4096, 4096, 128) == 4096 + 32 * 16 * 128 * 32 * 4
     big = lib.awq_workspace_bytes(2048, 4096, 4096, 128)            # optional: stream-K partial tiles
     assert big > 4096 and (big - 4096) % (256 * 256 * 4) == 0
-    assert lib.awq_workspace_bytes(2048, 4096 + 128, 4096, 128) == 0
+    # the same with an odd number of 128-channel slabs: the SM-pair kernel runs these shapes too (with an answer of
+    # 0 their tiles were balanced only after some other call had left a workspace, and the last bits with it)
+    assert lib.awq_workspace_bytes(2048, 4096 + 128, 4096, 128) == big
     assert lib.awq_workspace_bytes(8, 4096, 4096, 128) == 4096 + 256 * 2 * 8 * 128 * 4
 
 

@@ -73,3 +73,30 @@ def test_several_matrices_in_a_capture(M):
         eager = binding.linear_multi(x, mats, K, G)
         for y, want in zip(captured(), eager):
             assert torch.equal(y, want)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("N,K,M,multi", [
+    (1152, 8192, 130, False),     # 9 slabs: ten half-empty tiles, balanced over the SM pairs by stream-K
+    (1152, 8192, 130, True),
+    (1024, 8192, 130, True),
+])
+def test_same_bits_before_and_after_a_larger_call(N, K, M, multi):
+    import torch
+    from paper_2306_00978_b200 import binding
+    G = 128
+    torch.manual_seed(N + M)
+    qw = torch.randint(0, 256, (N * K // 2,), dtype=torch.uint8, device="cuda")
+    sc = (torch.rand((N // 16, K // G, 16), device="cuda") * 0.01 + 0.001).half()
+    zp = torch.randint(0, 256, (N // 32, K // G, 16), dtype=torch.uint8, device="cuda")
+    x = torch.randn((M, K), device="cuda").half()
+
+    def call():
+        return binding.linear_multi(x, [(qw, sc, zp, N)], K, G)[0] if multi else binding.linear(x, qw, sc, zp, N, K, G)
+
+    with _NoWorkspace():
+        first = call()
+        binding.ensure_workspace(1 << 28)
+        second = call()
+        binding.poll_status()
+        assert torch.equal(first, second)
