@@ -506,6 +506,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
 }
 
 // ------------------------------------------------------------------------------ host
+// stream-K's part of the workspace: a flag per pair in its head, one fp32 tile per pair behind that
+size_t streamk_bytes(int bn, int pairs) { return kCounterBytes + (size_t)pairs * 256 * bn * sizeof(float); }
+
 // pairs that can be resident at once on the current device (0 if the query fails); cached
 template <int G, int BN>
 int resident_pairs(int sms, cudaError_t* err) {
@@ -551,10 +554,8 @@ cudaError_t launch_pair(const CUtensorMap& xmap, const CUtensorMap& wmap, const 
     if (resident * 2 < sms - 4) { *launched = false; return cudaSuccess; }
     const long long tiles = (long long)((N + 255) / 256) * ((M + BN - 1) / BN);
     const long long stages = tiles * (K / kStageK);
-    // Stream-K needs one fp32 tile per pair behind the counters at the head of the workspace.
-    streamk = streamk && workspace != nullptr &&
-              workspace_bytes >= kCounterBytes + (size_t)resident * Cfg::kPartialFloats * sizeof(float) &&
-              (size_t)resident * sizeof(unsigned int) <= kCounterBytes;
+    // (choose_tile asked for room for sms / 2 pairs; resident ones are never more)
+    streamk = streamk && workspace_bytes >= streamk_bytes(BN, resident) && (size_t)resident * sizeof(unsigned int) <= kCounterBytes;
     long long want = tiles;
     if (streamk && stages / 4 > want) want = stages / 4;          // at least four stages per pair
     const int clusters = (int)(want < resident ? want : resident);
@@ -591,8 +592,11 @@ cudaError_t launch_pair(const CUtensorMap& xmap, const CUtensorMap& wmap, const 
 // whole tiles: idle pairs let the busy ones clock higher (an even split measured 5 % slower there).
 // 4096 -> 4096 at 333 tokens: 26.6 us with 256 tokens per tile (32 tiles for 74 pairs), 18.7 us with 128;
 // 5120 -> 13824 at 100 tokens 34 -> 24.6 us; 13824 -> 5120 at 2048 tokens 205 us (256, stream-K), 202 us (192).
+// Stream-K is offered only for tiles whose partial sums fit the workspace at hand, so that what was chosen
+// is what runs: 28672 -> 1152 at 130 tokens with room for 64-token tiles only takes those (28 us by the
+// estimate), with no room 64-token whole tiles (83 us; 256-token ones, 134 us).
 struct PairChoice { int bn; bool streamk; };
-PairChoice choose_tile(int M, int N, int K, int pairs, bool streamk_possible) {
+PairChoice choose_tile(int M, int N, int K, int pairs, size_t workspace_bytes) {
     static const struct { int bn; double start, stage, streamk; } kTiles[] = {
         {256, 9.0, 0.557, 10.0}, {192, 8.5, 0.425, 0.0}, {128, 7.0, 0.325, 0.0}, {64, 6.6, 0.330, 8.5}};
     PairChoice best = {256, false};
@@ -606,7 +610,7 @@ PairChoice choose_tile(int M, int N, int K, int pairs, bool streamk_possible) {
         if (plain < best_cost) { best_cost = plain; best = {t.bn, false}; }
         const long long share = (tiles * nks + pairs - 1) / pairs;
         const double even = bias * (t.start + (double)share * t.stage + t.streamk);
-        if (t.streamk > 0.0 && streamk_possible && (double)share * t.stage < 225.0 && even < best_cost) {
+        if (t.streamk > 0.0 && workspace_bytes >= streamk_bytes(t.bn, pairs) && (double)share * t.stage < 225.0 && even < best_cost) {
             best_cost = even;
             best = {t.bn, true};
         }
@@ -621,7 +625,7 @@ bool gemm_pair_applies(int M, int N) { return M > 64 || (M >= 32 && N >= 16384);
 
 // workspace with which the pair kernel balances its tiles over all SM pairs (stream-K)
 size_t gemm_pair_workspace_bytes(int sms) {
-    return kCounterBytes + (size_t)(sms / 2) * PairCfg<256>::kPartialFloats * sizeof(float);
+    return streamk_bytes(256, sms / 2);
 }
 
 // Launches the pair kernel if this device can keep (nearly) all its SMs busy with pairs;
@@ -630,7 +634,7 @@ cudaError_t launch_gemm_pair(const void* x, const CUtensorMap& wmap, const CUten
                              const void* scales, const void* zeros, int M, int N, int K, int group,
                              void* workspace, size_t workspace_bytes,
                              unsigned int* status_word, int sms, cudaStream_t st, bool* launched) {
-    const PairChoice c = choose_tile(M, N, K, sms / 2, workspace != nullptr);
+    const PairChoice c = choose_tile(M, N, K, sms / 2, workspace ? workspace_bytes : 0);
     CUtensorMap xmap;
     {
         // x as [M][K] fp16 in boxes of half a tile's tokens x one k-block, 128-byte swizzle

@@ -100,3 +100,40 @@ def test_same_bits_before_and_after_a_larger_call(N, K, M, multi):
         second = call()
         binding.poll_status()
         assert torch.equal(first, second)
+
+
+@pytest.mark.gpu
+def test_a_small_workspace_is_no_slower_than_none():
+    """130 tokens on 28672 -> 1152: ten tiles for all SM pairs.  With room for the partial sums of no tile width
+    the tile is the one that is best without them (not the one that would have been best with them)."""
+    import torch
+    from paper_2306_00978_b200 import binding
+    N, K, M, G = 1152, 28672, 130, 128
+    qw = torch.randint(0, 256, (N * K // 2,), dtype=torch.uint8, device="cuda")
+    sc = (torch.rand((N // 16, K // G, 16), device="cuda") * 0.01 + 0.001).half()
+    zp = torch.randint(0, 256, (N // 32, K // G, 16), dtype=torch.uint8, device="cuda")
+    x = torch.randn((M, K), device="cuda").half()
+    y = torch.empty((M, N), dtype=torch.float16, device="cuda")
+    L, us = binding.lib(), {}
+
+    def call():
+        assert L.awq_linear(x.data_ptr(), qw.data_ptr(), sc.data_ptr(), zp.data_ptr(), y.data_ptr(), M, N, K, G, None) == 0
+
+    with _NoWorkspace():
+        for nbytes in (0, 1 << 22, 5 << 20, 20 << 20):       # none, too small, one for 64-token tiles, one for all
+            buf = torch.empty(max(nbytes, 1), dtype=torch.uint8, device="cuda")
+            assert L.awq_set_workspace(buf.data_ptr() if nbytes else None, nbytes) == 0
+            best = float("inf")
+            for _ in range(20):
+                begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                begin.record()
+                for _ in range(4):
+                    call()
+                end.record()
+                end.synchronize()
+                best = min(best, begin.elapsed_time(end) * 250.0)
+            us[nbytes] = best
+            binding.poll_status()
+            assert L.awq_set_workspace(None, 0) == 0
+    print(us)
+    assert us[1 << 22] < 1.25 * us[0] and us[5 << 20] < us[0], us
