@@ -586,34 +586,36 @@ cudaError_t launch_pair(const CUtensorMap& xmap, const CUtensorMap& wmap, const 
 // 192 / 256 tokens); stream-K replaces the last wave by an even share but costs its pairs two more
 // drains and a pass over a partial tile (8.5 us at 64 tokens, 10 us at 256; at 128 and 192, with
 // sixteen dequantizer warps too few registers are left to fetch those sums in one go, 16 us and more: not
-// offered).  With all pairs busy a stage of any size takes up to 1.3 times as long, so the estimates
+// offered) and, where a tile is cut among many pairs, the addition of their sums one after the other by
+// the pair that finishes it (1.5 us each at 64 tokens, 4.4 us at 256).  With all pairs busy a stage of any size
+// takes up to 1.3 times as long, so the estimates
 // rank, they do not predict.  256 tokens are kept unless another tile promises 4 % (they move the
 // fewest bytes per product), and launches beyond about 0.3 ms, which run into the power limit, keep
 // whole tiles: idle pairs let the busy ones clock higher (an even split measured 5 % slower there).
 // 4096 -> 4096 at 333 tokens: 26.6 us with 256 tokens per tile (32 tiles for 74 pairs), 18.7 us with 128;
 // 5120 -> 13824 at 100 tokens 34 -> 24.6 us; 13824 -> 5120 at 2048 tokens 205 us (256, stream-K), 202 us (192).
+// Over 120 problems (N 256 .. 8192, K 4096 .. 28672, 70 .. 1000 tokens, every tile timed) the choice is 0.9 % off
+// the best on average and 19 % at worst (27 % and a factor of 5 without the term for the additions:
+// 28672 -> 1152 at 130 tokens 88.8 us with 256 tokens and stream-K, 35.3 us with 64).
 // Stream-K is offered only for tiles whose partial sums fit the workspace at hand, so that what was chosen
-// is what runs: 28672 -> 1152 at 130 tokens with room for 64-token tiles only takes those (28 us by the
-// estimate), with no room 64-token whole tiles (83 us; 256-token ones, 134 us).
-struct PairChoice { int bn; bool streamk; };
+// is what runs (28672 -> 1152 at 130 tokens with a workspace too small for any: 77.1 us, as without one).
+struct PairChoice { int bn; bool streamk; double us; };
 PairChoice choose_tile(int M, int N, int K, int pairs, size_t workspace_bytes) {
-    static const struct { int bn; double start, stage, streamk; } kTiles[] = {
-        {256, 9.0, 0.557, 10.0}, {192, 8.5, 0.425, 0.0}, {128, 7.0, 0.325, 0.0}, {64, 6.6, 0.330, 8.5}};
-    PairChoice best = {256, false};
-    double best_cost = 1e30;
+    static const struct { int bn; double start, stage, streamk, addition; } kTiles[] = {
+        {256, 9.0, 0.557, 10.0, 4.4}, {192, 8.5, 0.425, 0.0, 0.0}, {128, 7.0, 0.325, 0.0, 0.0}, {64, 6.6, 0.330, 8.5, 1.5}};
+    PairChoice best = {256, false, 1e30};
     const long long nks = K / kStageK;
     for (const auto& t : kTiles) {
         const long long tiles = (long long)((N + 255) / 256) * ((M + t.bn - 1) / t.bn);
         const long long waves = (tiles + pairs - 1) / pairs;
         const double bias = t.bn == 256 ? 1.0 : 1.04;
         const double plain = bias * (t.start + (double)(waves * nks) * t.stage);
-        if (plain < best_cost) { best_cost = plain; best = {t.bn, false}; }
-        const long long share = (tiles * nks + pairs - 1) / pairs;
-        const double even = bias * (t.start + (double)share * t.stage + t.streamk);
-        if (t.streamk > 0.0 && workspace_bytes >= streamk_bytes(t.bn, pairs) && (double)share * t.stage < 225.0 && even < best_cost) {
-            best_cost = even;
-            best = {t.bn, true};
-        }
+        if (plain < best.us) best = {t.bn, false, plain};
+        if (t.streamk == 0.0 || workspace_bytes < streamk_bytes(t.bn, pairs)) continue;
+        const long long share = (tiles * nks + pairs - 1) / pairs, range = share > 4 ? share : 4;     // (at least four stages per pair)
+        const double additions = nks > range ? (double)nks / (double)range - 1.0 : 0.0;
+        const double even = bias * (t.start + (double)share * t.stage + t.streamk + additions * t.addition);
+        if ((double)share * t.stage < 225.0 && even < best.us) best = {t.bn, true, even};
     }
     return best;
 }

@@ -103,9 +103,10 @@ def test_same_bits_before_and_after_a_larger_call(N, K, M, multi):
 
 
 @pytest.mark.gpu
-def test_a_small_workspace_is_no_slower_than_none():
+def test_a_workspace_is_no_slower_than_none():
     """130 tokens on 28672 -> 1152: ten tiles for all SM pairs.  With room for the partial sums of no tile width
-    the tile is the one that is best without them (not the one that would have been best with them)."""
+    the tile is the one that is best without them (not the one that would have been best with them); with
+    room for them a tile is not cut among so many pairs that adding their sums costs more than it saves."""
     import torch
     from paper_2306_00978_b200 import binding
     N, K, M, G = 1152, 28672, 130, 128
@@ -135,5 +136,4 @@ def test_a_small_workspace_is_no_slower_than_none():
             us[nbytes] = best
             binding.poll_status()
             assert L.awq_set_workspace(None, 0) == 0
-    print(us)
-    assert us[1 << 22] < 1.25 * us[0] and us[5 << 20] < us[0], us
+    assert us[1 << 22] < 1.25 * us[0] and us[5 << 20] < us[0] and us[20 << 20] < us[0], us
