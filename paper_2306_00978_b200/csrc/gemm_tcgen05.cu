@@ -429,6 +429,17 @@ int gemm_splits(int M, int N, int K, int group, int bn, int sms, size_t workspac
     return best;
 }
 
+// 65 .. 128 tokens on so few channels that all split-K ranges of all tiles run at once: with long rows seven
+// or so SMs per tile, none of which waits for another, beat the SM-pair kernel, which either leaves most
+// pairs idle or adds many pairs' sums one after the other.  A launch takes 18.6 us + 0.365 us per k-block of a
+// range (N = 256 at 4096 / 8192 / 13824 / 28672 input channels: 22 / 25 / 30 / 42 us, the SM-pair kernel 18 / 27 /
+// 40 / 70 us; N = 640: 22 / 26 / 30 / 40 us against 19 / 27 / 36 / 39 us); 5 % better is asked for.
+bool one_sm_preferred(int M, int N, int K, int splits, int sms, size_t workspace_bytes) {
+    if (M <= 64 || M > 128 || splits == 1 || (N / 128) * splits > sms) return false;
+    const int range = (K / kBK + splits - 1) / splits;
+    return 1.05 * (18.6 + 0.365 * range) < gemm_pair_estimate(M, N, K, sms, workspace_bytes);
+}
+
 }  // namespace
 
 cudaError_t launch_gemm(const void* x, const void* qweight, const void* scales, const void* zeros,
@@ -473,7 +484,9 @@ cudaError_t launch_gemm(const void* x, const void* qweight, const void* scales, 
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     CUtensorMap map, wmap;
-    if (path_pair_allowed && gemm_pair_applies(M, N)) {
+    const int splits = gemm_splits(M, N, K, group, bn, sms, workspace ? workspace_bytes : 0);
+    if (path_pair_allowed && gemm_pair_applies(M, N) &&
+        !one_sm_preferred(M, N, K, splits, sms, workspace ? workspace_bytes : 0)) {
         if (!make_w_map(&wmap, 256)) return cudaErrorInvalidValue;
         bool launched = false;
         e = launch_gemm_pair(x, wmap, ymap, scales, zeros, M, N, K, group, workspace, workspace_bytes,
@@ -481,7 +494,6 @@ cudaError_t launch_gemm(const void* x, const void* qweight, const void* scales, 
         if (e != cudaSuccess || launched) return e;
     }
     if (!make_x_map(&map, bn) || !make_w_map(&wmap, 128)) return cudaErrorInvalidValue;
-    const int splits = gemm_splits(M, N, K, group, bn, sms, workspace ? workspace_bytes : 0);
 #define AWQ_GEMM_CASE(GG, BNN) \
     return launch_one<GG, BNN>(map, wmap, ymap, scales, zeros, M, N, K, splits, workspace, status_word, sms, st)
     if (group == 128) {

@@ -630,6 +630,11 @@ size_t gemm_pair_workspace_bytes(int sms) {
     return streamk_bytes(256, sms / 2);
 }
 
+// its estimated time, us
+double gemm_pair_estimate(int M, int N, int K, int sms, size_t workspace_bytes) {
+    return choose_tile(M, N, K, sms / 2, workspace_bytes).us;
+}
+
 // Launches the pair kernel if this device can keep (nearly) all its SMs busy with pairs;
 // otherwise *launched is false and the caller uses the single-block kernel.
 cudaError_t launch_gemm_pair(const void* x, const CUtensorMap& wmap, const CUtensorMap& ymap,

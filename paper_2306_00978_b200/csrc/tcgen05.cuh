@@ -156,6 +156,7 @@ inline EncodeTiledFn encode_fn() {
 // tile balancing
 bool gemm_pair_applies(int M, int N);
 size_t gemm_pair_workspace_bytes(int sms);
+double gemm_pair_estimate(int M, int N, int K, int sms, size_t workspace_bytes);
 cudaError_t launch_gemm_pair(const void* x, const CUtensorMap& wmap, const CUtensorMap& ymap,
                              const void* scales, const void* zeros, int M, int N, int K, int group,
                              void* workspace, size_t workspace_bytes,
