@@ -76,7 +76,15 @@ struct LayerCall {
         y = *o;
         return true;
     }
-    void allocate() { if (!y.defined()) y = at::empty({(int64_t)M, (int64_t)N}, x->options()); }
+    // The output and every address, while the interpreter lock is held: a tensor without memory of its own
+    // (the wrapper that a function transform passes) throws here.
+    const void *px, *pq, *ps, *pz;
+    void* py;
+    void resolve() {
+        px = x->const_data_ptr(); pq = qweight->const_data_ptr(); ps = scales->const_data_ptr(); pz = zeros->const_data_ptr();
+        if (!y.defined()) y = at::empty({(int64_t)M, (int64_t)N}, x->options());
+        py = y.mutable_data_ptr();
+    }
     PyObject* result(int rc, const char* what) {
         if (rc != 0) return PyObject_CallFunction(g_check, "is", rc, what);          // raises
         if (out != Py_None) { Py_INCREF(out); return out; }
@@ -93,12 +101,11 @@ PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
     int path = 0;
     if (n != 9 || !g_linear_path || !c.parse(a) || !as_int(a[8], &path) || !workspace_suffices(c.dev, c.M, c.N, c.K, c.group))
         Py_RETURN_NONE;
-    c.allocate();
+    c.resolve();
     int rc;
     void* stream = current_stream(c.dev);
     Py_BEGIN_ALLOW_THREADS
-    rc = g_linear_path(c.x->const_data_ptr(), c.qweight->const_data_ptr(), c.scales->const_data_ptr(),
-                       c.zeros->const_data_ptr(), c.y.mutable_data_ptr(), c.M, c.N, c.K, c.group, path, stream);
+    rc = g_linear_path(c.px, c.pq, c.ps, c.pz, c.py, c.M, c.N, c.K, c.group, path, stream);
     Py_END_ALLOW_THREADS
     return c.result(rc, "awq_linear");
     END_HANDLE_TH_ERRORS
@@ -112,7 +119,7 @@ PyObject* linear_int3(PyObject*, PyObject* const* a, Py_ssize_t n) {
     LayerCall c;
     if (n != 8 || !g_linear_int3 || !c.parse(a) || !workspace_suffices(c.dev, c.M, c.N, c.K, c.group)) Py_RETURN_NONE;
     if (c.K < 1) Py_RETURN_NONE;
-    c.allocate();
+    c.resolve();
     at::Tensor scratch;
     int rc = 1;
     void* stream = current_stream(c.dev);
@@ -120,8 +127,7 @@ PyObject* linear_int3(PyObject*, PyObject* const* a, Py_ssize_t n) {
         if (pass == 1) scratch = at::empty({(int64_t)c.N * c.K / 2}, c.qweight->options());
         void* s = pass == 1 ? scratch.mutable_data_ptr() : nullptr;
         Py_BEGIN_ALLOW_THREADS
-        rc = g_linear_int3(c.x->const_data_ptr(), c.qweight->const_data_ptr(), c.scales->const_data_ptr(),
-                           c.zeros->const_data_ptr(), c.y.mutable_data_ptr(), s, c.M, c.N, c.K, c.group, stream);
+        rc = g_linear_int3(c.px, c.pq, c.ps, c.pz, c.py, s, c.M, c.N, c.K, c.group, stream);
         Py_END_ALLOW_THREADS
     }
     return c.result(rc, "awq_linear_int3");

@@ -43,3 +43,23 @@ def test_same_as_the_python_path(N, K, M):
         with pytest.raises(binding.AwqError):
             binding.linear(*bad)
     binding.poll_status()
+
+
+@pytest.mark.gpu
+def test_tensors_without_memory_raise():
+    """A function transform passes wrappers without memory of their own; asking for an address throws in C++,
+    which has to arrive as a Python exception from both calls."""
+    import torch
+    from paper_2306_00978_b200 import binding
+    case = Case(640, 256, 256, 3, 128, 0.5)
+    qw, sc, zp = oracle_packed_to_cuda(case)
+    x = to_cuda(case.x)
+    want = binding.linear(x, qw, sc, zp, 256, 256, 128)                      # registers the workspace
+    q3 = binding.pack_int3(qw & 0x77, 256, 256)
+    batch = torch.stack((x, x))
+    with pytest.raises(RuntimeError):
+        torch.func.vmap(lambda t: binding.linear(t, qw, sc, zp, 256, 256, 128))(batch)
+    with pytest.raises(RuntimeError):
+        torch.func.vmap(lambda t: binding.linear_int3(t, q3, sc, zp, 256, 256, 128))(batch)
+    assert torch.equal(binding.linear(x, qw, sc, zp, 256, 256, 128), want)
+    binding.poll_status()
