@@ -37,6 +37,7 @@ class _Problem(ctypes.Structure):
 _lib = None
 _native = None                 # csrc/native_calls.cpp, connected to the library when that is loaded
 _workspace: dict = {}          # device index -> torch tensor registered with the library
+_replaced: list = []           # smaller ones registered before: graphs captured then still write to them
 
 
 class AwqError(RuntimeError):
@@ -199,9 +200,13 @@ def ensure_workspace(nbytes: int) -> None:
     if torch.cuda.is_current_stream_capturing():
         return
     torch.cuda.synchronize()
-    buf = torch.empty(max(nbytes, 1 << 22), dtype=torch.uint8, device=f"cuda:{dev}")
+    # at least twice the last one: all the replaced ones together stay smaller than the one in use
+    least = 1 << 22 if cur is None else 2 * cur.numel()
+    buf = torch.empty(max(nbytes, least), dtype=torch.uint8, device=f"cuda:{dev}")
     _check(lib().awq_set_workspace(buf.data_ptr(), buf.numel()), "awq_set_workspace")
     _workspace[dev] = buf
+    if cur is not None:
+        _replaced.append(cur)
 
 
 def _workspace_for_multi(M: int, mats, K: int, group: int) -> None:

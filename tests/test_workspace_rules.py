@@ -21,6 +21,35 @@ def test_nothing_is_registered_while_capturing(monkeypatch):
     assert not binding._workspace
 
 
+def test_replaced_workspaces_stay_alive_and_bounded(monkeypatch):
+    """A graph holds the address of the workspace it was captured with, so growing must not free it."""
+    import torch
+    import weakref
+    from paper_2306_00978_b200 import binding
+
+    class Library:
+        def awq_set_workspace(self, address, nbytes):
+            return 0
+    real = torch.empty
+    monkeypatch.setattr(binding, "_workspace", {})
+    monkeypatch.setattr(binding, "_replaced", [], raising=False)
+    monkeypatch.setattr(binding, "lib", Library)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: False)
+    monkeypatch.setattr(torch.cuda, "synchronize", lambda: None)
+    monkeypatch.setattr(torch, "empty", lambda n, dtype, device: real(n, dtype=dtype))
+    seen = []
+    for need in (1 << 10, (1 << 22) + 1, (1 << 22) + 2, 9 << 20, 10 << 20, 40 << 20):
+        binding.ensure_workspace(need)
+        buf = binding._workspace[0]
+        assert buf.numel() >= need
+        if not seen or seen[-1]() is not buf:
+            seen.append(weakref.ref(buf))
+        del buf
+    assert len(seen) > 2 and all(r() is not None for r in seen)
+    assert sum(r().numel() for r in seen[:-1]) < binding._workspace[0].numel()
+
+
 class _NoWorkspace:
     """Nothing registered inside, what was registered is registered again afterwards."""
 
