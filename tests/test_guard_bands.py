@@ -41,7 +41,9 @@ def _check(buf, nbytes, what):
     (2432, 1152, 3, 64, 1),       # band kernel, x through the stages
     (2432, 8320, 2, 128, 1),      # band kernel, x resident
     (512, 1408, 9, 128, 3),       # split-K matrix-vector kernel
-    (1024, 1408, 13, 128, 5),     # chunked matrix-vector kernel
+    (1024, 1408, 7, 128, 5),      # chunked matrix-vector kernel
+    (640, 2304, 8, 64, 5),
+    (1024, 1408, 13, 128, 5),     # above 8 tokens the chunked tensor-core kernel
     (768, 2304, 24, 64, 5),
     (1024, 1408, 33, 128, 6),     # chunked tensor-core kernel
     (256, 640, 17, 64, 6),
@@ -107,7 +109,7 @@ def test_workspace_is_not_overrun():
     dev = torch.cuda.current_device()
     saved = binding._workspace.pop(dev, None)
     try:
-        for (N, K, M, G, path) in ((512, 1408, 9, 128, 3), (2432, 4096, 13, 128, 5), (1024, 1408, 24, 128, 5),
+        for (N, K, M, G, path) in ((512, 1408, 9, 128, 3), (2432, 4096, 8, 128, 5), (2432, 4096, 13, 128, 5), (1024, 1408, 24, 128, 5),
                                    (4096, 4096, 32, 128, 6), (1024, 1408, 64, 64, 6), (384, 4096, 100, 128, 4),
                                    (512, 4096, 300, 128, 2)):
             case = Case(7900 + N + K + M, N, K, M, G, 0.5)

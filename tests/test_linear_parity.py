@@ -197,9 +197,9 @@ def test_quantize_then_linear_back_to_back_on_one_stream():
 
 
 def test_auto_dispatch_between_9_and_16_tokens():
-    """awq_linear with 9..16 tokens: the chunked matrix-vector kernel when a workspace is registered
-    (the binding registers one), the tensor-core kernel otherwise.  Each result is bit-equal to its
-    forced path."""
+    """awq_linear with 9..16 tokens: the chunked tensor-core kernel when a workspace is registered
+    (the binding registers one), the prefill kernel otherwise.  Each result is bit-equal to its
+    forced path (AWQ_PATH_GEMV_MID is that kernel too above 8 tokens)."""
     import torch
     from paper_2306_00978_b200 import binding
     L = binding.lib()
@@ -209,7 +209,7 @@ def test_auto_dispatch_between_9_and_16_tokens():
         x = to_cuda(case.x)
         auto = binding.linear(x, qw, sc, zp, case.N, case.K, case.group)
         assert torch.equal(auto, binding.linear(x, qw, sc, zp, case.N, case.K, case.group, path=binding.PATH_GEMV_MID))
-        assert_parity(auto.cpu().numpy(), case.y_ref(), f"auto M=12, chunked kernel, K={K}")
+        assert_parity(auto.cpu().numpy(), case.y_ref(), f"auto M=12, chunked tensor-core kernel, K={K}")
     # a large matrix (random packed arrays: only the choice of kernel is checked here; parity at
     # this size is covered by the 70B sweep)
     N, K, G, M = 16384, 8192, 128, 12
@@ -290,17 +290,17 @@ def test_missing_workspace_is_reported():
 
 @pytest.mark.parametrize("N,K,M,G", [
     (512, 1024, 9, 128),      # one chunk
-    (1024, 1408, 16, 128),    # ragged second chunk (6 k-tiles)
-    (768, 4096, 17, 64),      # three token fragments, four chunks
-    (512, 2304, 32, 128),     # four token fragments, ragged last chunk
-    (640, 2048, 24, 64),      # 40 bands: a last unit of 8 bands
+    (1024, 1408, 16, 128),    # 16-token tile, ragged last chunk
+    (768, 4096, 17, 64),      # 32-token tile, several chunks
+    (512, 2304, 32, 128),     # full 32-token tile, ragged last chunk
+    (640, 2048, 24, 64),      # an odd number of slabs
     (2432, 4096, 13, 128),    # more units than blocks
-    (128, 8192, 10, 128),     # one unit of 8 bands per chunk
+    (128, 8192, 10, 128),     # one slab, many chunks
     (4224, 1152, 9, 128),     # units crossing from one chunk to the next inside a block
 ])
 def test_chunked_matrix_vector_kernel(N, K, M, G):
-    """AWQ_PATH_GEMV_MID: units of 16 bands x 1024 input channels, one band per warp; partial sums
-    per chunk, added by a second kernel.  Parity with the oracle and bit-reproducibility."""
+    """AWQ_PATH_GEMV_MID above 8 tokens, where it runs the chunked tensor-core kernel (below:
+    test_chunked_matrix_vector_kernel_up_to_8_tokens).  Parity with the oracle and bit-reproducibility."""
     from paper_2306_00978_b200 import binding
     case = Case(600 + N + K + M + G, N, K, M, G, 0.5)
     y = _run(case, binding.PATH_GEMV_MID)
@@ -335,10 +335,9 @@ def test_chunked_tensor_core_kernel(N, K, M, G, alpha):
 
 
 def test_auto_dispatch_between_17_and_64_tokens():
-    """awq_linear with 17..64 tokens and a registered workspace: the chunked matrix-vector kernel up
-    to 24 tokens on matrices of at least 2^25 weights, else the chunked tensor-core kernel; above 64
-    tokens, or where N is not a multiple of 128, the prefill kernels.  Each result is bit-equal to
-    its forced path."""
+    """awq_linear with 17..64 tokens and a registered workspace: the chunked tensor-core kernel
+    (AWQ_PATH_GEMV_MID is that kernel too above 8 tokens); above 64 tokens the prefill kernels.
+    Each result is bit-equal to its forced path."""
     import torch
     from paper_2306_00978_b200 import binding
     for (N, K, M, want) in ((1024, 1408, 20, binding.PATH_GEMM_SKINNY), (1024, 1408, 64, binding.PATH_GEMM_SKINNY),
@@ -359,3 +358,54 @@ def test_auto_dispatch_between_17_and_64_tokens():
         assert torch.equal(auto, forced), (N, K, M)
         if N * K < 1 << 24:
             assert_parity(auto.cpu().numpy(), case.y_ref(), f"auto M={M}")
+
+
+def _random_operands(N, K, M, G, seed):
+    import torch
+    torch.manual_seed(seed)
+    stored = min(G, 128)
+    qw = torch.randint(0, 256, (N * K // 2,), dtype=torch.uint8, device="cuda")
+    sc = (torch.rand((N // 16, K // stored, 16), device="cuda") * 0.01 + 0.001).half()
+    zp = torch.randint(0, 256, (N // 32, K // stored, 16), dtype=torch.uint8, device="cuda")
+    return qw, sc, zp, torch.randn((M, K), device="cuda").half()
+
+
+@pytest.mark.parametrize("N,K,M,G", [
+    (128, 128, 1, 128),       # half a unit, an eighth of a chunk
+    (1024, 1408, 8, 128),     # ragged second chunk (6 k-tiles)
+    (640, 2304, 5, 64),       # 40 bands: a last unit of 8 bands; ragged last chunk
+    (2432, 4096, 2, 128),     # a last unit of 8 bands in every chunk, chunks of 8 k-tiles
+    (4096, 4096, 7, 64),      # chunks of 8 k-tiles
+    (4224, 1152, 3, 128),     # more units than one chunk has, a short last chunk
+    (19072, 1152, 6, 128),    # more units than blocks: ranges that cross from one chunk to the next
+    (128, 8192, 4, 1024),     # one unit of 8 bands per chunk, groups stored per 128 columns
+])
+def test_chunked_matrix_vector_kernel_up_to_8_tokens(N, K, M, G):
+    """AWQ_PATH_GEMV_MID up to 8 tokens: units of 16 bands x a chunk of 512 or 1024 input channels, one band per
+    warp; partial sums per chunk, added by a second kernel.  Parity with the oracle and bit-reproducibility."""
+    from paper_2306_00978_b200 import binding
+    case = Case(640 + N + K + M + G, N, K, M, G, 0.5)
+    y = _run(case, binding.PATH_GEMV_MID)
+    assert_parity(y, case.y_ref(), f"chunked matrix-vector N={N} K={K} M={M} G={G}")
+    y2 = _run(case, binding.PATH_GEMV_MID)
+    assert np.array_equal(y.view(np.uint16), y2.view(np.uint16))
+
+
+@pytest.mark.parametrize("N,K,M,mid", [
+    (5504, 12288, 2, True), (5504, 12160, 2, False),        # 2 tokens: rows of at least 12288
+    (8192, 8320, 3, True), (8192, 8064, 4, False),          # 3, 4 tokens: at least 2^26 weights
+    (4096, 8320, 5, True), (4096, 8064, 8, False),          # 5 .. 8 tokens: at least 2^25 weights
+    (16384, 4096, 8, False),                                # rows of at most 4096: the band kernel
+])
+def test_auto_dispatch_up_to_8_tokens(N, K, M, mid):
+    """awq_linear up to 8 tokens on many output rows: the chunked matrix-vector kernel on long rows, else the band
+    kernel, whose sums are formed in another order."""
+    import torch
+    from paper_2306_00978_b200 import binding
+    qw, sc, zp, x = _random_operands(N, K, M, 128, N + K + M)
+    auto = binding.linear(x, qw, sc, zp, N, K, 128)
+    chunked = binding.linear(x, qw, sc, zp, N, K, 128, path=binding.PATH_GEMV_MID)
+    band = binding.linear(x, qw, sc, zp, N, K, 128, path=binding.PATH_GEMV)
+    binding.poll_status()
+    assert not torch.equal(chunked, band)
+    assert torch.equal(auto, chunked if mid else band)
