@@ -82,7 +82,8 @@ cudaError_t launch_gemv_mid(const void* x, const void* qweight, const void* scal
                             bool serialize, cudaStream_t st);
 
 // The chunked kernels (gemv_mid.cu, gemm_skinny.cu): first unit of every block (and the end of the
-// last one); units are in chunk-major order, `per_chunk` of them per chunk of K.  Blocks start in index order, the last
+// last one); units are in chunk-major order.  unit_starts is gemv_mid.cu's rule (gemm_skinny.cu cuts its ranges by
+// an estimate), `per_chunk` units per chunk of K.  Blocks start in index order, the last
 // ones on the SMs that the launch in front of this one frees last, so the blocks that hold one unit
 // more than the others are the first ones - except where the longer range would cross into the next
 // chunk, which costs a second slice of x (measured on 28672 -> 8192 at 8 tokens: 6 units 22.4 us, 7
@@ -115,7 +116,7 @@ inline UnitStarts unit_starts(int units, int per_chunk, int blocks) {
 // launched with programmatic stream serialization behind the kernel that wrote the partial sums
 cudaError_t launch_chunk_reduce(const float* partial, void* y, int chunks, size_t mn, cudaStream_t st);
 
-// 17 .. 64 tokens on the tensor cores (gemm_skinny.cu): units of one 128-channel slab x one chunk of
+// 9 .. 64 tokens, and fewer on few output rows, on the tensor cores (gemm_skinny.cu): units of one 128-channel slab x one chunk of
 // K, the chunk's slice of x resident in shared memory, partial sums per chunk in the workspace
 bool gemm_skinny_applies(int M, int N, int K, int group);
 // `count` matrices (1..kMaxMulti) sharing x, K and the group size in one launch (N: the sum of theirs);

@@ -1,5 +1,5 @@
-// The layer for 17 .. 64 tokens (Sec. 4.2: fused dequantize + product) on the tensor cores, where
-// the weights still set the time: every packed byte should cross HBM once and nothing else should
+// The layer for 9 .. 64 tokens (and fewer where the output rows are too few for the band kernel; Sec. 4.2:
+// fused dequantize + product) on the tensor cores, where the weights still set the time: every packed byte should cross HBM once and nothing else should
 // be slower than that.
 //
 // The prefill kernels (gemm_tcgen05*.cu) are built for many tokens: per 64-wide k-block a tile
@@ -64,6 +64,9 @@ constexpr int kSkMaxGroups = 16;                 // groups per chunk (one tensor
 constexpr int kSkParBytes = kSkMaxGroups * (8 * 32 + 4 * 16);   // a unit's scales [8 bands][groups][16] fp16 + zero bytes [4][groups][16]
 constexpr int kSkMaxSmem = 227 * 1024 - 64;          // dynamic part: a few static bytes come on top
 constexpr int kSkFixed = 1024 /*align*/ + 512 /*barriers*/ + 2 * kSkParBytes;
+// A stage may pass from the warps of one parity to the others' (an odd ring): what tells them apart is that a warp
+// has seen the products of five stages ago complete, so a ring is even or has at least five stages.
+static_assert((kSkMaxSmem - kSkFixed - kSkXBytes - kSkMaxParts * kSkPartTiles * kBK * 4) / kSkStageBytes >= 4, "ring");
 
 struct SkMaps {                                  // up to kMaxMulti matrices, slabs laid end to end
     CUtensorMap w[kMaxMulti], sc[kMaxMulti], z[kMaxMulti];
@@ -800,9 +803,9 @@ cudaError_t launch_gemm_skinny(const void* x, const GemvMatrix* mats, int count,
     cfg.attrs = attr;
     cfg.numAttrs = serialize ? 0 : 1;
     cudaError_t e;
-#define AWQ_SK_LAUNCH(GG, BNN, RR)                                                                                        \
-    e = inv_s ? launch_one_skinny<GG, BNN, true, RR>(cfg, xmap, maps, inv_s, partial, M, slabs, K, R, plan, status_word)  \
-              : launch_one_skinny<GG, BNN, false, RR>(cfg, xmap, maps, inv_s, partial, M, slabs, K, R, plan, status_word)
+#define AWQ_SK_LAUNCH(GG, BNN, EX)                                                                                        \
+    e = inv_s ? launch_one_skinny<GG, BNN, true, EX>(cfg, xmap, maps, inv_s, partial, M, slabs, K, R, plan, status_word)  \
+              : launch_one_skinny<GG, BNN, false, EX>(cfg, xmap, maps, inv_s, partial, M, slabs, K, R, plan, status_word)
 #define AWQ_SK_PICK(GG)                                                                             \
     do {                                                                                            \
         if (bn == 16) AWQ_SK_LAUNCH(GG, 16, true);                                           \

@@ -315,9 +315,9 @@ __device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
 __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
     f32x2 d; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c)); return d;
 }
-// The rounded product, as a * b + (-0.0) with the zero in a kernel argument: the assembler contracts
-// mul.rn.f32x2 with an add.rn.f32x2 behind it into one fused instruction (unlike the scalar forms with
-// explicit rounding), which the errors here must not be.
+// The rounded product, as a * b + (-0.0) with the zero in a kernel argument: with mul.rn.f32x2 and an
+// add.rn.f32x2 behind it about one group in 10^5 came out with another ratio than the definition, as if the
+// two had been fused (the scalar forms with explicit rounding did not); like this all agree.
 __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b, f32x2 minus_zero) { return fma2(a, b, minus_zero); }
 __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
     f32x2 d; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d;

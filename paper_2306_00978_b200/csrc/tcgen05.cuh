@@ -14,9 +14,8 @@ constexpr int kBK = 64;   // k-block: 64 input channels = one 128-byte swizzle r
 // ------------------------------------------------------------------ small PTX wrappers
 // One lane of a converged warp, chosen the same way every time.  The warps that issue copies and products
 // run their whole loop converged - every lane polls the barriers and forms the operands - and only the
-// instruction itself is predicated on this lane: descriptors and addresses then stay in uniform
-// registers.  With the loop inside `if (lane == 0)` every product first moved its operands there, and one
-// thread issued a product per ~80 - 105 cycles (8192 -> 28672 at 32 tokens 64 -> 50 us).
+// instruction itself is predicated on this lane.  With the loop inside `if (lane == 0)` a thread issued a
+// product per ~80 - 105 cycles; converged, 8192 -> 28672 at 32 tokens went from 64 to 49 us.
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p) :: "memory");
@@ -99,9 +98,9 @@ __device__ __forceinline__ uint32_t hmul2_u32(uint32_t a, uint32_t b) {
 }
 
 // Two codes of a packed word as fp16: (w & mask) | 0x6400 in both halves, i.e. 1024 + q (low nibbles) or
-// 1024 + 16 q (high ones).  As one three-input instruction with both constants in registers: written as
-// C it became two, since an instruction holds one immediate (16 packed words with four tensor-memory stores
-// of four warps per scheduler: 420 -> 340 cycles a warp).
+// 1024 + 16 q (high ones).  Asked for as one three-input instruction with both constants in registers: written
+// as C, 16 packed words with four tensor-memory stores of four warps per scheduler took 420 cycles a warp, like
+// this they take 340.
 __device__ __forceinline__ uint32_t code_pair(uint32_t w, uint32_t mask) {
     uint32_t d; asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(d) : "r"(w), "r"(mask), "r"(0x64006400u)); return d;
 }
