@@ -113,9 +113,9 @@ def test_quantize_pack_coarse_groups_bit_exact(N, K, G, alpha, bits, symmetric, 
     (768, 4096, 40, 512), (512, 1024, 100, 256), (512, 2048, 300, 1024),
 ])
 def test_layer_on_coarse_groups(N, K, M, G):
-    """Every kernel family of awq_linear (band and split-K matrix-vector, chunked matrix-vector,
-    chunked tensor-core, one-SM and SM-pair prefill kernels) on arrays quantized with a coarse group,
-    quantized on the GPU and by the oracle."""
+    """The kernels that awq_linear takes at these sizes (band matrix-vector, chunked tensor-core, SM-pair
+    prefill) and the split-K matrix-vector kernel on arrays quantized with a coarse group, quantized on the
+    GPU and by the oracle."""
     import torch
     from paper_2306_00978_b200 import binding
     case = Case(5200 + N + K + M + G, N, K, M, G, 0.5)

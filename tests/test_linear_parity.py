@@ -85,9 +85,9 @@ def _run_gemm_without_workspace(case):
 @pytest.mark.parametrize("mode", ["auto", "one-sm", "no-workspace"])
 @pytest.mark.parametrize("N,K,M,G,alpha", GEMM_CASES)
 def test_gemm_parity(N, K, M, G, alpha, mode):
-    """PATH_GEMM runs SM pairs when N % 256 == 0 and M > 128, or less on wide matrices (stream-K over the registered
-    workspace, or whole tiles round-robin without one) and one SM per tile otherwise;
-    PATH_GEMM_1SM forces the latter on every case."""
+    """PATH_GEMM runs SM pairs above 64 tokens, or from 32 on wide matrices (stream-K over the registered
+    workspace where that pays, else whole tiles round-robin), and one SM per tile otherwise and for few
+    channels with long rows up to 128 tokens; PATH_GEMM_1SM forces the latter on every case."""
     from paper_2306_00978_b200 import binding
     case = Case(3000 + N + K + M, N, K, M, G, alpha)
     if mode == "no-workspace":
