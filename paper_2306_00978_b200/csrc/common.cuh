@@ -112,6 +112,26 @@ inline UnitStarts unit_starts(int units, int per_chunk, int blocks) {
     return s;
 }
 
+#ifdef __CUDACC__
+// p[0] + p[stride] + ... over the chunks, ascending, four neighbours at a time; the loads of B chunks leave
+// before the first addition (8192 -> 4096 at 5 tokens: 9.9 us in a plain loop of loads through L2, 9.4 us in a
+// plain loop of read-only loads, 8.6 us with B = 8).
+template <int B>
+__device__ __forceinline__ float4 add_chunks(const float* p, int chunks, size_t stride) {
+    float4 s = __ldcg(reinterpret_cast<const float4*>(p));
+    for (int c = 1; c < chunks; c += B) {
+        float4 v[B];
+#pragma unroll
+        for (int q = 0; q < B; ++q)
+            if (c + q < chunks) v[q] = __ldcg(reinterpret_cast<const float4*>(p + (size_t)(c + q) * stride));
+#pragma unroll
+        for (int q = 0; q < B; ++q)
+            if (c + q < chunks) { s.x += v[q].x; s.y += v[q].y; s.z += v[q].z; s.w += v[q].w; }
+    }
+    return s;
+}
+#endif
+
 // y[m][n] = fp16(sum over the chunks, ascending, of partial[c][m][n]), mn = M * N a multiple of 4;
 // launched with programmatic stream serialization behind the kernel that wrote the partial sums
 cudaError_t launch_chunk_reduce(const float* partial, void* y, int chunks, size_t mn, cudaStream_t st);

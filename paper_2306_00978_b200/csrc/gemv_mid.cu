@@ -305,11 +305,7 @@ gemv_mid_reduce_kernel(const float* partial, __half* __restrict__ y, int chunks,
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (i >= mn) return;
-    float4 s = __ldcg(reinterpret_cast<const float4*>(partial + i));
-    for (int c = 1; c < chunks; ++c) {
-        const float4 v = __ldcg(reinterpret_cast<const float4*>(partial + (size_t)c * mn + i));
-        s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-    }
+    const float4 s = add_chunks<8>(partial + i, chunks, mn);
     const __half2 lo = __floats2half2_rn(s.x, s.y), hi = __floats2half2_rn(s.z, s.w);
     uint2 o;
     o.x = *reinterpret_cast<const uint32_t*>(&lo);
