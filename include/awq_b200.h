@@ -70,26 +70,28 @@ typedef enum AwqStatus {
 typedef enum AwqPath {
     AWQ_PATH_AUTO = 0,          /* what awq_linear does.  M <= 8: the matrix-vector kernels, and where
                                    K > 4096 from 3 tokens (N * K >= 2^26; from 2 where K >= 12288) or 5
-                                   tokens (N * K >= 2^25) the chunked one; M <= 64: the chunked
-                                   tensor-core kernel (below 9 tokens only where N/16 is well below the
-                                   SM count) - the chunked kernels if a workspace of
-                                   awq_workspace_bytes is registered; else the tensor-core prefill
-                                   kernels (M <= 8: the band or split-K kernel) */
+                                   tokens (N * K >= 2^25) the chunked one; M <= 64: the stream
+                                   kernel (below 9 tokens only where N/16 is well below the SM
+                                   count), up to 256 where its estimate is the best - these if a
+                                   workspace of awq_workspace_bytes is registered; else the tensor-core
+                                   prefill kernels (M <= 8: the band or split-K kernel) */
     AWQ_PATH_GEMV = 1,          /* fused dequant matrix-vector kernel, M <= 16: band kernel when
                                    M <= 8 and N/16 is not much below the SM count, else split-K */
-    AWQ_PATH_GEMM = 2,          /* tcgen05 tensor-core kernel, any M >= 1: pairs of SMs
-                                   (cta_group::2, 256 channels x 64 .. 256 tokens per tile) when
-                                   M > 64 (M >= 32 from N = 16384; up to 128 tokens not on few
-                                   channels with long rows), else one SM per tile */
+    AWQ_PATH_GEMM = 2,          /* tcgen05 tensor-core kernels, any M >= 1: at 65 .. 256 tokens on few
+                                   tiles or long rows the stream kernel (with a workspace), else
+                                   pairs of SMs (cta_group::2, 256 channels x 64 .. 256 tokens per
+                                   tile) when M > 64 (M >= 32 from N = 16384; up to 128 tokens not on
+                                   few channels with long rows), else one SM per tile */
     AWQ_PATH_GEMV_SPLITK = 3,   /* the split-K matrix-vector kernel, M <= 16 */
     AWQ_PATH_GEMM_1SM = 4,      /* the tensor-core kernel with one SM per tile, any M >= 1 */
     AWQ_PATH_GEMV_MID = 5,      /* M <= 8: the chunked matrix-vector kernel: work units of 16 bands
                                    x 1024 input channels, the unit's slice of x in shared memory, one
-                                   band per warp; 9 <= M <= 32: the chunked tensor-core kernel; needs a
+                                   band per warp; 9 <= M <= 32: the stream kernel; needs a
                                    workspace of awq_workspace_bytes (fp32 partial sums per chunk of K) */
-    AWQ_PATH_GEMM_SKINNY = 6    /* the chunked tensor-core kernel, M <= 64, N a multiple of 128: work
-                                   units of 128 channels x a chunk of K, the chunk's slice of x resident
-                                   in shared memory; needs a workspace of awq_workspace_bytes */
+    AWQ_PATH_GEMM_SKINNY = 6    /* the stream kernel, M <= 64, N a multiple of 128: pairs of SMs
+                                   (cta_group::2, 256 channels x up to 128 tokens per tile), the tiles' K
+                                   loops laid end to end and cut into one range per pair; needs a
+                                   workspace of awq_workspace_bytes */
 } AwqPath;
 
 /* Sizes of the packed arrays, in bytes (0 if the shape is not accepted). */
@@ -160,17 +162,17 @@ int awq_channel_scale(const float* act_mean_abs, float alpha, float* s, int K, v
  * x: in, fp16 [M][K].  y: out, fp16 [M][N], fully overwritten; must not alias an input.
  * Which kernel runs is listed under AWQ_PATH_AUTO.  The matrix-vector kernels (M <= 8) are HBM-bound:
  * the 4-bit codes enter warp-level tensor-core products exactly, accumulation, zero point and Delta
- * are fp32, one rounding to fp16 at the end.  The chunked tensor-core kernel forms q - z exactly and
+ * are fp32, one rounding to fp16 at the end.  The stream kernel forms q - z exactly and
  * applies Delta in fp32 up to 32 tokens; from 33 tokens, like the prefill kernels, it rounds
  * (q - z) * Delta once to fp16 and accumulates in fp32 in tensor memory.  Results are
  * bit-reproducible.
  * Workspace.  The split-K matrix-vector kernel (small N, M <= 16) needs the registered workspace;
- * the chunked kernels (partial sums per chunk of K, added in ascending order by a second small
- * kernel) and the prefill kernels' split-K / stream-K use it when it holds awq_workspace_bytes,
+ * the chunked matrix-vector and the stream kernel (partial sums per part of K, added in ascending order by
+ * a second small kernel) and the prefill kernels' split-K / stream-K use it when it holds awq_workspace_bytes,
  * else awq_linear falls back to a kernel that needs none.  Calls that use the workspace must not
  * overlap on the GPU (issue them on one stream).
  * Stream order.  x and y follow plain stream order.  The packed arrays are treated as constants
- * of the layer: the band and chunked kernels are launched with programmatic stream serialization
+ * of the layer: the band, chunked and stream kernels are launched with programmatic stream serialization
  * and start copying qweight, scales and zeros into shared memory BEFORE the work in front of them
  * in the stream has completed; only their reads of x and their writes of y and of the workspace
  * wait for that work.  The library covers its own writers: the first
@@ -192,7 +194,8 @@ int awq_linear(const void* x, const void* qweight, const void* scales, const voi
  * comparable to its launch overhead).  y_i = x . dequant(Wq_i)^T for i < count, count <= 4; all
  * matrices share K and `group`, each has its own N.  `problems` is a HOST array read during the
  * call.  For M <= 8 with enough output rows in total the matrices are served by ONE launch of
- * the matrix-vector band kernel, for other M <= 64 by one launch of the chunked tensor-core kernel if
+ * the matrix-vector band kernel (from 4 tokens on long rows, K > 4096, of the stream kernel), for other M <= 64,
+ * and up to 256 where its estimate is below that of separate calls, by one launch of the stream kernel if
  * the workspace holds awq_workspace_bytes(M, sum of the N, K, group); otherwise this is the same as
  * `count` awq_linear calls.  Each output is what awq_linear would give with the band kernel (bit-identical when awq_linear picks
  * that kernel for the matrix on its own, within the usual tolerance otherwise).
@@ -222,12 +225,12 @@ int awq_linear_multi(const void* x, const AwqLinearProblem* problems, int count,
  * result for a few elements in a thousand, which the method does not care about as long as the
  * quantizer's s and this inv_s belong together.)
  * Where the band matrix-vector kernel serves the call (M <= 8, enough output rows) and can keep x
- * on chip (K = 4096, or M <= 2 and M * K small enough for shared memory), or where the chunked
- * tensor-core kernel serves it (see awq_linear_multi), the scaling happens while
+ * on chip (K = 4096, or M <= 2 and M * K small enough for shared memory), or where the stream
+ * kernel serves it (see awq_linear_multi), the scaling happens while
  * the kernel fetches x: no extra launch, no extra memory.  Otherwise x' is first written to
  * x_scratch (device, fp16 [M][K], caller-owned) by a small kernel and the plain call follows;
  * x_scratch may be NULL if awq_linear_scaled_needs_scratch(M, N, K, group) returns 0 (for the
- * multi call: N = the sum of the matrices' N), else AWQ_ERR_NULL_POINTER (whether the chunked kernel runs
+ * multi call: N = the sum of the matrices' N), else AWQ_ERR_NULL_POINTER (whether the stream kernel runs
  * depends on the registered workspace, so above 8 tokens the answer is always 1).
  */
 int awq_linear_scaled(const void* x, const float* inv_s, void* x_scratch, const void* qweight, const void* scales,
@@ -328,9 +331,9 @@ int awq_search_alpha(const void* W, const float* act_mean_abs, const void* X, in
  * awq_workspace_bytes: bytes awq_linear can use for this problem (0 if none).  For M <= 16 the
  * split-K matrix-vector kernel (small N) REQUIRES them.  For everything else they are OPTIONAL and
  * decide which kernel awq_linear takes:
- *  - the chunked kernels (AWQ_PATH_GEMV_MID up to 8 tokens, AWQ_PATH_GEMM_SKINNY up to 64) keep one
- *    fp32 [M][N] array of partial sums per chunk of K there; a second small kernel adds the chunks
- *    in ascending order.  Without a workspace of this size awq_linear takes the band
+ *  - the chunked matrix-vector kernel (AWQ_PATH_GEMV_MID, up to 8 tokens) keeps one fp32 [M][N] array of partial
+ *    sums per chunk of K there, the stream kernel (AWQ_PATH_GEMM_SKINNY, and up to 256 tokens) the
+ *    parts of the tiles that two or more SM pairs share; a second small kernel adds them in ascending order.  Without a workspace of this size awq_linear takes the band
  *    matrix-vector kernel (M <= 8) or the prefill kernels instead (same result within the
  *    tolerance, slower);
  *  - the one-SM prefill kernel (M <= 128) splits each tile's K loop over several SMs (up to 16

@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB_NAME = "libawq_b200.so"
 LIB_PATH = os.path.join(HERE, LIB_NAME)
 NATIVE_PATH = os.path.join(HERE, "_native.so")
-SOURCES = ("api.cu", "quantize_pack.cu", "gemv.cu", "gemv_mid.cu", "gemm_tcgen05.cu", "gemm_tcgen05_pair.cu", "gemm_skinny.cu", "search.cu")
+SOURCES = ("api.cu", "quantize_pack.cu", "gemv.cu", "gemv_mid.cu", "gemm_tcgen05.cu", "gemm_tcgen05_pair.cu", "gemm_stream.cu", "search.cu")
 NVCC_FLAGS = (
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "--std=c++17",
     "-Xcompiler", "-fPIC",

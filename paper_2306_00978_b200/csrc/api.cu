@@ -183,14 +183,38 @@ static bool mid_kernel_preferred(int M, int N, int K) {
     return M <= 8 && K > 4096 && nk >= (M <= 4 ? (1LL << 26) : (1LL << 25));
 }
 
-// Where the chunked tensor-core kernel runs: 9 .. 64 tokens, and below where the output rows are too few
-// for the band kernel.  Measured, us, against what ran there before: the chunked matrix-vector kernel with
-// more than one token fragment (4096 -> 4096 / 4096 -> 11008 / 11008 -> 4096 / 8192 -> 28672 at 16 tokens
-// 7.1 / 12.7 / 12.8 / 37.9 against 7.7 / 13.3 / 14.7 / 39.1, at 24 tokens 8.2 / 15.1 / 15.2 / 43.9 against
-// 9.7 / 16.8 / 18.3 / 52.0), and the split-K kernel (1024 -> 1024 at 4 / 8 tokens 4.5 / 4.5 against 7.9 /
-// 10.0, 2048 -> 1536 5.3 / 5.2 against 7.9 / 10.2).
-static bool skinny_kernel_preferred(int M, int total_n, int K, int group, int sms) {
-    return M <= 64 && (M > 8 || !gemv_uses_band_kernel(M, total_n, sms)) && gemm_skinny_applies(M, total_n, K, group);
+// Where the stream kernel runs up to 64 tokens: from 9, and below where the output rows are too few for the band kernel
+// (1024 -> 8192 at 3 / 8 tokens 4.8 / 4.9 us; the split-K kernel 8 and 10 us).  Calls of several matrices, which the chunked
+// matrix-vector kernel does not serve, take it from 4 tokens where x does not stay in the band kernel's registers (stream / band,
+// us: 11008 -> 4096 at 4 / 8 tokens 10.5 / 10.4 against 10.9 / 16.1, 8192 -> 28672 32.1 / 32.7 against 34.7 / 49.1).
+static bool stream_kernel_preferred(int M, int total_n, int K, int group, int sms, bool several = false) {
+    if (M > 64 || !gemm_stream_applies(M, total_n, K, group)) return false;
+    if (M > 8 || !gemv_uses_band_kernel(M, total_n, sms)) return true;
+    return several && M >= 4 && K > 4096 && (long long)total_n * K >= (1LL << 25);
+}
+
+// Above 64 tokens the stream kernel is taken where its estimate is 5 % below the prefill kernels' (few tiles for many
+// pairs, long rows): 4096 -> 4096 at 100 tokens 11.5 against 17.5 us, 11008 -> 4096 17.6 against 27.0, 28672 -> 8192
+// 59 against 175; at 200 tokens 11008 -> 4096 27 against 32, while 4096 -> 11008 keeps them (28 against 22).  Beyond two
+// tiles of 128 tokens they won everywhere.  The one-SM kernel keeps the shapes that it had.
+static bool stream_beats_prefill(const DeviceState* d, const AwqLinearProblem* problems, int count, int M, int K, int group) {
+    if (M <= 64 || M > 256) return false;
+    size_t have = 0;
+    {
+        std::lock_guard<std::mutex> lock(g_mutex);
+        have = d->workspace_bytes;
+    }
+    if (have < gemm_stream_workspace_bytes(M, d->sms)) return false;
+    double others = 0.0;
+    int slabs = 0;
+    for (int i = 0; i < count; ++i) {
+        bool one_sm = false;
+        if (!gemm_stream_applies(M, problems[i].N, K, group)) return false;
+        others += gemm_prefill_estimate(M, problems[i].N, K, group, d->sms, have, &one_sm);
+        if (one_sm) return false;
+        slabs += (problems[i].N + 255) / 256;
+    }
+    return 1.05 * gemm_stream_estimate(M, slabs, K, d->sms) < others;
 }
 
 static int resolve_path(int M, int K, int path) {
@@ -210,13 +234,13 @@ size_t awq_workspace_bytes(int M, int N, int K, int group) {
     }
     size_t gemm = gemm_workspace_bytes(M, N, sms);
     const size_t mid = (M <= 8 && gemv_mid_applies(M, N, K, group, sms)) ? gemv_mid_workspace_bytes(M, N, K) : 0;
-    const size_t skinny = skinny_kernel_preferred(M, N, K, group, sms) ? gemm_skinny_workspace_bytes(M, N, K, group, sms) : 0;
-    if (skinny > gemm) gemm = skinny;
+    const size_t parts = stream_kernel_preferred(M, N, K, group, sms) ? gemm_stream_workspace_bytes(M, sms) : 0;
+    if (parts > gemm) gemm = parts;
     if (M > 16) return gemm;
     size_t gemv = gemv_workspace_bytes(M);         // required by the split-K matrix-vector kernel
     if (M > 8) return gemv > gemm ? gemv : gemm;
     if (mid > gemv) gemv = mid;                    // awq_linear takes no prefill kernel here
-    return gemv > skinny ? gemv : skinny;
+    return gemv > parts ? gemv : parts;
 }
 
 int awq_set_workspace(void* dev_ptr, size_t bytes) {
@@ -250,14 +274,14 @@ int awq_linear_path(const void* x, const void* qweight, const void* scales, cons
     if (path == AWQ_PATH_GEMV_MID) {
         if (M > 32 || K > 65536) return AWQ_ERR_BAD_SHAPE;
     } else if (path == AWQ_PATH_GEMM_SKINNY) {
-        if (!gemm_skinny_applies(M, N, K, group)) return AWQ_ERR_BAD_SHAPE;
+        if ((M > 64 || !gemm_stream_applies(M, N, K, group))) return AWQ_ERR_BAD_SHAPE;
     } else if (path != AWQ_PATH_GEMM && path != AWQ_PATH_GEMM_1SM && (M > 16 || K > 65536)) {
         return AWQ_ERR_BAD_SHAPE;
     }
     DeviceState* d;
     if (int rc = device_state(&d)) return rc;
-    if (automatic && skinny_kernel_preferred(M, N, K, group, d->sms)) {
-        const size_t need = gemm_skinny_workspace_bytes(M, N, K, group, d->sms);
+    if (automatic && stream_kernel_preferred(M, N, K, group, d->sms)) {
+        const size_t need = gemm_stream_workspace_bytes(M, d->sms);
         std::lock_guard<std::mutex> lock(g_mutex);
         if (d->workspace_bytes >= need) path = AWQ_PATH_GEMM_SKINNY;
     }
@@ -265,7 +289,11 @@ int awq_linear_path(const void* x, const void* qweight, const void* scales, cons
         std::lock_guard<std::mutex> lock(g_mutex);
         if (d->workspace_bytes >= gemv_mid_workspace_bytes(M, N, K)) path = AWQ_PATH_GEMV_MID;
     }
-    if (path == AWQ_PATH_GEMV_MID && M > 8 && gemm_skinny_applies(M, N, K, group)) path = AWQ_PATH_GEMM_SKINNY;
+    if (path == AWQ_PATH_GEMM) {
+        const AwqLinearProblem one = {qweight, scales, zeros, y, N};
+        if (stream_beats_prefill(d, &one, 1, M, K, group)) path = AWQ_PATH_GEMM_SKINNY;
+    }
+    if (path == AWQ_PATH_GEMV_MID && M > 8 && gemm_stream_applies(M, N, K, group)) path = AWQ_PATH_GEMM_SKINNY;
     if (path == AWQ_PATH_GEMV_MID) {
         if (!gemv_mid_applies(M, N, K, group, d->sms)) return AWQ_ERR_BAD_SHAPE;
         void* ws = nullptr;
@@ -278,7 +306,7 @@ int awq_linear_path(const void* x, const void* qweight, const void* scales, cons
                                          take_packed_written(d), (cudaStream_t)stream));
     }
     if (path == AWQ_PATH_GEMM_SKINNY) {
-        const size_t need = gemm_skinny_workspace_bytes(M, N, K, group, d->sms);
+        const size_t need = gemm_stream_workspace_bytes(M, d->sms);
         void* ws = nullptr;
         {
             std::lock_guard<std::mutex> lock(g_mutex);
@@ -286,7 +314,7 @@ int awq_linear_path(const void* x, const void* qweight, const void* scales, cons
             ws = d->workspace;
         }
         const GemvMatrix one = {qweight, scales, zeros, y, N};
-        return note_cuda(launch_gemm_skinny(x, &one, 1, M, K, group, nullptr, ws, d->status_word,
+        return note_cuda(launch_gemm_stream(x, &one, 1, M, K, group, nullptr, ws, d->status_word,
                                             d->sms, take_packed_written(d), (cudaStream_t)stream));
     }
     const bool tensor_path = path == AWQ_PATH_GEMM || path == AWQ_PATH_GEMM_1SM;
@@ -367,10 +395,10 @@ int awq_static_scratch_fill(int value, void* stream) {
     return note_cuda(cudaMemsetAsync(scratch, value & 0xFF, kCounterBytes, (cudaStream_t)stream));
 }
 
-// All matrices in one launch of the chunked tensor-core kernel, if the workspace holds their partial sums.
-static int linear_multi_skinny(DeviceState* d, const void* x, const float* inv_s, const AwqLinearProblem* problems,
-                               int count, int total_n, int M, int K, int group, void* stream, bool* launched) {
-    const size_t need = gemm_skinny_workspace_bytes(M, total_n, K, group, d->sms);
+// All matrices in one launch of the stream kernel, if the workspace holds their partial sums.
+static int linear_multi_stream(DeviceState* d, const void* x, const float* inv_s, const AwqLinearProblem* problems,
+                               int count, int M, int K, int group, void* stream, bool* launched) {
+    const size_t need = gemm_stream_workspace_bytes(M, d->sms);
     void* ws = nullptr;
     {
         std::lock_guard<std::mutex> lock(g_mutex);
@@ -381,7 +409,7 @@ static int linear_multi_skinny(DeviceState* d, const void* x, const float* inv_s
     for (int i = 0; i < count; ++i)
         mats[i] = GemvMatrix{problems[i].qweight, problems[i].scales, problems[i].zeros, problems[i].y, problems[i].N};
     *launched = true;
-    return note_cuda(launch_gemm_skinny(x, mats, count, M, K, group, inv_s, ws, d->status_word, d->sms,
+    return note_cuda(launch_gemm_stream(x, mats, count, M, K, group, inv_s, ws, d->status_word, d->sms,
                                         take_packed_written(d), (cudaStream_t)stream));
 }
 
@@ -403,6 +431,11 @@ int awq_linear_multi(const void* x, const AwqLinearProblem* problems, int count,
     if (!aligned16(x)) return AWQ_ERR_MISALIGNED;
     DeviceState* d;
     if (int rc = device_state(&d)) return rc;
+    if (stream_kernel_preferred(M, total_n, K, group, d->sms, count > 1) || (count > 1 && stream_beats_prefill(d, problems, count, M, K, group))) {
+        bool launched = false;
+        const int rc = linear_multi_stream(d, x, nullptr, problems, count, M, K, group, stream, &launched);
+        if (rc != AWQ_OK || launched) return rc;
+    }
     if (M <= 8 && K <= 65536 && gemv_uses_band_kernel(M, total_n, d->sms)) {
         GemvMatrix mats[kMaxMulti];
         for (int i = 0; i < count; ++i)
@@ -410,11 +443,6 @@ int awq_linear_multi(const void* x, const AwqLinearProblem* problems, int count,
                                  problems[i].N};
         return note_cuda(launch_gemv_band(x, mats, count, M, K, group, d->status_word, d->sms,
                                           take_packed_written(d), (cudaStream_t)stream));
-    }
-    if (skinny_kernel_preferred(M, total_n, K, group, d->sms)) {
-        bool launched = false;
-        const int rc = linear_multi_skinny(d, x, nullptr, problems, count, total_n, M, K, group, stream, &launched);
-        if (rc != AWQ_OK || launched) return rc;
     }
     // otherwise one call per matrix, as awq_linear would run it
     for (int i = 0; i < count; ++i) {
@@ -473,9 +501,9 @@ int awq_linear_multi_scaled(const void* x, const float* inv_s, void* x_scratch, 
                                           take_packed_written(d), (cudaStream_t)stream, inv_s));
     }
     if (!x_scratch) return AWQ_ERR_NULL_POINTER;
-    if (skinny_kernel_preferred(M, total_n, K, group, d->sms)) {
+    if (stream_kernel_preferred(M, total_n, K, group, d->sms, count > 1) || stream_beats_prefill(d, problems, count, M, K, group)) {
         bool launched = false;
-        const int rc = linear_multi_skinny(d, x, inv_s, problems, count, total_n, M, K, group, stream, &launched);
+        const int rc = linear_multi_stream(d, x, inv_s, problems, count, M, K, group, stream, &launched);
         if (rc != AWQ_OK || launched) return rc;
     }
     // no kernel to fold it into: scale first (one more launch), then the plain calls

@@ -81,9 +81,8 @@ cudaError_t launch_gemv_mid(const void* x, const void* qweight, const void* scal
                             int M, int N, int K, int group, void* workspace, unsigned int* status_word, int sms,
                             bool serialize, cudaStream_t st);
 
-// The chunked kernels (gemv_mid.cu, gemm_skinny.cu): first unit of every block (and the end of the
-// last one); units are in chunk-major order.  unit_starts is gemv_mid.cu's rule (gemm_skinny.cu cuts its ranges by
-// an estimate), `per_chunk` units per chunk of K.  Blocks start in index order, the last
+// The chunked kernel (gemv_mid.cu): first unit of every block (and the end of the last one); units are in
+// chunk-major order, `per_chunk` units per chunk of K.  Blocks start in index order, the last
 // ones on the SMs that the launch in front of this one frees last, so the blocks that hold one unit
 // more than the others are the first ones - except where the longer range would cross into the next
 // chunk, which costs a second slice of x (measured on 28672 -> 8192 at 8 tokens: 6 units 22.4 us, 7
@@ -136,14 +135,15 @@ __device__ __forceinline__ float4 add_chunks(const float* p, int chunks, size_t 
 // launched with programmatic stream serialization behind the kernel that wrote the partial sums
 cudaError_t launch_chunk_reduce(const float* partial, void* y, int chunks, size_t mn, cudaStream_t st);
 
-// 9 .. 64 tokens, and fewer on few output rows, on the tensor cores (gemm_skinny.cu): units of one 128-channel slab x one chunk of
-// K, the chunk's slice of x resident in shared memory, partial sums per chunk in the workspace
-bool gemm_skinny_applies(int M, int N, int K, int group);
-// `count` matrices (1..kMaxMulti) sharing x, K and the group size in one launch (N: the sum of theirs);
+// The stream kernel (gemm_stream.cu): 9 tokens and more, and fewer on few output rows, on the tensor cores of SM pairs;
+// the tiles' K loops laid end to end and cut into one range per pair, partial sums in the workspace.
+bool gemm_stream_applies(int M, int N, int K, int group);
+// `count` matrices (1..kMaxMulti) sharing x, K and the group size in one launch;
 // inv_s: nullptr, or the inverse channel scales (fp32 [K], device), multiplied into x on the way.
 // Up to 32 tokens q - z enters the products as an integer and Delta is applied in fp32; above, fp16 (q - z) * Delta does.
-size_t gemm_skinny_workspace_bytes(int M, int N, int K, int group, int sms);
-cudaError_t launch_gemm_skinny(const void* x, const GemvMatrix* mats, int count, int M, int K, int group,
+size_t gemm_stream_workspace_bytes(int M, int sms);
+double gemm_stream_estimate(int M, int slabs, int K, int sms);     // us, above 64 tokens; slabs of 256 channels, all matrices'
+cudaError_t launch_gemm_stream(const void* x, const GemvMatrix* mats, int count, int M, int K, int group,
                                const float* inv_s, void* workspace, unsigned int* status_word, int sms,
                                bool serialize, cudaStream_t st);
 
@@ -169,6 +169,8 @@ cudaError_t launch_gemm(const void* x, const void* qweight, const void* scales, 
                         void* y, int M, int N, int K, int group, bool path_pair_allowed,
                         void* workspace, size_t workspace_bytes,
                         unsigned int* status_word, cudaStream_t st);
+// what launch_gemm takes, us (an estimate that ranks), and whether it is the one-SM kernel
+double gemm_prefill_estimate(int M, int N, int K, int group, int sms, size_t workspace_bytes, bool* one_sm);
 // optional workspace of the tensor-core path (0 if the shape has no use for one)
 size_t gemm_workspace_bytes(int M, int N, int sms);
 

@@ -506,6 +506,12 @@ cudaError_t launch_gemm(const void* x, const void* qweight, const void* scales, 
 #undef AWQ_GEMM_CASE
 }
 
+double gemm_prefill_estimate(int M, int N, int K, int group, int sms, size_t workspace_bytes, bool* one_sm) {
+    const int bn = M > 128 ? 256 : 128;
+    *one_sm = one_sm_preferred(M, N, K, gemm_splits(M, N, K, group, bn, sms, workspace_bytes), sms, workspace_bytes);
+    return gemm_pair_estimate(M, N, K, sms, workspace_bytes);
+}
+
 size_t gemm_workspace_bytes(int M, int N, int sms) {
     if (gemm_pair_applies(M, N)) return gemm_pair_workspace_bytes(sms);
     // split-K of the one-SM kernel: the most it can use for this M and N (any K)
