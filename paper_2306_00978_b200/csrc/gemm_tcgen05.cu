@@ -89,7 +89,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ C
     auto acc_full = [&](int b) { return bars + 8u * (uint32_t)(3 * S + b); };
     auto acc_empty = [&](int b) { return bars + 8u * (uint32_t)(3 * S + 2 + b); };
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (the shuffle tells the compiler that all lanes of a warp take the same role: addresses stay in uniform registers)
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int m_tiles = (M + BN - 1) / BN;
     const int total_tiles = (N / 128) * m_tiles;
     // split-K: a work item is (tile, split); split sp of a tile covers the groups

@@ -181,7 +181,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     auto acc_full = [&](uint32_t b) { return bars + 8u * ((uint32_t)(3 * S + SL) + b); };        // accumulator complete
     auto acc_empty = [&](uint32_t b) { return bars + 8u * ((uint32_t)(3 * S + SL + 2) + b); };   // leader: accumulator drained
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (the shuffle tells the compiler that all lanes of a warp take the same role: addresses stay in uniform registers)
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const int m_tiles = (M + BN - 1) / BN;
     const int total_tiles = ((N + 255) / 256) * m_tiles;     // an odd last slab of 128 channels pairs with an absent one
@@ -213,7 +214,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     __syncthreads();
     cluster_sync_all();                      // both blocks' barriers exist before anyone arrives remotely
     tc_fence_after();
-    const uint32_t tmem_base = s_tmem_base;
+    constexpr uint32_t tmem_base = 0;        // all 512 columns are this block's
     const WaitCtl ctl{status_word, &s_abort};
 
     if (warp == 0) {
