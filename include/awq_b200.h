@@ -309,8 +309,9 @@ int awq_static_scratch_fill(int value, void* stream);
  * the paper does not name its norm: the mean squared difference has the same minimizer as any other
  * monotone function of the Frobenius norm).  The quantizer and the layer are the library's own
  * kernels, so the search scores exactly what deployment runs; the fp16 reference product W X is a
- * dense GEMM kernel of this library with fp32 accumulation and output.  Nothing is allocated: all
- * intermediate arrays live in `scratch`.  The paper uses 20 grid points over [0, 1]; the grid is the
+ * dense GEMM kernel of this library with fp32 accumulation and output.  Grid points are evaluated several at a
+ * time, as many as 384 MB of x / s, packed arrays and y hold (above 64 tokens their products are one launch of the
+ * SM-pair kernel).  Nothing is allocated: all intermediate arrays live in `scratch`.  The paper uses 20 grid points over [0, 1]; the grid is the
  * caller's.
  * W: in, fp16 [N][K] (device).  act_mean_abs: in, fp32 [K] (device).  X: in, fp16 [M][K] calibration
  * activations (device), M >= 1.  alphas: in, HOST array of n_alphas <= 64 values in [0, 1].

@@ -32,6 +32,7 @@ cudaError_t launch_quantize_pack(const __half* W, const float* a, float alpha, i
                                  bool symmetric, const float* clip, uint32_t* qweight, __half* scales, uint8_t* zeros,
                                  int N, int K, cudaStream_t st);
 constexpr int kMaxClipRatios = 32;
+constexpr int kMaxSearchAlphas = 64;
 // ratios: HOST array of n_ratios <= kMaxClipRatios values; clip: device out, fp32 [N][K/group]
 cudaError_t launch_clip_search(const __half* W, const float* a, float alpha, int group, int bits,
                                const float* ratios, int n_ratios, float* clip, int N, int K,
@@ -148,18 +149,41 @@ cudaError_t launch_gemm_stream(const void* x, const GemvMatrix* mats, int count,
                                bool serialize, cudaStream_t st);
 
 // scale search (search.cu)
-constexpr int kMaxSearchAlphas = 64;
-size_t search_scratch_bytes(int M, int N, int K, int group);
-void search_carve(void* base, int M, int N, int K, int group, float** s, void** xs, void** qweight,
-                  void** scales, void** zeros, void** yq, float** yref, double** partials, float** losses);
+// Scratch of a search: `batch` grid points at a time, each with `rows` >= M rows of x / s and y and packed arrays of its own.
+struct SearchPlan {
+    int batch, rows;
+    float* s;                                // [kMaxSearchAlphas][K]
+    __half* xs;
+    unsigned char* qweight;
+    unsigned char* scales;
+    unsigned char* zeros;
+    __half* yq;
+    float* yref;
+    double* partials;
+    float* losses;
+    size_t total;
+};
+SearchPlan search_plan(void* scratch, int M, int N, int K, int group);
 cudaError_t launch_reference_product(const void* W, const void* X, float* yref, int M, int N, int K,
                                      cudaStream_t st);
-cudaError_t launch_divide_by_scale(const void* X, const float* s, void* xs, int M, int K, cudaStream_t st);
+// xs[i] = fp16_rne(fp32(X) / s[i]) for `count` scale arrays, `rows` rows apart
+cudaError_t launch_divide_by_scale(const void* X, const float* s, int count, void* xs, int M, int rows, int K, cudaStream_t st);
 // xs = fp16_rne(fp32(X) * inv_s); inverse_scale: inv_s = fp32(1 / s), correctly rounded
 cudaError_t launch_multiply_by_inverse(const void* X, const float* inv_s, void* xs, int M, int K, cudaStream_t st);
 cudaError_t launch_inverse_scale(const float* s, float* inv_s, int K, cudaStream_t st);
-cudaError_t launch_mean_squared_difference(const void* yq, const float* yref, size_t n, double* partials,
-                                           float* out, cudaStream_t st);
+// partial sums of (yq[i] - yref)^2 for `count` arrays (search_partials(plan, first) is where the first one's go), then the means
+cudaError_t launch_squared_difference(const void* yq, const float* yref, int count, int M, int rows, int N, double* partials,
+                                      cudaStream_t st);
+cudaError_t launch_losses(const double* partials, int count, size_t n, float* losses, cudaStream_t st);
+double* search_partials(const SearchPlan& p, int first);
+// s[i] of n alphas (a HOST array); W quantized with each of `count` scale arrays, packed arrays end to end
+cudaError_t launch_channel_scales(const float* a, const float* alphas, int n, float* s, int K, cudaStream_t st);
+cudaError_t launch_quantize_pack_many(const __half* W, const float* s, int count, int group, uint32_t* qweight, __half* scales,
+                                      uint8_t* zeros, int N, int K, cudaStream_t st);
+// `count` products of the same shape in one launch (gemm_tcgen05.cu)
+cudaError_t launch_gemm_blocks(const void* x, const void* qweight, const void* scales, const void* zeros, void* y, int count,
+                               int M, int rows, int N, int K, int group, void* workspace, size_t workspace_bytes,
+                               unsigned int* status_word, int sms, cudaStream_t st, bool* launched);
 
 // the matrix-vector kernel's built-in scratch (no allocation): address on the current device
 cudaError_t gemv_static_scratch(void** out);

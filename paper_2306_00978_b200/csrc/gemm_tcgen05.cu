@@ -507,6 +507,30 @@ cudaError_t launch_gemm(const void* x, const void* qweight, const void* scales, 
 #undef AWQ_GEMM_CASE
 }
 
+// `count` products with x [rows] x K, N channels and y [rows] x N each (M of the rows are used; rows a multiple of 32, N of
+// 256), all arrays end to end, in one launch of the SM-pair kernel.  *launched is false where it cannot run.
+cudaError_t launch_gemm_blocks(const void* x, const void* qweight, const void* scales, const void* zeros, void* y, int count,
+                               int M, int rows, int N, int K, int group, void* workspace, size_t workspace_bytes,
+                               unsigned int* status_word, int sms, cudaStream_t st, bool* launched) {
+    EncodeTiledFn enc = encode_fn();
+    *launched = false;
+    if (!enc || N % 256 != 0 || rows % 32 != 0) return cudaSuccess;
+    const cuuint32_t estr[2] = {1, 1};
+    CUtensorMap wmap, ymap;
+    const cuuint64_t wdims[2] = {(cuuint64_t)K * 2, (cuuint64_t)count * (N / 16)}, wstrides[1] = {(cuuint64_t)K * 8};
+    const cuuint32_t wbox[2] = {256, 8};
+    const cuuint64_t ydims[2] = {(cuuint64_t)N, (cuuint64_t)count * rows}, ystrides[1] = {(cuuint64_t)N * 2};
+    const cuuint32_t ybox[2] = {32, 32};
+    if (enc(&wmap, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<void*>(qweight), wdims, wstrides, wbox, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
+        enc(&ymap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, y, ydims, ystrides, ybox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    return launch_gemm_pair(x, wmap, ymap, scales, zeros, M, count * N, K, group, workspace, workspace_bytes, status_word, sms,
+                            st, launched, count, rows);
+}
+
 double gemm_prefill_estimate(int M, int N, int K, int group, int sms, size_t workspace_bytes, bool* one_sm) {
     const int bn = M > 128 ? 256 : 128;
     *one_sm = one_sm_preferred(M, N, K, gemm_splits(M, N, K, group, bn, sms, workspace_bytes), sms, workspace_bytes);

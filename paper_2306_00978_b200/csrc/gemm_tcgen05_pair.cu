@@ -150,6 +150,14 @@ __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
     return v;
 }
 
+// Several products of the same shape end to end (the scale search): their channels stacked in the packed arrays, each with
+// `rows` rows of x and y of its own.  One product: all slabs, rows 0.
+struct PairBlocks {
+    int slabs;                       // 256-channel slabs of a product
+    int n;                           // its channels
+    int rows;                        // rows from a product's x (and y) to the next one's
+};
+
 // ------------------------------------------------------------------------- the kernel
 template <int G, int BN>
 __global__ void __launch_bounds__(PairCfg<BN>::kThreads, 1)
@@ -157,7 +165,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                  const __grid_constant__ CUtensorMap y_map,
                  const __half* __restrict__ scales, const unsigned char* __restrict__ zeros,
                  int M, int N, int K, unsigned int* status_word,
-                 float* partials, unsigned int* flags) {
+                 float* partials, unsigned int* flags, const PairBlocks blocks) {
     using Cfg = PairCfg<BN>;
     constexpr int S = Cfg::kStages, SL = Cfg::kSlots;
     constexpr uint32_t NACC = Cfg::kNumAcc;
@@ -226,7 +234,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         bool ok = true;
         while (ok && pieces.next(tile, k0, k1)) {
             const int slab = (tile / m_tiles) * 2 + (int)rank;              // 128-channel slab of this block
-            const int tok0 = (tile % m_tiles) * BN + (int)rank * Cfg::kHalf;
+            const int tok0 = (tile / m_tiles / blocks.slabs) * blocks.rows + (tile % m_tiles) * BN + (int)rank * Cfg::kHalf;
             for (int ks = k0; ks < k1; ++ks) {
                 if (!mbar_wait_warp(empty(stage), phase ^ 1u, ctl)) { ok = false; break; }
                 if (lead) {
@@ -386,7 +394,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         int obuf = 0;
         bool ok = true;
         while (ok && pieces.next(tile, k0, k1)) {
-            const int slab = (tile / m_tiles) * 2 + (int)rank, mt = tile % m_tiles;
+            const int block = tile / m_tiles / blocks.slabs, mt = tile % m_tiles;
+            const int slab = (tile / m_tiles - block * blocks.slabs) * 2 + (int)rank;
             // A piece that does not start the tile is a contribution: its fp32 sums go to this pair's
             // slot of the workspace.  A piece that starts the tile but does not end it waits for the
             // contributions of the pairs after this one (they were produced at the start of those
@@ -463,7 +472,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 }
                 // stage the 32 x 32 block as [token][channel] fp16 and hand it to the copy engine
                 // (rows past M are clipped by the tensor map; blocks that lie outside y are left out)
-                if (n0 >= N || m0 + c >= M) continue;
+                if (n0 >= blocks.n || m0 + c >= M) continue;
                 if (lane == 0) bulk_wait_read_1();                  // the store that last used this buffer
                 __syncwarp();
                 const uint32_t tb = out_base + (uint32_t)(((half * 4 + quad) * 2 + obuf) * 2048);
@@ -474,7 +483,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                    tma_store_2d(&y_map, n0, m0 + c, tb);
+                    tma_store_2d(&y_map, n0, block * blocks.rows + m0 + c, tb);
                     bulk_commit_group();
                 }
                 obuf ^= 1;
@@ -545,7 +554,7 @@ int resident_pairs(int sms, cudaError_t* err) {
 template <int G, int BN>
 cudaError_t launch_pair(const CUtensorMap& xmap, const CUtensorMap& wmap, const CUtensorMap& ymap,
                         const void* scales, const void* zeros, int M, int N, int K, bool streamk,
-                        void* workspace, size_t workspace_bytes,
+                        void* workspace, size_t workspace_bytes, const PairBlocks& blocks,
                         unsigned int* status_word, int sms, cudaStream_t st, bool* launched) {
     using Cfg = PairCfg<BN>;
     cudaError_t e;
@@ -574,7 +583,7 @@ cudaError_t launch_pair(const CUtensorMap& xmap, const CUtensorMap& wmap, const 
                               : nullptr;
     unsigned int* flags = static_cast<unsigned int*>(workspace);
     e = cudaLaunchKernelEx(&cfg, gemm_pair_kernel<G, BN>, xmap, wmap, ymap, reinterpret_cast<const __half*>(scales),
-                           reinterpret_cast<const unsigned char*>(zeros), M, N, K, status_word, partials, flags);
+                           reinterpret_cast<const unsigned char*>(zeros), M, N, K, status_word, partials, flags, blocks);
     if (e != cudaSuccess) return e;
     count_launch();
     *launched = true;
@@ -641,12 +650,13 @@ double gemm_pair_estimate(int M, int N, int K, int sms, size_t workspace_bytes) 
 cudaError_t launch_gemm_pair(const void* x, const CUtensorMap& wmap, const CUtensorMap& ymap,
                              const void* scales, const void* zeros, int M, int N, int K, int group,
                              void* workspace, size_t workspace_bytes,
-                             unsigned int* status_word, int sms, cudaStream_t st, bool* launched) {
+                             unsigned int* status_word, int sms, cudaStream_t st, bool* launched, int count, int rows) {
+    const PairBlocks blocks = {(N / count + 255) / 256, N / count, rows};
     const PairChoice c = choose_tile(M, N, K, sms / 2, workspace ? workspace_bytes : 0);
     CUtensorMap xmap;
     {
         // x as [M][K] fp16 in boxes of half a tile's tokens x one k-block, 128-byte swizzle
-        const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)M};
+        const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)(count > 1 ? (long long)count * rows : M)};
         const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
         const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)(c.bn / 2)}, estr[2] = {1, 1};
         if (encode_fn()(&xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(x), dims, strides, box, estr,
@@ -655,7 +665,7 @@ cudaError_t launch_gemm_pair(const void* x, const CUtensorMap& wmap, const CUten
             return cudaErrorInvalidValue;
     }
 #define AWQ_PAIR_CASE(GG, BNN)                                                                                     \
-    return launch_pair<GG, BNN>(xmap, wmap, ymap, scales, zeros, M, N, K, c.streamk, workspace, workspace_bytes,  \
+    return launch_pair<GG, BNN>(xmap, wmap, ymap, scales, zeros, M, N, K, c.streamk, workspace, workspace_bytes, blocks, \
                                 status_word, sms, st, launched)
     if (group == 128) {
         switch (c.bn) { case 64: AWQ_PAIR_CASE(128, 64); case 128: AWQ_PAIR_CASE(128, 128);

@@ -29,6 +29,16 @@ __global__ void channel_scale_kernel(const float* __restrict__ a, float alpha, i
     if (k < K) s[k] = channel_scale_one(mode == kAlphaZero ? 1.0f : a[k], alpha, mode);
 }
 
+// s of several alphas: blockIdx.y counts them
+struct Alphas {
+    float v[kMaxSearchAlphas];
+    int mode[kMaxSearchAlphas];
+};
+__global__ void channel_scales_kernel(const float* __restrict__ a, const __grid_constant__ Alphas alphas, float* __restrict__ s, int K) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y, mode = alphas.mode[i];
+    if (k < K) s[(size_t)i * K + k] = channel_scale_one(mode == kAlphaZero ? 1.0f : a[k], alphas.v[i], mode);
+}
+
 __device__ __forceinline__ uint2 ldg_stream(const uint2* p) {
     uint2 v;
     asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
@@ -115,12 +125,14 @@ template <int G> struct QCfg {
     static constexpr int kStored = G < 128 ? G : 128;               // columns per stored scale / zero point
 };
 
-template <int G, int BITS, bool CLIP, bool SYM>
-__global__ void __launch_bounds__(QCfg<G>::kThreads, 1024 / QCfg<G>::kThreads)
+// MANY (the scale search): `a` is `many` arrays of K scales; W is quantized with each, its 32 values per lane loaded once,
+// and the packed arrays follow one another (4096 x 4096 with 20 arrays: 12.3 us each in launches of their own, 9.9 us here).
+template <int G, int BITS, bool CLIP, bool SYM, bool MANY = false>
+__global__ void __launch_bounds__(QCfg<G>::kThreads, (MANY ? 640 : 1024) / QCfg<G>::kThreads)
 quantize_pack_tile_kernel(const __half* __restrict__ W, const float* __restrict__ a, float alpha,
                           int mode, const float* __restrict__ clip,
                           uint32_t* __restrict__ qweight, __half* __restrict__ scales,
-                          uint8_t* __restrict__ zeros, int N, int K) {
+                          uint8_t* __restrict__ zeros, int N, int K, int many) {
     constexpr float top = (float)((1 << BITS) - 1);       // largest code
     constexpr int kQBands = QCfg<G>::kBands, kQBlocks = QCfg<G>::kBlocks, kQThreads = QCfg<G>::kThreads;
     __shared__ __align__(16) float s_sm[kQBlocks * 64];
@@ -139,9 +151,19 @@ quantize_pack_tile_kernel(const __half* __restrict__ W, const float* __restrict_
         for (int j = 0; j < 4; ++j)
             raw[h][j] = ldg_stream(reinterpret_cast<const uint2*>(
                 W + (size_t)(n0 + 8 * h) * K + kbase + ti * 64 + 16 * j + 4 * t));
-    for (int i = threadIdx.x; i < kQBlocks * 64; i += kQThreads) {
-        const int k = kbase + i;
-        s_sm[i] = channel_scale_one(mode == kAlphaZero ? 1.0f : a[k], alpha, mode);
+    static_assert(!MANY || kQBlocks * 64 == kQThreads, "one scale per thread");
+    float s_next = 0.0f;
+    if (MANY) s_next = a[kbase + (int)threadIdx.x];
+    for (int rest = MANY ? many : 1; rest > 0; --rest) {
+    if (MANY) {
+        s_sm[threadIdx.x] = s_next;
+        a += K;
+        if (rest > 1) s_next = a[kbase + (int)threadIdx.x];
+    } else {
+        for (int i = threadIdx.x; i < kQBlocks * 64; i += kQThreads) {
+            const int k = kbase + i;
+            s_sm[i] = channel_scale_one(mode == kAlphaZero ? 1.0f : a[k], alpha, mode);
+        }
     }
     __syncthreads();
 
@@ -278,6 +300,13 @@ quantize_pack_tile_kernel(const __half* __restrict__ W, const float* __restrict_
         scales[(band * nsg + sgi) * 16 + g + 8] = d16[1];
         zeros[((band >> 1) * nsg + sgi) * 16 + (band & 1) * 8 + g] =
             (uint8_t)((uint32_t)z[0] | ((uint32_t)z[1] << 4));
+    }
+    if (MANY) {
+        qweight += (size_t)N * K / 8;
+        scales += (size_t)N * (K / QCfg<G>::kStored);
+        zeros += (size_t)N * (K / QCfg<G>::kStored) / 2;
+        __syncthreads();                                     // s_sm and s_mm have been read
+    }
     }
 }
 
@@ -487,13 +516,33 @@ cudaError_t launch_channel_scale(const float* a, float alpha, float* s, int K, c
     return cudaGetLastError();
 }
 
+cudaError_t launch_channel_scales(const float* a, const float* alphas, int n, float* s, int K, cudaStream_t st) {
+    Alphas list = {};
+    for (int i = 0; i < n; ++i) { list.v[i] = alphas[i]; list.mode[i] = (int)alpha_mode(alphas[i]); }
+    channel_scales_kernel<<<dim3((K + 255) / 256, n), 256, 0, st>>>(a, list, s, K);
+    count_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_quantize_pack_many(const __half* W, const float* s, int count, int group, uint32_t* qweight, __half* scales,
+                                      uint8_t* zeros, int N, int K, cudaStream_t st) {
+    if (group == 64)
+        quantize_pack_tile_kernel<64, 4, false, false, true><<<dim3(K / 128, N / (16 * QCfg<64>::kBands)), QCfg<64>::kThreads, 0, st>>>(
+            W, s, 1.0f, kAlphaOne, nullptr, qweight, scales, zeros, N, K, count);
+    else
+        quantize_pack_tile_kernel<128, 4, false, false, true><<<dim3(K / 128, N / (16 * QCfg<128>::kBands)), QCfg<128>::kThreads, 0, st>>>(
+            W, s, 1.0f, kAlphaOne, nullptr, qweight, scales, zeros, N, K, count);
+    count_launch();
+    return cudaGetLastError();
+}
+
 cudaError_t launch_quantize_pack(const __half* W, const float* a, float alpha, int group, int bits,
                                  bool symmetric, const float* clip, uint32_t* qweight, __half* scales, uint8_t* zeros,
                                  int N, int K, cudaStream_t st) {
     const int mode = (int)alpha_mode(alpha);
 #define AWQ_QP_LAUNCH(GG, BB, CC, SS)                                                                           \
     quantize_pack_tile_kernel<GG, BB, CC, SS><<<dim3(K / (QCfg<GG>::kBlocks * 64), N / (16 * QCfg<GG>::kBands)), \
-                                                QCfg<GG>::kThreads, 0, st>>>(W, a, alpha, mode, clip, qweight, scales, zeros, N, K)
+                                                QCfg<GG>::kThreads, 0, st>>>(W, a, alpha, mode, clip, qweight, scales, zeros, N, K, 1)
 #define AWQ_QP_PICK2(GG, SS)                                             \
     do {                                                                 \
         if (bits == 4 && !clip) AWQ_QP_LAUNCH(GG, 4, false, SS);         \

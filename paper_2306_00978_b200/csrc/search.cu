@@ -11,27 +11,30 @@ namespace awq {
 
 namespace {
 
-constexpr int kLossBlocks = 1024;
+constexpr int kLossBlocks = 296;
 
-// xs[m][k] = fp16_rne(fp32(X[m][k]) / s[k]): the caller's side of Eq. 4, one IEEE division and
-// one rounding per element; eight elements per thread (K is a multiple of 128).
+// xs[b][m][k] = fp16_rne(fp32(X[m][k]) / s[b][k]): the caller's side of Eq. 4, one IEEE division and
+// one rounding per element; eight elements per thread (K is a multiple of 128), one scale array per blockIdx.y.
 __global__ void divide_by_scale_kernel(const __half* __restrict__ X, const float* __restrict__ s,
-                                       __half* __restrict__ xs, size_t chunks, int K) {
+                                       __half* __restrict__ xs, size_t chunks, size_t block_chunks, int K) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= chunks) return;
+    s += (size_t)blockIdx.y * K;
     const int k0 = (int)((i * 8) % (size_t)K);
     const uint4 h = reinterpret_cast<const uint4*>(X)[i];
     const uint32_t w[4] = {h.x, h.y, h.z, h.w};
+    const float4 s0 = *reinterpret_cast<const float4*>(s + k0), s1 = *reinterpret_cast<const float4*>(s + k0 + 4);
+    const float sk[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
     uint32_t o[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         const float lo = __half2float(__ushort_as_half((unsigned short)(w[e] & 0xFFFFu)));
         const float hi = __half2float(__ushort_as_half((unsigned short)(w[e] >> 16)));
-        const unsigned short a = __half_as_ushort(__float2half_rn(__fdiv_rn(lo, s[k0 + 2 * e])));
-        const unsigned short b = __half_as_ushort(__float2half_rn(__fdiv_rn(hi, s[k0 + 2 * e + 1])));
+        const unsigned short a = __half_as_ushort(__float2half_rn(__fdiv_rn(lo, sk[2 * e])));
+        const unsigned short b = __half_as_ushort(__float2half_rn(__fdiv_rn(hi, sk[2 * e + 1])));
         o[e] = (uint32_t)a | ((uint32_t)b << 16);
     }
-    reinterpret_cast<uint4*>(xs)[i] = make_uint4(o[0], o[1], o[2], o[3]);
+    reinterpret_cast<uint4*>(xs)[blockIdx.y * block_chunks + i] = make_uint4(o[0], o[1], o[2], o[3]);
 }
 
 // xs[m][k] = fp16_rne(fp32(X[m][k]) * inv_s[k]): what awq_linear_scaled computes inside the layer,
@@ -57,59 +60,67 @@ __global__ void inverse_scale_kernel(const float* __restrict__ s, float* __restr
     if (k < K) inv_s[k] = __frcp_rn(s[k]);
 }
 
-// Sum of (y_q - y_ref)^2: every block adds a fixed, interleaved share of the elements in fp64
-// and the last kernel adds the blocks' sums in block order, so the loss is reproducible.
-__global__ void __launch_bounds__(256)
-sqdiff_partial_kernel(const __half* __restrict__ yq, const float* __restrict__ yref, size_t n,
-                      double* __restrict__ partials) {
+// Sums of (y_q - y_ref)^2, one y_q per blockIdx.y: every block adds a fixed, interleaved share of the elements in fp64
+// (eight at a time: N is a multiple of 128) and the last kernel adds the blocks' sums in a fixed tree, so the loss is
+// reproducible.  (One element at a time and one thread for the last step: 30 us of a grid point's 85.)
+__device__ __forceinline__ double block_sum(double acc) {
     __shared__ double s_sum[256];
-    double acc = 0.0;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float d = __half2float(yq[i]) - yref[i];
-        acc += (double)d * (double)d;
-    }
     s_sum[threadIdx.x] = acc;
     __syncthreads();
     for (int off = 128; off >= 1; off >>= 1) {
         if ((int)threadIdx.x < off) s_sum[threadIdx.x] += s_sum[threadIdx.x + off];
         __syncthreads();
     }
-    if (threadIdx.x == 0) partials[blockIdx.x] = s_sum[0];
+    return s_sum[0];
 }
-__global__ void sqdiff_final_kernel(const double* __restrict__ partials, int blocks, double inv_count,
-                                    float* __restrict__ out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+__global__ void __launch_bounds__(256)
+sqdiff_partial_kernel(const __half* __restrict__ yq, const float* __restrict__ yref, size_t chunks, size_t block_chunks,
+                      double* __restrict__ partials) {
+    const uint4* y = reinterpret_cast<const uint4*>(yq) + blockIdx.y * block_chunks;
+    double acc = 0.0;
+    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < chunks; i += (size_t)gridDim.x * 256) {
+        const uint4 h = y[i];
+        const float4 r0 = reinterpret_cast<const float4*>(yref)[2 * i], r1 = reinterpret_cast<const float4*>(yref)[2 * i + 1];
+        const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&h.x)), b = __half22float2(*reinterpret_cast<const __half2*>(&h.y));
+        const float2 c = __half22float2(*reinterpret_cast<const __half2*>(&h.z)), d = __half22float2(*reinterpret_cast<const __half2*>(&h.w));
+        const float e[8] = {a.x - r0.x, a.y - r0.y, b.x - r0.z, b.y - r0.w, c.x - r1.x, c.y - r1.y, d.x - r1.z, d.y - r1.w};
+#pragma unroll
+        for (int k = 0; k < 8; ++k) acc += (double)e[k] * (double)e[k];
+    }
+    const double sum = block_sum(acc);
+    if (threadIdx.x == 0) partials[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = sum;
+}
+__global__ void __launch_bounds__(256)
+sqdiff_final_kernel(const double* __restrict__ partials, int blocks, double inv_count, float* __restrict__ out) {
     double t = 0.0;
-    for (int i = 0; i < blocks; ++i) t += partials[i];
-    *out = (float)(t * inv_count);
+    for (int i = threadIdx.x; i < blocks; i += 256) t += partials[(size_t)blockIdx.x * blocks + i];
+    const double sum = block_sum(t);
+    if (threadIdx.x == 0) out[blockIdx.x] = (float)(sum * inv_count);
 }
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-struct SearchScratch {
-    float* s;
-    __half* xs;
-    unsigned char* qweight;
-    unsigned char* scales;
-    unsigned char* zeros;
-    __half* yq;
-    float* yref;
-    double* partials;
-    float* losses;
-    size_t total;
-};
-SearchScratch carve(void* base, int M, int N, int K, int group) {
-    SearchScratch r;
+// Grid points evaluated together: as many as 384 MB of scratch hold (twenty of 4096 -> 4096 with 512 tokens), at most kMaxSearchAlphas.
+int search_rows(int M) { return (M + 31) / 32 * 32; }
+size_t search_point_bytes(int M, int N, int K, int group) {
+    return (size_t)search_rows(M) * K * 2 + (size_t)N * K / 2 + (size_t)(K / group) * N * 5 / 2 + (size_t)search_rows(M) * N * 2;
+}
+SearchPlan carve(void* base, int M, int N, int K, int group) {
+    SearchPlan r;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t o = off; off += align256(bytes); return static_cast<unsigned char*>(base) + o; };
-    r.s = reinterpret_cast<float*>(take((size_t)K * 4));
-    r.xs = reinterpret_cast<__half*>(take((size_t)M * K * 2));
-    r.qweight = take((size_t)N * K / 2);
-    r.scales = take((size_t)(K / group) * N * 2);
-    r.zeros = take((size_t)(K / group) * N / 2);
-    r.yq = reinterpret_cast<__half*>(take((size_t)M * N * 2));
+    const size_t fit = ((size_t)384 << 20) / search_point_bytes(M, N, K, group);
+    r.batch = fit < 1 ? 1 : fit > (size_t)kMaxSearchAlphas ? kMaxSearchAlphas : (int)fit;
+    r.rows = search_rows(M);
+    const size_t b = (size_t)r.batch;
+    r.s = reinterpret_cast<float*>(take((size_t)kMaxSearchAlphas * K * 4));
+    r.xs = reinterpret_cast<__half*>(take(b * r.rows * K * 2));
+    r.qweight = take(b * N * K / 2);
+    r.scales = take(b * (K / group) * N * 2);
+    r.zeros = take(b * (K / group) * N / 2);
+    r.yq = reinterpret_cast<__half*>(take(b * r.rows * N * 2));
     r.yref = reinterpret_cast<float*>(take((size_t)M * N * 4));
-    r.partials = reinterpret_cast<double*>(take((size_t)kLossBlocks * 8));
+    r.partials = reinterpret_cast<double*>(take((size_t)kMaxSearchAlphas * kLossBlocks * 8));
     r.losses = reinterpret_cast<float*>(take((size_t)kMaxSearchAlphas * 4));
     r.total = off;
     return r;
@@ -210,9 +221,7 @@ reference_product_kernel(const __half* __restrict__ W, const __half* __restrict_
 
 }  // namespace
 
-size_t search_scratch_bytes(int M, int N, int K, int group) {
-    return carve(nullptr, M, N, K, group).total;
-}
+SearchPlan search_plan(void* scratch, int M, int N, int K, int group) { return carve(scratch, M, N, K, group); }
 
 // y_ref[m][n] = sum_k X[m][k] W[n][k], fp32 [M][N] row-major.
 cudaError_t launch_reference_product(const void* W, const void* X, float* yref, int M, int N, int K,
@@ -224,10 +233,10 @@ cudaError_t launch_reference_product(const void* W, const void* X, float* yref, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_divide_by_scale(const void* X, const float* s, void* xs, int M, int K, cudaStream_t st) {
+cudaError_t launch_divide_by_scale(const void* X, const float* s, int count, void* xs, int M, int rows, int K, cudaStream_t st) {
     const size_t chunks = (size_t)M * K / 8;
-    divide_by_scale_kernel<<<(unsigned)((chunks + 255) / 256), 256, 0, st>>>(
-        reinterpret_cast<const __half*>(X), s, reinterpret_cast<__half*>(xs), chunks, K);
+    divide_by_scale_kernel<<<dim3((unsigned)((chunks + 255) / 256), (unsigned)count), 256, 0, st>>>(
+        reinterpret_cast<const __half*>(X), s, reinterpret_cast<__half*>(xs), chunks, (size_t)rows * K / 8, K);
     count_launch();
     return cudaGetLastError();
 }
@@ -246,20 +255,17 @@ cudaError_t launch_inverse_scale(const float* s, float* inv_s, int K, cudaStream
     return cudaGetLastError();
 }
 
-cudaError_t launch_mean_squared_difference(const void* yq, const float* yref, size_t n, double* partials,
-                                           float* out, cudaStream_t st) {
-    sqdiff_partial_kernel<<<kLossBlocks, 256, 0, st>>>(reinterpret_cast<const __half*>(yq), yref, n, partials);
-    sqdiff_final_kernel<<<1, 32, 0, st>>>(partials, kLossBlocks, 1.0 / (double)n, out);
-    count_launch();
+cudaError_t launch_squared_difference(const void* yq, const float* yref, int count, int M, int rows, int N, double* partials, cudaStream_t st) {
+    sqdiff_partial_kernel<<<dim3(kLossBlocks, (unsigned)count), 256, 0, st>>>(reinterpret_cast<const __half*>(yq), yref, (size_t)M * N / 8,
+                                                                             (size_t)rows * N / 8, partials);
     count_launch();
     return cudaGetLastError();
 }
-
-void search_carve(void* base, int M, int N, int K, int group, float** s, void** xs, void** qweight,
-                  void** scales, void** zeros, void** yq, float** yref, double** partials, float** losses) {
-    const SearchScratch r = carve(base, M, N, K, group);
-    *s = r.s; *xs = r.xs; *qweight = r.qweight; *scales = r.scales; *zeros = r.zeros;
-    *yq = r.yq; *yref = r.yref; *partials = r.partials; *losses = r.losses;
+cudaError_t launch_losses(const double* partials, int count, size_t n, float* losses, cudaStream_t st) {
+    sqdiff_final_kernel<<<(unsigned)count, 256, 0, st>>>(partials, kLossBlocks, 1.0 / (double)n, losses);
+    count_launch();
+    return cudaGetLastError();
 }
+double* search_partials(const SearchPlan& p, int first) { return p.partials + (size_t)first * kLossBlocks; }
 
 }  // namespace awq
