@@ -362,7 +362,9 @@ gemv_band_kernel(const BandProblems probs, const __half* __restrict__ x, int M, 
     const int b0 = bq * (int)blockIdx.x + min((int)blockIdx.x, br);
     const int b1 = b0 + bq + ((int)blockIdx.x < br ? 1 : 0);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (the shuffle tells the compiler that all lanes of a warp take the same role: addresses and barriers stay in uniform
+    // registers; 4096 -> 22016 at one token 10.3 -> 9.7 us, 8192 -> 28672 26.8 -> 25.1 us)
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     if (threadIdx.x < (unsigned)S) {
         mbar_init(bars + 8u * threadIdx.x, 1);                      // full: the copy warp's byte count
         // empty: math warps and the flush warp; with one-stage bands the flush warp alone (it has
@@ -895,7 +897,7 @@ gemv_splitk_kernel(const unsigned char* __restrict__ qweight, const __half* __re
     const int ul = max(u0, ((u1 - 1) / rg.ups) * rg.ups);     // first unit of the last segment
     const int nl = (ul == u0) ? 0 : u1 - ul;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
     if (threadIdx.x < (unsigned)S) {
         mbar_init(bars + 8u * threadIdx.x, 1);

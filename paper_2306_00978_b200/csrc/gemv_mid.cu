@@ -109,7 +109,8 @@ gemv_mid_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant
     const int u0 = starts.v[blockIdx.x], u1 = starts.v[blockIdx.x + 1];
     (void)units;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (the shuffle: as in gemv.cu; 8192 -> 28672 at 8 tokens 30.8 -> 29.3 us)
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     if (threadIdx.x < (unsigned)S) {
         mbar_init(bars + 8u * threadIdx.x, 1);                           // full: the producer's byte count
         mbar_init(bars + 64u + 8u * threadIdx.x, kMidMathWarps);         // empty: every math warp is done with it
