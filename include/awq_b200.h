@@ -172,7 +172,7 @@ int awq_channel_scale(const float* act_mean_abs, float alpha, float* s, int K, v
  * else awq_linear falls back to a kernel that needs none.  Calls that use the workspace must not
  * overlap on the GPU (issue them on one stream).
  * Stream order.  x and y follow plain stream order.  The packed arrays are treated as constants
- * of the layer: the band, chunked and stream kernels are launched with programmatic stream serialization
+ * of the layer: the band, chunked, stream and SM-pair kernels are launched with programmatic stream serialization
  * and start copying qweight, scales and zeros into shared memory BEFORE the work in front of them
  * in the stream has completed; only their reads of x and their writes of y and of the workspace
  * wait for that work.  The library covers its own writers: the first

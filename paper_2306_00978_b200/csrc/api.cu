@@ -324,7 +324,7 @@ int awq_linear_path(const void* x, const void* qweight, const void* scales, cons
         return note_cuda(launch_gemv_band(x, &one, 1, M, K, group, d->status_word, d->sms,
                                           take_packed_written(d), st));
     }
-    (void)take_packed_written(d);               // every other kernel is plainly stream-ordered
+    const bool serialize = take_packed_written(d);   // (split-K and one-SM kernels are plainly stream-ordered)
     if (path == AWQ_PATH_GEMV || path == AWQ_PATH_GEMV_SPLITK) {
         void* ws = nullptr;
         {
@@ -349,7 +349,7 @@ int awq_linear_path(const void* x, const void* qweight, const void* scales, cons
         ws_bytes = d->workspace_bytes;
     }
     return note_cuda(launch_gemm(x, qweight, scales, zeros, y, M, N, K, group, path != AWQ_PATH_GEMM_1SM,
-                                 ws, ws_bytes, d->status_word, st));
+                                 ws, ws_bytes, d->status_word, serialize, st));
 }
 
 int awq_linear_gemv_static(const void* x, const void* qweight, const void* scales, const void* zeros,

@@ -192,7 +192,7 @@ int gemv_static_max_m();
 cudaError_t launch_gemm(const void* x, const void* qweight, const void* scales, const void* zeros,
                         void* y, int M, int N, int K, int group, bool path_pair_allowed,
                         void* workspace, size_t workspace_bytes,
-                        unsigned int* status_word, cudaStream_t st);
+                        unsigned int* status_word, bool serialize, cudaStream_t st);
 // what launch_gemm takes, us (an estimate that ranks), and whether it is the one-SM kernel
 double gemm_prefill_estimate(int M, int N, int K, int group, int sms, size_t workspace_bytes, bool* one_sm);
 // optional workspace of the tensor-core path (0 if the shape has no use for one)

@@ -446,7 +446,7 @@ bool one_sm_preferred(int M, int N, int K, int splits, int sms, size_t workspace
 cudaError_t launch_gemm(const void* x, const void* qweight, const void* scales, const void* zeros,
                         void* y, int M, int N, int K, int group, bool path_pair_allowed,
                         void* workspace, size_t workspace_bytes,
-                        unsigned int* status_word, cudaStream_t st) {
+                        unsigned int* status_word, bool serialize, cudaStream_t st) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
     const int bn = M > 128 ? 256 : M > 64 ? 128 : M > 32 ? 64 : 32;
@@ -491,7 +491,7 @@ cudaError_t launch_gemm(const void* x, const void* qweight, const void* scales, 
         if (!make_w_map(&wmap, 256)) return cudaErrorInvalidValue;
         bool launched = false;
         e = launch_gemm_pair(x, wmap, ymap, scales, zeros, M, N, K, group, workspace, workspace_bytes,
-                             status_word, sms, st, &launched);
+                             status_word, sms, serialize, st, &launched);
         if (e != cudaSuccess || launched) return e;
     }
     if (!make_x_map(&map, bn) || !make_w_map(&wmap, 128)) return cudaErrorInvalidValue;
@@ -528,7 +528,7 @@ cudaError_t launch_gemm_blocks(const void* x, const void* qweight, const void* s
             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
     return launch_gemm_pair(x, wmap, ymap, scales, zeros, M, count * N, K, group, workspace, workspace_bytes, status_word, sms,
-                            st, launched, count, rows);
+                            true, st, launched, count, rows);
 }
 
 double gemm_prefill_estimate(int M, int N, int K, int group, int sms, size_t workspace_bytes, bool* one_sm) {

@@ -14,6 +14,10 @@
 // memory (128 tokens, one tile per pair, 108 stages: 55 us with four stages, 42 us with eight; 256 tokens gain
 // nothing from a fifth).
 //
+// The start of a launch: chained to the one in front by programmatic dependent launch, weight copies (a warp of their own, x's are
+// another's) issued before tensor memory and the cluster are ready.  Chained calls, before and after: 333 tokens on
+// 4096 -> 4096 19.3 -> 15.7 us, 700 on 2048 -> 2048 13.5 -> 10.7, 100 on 5120 -> 13824 22.7 -> 19.2, 8192 on 4096 -> 11008 610 -> 537.
+//
 // Block r of a pair (r = rank in the cluster) owns
 //   - A: output channels 128 r .. 128 r + 127 of the 256-channel slab, dequantized by its own
 //        warps into its own tensor memory (64 columns per stage),
@@ -85,9 +89,9 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
+// (what is handed over in front of it is the barriers' initialisation, which has a fence of its own)
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // x tile copy whose bytes are counted on a barrier of the pair's leader
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1,
                                                  uint32_t leader_bar) {
@@ -204,44 +208,49 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     pieces.tile = cluster; pieces.tile_step = num_clusters; pieces.total_tiles = total_tiles; pieces.nks = nks;
     int tile, k0, k1;
 
-    if (threadIdx.x == 0) {
-        s_abort = 0u;
-        for (int s = 0; s < S; ++s) {
-            mbar_init(w_full(s), 1); mbar_init(x_full(s), 1); mbar_init(empty(s), 1);
+    // the weight copies need nothing but their own block's barriers: they start before tensor memory and the cluster are ready
+    if (warp == 0) {
+        if (lane == 0) {
+            s_abort = 0u;
+            for (int s = 0; s < S; ++s) {
+                mbar_init(w_full(s), 1); mbar_init(x_full(s), 1); mbar_init(empty(s), 1);
+            }
+            for (int s = 0; s < SL; ++s) mbar_init(a_full(s), 16);
+            for (uint32_t b = 0; b < NACC; ++b) { mbar_init(acc_full(b), 1); mbar_init(acc_empty(b), 16); }
+            mbar_fence_init();
         }
-        for (int s = 0; s < SL; ++s) mbar_init(a_full(s), 16);
-        for (uint32_t b = 0; b < NACC; ++b) { mbar_init(acc_full(b), 1); mbar_init(acc_empty(b), 16); }
-        mbar_fence_init();
+        __syncwarp();
+        asm volatile("bar.arrive 1, %0;" ::"r"(Cfg::kThreads) : "memory");
+        cluster_arrive();
+    } else {
+        if (warp == 1) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
+                         ::"r"(smem_u32(&s_tmem_base)), "r"((uint32_t)Cfg::kTmemCols) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+            tc_fence_before();
+        }
+        named_barrier_sync(1, Cfg::kThreads);
+        cluster_arrive();
+        cluster_wait();                      // both blocks' barriers exist before anyone arrives remotely
+        tc_fence_after();
     }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(&s_tmem_base)), "r"((uint32_t)Cfg::kTmemCols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    }
-    tc_fence_before();
-    __syncthreads();
-    cluster_sync_all();                      // both blocks' barriers exist before anyone arrives remotely
-    tc_fence_after();
     constexpr uint32_t tmem_base = 0;        // all 512 columns are this block's
     const WaitCtl ctl{status_word, &s_abort};
+    // programmatic dependent launch: the packed arrays are constants of the layer and are read before the work in front of
+    // this launch has completed; x is read and y and the workspace are written after it
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (warp == 0) {
-        // ------------------------------------------------------------------ producer
+        // ------------------------------------------------------------------ weight copies
         const bool lead = elect_one();
-        const uint32_t leader_x_full0 = map_to_rank(x_full(0), 0);
         uint32_t stage = 0, phase = 0;
         unsigned int issued = 0;
         bool ok = true;
         while (ok && pieces.next(tile, k0, k1)) {
             const int slab = (tile / m_tiles) * 2 + (int)rank;              // 128-channel slab of this block
-            const int tok0 = (tile / m_tiles / blocks.slabs) * blocks.rows + (tile % m_tiles) * BN + (int)rank * Cfg::kHalf;
             for (int ks = k0; ks < k1; ++ks) {
                 if (!mbar_wait_warp(empty(stage), phase ^ 1u, ctl)) { ok = false; break; }
                 if (lead) {
-                    if (rank == 0) mbar_arrive_expect_tx(x_full(stage), 2u * Cfg::kXTileBytes);
-                    const uint32_t xbar = leader_x_full0 + 8u * stage;
-                    tma_load_2d_pair(x_addr(stage), &x_map, ks * kStageK, tok0, xbar);
-                    tma_load_2d_pair(x_addr(stage) + Cfg::kXHalfBytes, &x_map, ks * kStageK + kBK, tok0, xbar);
                     const uint32_t bar = w_full(stage);
                     mbar_arrive_expect_tx(bar, (uint32_t)Cfg::kWBytes);
                     // weights: box of 8 bands x 1 KB (256 words: two k-tiles) at (stage, first band)
@@ -261,7 +270,30 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 const unsigned long long t0 = global_ns();
                 while (!mbar_try_wait(w_full(st), ph) && global_ns() - t0 < 100000000ull) {}
             }
-            const unsigned long long t1 = global_ns();              // and the x halves (counted on the leader)
+        }
+    } else if (warp == 2) {
+        // ------------------------------------------------------------------ x copies
+        const bool lead = elect_one();
+        const uint32_t leader_x_full0 = map_to_rank(x_full(0), 0);
+        uint32_t stage = 0, phase = 0;
+        bool ok = true;
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        while (ok && pieces.next(tile, k0, k1)) {
+            const int tok0 = (tile / m_tiles / blocks.slabs) * blocks.rows + (tile % m_tiles) * BN + (int)rank * Cfg::kHalf;
+            for (int ks = k0; ks < k1; ++ks) {
+                if (!mbar_wait_warp(empty(stage), phase ^ 1u, ctl)) { ok = false; break; }
+                if (lead) {
+                    if (rank == 0) mbar_arrive_expect_tx(x_full(stage), 2u * Cfg::kXTileBytes);
+                    const uint32_t xbar = leader_x_full0 + 8u * stage;
+                    tma_load_2d_pair(x_addr(stage), &x_map, ks * kStageK, tok0, xbar);
+                    tma_load_2d_pair(x_addr(stage) + Cfg::kXHalfBytes, &x_map, ks * kStageK + kBK, tok0, xbar);
+                }
+                __syncwarp();
+                if (++stage == S) { stage = 0; phase ^= 1u; }
+            }
+        }
+        if (!ok) {                                                  // giving up: the x halves are counted on the leader
+            const unsigned long long t1 = global_ns();
             while (global_ns() - t1 < 1000000ull) __nanosleep(1000);
         }
     } else if (warp == 1) {
@@ -385,6 +417,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     } else if (warp >= 4) {
         // ------------------------------------------------------------------ epilogue
         // warps 4-7 drain the first half of the accumulator's token columns, the last four warps the second
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         const int quad = warp & 3;                     // TMEM lanes 32*quad .. +31
         const int half = warp >= Cfg::kEpilogueWarp1 ? 1 : 0;
         const uint32_t leader_acc_empty0 = map_to_rank(acc_empty(0), 0);
@@ -394,8 +427,6 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         int obuf = 0;
         bool ok = true;
         while (ok && pieces.next(tile, k0, k1)) {
-            const int block = tile / m_tiles / blocks.slabs, mt = tile % m_tiles;
-            const int slab = (tile / m_tiles - block * blocks.slabs) * 2 + (int)rank;
             // A piece that does not start the tile is a contribution: its fp32 sums go to this pair's
             // slot of the workspace.  A piece that starts the tile but does not end it waits for the
             // contributions of the pairs after this one (they were produced at the start of those
@@ -435,8 +466,10 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
             tc_fence_after();
-            const int n0 = slab * 128 + quad * 32;
-            const int m0 = mt * BN + half * Cfg::kHalf;
+            int row = (tile % m_tiles) * BN + half * Cfg::kHalf;        // this warp's first token, then its row of y
+            const int block = tile / m_tiles / blocks.slabs, n0 = ((tile / m_tiles - block * blocks.slabs) * 2 + (int)rank) * 128 + quad * 32;
+            const int rows = n0 < blocks.n ? M - row : 0;               // what there is to store
+            row += block * blocks.rows;
             const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + acc * (uint32_t)BN + (uint32_t)(half * Cfg::kHalf);
 #pragma unroll 1
             for (int c = 0; c < Cfg::kHalf; c += 32) {
@@ -472,7 +505,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 }
                 // stage the 32 x 32 block as [token][channel] fp16 and hand it to the copy engine
                 // (rows past M are clipped by the tensor map; blocks that lie outside y are left out)
-                if (n0 >= blocks.n || m0 + c >= M) continue;
+                if (c >= rows) continue;
                 if (lane == 0) bulk_wait_read_1();                  // the store that last used this buffer
                 __syncwarp();
                 const uint32_t tb = out_base + (uint32_t)(((half * 4 + quad) * 2 + obuf) * 2048);
@@ -483,7 +516,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                    tma_store_2d(&y_map, n0, block * blocks.rows + m0 + c, tb);
+                    tma_store_2d(&y_map, n0, row + c, tb);
                     bulk_commit_group();
                 }
                 obuf ^= 1;
@@ -505,9 +538,11 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     }
 
     __syncwarp();
+    if (warp == 0) cluster_wait();
     tc_fence_before();
     __syncthreads();
-    cluster_sync_all();                      // nothing of the pair still refers to this block
+    cluster_arrive();
+    cluster_wait();                          // nothing of the pair still refers to this block
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;"
@@ -555,7 +590,7 @@ template <int G, int BN>
 cudaError_t launch_pair(const CUtensorMap& xmap, const CUtensorMap& wmap, const CUtensorMap& ymap,
                         const void* scales, const void* zeros, int M, int N, int K, bool streamk,
                         void* workspace, size_t workspace_bytes, const PairBlocks& blocks,
-                        unsigned int* status_word, int sms, cudaStream_t st, bool* launched) {
+                        unsigned int* status_word, int sms, bool serialize, cudaStream_t st, bool* launched) {
     using Cfg = PairCfg<BN>;
     cudaError_t e;
     const int resident = resident_pairs<G, BN>(sms, &e);
@@ -570,15 +605,17 @@ cudaError_t launch_pair(const CUtensorMap& xmap, const CUtensorMap& wmap, const 
     if (streamk && stages / 4 > want) want = stages / 4;          // at least four stages per pair
     const int clusters = (int)(want < resident ? want : resident);
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3((unsigned)(2 * clusters));
     cfg.blockDim = dim3(Cfg::kThreads);
     cfg.dynamicSmemBytes = Cfg::kSmemBytes;
     cfg.stream = st;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = serialize ? 1 : 2;
     float* partials = streamk ? reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + kCounterBytes)
                               : nullptr;
     unsigned int* flags = static_cast<unsigned int*>(workspace);
@@ -650,7 +687,7 @@ double gemm_pair_estimate(int M, int N, int K, int sms, size_t workspace_bytes) 
 cudaError_t launch_gemm_pair(const void* x, const CUtensorMap& wmap, const CUtensorMap& ymap,
                              const void* scales, const void* zeros, int M, int N, int K, int group,
                              void* workspace, size_t workspace_bytes,
-                             unsigned int* status_word, int sms, cudaStream_t st, bool* launched, int count, int rows) {
+                             unsigned int* status_word, int sms, bool serialize, cudaStream_t st, bool* launched, int count, int rows) {
     const PairBlocks blocks = {(N / count + 255) / 256, N / count, rows};
     const PairChoice c = choose_tile(M, N, K, sms / 2, workspace ? workspace_bytes : 0);
     CUtensorMap xmap;
@@ -666,7 +703,7 @@ cudaError_t launch_gemm_pair(const void* x, const CUtensorMap& wmap, const CUten
     }
 #define AWQ_PAIR_CASE(GG, BNN)                                                                                     \
     return launch_pair<GG, BNN>(xmap, wmap, ymap, scales, zeros, M, N, K, c.streamk, workspace, workspace_bytes, blocks, \
-                                status_word, sms, st, launched)
+                                status_word, sms, serialize, st, launched)
     if (group == 128) {
         switch (c.bn) { case 64: AWQ_PAIR_CASE(128, 64); case 128: AWQ_PAIR_CASE(128, 128);
                         case 192: AWQ_PAIR_CASE(128, 192); default: AWQ_PAIR_CASE(128, 256); }

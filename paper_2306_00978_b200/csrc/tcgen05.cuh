@@ -159,7 +159,7 @@ double gemm_pair_estimate(int M, int N, int K, int sms, size_t workspace_bytes);
 cudaError_t launch_gemm_pair(const void* x, const CUtensorMap& wmap, const CUtensorMap& ymap,
                              const void* scales, const void* zeros, int M, int N, int K, int group,
                              void* workspace, size_t workspace_bytes,
-                             unsigned int* status_word, int sms, cudaStream_t st, bool* launched,
+                             unsigned int* status_word, int sms, bool serialize, cudaStream_t st, bool* launched,
                              int count = 1, int rows = 0);     // count products of N / count channels, rows of x and y apart
 
 }  // namespace awq
