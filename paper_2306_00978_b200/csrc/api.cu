@@ -193,10 +193,11 @@ static bool stream_kernel_preferred(int M, int total_n, int K, int group, int sm
     return several && M >= 4 && K > 4096 && (long long)total_n * K >= (1LL << 25);
 }
 
-// Above 64 tokens the stream kernel is taken where its estimate is 5 % below the prefill kernels' (few tiles for many
-// pairs, long rows): 4096 -> 4096 at 100 tokens 11.5 against 17.5 us, 11008 -> 4096 17.6 against 27.0, 28672 -> 8192
-// 59 against 175; at 200 tokens 11008 -> 4096 27 against 32, while 4096 -> 11008 keeps them (28 against 22).  Beyond two
-// tiles of 128 tokens they won everywhere.  The one-SM kernel keeps the shapes that it had.
+// Above 64 tokens the stream kernel is taken where its estimate is below the prefill kernels' (few tiles for many pairs, long
+// rows).  Stream / SM-pair kernel, us: 4096 -> 4096 at 65 / 100 / 128 tokens 10.1 / 11.2 / 11.9 against 14.1 / 14.3 / 14.3,
+// 11008 -> 4096 at 100 / 256 tokens 16.8 / 27.7 against 23.8 / 31.8, 8192 -> 3072 at 256 tokens 19.9 against 25.9; but 4096 -> 11008
+// at 100 tokens 18.3 against 16.2, 4096 -> 4096 at 256 tokens 17.1 against 15.9, 8192 -> 8192 38.2 against 28.8.  Beyond two tiles of
+// 128 tokens the latter won everywhere.  The one-SM kernel keeps the shapes that it had.
 static bool stream_beats_prefill(const DeviceState* d, const AwqLinearProblem* problems, int count, int M, int K, int group) {
     if (M <= 64 || M > 256) return false;
     size_t have = 0;
@@ -214,7 +215,7 @@ static bool stream_beats_prefill(const DeviceState* d, const AwqLinearProblem* p
         if (one_sm) return false;
         slabs += (problems[i].N + 255) / 256;
     }
-    return 1.05 * gemm_stream_estimate(M, slabs, K, d->sms) < others;
+    return gemm_stream_estimate(M, slabs, K, d->sms) < others;
 }
 
 static int resolve_path(int M, int K, int path) {

@@ -785,15 +785,15 @@ size_t gemm_stream_workspace_bytes(int M, int sms) {
     return kCounterBytes + (size_t)(sms / 2) * 2 * 256 * (bn < M ? bn : M) * sizeof(float);
 }
 
-// Estimated time above 64 tokens, us: start, stages of the longest range, and the parts that a pair leaves (and the second kernel
-// reads).  A fit to 70 / 100 / 128 / 192 / 256 tokens on 7 shapes (2048 -> 2048 .. 28672 -> 8192); on 36 other problems (N 1024 ..
-// 28672, K 1024 .. 28672, 65 .. 224 tokens) it is 5 % off on average, 28 % at worst (4096 -> 1024, cut among 64 pairs).
+// Estimated time above 64 tokens, us: start, stages of the longest range, the parts that a pair leaves, and how many of them
+// make up a tile.  A fit to 70 / 100 / 128 / 192 / 256 tokens on 7 shapes (2048 -> 2048 .. 28672 -> 8192); on 36 other problems
+// (N 1024 .. 28672, K 1024 .. 28672, 65 .. 224 tokens) it is 5 % off on average.
 double gemm_stream_estimate(int M, int slabs, int K, int sms) {
     const int bn = st_tile_tokens(M), nks = (K + kStStageK - 1) / kStStageK;
     const long long total = (long long)slabs * ((M + bn - 1) / bn) * nks, pairs = sms / 2;
     const double share = total < pairs ? 1.0 : (double)total / (double)pairs;
-    const double parts = 1.0 + (share < nks ? share / nks : 1.0);
-    return 1.6 + (double)((long long)(share + 0.999)) * (0.45 + 0.0048 * bn) + (2.63 + 0.0208 * bn) * parts;
+    const double parts = 1.0 + (share < nks ? share / nks : 1.0), per_tile = (double)nks / share;
+    return 1.6 + (double)((long long)(share + 0.999)) * (0.45 + 0.0048 * bn) + (2.63 + 0.0208 * bn) * parts + 0.1 * per_tile;
 }
 
 cudaError_t launch_gemm_stream(const void* x, const GemvMatrix* mats, int count, int M, int K, int group,

@@ -438,7 +438,8 @@ int gemm_splits(int M, int N, int K, int group, int bn, int sms, size_t workspac
 bool one_sm_preferred(int M, int N, int K, int splits, int sms, size_t workspace_bytes) {
     if (M <= 64 || M > 128 || splits == 1 || (N / 128) * splits > sms) return false;
     const int range = (K / kBK + splits - 1) / splits;
-    return 1.05 * (18.6 + 0.365 * range) < gemm_pair_estimate(M, N, K, sms, workspace_bytes);
+    // (both as launches by themselves, which the times above are: the pair kernel's estimate is a chained launch's)
+    return 1.05 * (18.6 + 0.365 * range) < gemm_pair_estimate(M, N, K, sms, workspace_bytes) + 3.0;
 }
 
 }  // namespace

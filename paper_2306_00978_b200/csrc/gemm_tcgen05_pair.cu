@@ -630,7 +630,7 @@ cudaError_t launch_pair(const CUtensorMap& xmap, const CUtensorMap& wmap, const 
 // Tokens per tile, and whether to cut the tiles' K loops into equal ranges (stream-K).  A launch takes `start`
 // us plus `stage` us per 128 input channels of each wave of tiles (both measured with one tile per pair, on
 // 4096 -> 4096 and 13824 -> 5120: 17.4 / 17.2 / 21.9 / 26.8 and 42.8 / 42.2 / 54.8 / 69.2 us with 64 / 128 /
-// 192 / 256 tokens); stream-K replaces the last wave by an even share but costs its pairs two more
+// 192 / 256 tokens, a launch by itself; chained ones start 3 us sooner, which is in `start`); stream-K replaces the last wave by an even share but costs its pairs two more
 // drains and a pass over a partial tile (8.5 us at 64 tokens, 10 us at 256; at 128 and 192, with
 // sixteen dequantizer warps too few registers are left to fetch those sums in one go, 16 us and more: not
 // offered) and, where a tile is cut among many pairs, the addition of their sums one after the other by
@@ -649,20 +649,21 @@ cudaError_t launch_pair(const CUtensorMap& xmap, const CUtensorMap& wmap, const 
 struct PairChoice { int bn; bool streamk; double us; };
 PairChoice choose_tile(int M, int N, int K, int pairs, size_t workspace_bytes) {
     static const struct { int bn; double start, stage, streamk, addition; } kTiles[] = {
-        {256, 9.0, 0.557, 10.0, 4.4}, {192, 8.5, 0.425, 0.0, 0.0}, {128, 7.0, 0.325, 0.0, 0.0}, {64, 6.6, 0.330, 8.5, 1.5}};
+        {256, 6.0, 0.557, 10.0, 4.4}, {192, 5.5, 0.425, 0.0, 0.0}, {128, 4.0, 0.325, 0.0, 0.0}, {64, 3.6, 0.330, 8.5, 1.5}};
     PairChoice best = {256, false, 1e30};
+    double least = 1e30;                             // with the bias
     const long long nks = K / kStageK;
     for (const auto& t : kTiles) {
         const long long tiles = (long long)((N + 255) / 256) * ((M + t.bn - 1) / t.bn);
         const long long waves = (tiles + pairs - 1) / pairs;
         const double bias = t.bn == 256 ? 1.0 : 1.04;
-        const double plain = bias * (t.start + (double)(waves * nks) * t.stage);
-        if (plain < best.us) best = {t.bn, false, plain};
+        const double plain = t.start + (double)(waves * nks) * t.stage;
+        if (bias * plain < least) { least = bias * plain; best = {t.bn, false, plain}; }
         if (t.streamk == 0.0 || workspace_bytes < streamk_bytes(t.bn, pairs)) continue;
         const long long share = (tiles * nks + pairs - 1) / pairs, range = share > 4 ? share : 4;     // (at least four stages per pair)
         const double additions = nks > range ? (double)nks / (double)range - 1.0 : 0.0;
-        const double even = bias * (t.start + (double)share * t.stage + t.streamk + additions * t.addition);
-        if ((double)share * t.stage < 225.0 && even < best.us) best = {t.bn, true, even};
+        const double even = t.start + (double)share * t.stage + t.streamk + additions * t.addition;
+        if ((double)share * t.stage < 225.0 && bias * even < least) { least = bias * even; best = {t.bn, true, even}; }
     }
     return best;
 }
