@@ -606,7 +606,7 @@ int awq_search_alpha(const void* W, const float* act_mean_abs, const void* X, in
         ws_bytes = d->workspace_bytes;
         d->packed_written = true;
     }
-    if (int rc = note_cuda(launch_reference_product(W, X, p.yref, M, N, K, st))) return rc;
+    if (int rc = note_cuda(launch_reference_product(W, X, p.yref, M, N, K, d->status_word, st))) return rc;
     if (int rc = note_cuda(launch_channel_scales(act_mean_abs, alphas, n_alphas, p.s, K, st))) return rc;
     const int batches = (n_alphas + p.batch - 1) / p.batch, most = (n_alphas + batches - 1) / batches;
     for (int i0 = 0; i0 < n_alphas; i0 += most) {

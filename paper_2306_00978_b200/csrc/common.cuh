@@ -165,7 +165,7 @@ struct SearchPlan {
 };
 SearchPlan search_plan(void* scratch, int M, int N, int K, int group);
 cudaError_t launch_reference_product(const void* W, const void* X, float* yref, int M, int N, int K,
-                                     cudaStream_t st);
+                                     unsigned int* status_word, cudaStream_t st);
 // xs[i] = fp16_rne(fp32(X) / s[i]) for `count` scale arrays, `rows` rows apart
 cudaError_t launch_divide_by_scale(const void* X, const float* s, int count, void* xs, int M, int rows, int K, cudaStream_t st);
 // xs = fp16_rne(fp32(X) * inv_s); inverse_scale: inv_s = fp32(1 / s), correctly rounded

@@ -3,9 +3,8 @@
 // diag(s)^-1 X, and measure the output error against the fp16 layer W X (Eq. 4).  Everything
 // that the search evaluates is therefore exactly what deployment will run.  The reference product
 // W X is a plain dense fp16 GEMM with fp32 accumulation and output; it runs once per search, on
-// a small warp-level tensor-core kernel of this file (no library call, no allocation).
-#include "async_copy.cuh"
-#include "common.cuh"
+// a tcgen05 kernel of this file (no library call, no allocation).
+#include "tcgen05.cuh"
 
 namespace awq {
 
@@ -127,96 +126,109 @@ SearchPlan carve(void* base, int M, int N, int K, int group) {
 }
 
 // ---------------------------------------------------------------- dense reference product
-// C[m][n] = sum_k X[m][k] * W[n][k]: both operands have K contiguous, which is the row / column
-// operand form of the warp-level m16n8k16 product.  128 tokens x 128 channels per block, 32
-// input channels per step, two shared-memory buffers filled by 16-byte asynchronous copies, eight
-// warps of 64 x 32 outputs each.  Rows of 80 bytes keep the 8 x 16-byte row reads of a matrix
-// load on distinct banks.
-constexpr int kRefBM = 128, kRefBN = 128, kRefBK = 32, kRefRow = 80;   // bytes per staged row
-constexpr int kRefTile = 128 * kRefRow;                                // one operand tile of one buffer
+// C[m][n] = sum_k X[m][k] * W[n][k]: both operands have K contiguous.  A block takes 128 channels (A, the lanes of tensor
+// memory) x 128 tokens: one warp copies 64 input channels of both per stage (128-byte swizzle), one issues the products, four
+// store the accumulator, a lane a channel, so that a token's 32 channels are one 128-byte store.  Three stages, two blocks per
+// SM: one block's start and stores run under the other's products.  4096 channels x 4096 x 512 tokens: 28.6 us; 94 us on warp-level
+// m16n8k16 products of 128 x 128 x 32 tiles in two shared-memory buffers.
+constexpr int kRefTile = 128, kRefStages = 3, kRefOperand = kRefTile * kBK * 2, kRefThreads = 192;
+constexpr int kRefSmem = kRefStages * 2 * kRefOperand + 1024;
 
-__device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src, bool valid) {
-    const int n = valid ? 16 : 0;                                     // 0: the 16 bytes are zero-filled
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+__device__ __forceinline__ void umma_f16_smem(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
-__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
 
-__global__ void __launch_bounds__(256)
-reference_product_kernel(const __half* __restrict__ W, const __half* __restrict__ X, float* __restrict__ C,
-                         int M, int N, int K) {
-    __shared__ __align__(16) unsigned char sm[2 * 2 * kRefTile];      // [buffer][X tile | W tile]
-    const uint32_t sbase = smem_u32(sm);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.y * kRefBM, n0 = blockIdx.x * kRefBN;
-    const int wm = (warp >> 2) * 64, wn = (warp & 3) * 32;            // this warp's corner inside the tile
-
-    auto fill = [&](int buf, int k0) {
-        // 128 rows x 4 pieces of 16 bytes per operand: two pieces of each operand per thread
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int piece = tid + i * 256, row = piece >> 2, c = piece & 3;
-            const uint32_t dst = sbase + buf * (2 * kRefTile) + row * kRefRow + c * 16;
-            const bool ok = m0 + row < M;
-            cp_async_16(dst, X + (size_t)(ok ? m0 + row : 0) * K + k0 + c * 8, ok);
-            cp_async_16(dst + kRefTile, W + (size_t)(n0 + row) * K + k0 + c * 8, true);
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-
-    float acc[4][4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.0f;
-
-    const int steps = K / kRefBK;
-    fill(0, 0);
-    for (int s = 0; s < steps; ++s) {
-        if (s + 1 < steps) {
-            fill((s + 1) & 1, (s + 1) * kRefBK);
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-        } else {
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-        }
-        __syncthreads();
-        const uint32_t xa = sbase + (s & 1) * (2 * kRefTile), wa = xa + kRefTile;
-#pragma unroll
-        for (int kk = 0; kk < kRefBK; kk += 16) {
-            uint32_t a[4][4], b[2][4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)   // rows wm + 16 i + (lane % 16), columns kk + 8 (lane / 16)
-                ldmatrix_x4(a[i], xa + (wm + 16 * i + (lane & 15)) * kRefRow + (kk + 8 * (lane >> 4)) * 2);
-#pragma unroll
-            for (int j = 0; j < 2; ++j)   // channels wn + 16 j + (lane % 8) + 8 (lane / 16), columns kk + 8 ((lane / 8) % 2)
-                ldmatrix_x4(b[j], wa + (wn + 16 * j + (lane & 7) + 8 * (lane >> 4)) * kRefRow + (kk + 8 * ((lane >> 3) & 1)) * 2);
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint32_t b0 = b[j >> 1][2 * (j & 1)], b1 = b[j >> 1][2 * (j & 1) + 1];
-                    asm volatile(
-                        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                        : "+f"(acc[i][j][0]), "+f"(acc[i][j][1]), "+f"(acc[i][j][2]), "+f"(acc[i][j][3])
-                        : "r"(a[i][0]), "r"(a[i][1]), "r"(a[i][2]), "r"(a[i][3]), "r"(b0), "r"(b1));
-                }
-        }
-        __syncthreads();                                              // the buffer is refilled two steps on
+__global__ void __launch_bounds__(kRefThreads)
+reference_product_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap x_map, float* __restrict__ C,
+                         int M, int N, int K, unsigned int* status_word) {
+    extern __shared__ unsigned char smem_dyn[];
+    __shared__ __align__(8) unsigned long long s_bars[2 * kRefStages + 1];
+    __shared__ unsigned int s_abort;
+    __shared__ uint32_t s_tmem_base;
+    const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u, bars = smem_u32(s_bars);
+    auto full = [&](uint32_t s) { return bars + 8u * s; };
+    auto empty = [&](uint32_t s) { return bars + 8u * (uint32_t)(kRefStages + s); };
+    const uint32_t acc_full = bars + 16u * (uint32_t)kRefStages;
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const int n0 = blockIdx.x * kRefTile, m0 = blockIdx.y * kRefTile, steps = K / kBK;
+    if (threadIdx.x == 0) {
+        s_abort = 0u;
+        for (uint32_t s = 0; s < (uint32_t)kRefStages; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
+        mbar_init(acc_full, 1);
+        mbar_fence_init();
     }
-    const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int col = n0 + wn + 8 * j + 2 * t;
-            const int r0 = m0 + wm + 16 * i + g, r1 = r0 + 8;
-            if (r0 < M) *reinterpret_cast<float2*>(C + (size_t)r0 * N + col) = make_float2(acc[i][j][0], acc[i][j][1]);
-            if (r1 < M) *reinterpret_cast<float2*>(C + (size_t)r1 * N + col) = make_float2(acc[i][j][2], acc[i][j][3]);
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "r"(128u) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = s_tmem_base;
+    const WaitCtl ctl{status_word, &s_abort};
+    if (warp == 0) {
+        const bool lead = elect_one();
+        uint32_t stage = 0, phase = 0;
+        int i = 0;
+        for (; i < steps; ++i) {
+            if (!mbar_wait_warp(empty(stage), phase ^ 1u, ctl)) break;
+            if (lead) {
+                mbar_arrive_expect_tx(full(stage), 2 * kRefOperand);
+                tma_load_2d(base + stage * (2 * kRefOperand), &w_map, i * kBK, n0, full(stage));
+                tma_load_2d(base + stage * (2 * kRefOperand) + kRefOperand, &x_map, i * kBK, m0, full(stage));   // rows past M: zeros
+            }
+            __syncwarp();
+            if (++stage == kRefStages) { stage = 0; phase ^= 1u; }
         }
+        if (i < steps)                                               // giving up: the copies in flight land first
+            for (int q = 0; q < kRefStages && q < i; ++q) {
+                if (stage == 0) { stage = kRefStages - 1; phase ^= 1u; } else { --stage; }
+                const unsigned long long t0 = global_ns();
+                while (!mbar_try_wait(full(stage), phase) && global_ns() - t0 < drain_limit_ns(ctl)) {}
+            }
+    } else if (warp == 1) {
+        const bool lead = elect_one();
+        constexpr uint32_t idesc = instr_desc(kRefTile);
+        uint32_t stage = 0, phase = 0;
+        int i = 0;
+        for (; i < steps; ++i) {
+            if (!mbar_wait_warp(full(stage), phase, ctl)) break;
+            tc_fence_after();
+            const uint64_t a = smem_desc_sw128(base + stage * (2 * kRefOperand)), b = smem_desc_sw128(base + stage * (2 * kRefOperand) + kRefOperand);
+            if (lead) {
+#pragma unroll
+                for (int k = 0; k < kBK / 16; ++k)
+                    umma_f16_smem(tmem_base, a + (uint64_t)(2 * k), b + (uint64_t)(2 * k), idesc, (i > 0 || k > 0) ? 1u : 0u);
+                umma_commit(empty(stage));
+                if (i + 1 == steps) umma_commit(acc_full);
+            }
+            __syncwarp();
+            if (++stage == kRefStages) { stage = 0; phase ^= 1u; }
+        }
+    } else if (mbar_wait_warp(acc_full, 0u, ctl)) {
+        tc_fence_after();
+        const int quad = warp & 3, n = n0 + quad * 32 + lane;
+#pragma unroll 1
+        for (int c = 0; c < kRefTile; c += 32) {
+            uint32_t r[32];
+            tmem_ld_32cols(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)c, r);
+            tmem_ld_wait(r);
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                if (m0 + c + i < M) C[(size_t)(m0 + c + i) * N + n] = __uint_as_float(r[i]);
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(128u) : "memory");
+    }
 }
 
 }  // namespace
@@ -224,11 +236,23 @@ reference_product_kernel(const __half* __restrict__ W, const __half* __restrict_
 SearchPlan search_plan(void* scratch, int M, int N, int K, int group) { return carve(scratch, M, N, K, group); }
 
 // y_ref[m][n] = sum_k X[m][k] W[n][k], fp32 [M][N] row-major.
-cudaError_t launch_reference_product(const void* W, const void* X, float* yref, int M, int N, int K,
+cudaError_t launch_reference_product(const void* W, const void* X, float* yref, int M, int N, int K, unsigned int* status_word,
                                      cudaStream_t st) {
-    const dim3 grid((unsigned)(N / kRefBN), (unsigned)((M + kRefBM - 1) / kRefBM));
-    reference_product_kernel<<<grid, 256, 0, st>>>(reinterpret_cast<const __half*>(W),
-                                                   reinterpret_cast<const __half*>(X), yref, M, N, K);
+    EncodeTiledFn enc = encode_fn();
+    if (!enc) return cudaErrorNotSupported;
+    CUtensorMap maps[2];
+    for (int i = 0; i < 2; ++i) {
+        const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)(i ? M : N)}, strides[1] = {(cuuint64_t)K * 2};
+        const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)kRefTile}, estr[2] = {1, 1};
+        if (enc(&maps[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(i ? X : W), dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    const cudaError_t e = cudaFuncSetAttribute(reference_product_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRefSmem);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((unsigned)(N / kRefTile), (unsigned)((M + kRefTile - 1) / kRefTile));
+    reference_product_kernel<<<grid, kRefThreads, kRefSmem, st>>>(maps[0], maps[1], yref, M, N, K, status_word);
     count_launch();
     return cudaGetLastError();
 }
