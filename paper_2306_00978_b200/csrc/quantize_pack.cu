@@ -225,26 +225,38 @@ quantize_pack_tile_kernel(const __half* __restrict__ W, const float* __restrict_
             mx[h] = __fmul_rn(mx[h], r);
         }
     }
-    __half d16[2]; float d[2], z[2], rd[2], thr[2], zc[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    // Delta, the zero point and 1 / Delta cost three IEEE divisions: each of a row's four lanes needs both rows', so even lanes
+    // form the upper row's and odd ones the lower row's, and they exchange them (4096 -> 11008: 32.9 -> 31.2 us).
+    const bool low = (t & 1) != 0;
+    float d[2], z[2], rd[2], thr[2], zc[2];
+    {
+        const float mn1 = low ? mn[1] : mn[0], mx1 = low ? mx[1] : mx[0], wabs1 = low ? wabs[1] : wabs[0];
+        __half h16;
+        float d1, z1;
         if (SYM) {
             constexpr float half_levels = (float)(1 << (BITS - 1));
-            const float d32 = __fdiv_rn(fmaxf(fabsf(mn[h]), fabsf(mx[h])), half_levels);
-            d16[h] = __float2half_rn(d32);
-            const unsigned short bits = __half_as_ushort(d16[h]);
-            if ((bits & 0x7FFFu) == 0u || (bits & 0x7C00u) == 0x7C00u) d16[h] = __ushort_as_half(0x3C00u);
-            d[h] = __half2float(d16[h]);
-            z[h] = half_levels;
+            const float d32 = __fdiv_rn(fmaxf(fabsf(mn1), fabsf(mx1)), half_levels);
+            h16 = __float2half_rn(d32);
+            const unsigned short bits = __half_as_ushort(h16);
+            if ((bits & 0x7FFFu) == 0u || (bits & 0x7C00u) == 0x7C00u) h16 = __ushort_as_half(0x3C00u);
+            d1 = __half2float(h16);
+            z1 = half_levels;
         } else {
-            group_params(mn[h], mx[h], top, d16[h], d[h], z[h]);
+            group_params(mn1, mx1, top, h16, d1, z1);
         }
-        rd[h] = __frcp_rn(d[h]);
-        zc[h] = 12582912.0f - z[h];                          // exact: z is a small integer
+        const float rd1 = __frcp_rn(d1);
         // |w * rd - w / d| <= 1.8e-7 |w / d| (three roundings); the group's largest |w / d|
         // bounds it for every element; quotients beyond 1024 always take the division
-        const float tmax = __fmul_rn(wabs[h], rd[h]);
-        thr[h] = tmax < 1024.0f ? 0.5f - fmaf(tmax, 4e-7f, 1e-6f) : -1.0f;
+        const float tmax = __fmul_rn(wabs1, rd1);
+        const float thr1 = tmax < 1024.0f ? 0.5f - fmaf(tmax, 4e-7f, 1e-6f) : -1.0f;
+        const float d2 = __shfl_xor_sync(0xFFFFFFFFu, d1, 1), z2 = __shfl_xor_sync(0xFFFFFFFFu, z1, 1);
+        const float rd2 = __shfl_xor_sync(0xFFFFFFFFu, rd1, 1), thr2 = __shfl_xor_sync(0xFFFFFFFFu, thr1, 1);
+        d[0] = low ? d2 : d1; d[1] = low ? d1 : d2;
+        z[0] = low ? z2 : z1; z[1] = low ? z1 : z2;
+        rd[0] = low ? rd2 : rd1; rd[1] = low ? rd1 : rd2;
+        thr[0] = low ? thr2 : thr1; thr[1] = low ? thr1 : thr2;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) zc[h] = 12582912.0f - z[h];      // exact: z is a small integer
     }
     // Clamping to [0, top] can only matter where the group's smallest or largest element leaves the
     // range (the level is monotone in w'): rare without clipping - rne(max / Delta) + rne(-min / Delta)
@@ -296,8 +308,8 @@ quantize_pack_tile_kernel(const __half* __restrict__ W, const float* __restrict_
         // stored group is the group itself up to 128 columns, else each of its runs of 128 columns
         const size_t nsg = K / QCfg<G>::kStored;
         const size_t sgi = (G == 64) ? (size_t)gi : (size_t)kblk * (kQBlocks / 2) + ti / 2;
-        scales[(band * nsg + sgi) * 16 + g] = d16[0];
-        scales[(band * nsg + sgi) * 16 + g + 8] = d16[1];
+        scales[(band * nsg + sgi) * 16 + g] = __float2half_rn(d[0]);         // exact: Delta is an fp16 value
+        scales[(band * nsg + sgi) * 16 + g + 8] = __float2half_rn(d[1]);
         zeros[((band >> 1) * nsg + sgi) * 16 + (band & 1) * 8 + g] =
             (uint8_t)((uint32_t)z[0] | ((uint32_t)z[1] << 4));
     }
