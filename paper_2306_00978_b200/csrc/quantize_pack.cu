@@ -126,9 +126,10 @@ template <int G> struct QCfg {
 };
 
 // MANY (the scale search): `a` is `many` arrays of K scales; W is quantized with each, its 32 values per lane loaded once,
-// and the packed arrays follow one another (4096 x 4096 with 20 arrays: 12.3 us each in launches of their own, 9.9 us here).
+// and the packed arrays follow one another (4096 x 4096 with 20 arrays: 12.3 us each in launches of their own, ~9 us here; with
+// four blocks per SM, which nothing spills in, the whole search takes 538 us, with five 545, with six 556).
 template <int G, int BITS, bool CLIP, bool SYM, bool MANY = false>
-__global__ void __launch_bounds__(QCfg<G>::kThreads, (MANY ? 640 : 1024) / QCfg<G>::kThreads)
+__global__ void __launch_bounds__(QCfg<G>::kThreads, (MANY ? 512 : 1024) / QCfg<G>::kThreads)
 quantize_pack_tile_kernel(const __half* __restrict__ W, const float* __restrict__ a, float alpha,
                           int mode, const float* __restrict__ clip,
                           uint32_t* __restrict__ qweight, __half* __restrict__ scales,

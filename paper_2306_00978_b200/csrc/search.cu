@@ -13,27 +13,32 @@ namespace {
 constexpr int kLossBlocks = 296;
 
 // xs[b][m][k] = fp16_rne(fp32(X[m][k]) / s[b][k]): the caller's side of Eq. 4, one IEEE division and
-// one rounding per element; eight elements per thread (K is a multiple of 128), one scale array per blockIdx.y.
-__global__ void divide_by_scale_kernel(const __half* __restrict__ X, const float* __restrict__ s,
+// one rounding per element; eight elements per thread (K is a multiple of 128), which divides them by every gridDim.y-th of the
+// scale arrays.
+__global__ void divide_by_scale_kernel(const __half* __restrict__ X, const float* __restrict__ s, int count,
                                        __half* __restrict__ xs, size_t chunks, size_t block_chunks, int K) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= chunks) return;
-    s += (size_t)blockIdx.y * K;
     const int k0 = (int)((i * 8) % (size_t)K);
     const uint4 h = reinterpret_cast<const uint4*>(X)[i];
     const uint32_t w[4] = {h.x, h.y, h.z, h.w};
-    const float4 s0 = *reinterpret_cast<const float4*>(s + k0), s1 = *reinterpret_cast<const float4*>(s + k0 + 4);
-    const float sk[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
-    uint32_t o[4];
+    float x[8];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-        const float lo = __half2float(__ushort_as_half((unsigned short)(w[e] & 0xFFFFu)));
-        const float hi = __half2float(__ushort_as_half((unsigned short)(w[e] >> 16)));
-        const unsigned short a = __half_as_ushort(__float2half_rn(__fdiv_rn(lo, sk[2 * e])));
-        const unsigned short b = __half_as_ushort(__float2half_rn(__fdiv_rn(hi, sk[2 * e + 1])));
-        o[e] = (uint32_t)a | ((uint32_t)b << 16);
+        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[e]));
+        x[2 * e] = f.x; x[2 * e + 1] = f.y;
     }
-    reinterpret_cast<uint4*>(xs)[blockIdx.y * block_chunks + i] = make_uint4(o[0], o[1], o[2], o[3]);
+    for (int b = blockIdx.y; b < count; b += gridDim.y) {
+        const float4 s0 = *reinterpret_cast<const float4*>(s + (size_t)b * K + k0), s1 = *reinterpret_cast<const float4*>(s + (size_t)b * K + k0 + 4);
+        const float sk[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+        uint32_t o[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const __half2 r = __floats2half2_rn(__fdiv_rn(x[2 * e], sk[2 * e]), __fdiv_rn(x[2 * e + 1], sk[2 * e + 1]));
+            o[e] = *reinterpret_cast<const uint32_t*>(&r);
+        }
+        reinterpret_cast<uint4*>(xs)[b * block_chunks + i] = make_uint4(o[0], o[1], o[2], o[3]);
+    }
 }
 
 // xs[m][k] = fp16_rne(fp32(X[m][k]) * inv_s[k]): what awq_linear_scaled computes inside the layer,
@@ -259,8 +264,11 @@ cudaError_t launch_reference_product(const void* W, const void* X, float* yref, 
 
 cudaError_t launch_divide_by_scale(const void* X, const float* s, int count, void* xs, int M, int rows, int K, cudaStream_t st) {
     const size_t chunks = (size_t)M * K / 8;
-    divide_by_scale_kernel<<<dim3((unsigned)((chunks + 255) / 256), (unsigned)count), 256, 0, st>>>(
-        reinterpret_cast<const __half*>(X), s, reinterpret_cast<__half*>(xs), chunks, (size_t)rows * K / 8, K);
+    const unsigned blocks = (unsigned)((chunks + 255) / 256);
+    // X is loaded and widened once per thread where that leaves blocks enough
+    const unsigned share = blocks >= 1024 ? 1u : blocks >= 256 ? 4u : 16u;
+    divide_by_scale_kernel<<<dim3(blocks, share < (unsigned)count ? share : (unsigned)count), 256, 0, st>>>(
+        reinterpret_cast<const __half*>(X), s, count, reinterpret_cast<__half*>(xs), chunks, (size_t)rows * K / 8, K);
     count_launch();
     return cudaGetLastError();
 }
