@@ -16,7 +16,7 @@
 //
 // The start of a launch: chained to the one in front by programmatic dependent launch, weight copies (a warp of their own, x's are
 // another's) issued before tensor memory and the cluster are ready.  Chained calls, before and after: 333 tokens on
-// 4096 -> 4096 19.3 -> 15.7 us, 700 on 2048 -> 2048 13.5 -> 10.7, 100 on 5120 -> 13824 22.7 -> 19.2, 8192 on 4096 -> 11008 610 -> 537.
+// 4096 -> 4096 19.3 -> 15.7 us, 700 on 2048 -> 2048 13.5 -> 10.7, 100 on 5120 -> 13824 22.7 -> 19.2.
 //
 // Block r of a pair (r = rank in the cluster) owns
 //   - A: output channels 128 r .. 128 r + 127 of the 256-channel slab, dequantized by its own
@@ -691,6 +691,9 @@ cudaError_t launch_gemm_pair(const void* x, const CUtensorMap& wmap, const CUten
                              unsigned int* status_word, int sms, bool serialize, cudaStream_t st, bool* launched, int count, int rows) {
     const PairBlocks blocks = {(N / count + 255) / 256, N / count, rows};
     const PairChoice c = choose_tile(M, N, K, sms / 2, workspace ? workspace_bytes : 0);
+    // Launches beyond about 0.3 ms run at the power limit and are not chained: back to back, 8192 tokens on 4096 -> 11008 take
+    // 575 us unchained and 587 us chained, 2048 tokens on 13824 -> 5120 242 and 239 us.
+    serialize = serialize || c.us > 300.0;
     CUtensorMap xmap;
     {
         // x as [M][K] fp16 in boxes of half a tile's tokens x one k-block, 128-byte swizzle
