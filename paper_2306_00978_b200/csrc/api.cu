@@ -188,9 +188,11 @@ static bool mid_kernel_preferred(int M, int N, int K) {
 // matrix-vector kernel does not serve, take it from 4 tokens where x does not stay in the band kernel's registers (stream / band,
 // us: 11008 -> 4096 at 4 / 8 tokens 10.5 / 10.4 against 10.9 / 16.1, 8192 -> 28672 32.1 / 32.7 against 34.7 / 49.1).
 static bool stream_kernel_preferred(int M, int total_n, int K, int group, int sms, bool several = false) {
-    if (M > 64 || !gemm_stream_applies(M, total_n, K, group)) return false;
-    if (M > 8 || !gemv_uses_band_kernel(M, total_n, sms)) return true;
-    return several && M >= 4 && K > 4096 && (long long)total_n * K >= (1LL << 25);
+    if (M > 64) return false;
+    if (M <= 8 && gemv_uses_band_kernel(M, total_n, sms) &&
+        !(several && M >= 4 && K > 4096 && (long long)total_n * K >= (1LL << 25)))
+        return false;
+    return gemm_stream_applies(M, total_n, K, group);
 }
 
 // Above 64 tokens the stream kernel is taken where its estimate is below the prefill kernels' (few tiles for many pairs, long
