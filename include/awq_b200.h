@@ -194,7 +194,7 @@ int awq_linear(const void* x, const void* qweight, const void* scales, const voi
  * comparable to its launch overhead).  y_i = x . dequant(Wq_i)^T for i < count, count <= 4; all
  * matrices share K and `group`, each has its own N.  `problems` is a HOST array read during the
  * call.  For M <= 8 with enough output rows in total the matrices are served by ONE launch of
- * the matrix-vector band kernel (from 4 tokens on long rows, K > 4096, of the stream kernel), for other M <= 64,
+ * the matrix-vector band kernel, which uses no workspace, for other M <= 64,
  * and up to 256 where its estimate is below that of separate calls, by one launch of the stream kernel if
  * the workspace holds awq_workspace_bytes(M, sum of the N, K, group); otherwise this is the same as
  * `count` awq_linear calls.  Each output is what awq_linear would give with the band kernel (bit-identical when awq_linear picks

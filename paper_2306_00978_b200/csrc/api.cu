@@ -184,15 +184,12 @@ static bool mid_kernel_preferred(int M, int N, int K) {
 }
 
 // Where the stream kernel runs up to 64 tokens: from 9, and below where the output rows are too few for the band kernel
-// (1024 -> 8192 at 3 / 8 tokens 4.8 / 4.9 us; the split-K kernel 8 and 10 us).  Calls of several matrices, which the chunked
-// matrix-vector kernel does not serve, take it from 4 tokens where x does not stay in the band kernel's registers (stream / band,
-// us: 11008 -> 4096 at 4 / 8 tokens 10.5 / 10.4 against 10.9 / 16.1, 8192 -> 28672 32.1 / 32.7 against 34.7 / 49.1).
-static bool stream_kernel_preferred(int M, int total_n, int K, int group, int sms, bool several = false) {
-    if (M > 64) return false;
-    if (M <= 8 && gemv_uses_band_kernel(M, total_n, sms) &&
-        !(several && M >= 4 && K > 4096 && (long long)total_n * K >= (1LL << 25)))
-        return false;
-    return gemm_stream_applies(M, total_n, K, group);
+// (1024 -> 8192 at 3 / 8 tokens 4.8 / 4.9 us; the split-K kernel 8 and 10 us).  Calls of several matrices with rows enough stay on the
+// band kernel up to 8 tokens, although on long rows it is the slower one from 4 (stream / band, us: 8192 -> 28672 at 4 / 8 tokens
+// 32.1 / 32.7 against 34.7 / 49.1): it gives the bits that each matrix gets by itself, and it touches no workspace, so such calls may run
+// on several streams at once.
+static bool stream_kernel_preferred(int M, int total_n, int K, int group, int sms) {
+    return M <= 64 && (M > 8 || !gemv_uses_band_kernel(M, total_n, sms)) && gemm_stream_applies(M, total_n, K, group);
 }
 
 // Above 64 tokens the stream kernel is taken where its estimate is below the prefill kernels' (few tiles for many pairs, long
@@ -434,7 +431,7 @@ int awq_linear_multi(const void* x, const AwqLinearProblem* problems, int count,
     if (!aligned16(x)) return AWQ_ERR_MISALIGNED;
     DeviceState* d;
     if (int rc = device_state(&d)) return rc;
-    if (stream_kernel_preferred(M, total_n, K, group, d->sms, count > 1) || (count > 1 && stream_beats_prefill(d, problems, count, M, K, group))) {
+    if (stream_kernel_preferred(M, total_n, K, group, d->sms) || (count > 1 && stream_beats_prefill(d, problems, count, M, K, group))) {
         bool launched = false;
         const int rc = linear_multi_stream(d, x, nullptr, problems, count, M, K, group, stream, &launched);
         if (rc != AWQ_OK || launched) return rc;
@@ -504,7 +501,7 @@ int awq_linear_multi_scaled(const void* x, const float* inv_s, void* x_scratch, 
                                           take_packed_written(d), (cudaStream_t)stream, inv_s));
     }
     if (!x_scratch) return AWQ_ERR_NULL_POINTER;
-    if (stream_kernel_preferred(M, total_n, K, group, d->sms, count > 1) || stream_beats_prefill(d, problems, count, M, K, group)) {
+    if (stream_kernel_preferred(M, total_n, K, group, d->sms) || stream_beats_prefill(d, problems, count, M, K, group)) {
         bool launched = false;
         const int rc = linear_multi_stream(d, x, inv_s, problems, count, M, K, group, stream, &launched);
         if (rc != AWQ_OK || launched) return rc;
