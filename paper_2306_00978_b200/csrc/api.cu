@@ -15,6 +15,43 @@ constexpr int kMaxDevices = 64;
 std::atomic<unsigned long long> g_launches{0};
 thread_local char t_cuda_error[256] = "";
 
+// A stream, and the capture that it is in (0: none).  A handle that comes back after cudaStreamDestroy is no harm: the new stream's
+// first launch waits once for nothing.  (cudaStreamGetId would tell them apart, but it invalidates a capture.)
+struct StreamKey {
+    unsigned long long stream, capture;
+    bool operator==(const StreamKey& o) const { return stream == o.stream && capture == o.capture; }
+};
+// Streams on which one of this library's kernels that write packed arrays (quantizer, 3-bit packing and expansion) has been
+// enqueued and no layer call since.  Most layer kernels copy weights before the launch in front of them has completed, so the
+// first one behind such a writer on the same stream is launched fully serialized; what runs on other streams changes nothing.
+struct PendingWriters {
+    static constexpr int kMost = 64;
+    struct Entry { StreamKey key; unsigned long long serial; };
+    Entry list[kMost];
+    int count = 0;
+    unsigned long long serial = 0;         // of the last writer
+    bool overflow = false;                 // more streams than fit: every launch is serialized until the device has been waited for
+
+    void add(const StreamKey& key) {
+        ++serial;
+        for (int i = 0; i < count; ++i)
+            // a stream is in one capture at a time: a writer in an earlier one can have no reader any more
+            if (list[i].key.stream == key.stream && (list[i].key.capture != 0) == (key.capture != 0)) { list[i] = {key, serial}; return; }
+        if (count < kMost) list[count++] = {key, serial}; else overflow = true;
+    }
+    unsigned long long pending(const StreamKey& key) const {         // the writer's serial, 0: none
+        for (int i = 0; i < count; ++i) if (list[i].key == key) return list[i].serial;
+        return 0;
+    }
+    void remove(const StreamKey& key, unsigned long long upto) {
+        for (int i = 0; i < count; ++i) if (list[i].key == key && list[i].serial <= upto) { list[i] = list[--count]; return; }
+    }
+    void completed(unsigned long long upto) {                        // all work enqueued before this serial's writer, and it, has ended
+        for (int i = 0; i < count;) if (list[i].key.capture == 0 && list[i].serial <= upto) list[i] = list[--count]; else ++i;
+        if (upto == serial) overflow = false;
+    }
+};
+
 struct DeviceState {
     void* workspace = nullptr;
     size_t workspace_bytes = 0;
@@ -22,13 +59,10 @@ struct DeviceState {
     int cc_major = -1;
     int sms = 0;
     int tx_surplus_once = 0;               // time-out test: see awq_test_stall_next_gemv
-    // Set when one of this library's kernels that writes packed arrays (the quantizer) has been
-    // enqueued since the last matrix-vector launch: the band kernel prefetches weights before its
-    // stream dependency resolves, so the first launch after such a writer is fully serialized.
-    bool packed_written = false;
+    PendingWriters writers;
 };
 DeviceState g_dev[kMaxDevices];
-std::mutex g_mutex;
+std::mutex g_mutex;                        // DeviceState's fields
 
 // [0]: 0, or a code written by a kernel that gave up a wait; [1]: limit of a device-side wait in
 // microseconds (0 = the built-in default)
@@ -69,12 +103,55 @@ int device_state(DeviceState** out) {
     return AWQ_OK;
 }
 
-// True once after a packed-array writer of this library was enqueued on the device.
-bool take_packed_written(DeviceState* d) {
+thread_local char t_per_thread_stream;     // its address stands for the calling thread's cudaStreamPerThread
+
+StreamKey stream_key(cudaStream_t st) {
+    StreamKey key = {(unsigned long long)(uintptr_t)st, 0};
+    if (st == cudaStreamLegacy) key.stream = 0;
+    if (st == cudaStreamPerThread) key.stream = (unsigned long long)(uintptr_t)&t_per_thread_stream;
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) (void)cudaGetLastError();
+    else if (status != cudaStreamCaptureStatusNone) key.capture = id;
+    return key;
+}
+
+// Called after a writer of packed arrays has been enqueued.  (Not before: another thread's layer call on the same stream could take
+// the entry and be enqueued in front of the writer.)
+void note_packed_writer(DeviceState* d, void* stream) {
+    const StreamKey key = stream_key((cudaStream_t)stream);
     std::lock_guard<std::mutex> lock(g_mutex);
-    const bool w = d->packed_written;
-    d->packed_written = false;
-    return w;
+    d->writers.add(key);
+}
+
+// How a layer's launch is ordered behind the work in front of it.
+struct LaunchOrder {
+    DeviceState* d;
+    StreamKey key;
+    unsigned long long writer;             // serial of the writer that it waits for, 0: none is known
+    bool serialize;
+    // the kernel is in the stream: the launches behind it need not wait for that writer any more
+    cudaError_t launched(cudaError_t e) const {
+        if (e == cudaSuccess && writer != 0) {
+            std::lock_guard<std::mutex> lock(g_mutex);
+            d->writers.remove(key, writer);
+        }
+        return e;
+    }
+};
+// behind_writer: the call itself has just enqueued a kernel that writes what this launch reads
+LaunchOrder launch_order(DeviceState* d, void* stream, bool behind_writer = false) {
+    LaunchOrder o = {d, {0, 0}, 0, behind_writer};
+    {
+        std::lock_guard<std::mutex> lock(g_mutex);
+        if (d->writers.overflow) o.serialize = true;
+        if (d->writers.count == 0) return o;
+    }
+    o.key = stream_key((cudaStream_t)stream);
+    std::lock_guard<std::mutex> lock(g_mutex);
+    o.writer = d->writers.pending(o.key);
+    if (o.writer != 0) o.serialize = true;
+    return o;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -132,14 +209,12 @@ int awq_quantize_pack_ex(const void* W, const float* act_mean_abs, float alpha, 
         return AWQ_ERR_MISALIGNED;
     DeviceState* d;
     if (int rc = device_state(&d)) return rc;
-    {
-        std::lock_guard<std::mutex> lock(g_mutex);
-        d->packed_written = true;
-    }
-    return note_cuda(launch_quantize_pack(reinterpret_cast<const __half*>(W), act_mean_abs, alpha, group, bits,
-                                          symmetric != 0, clip_ratio, reinterpret_cast<uint32_t*>(qweight),
-                                          reinterpret_cast<__half*>(scales),
-                                          reinterpret_cast<uint8_t*>(zeros), N, K, (cudaStream_t)stream));
+    const int rc = note_cuda(launch_quantize_pack(reinterpret_cast<const __half*>(W), act_mean_abs, alpha, group, bits,
+                                                  symmetric != 0, clip_ratio, reinterpret_cast<uint32_t*>(qweight),
+                                                  reinterpret_cast<__half*>(scales),
+                                                  reinterpret_cast<uint8_t*>(zeros), N, K, (cudaStream_t)stream));
+    note_packed_writer(d, stream);
+    return rc;
 }
 
 int awq_quantize_pack(const void* W, const float* act_mean_abs, float alpha, int group,
@@ -294,6 +369,8 @@ int awq_linear_path(const void* x, const void* qweight, const void* scales, cons
         if (stream_beats_prefill(d, &one, 1, M, K, group)) path = AWQ_PATH_GEMM_SKINNY;
     }
     if (path == AWQ_PATH_GEMV_MID && M > 8 && gemm_stream_applies(M, N, K, group)) path = AWQ_PATH_GEMM_SKINNY;
+    const cudaStream_t st = (cudaStream_t)stream;
+    const LaunchOrder order = launch_order(d, stream);
     if (path == AWQ_PATH_GEMV_MID) {
         if (!gemv_mid_applies(M, N, K, group, d->sms)) return AWQ_ERR_BAD_SHAPE;
         void* ws = nullptr;
@@ -302,8 +379,8 @@ int awq_linear_path(const void* x, const void* qweight, const void* scales, cons
             if (d->workspace_bytes < gemv_mid_workspace_bytes(M, N, K)) return AWQ_ERR_NO_WORKSPACE;
             ws = d->workspace;
         }
-        return note_cuda(launch_gemv_mid(x, qweight, scales, zeros, y, M, N, K, group, ws, d->status_word, d->sms,
-                                         take_packed_written(d), (cudaStream_t)stream));
+        return note_cuda(order.launched(launch_gemv_mid(x, qweight, scales, zeros, y, M, N, K, group, ws, d->status_word, d->sms,
+                                                        order.serialize, st)));
     }
     if (path == AWQ_PATH_GEMM_SKINNY) {
         const size_t need = gemm_stream_workspace_bytes(M, d->sms);
@@ -314,17 +391,14 @@ int awq_linear_path(const void* x, const void* qweight, const void* scales, cons
             ws = d->workspace;
         }
         const GemvMatrix one = {qweight, scales, zeros, y, N};
-        return note_cuda(launch_gemm_stream(x, &one, 1, M, K, group, nullptr, ws, d->status_word,
-                                            d->sms, take_packed_written(d), (cudaStream_t)stream));
+        return note_cuda(order.launched(launch_gemm_stream(x, &one, 1, M, K, group, nullptr, ws, d->status_word,
+                                                           d->sms, order.serialize, st)));
     }
-    const bool tensor_path = path == AWQ_PATH_GEMM || path == AWQ_PATH_GEMM_1SM;
-    const cudaStream_t st = (cudaStream_t)stream;
     if (path == AWQ_PATH_GEMV && gemv_uses_band_kernel(M, N, d->sms)) {
         const GemvMatrix one = {qweight, scales, zeros, y, N};
-        return note_cuda(launch_gemv_band(x, &one, 1, M, K, group, d->status_word, d->sms,
-                                          take_packed_written(d), st));
+        return note_cuda(order.launched(launch_gemv_band(x, &one, 1, M, K, group, d->status_word, d->sms, order.serialize, st)));
     }
-    const bool serialize = take_packed_written(d);   // (split-K and one-SM kernels are plainly stream-ordered)
+    // (split-K and one-SM kernels are plainly stream-ordered)
     if (path == AWQ_PATH_GEMV || path == AWQ_PATH_GEMV_SPLITK) {
         void* ws = nullptr;
         {
@@ -338,8 +412,8 @@ int awq_linear_path(const void* x, const void* qweight, const void* scales, cons
             surplus = d->tx_surplus_once;
             d->tx_surplus_once = 0;
         }
-        return note_cuda(launch_gemv_splitk(x, qweight, scales, zeros, y, M, N, K, group, ws, d->status_word,
-                                            d->sms, st, surplus));
+        return note_cuda(order.launched(launch_gemv_splitk(x, qweight, scales, zeros, y, M, N, K, group, ws, d->status_word,
+                                                           d->sms, st, surplus)));
     }
     void* ws = nullptr;
     size_t ws_bytes = 0;
@@ -348,8 +422,8 @@ int awq_linear_path(const void* x, const void* qweight, const void* scales, cons
         ws = d->workspace;
         ws_bytes = d->workspace_bytes;
     }
-    return note_cuda(launch_gemm(x, qweight, scales, zeros, y, M, N, K, group, path != AWQ_PATH_GEMM_1SM,
-                                 ws, ws_bytes, d->status_word, serialize, st));
+    return note_cuda(order.launched(launch_gemm(x, qweight, scales, zeros, y, M, N, K, group, path != AWQ_PATH_GEMM_1SM,
+                                                ws, ws_bytes, d->status_word, order.serialize, st)));
 }
 
 int awq_linear_gemv_static(const void* x, const void* qweight, const void* scales, const void* zeros,
@@ -409,8 +483,9 @@ static int linear_multi_stream(DeviceState* d, const void* x, const float* inv_s
     for (int i = 0; i < count; ++i)
         mats[i] = GemvMatrix{problems[i].qweight, problems[i].scales, problems[i].zeros, problems[i].y, problems[i].N};
     *launched = true;
-    return note_cuda(launch_gemm_stream(x, mats, count, M, K, group, inv_s, ws, d->status_word, d->sms,
-                                        take_packed_written(d), (cudaStream_t)stream));
+    const LaunchOrder order = launch_order(d, stream);
+    return note_cuda(order.launched(launch_gemm_stream(x, mats, count, M, K, group, inv_s, ws, d->status_word, d->sms,
+                                                       order.serialize, (cudaStream_t)stream)));
 }
 
 int awq_linear_multi(const void* x, const AwqLinearProblem* problems, int count,
@@ -441,8 +516,9 @@ int awq_linear_multi(const void* x, const AwqLinearProblem* problems, int count,
         for (int i = 0; i < count; ++i)
             mats[i] = GemvMatrix{problems[i].qweight, problems[i].scales, problems[i].zeros, problems[i].y,
                                  problems[i].N};
-        return note_cuda(launch_gemv_band(x, mats, count, M, K, group, d->status_word, d->sms,
-                                          take_packed_written(d), (cudaStream_t)stream));
+        const LaunchOrder order = launch_order(d, stream);
+        return note_cuda(order.launched(launch_gemv_band(x, mats, count, M, K, group, d->status_word, d->sms, order.serialize,
+                                                         (cudaStream_t)stream)));
     }
     // otherwise one call per matrix, as awq_linear would run it
     for (int i = 0; i < count; ++i) {
@@ -497,8 +573,9 @@ int awq_linear_multi_scaled(const void* x, const float* inv_s, void* x_scratch, 
         for (int i = 0; i < count; ++i)
             mats[i] = GemvMatrix{problems[i].qweight, problems[i].scales, problems[i].zeros, problems[i].y,
                                  problems[i].N};
-        return note_cuda(launch_gemv_band(x, mats, count, M, K, group, d->status_word, d->sms,
-                                          take_packed_written(d), (cudaStream_t)stream, inv_s));
+        const LaunchOrder order = launch_order(d, stream);
+        return note_cuda(order.launched(launch_gemv_band(x, mats, count, M, K, group, d->status_word, d->sms, order.serialize,
+                                                         (cudaStream_t)stream, inv_s)));
     }
     if (!x_scratch) return AWQ_ERR_NULL_POINTER;
     if (stream_kernel_preferred(M, total_n, K, group, d->sms) || stream_beats_prefill(d, problems, count, M, K, group)) {
@@ -528,11 +605,9 @@ int awq_pack_int3(const void* qweight, void* qweight3, int N, int K, void* strea
     if (!aligned16(qweight) || !aligned16(qweight3)) return AWQ_ERR_MISALIGNED;
     DeviceState* d;
     if (int rc = device_state(&d)) return rc;
-    {
-        std::lock_guard<std::mutex> lock(g_mutex);
-        d->packed_written = true;
-    }
-    return note_cuda(launch_pack_int3(qweight, qweight3, N, K, (cudaStream_t)stream));
+    const int rc = note_cuda(launch_pack_int3(qweight, qweight3, N, K, (cudaStream_t)stream));
+    note_packed_writer(d, stream);
+    return rc;
 }
 
 int awq_unpack_int3(const void* qweight3, void* qweight, int N, int K, void* stream) {
@@ -541,11 +616,9 @@ int awq_unpack_int3(const void* qweight3, void* qweight, int N, int K, void* str
     if (!aligned16(qweight) || !aligned16(qweight3)) return AWQ_ERR_MISALIGNED;
     DeviceState* d;
     if (int rc = device_state(&d)) return rc;
-    {
-        std::lock_guard<std::mutex> lock(g_mutex);
-        d->packed_written = true;
-    }
-    return note_cuda(launch_unpack_int3(qweight3, qweight, N, K, (cudaStream_t)stream));
+    const int rc = note_cuda(launch_unpack_int3(qweight3, qweight, N, K, (cudaStream_t)stream));
+    note_packed_writer(d, stream);
+    return rc;
 }
 
 int awq_linear_int3(const void* x, const void* qweight3, const void* scales, const void* zeros, void* y,
@@ -561,8 +634,9 @@ int awq_linear_int3(const void* x, const void* qweight3, const void* scales, con
     if (int rc = device_state(&d)) return rc;
     if (M <= 8 && K <= 65536 && gemv_uses_band_kernel(M, N, d->sms)) {
         const GemvMatrix one = {qweight3, scales, zeros, y, N};
-        return note_cuda(launch_gemv_band(x, &one, 1, M, K, group, d->status_word, d->sms,
-                                          take_packed_written(d), (cudaStream_t)stream, nullptr, 3));
+        const LaunchOrder order = launch_order(d, stream);
+        return note_cuda(order.launched(launch_gemv_band(x, &one, 1, M, K, group, d->status_word, d->sms, order.serialize,
+                                                         (cudaStream_t)stream, nullptr, 3)));
     }
     // every other kernel reads the 4-bit layout: expand first (one more launch), then the plain call
     if (!qweight_scratch) return AWQ_ERR_NULL_POINTER;
@@ -603,7 +677,6 @@ int awq_search_alpha(const void* W, const float* act_mean_abs, const void* X, in
         std::lock_guard<std::mutex> lock(g_mutex);
         ws = d->workspace;
         ws_bytes = d->workspace_bytes;
-        d->packed_written = true;
     }
     if (int rc = note_cuda(launch_reference_product(W, X, p.yref, M, N, K, d->status_word, st))) return rc;
     if (int rc = note_cuda(launch_channel_scales(act_mean_abs, alphas, n_alphas, p.s, K, st))) return rc;
@@ -615,6 +688,7 @@ int awq_search_alpha(const void* W, const float* act_mean_abs, const void* X, in
                                                          reinterpret_cast<uint32_t*>(p.qweight), reinterpret_cast<__half*>(p.scales),
                                                          p.zeros, N, K, st)))
             return rc;
+        // (the plainly ordered division stands between this writer and its readers)
         if (int rc = note_cuda(launch_divide_by_scale(X, s, b, p.xs, M, p.rows, K, st))) return rc;
         // all products at once where the layer's kernel rounds (q - z) * Delta to fp16 too (above 64 tokens)
         bool launched = false;
@@ -661,7 +735,16 @@ int awq_unpack_canonical(const void* qweight, const void* scales, const void* ze
 int awq_poll_status(void) {
     DeviceState* d;
     if (int rc = device_state(&d)) return rc;
+    unsigned long long upto = 0;
+    {
+        std::lock_guard<std::mutex> lock(g_mutex);
+        upto = d->writers.serial;
+    }
     if (int rc = note_cuda(cudaDeviceSynchronize())) return rc;
+    {
+        std::lock_guard<std::mutex> lock(g_mutex);
+        d->writers.completed(upto);
+    }
     unsigned int v = 0;
     if (int rc = note_cuda(cudaMemcpy(&v, d->status_word, sizeof(v), cudaMemcpyDeviceToHost))) return rc;
     if (v != 0) {

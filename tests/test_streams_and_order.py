@@ -1,4 +1,8 @@
-"""Calls on several streams and threads: those that need no workspace may overlap."""
+"""Calls on several streams and threads: a layer call behind a writer of its packed arrays waits for it whatever runs elsewhere
+on the device, and calls that need no workspace may overlap.  How a launch is ordered behind the one in front is read from the
+edges of a captured graph, which is not launched."""
+import contextlib
+import ctypes
 import threading
 
 import numpy as np
@@ -7,6 +11,72 @@ import pytest
 from tests.util import Case, oracle_packed_to_cuda, to_cuda
 
 pytestmark = pytest.mark.gpu
+
+FULL, PROGRAMMATIC = 0, 1                # cudaGraphDependencyType
+
+
+class _EdgeData(ctypes.Structure):
+    _fields_ = [("from_port", ctypes.c_ubyte), ("to_port", ctypes.c_ubyte), ("type", ctypes.c_ubyte), ("reserved", ctypes.c_ubyte * 5)]
+
+
+@contextlib.contextmanager
+def _captured_edges(stream):
+    """Captures what is enqueued on `stream` inside; yields a list that holds the edges' types afterwards, in stream order."""
+    rt = ctypes.CDLL("libcudart.so.12")
+    ptr, size, types = ctypes.c_void_p, ctypes.c_size_t, []
+    handle, graph, n = ptr(stream.cuda_stream), ptr(), size()
+    assert rt.cudaStreamBeginCapture(handle, 2) == 0                      # relaxed: other streams go on as before
+    try:
+        yield types
+    finally:
+        assert rt.cudaStreamEndCapture(handle, ctypes.byref(graph)) == 0
+    assert rt.cudaGraphGetEdges_v2(graph, None, None, None, ctypes.byref(n)) == 0
+    begin, end, data = (ptr * n.value)(), (ptr * n.value)(), (_EdgeData * n.value)()
+    assert rt.cudaGraphGetEdges_v2(graph, begin, end, data, ctypes.byref(n)) == 0
+    follow = {b: (e, d.type) for b, e, d in zip(begin, end, data)}
+    assert len(follow) == n.value                                         # a chain
+    node = next(b for b in follow if b not in set(end))
+    while node in follow:
+        node, kind = follow[node]
+        types.append(kind)
+    assert rt.cudaGraphDestroy(graph) == 0
+
+
+def _operands(N, K, M, G, bits=4):
+    import torch
+    torch.manual_seed(N + K + M)
+    qw = torch.randint(0, 256, (N * K * bits // 8,), dtype=torch.uint8, device="cuda")
+    sc = (torch.rand((N // 16, K // G, 16), device="cuda") * 0.01 + 0.001).half()
+    zp = torch.randint(0, 256, (N // 32, K // G, 16), dtype=torch.uint8, device="cuda")
+    return torch.randn((M, K), device="cuda").half(), qw, sc, zp, torch.empty((M, N), dtype=torch.float16, device="cuda")
+
+
+@pytest.mark.parametrize("M", [1, 5, 16, 100, 300])      # band, chunked, stream and SM-pair kernel
+def test_a_call_on_another_stream_does_not_release_the_reader(M):
+    import torch
+    from paper_2306_00978_b200 import binding
+    N, K, G = (8192, 4096, 128) if M != 5 else (4096, 8320, 128)
+    L = binding.lib()
+    x, qw, sc, zp, y = _operands(N, K, M, G)
+    other = _operands(N, K, M, G)
+    W = (torch.randn((N, K), device="cuda") * 0.02).half()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+
+    def layer(stream, x, qw, sc, zp, y):
+        assert L.awq_linear(x.data_ptr(), qw.data_ptr(), sc.data_ptr(), zp.data_ptr(), y.data_ptr(), M, N, K, G, stream.cuda_stream) == 0
+
+    binding.linear(x, qw, sc, zp, N, K, G, out=y)
+    torch.cuda.synchronize()
+    layer(a, x, qw, sc, zp, y)
+    torch.cuda.synchronize()
+    with _captured_edges(a) as types:
+        assert L.awq_quantize_pack(W.data_ptr(), None, 0.0, G, qw.data_ptr(), sc.data_ptr(), zp.data_ptr(), N, K, a.cuda_stream) == 0
+        layer(b, *other)
+        layer(a, x, qw, sc, zp, y)
+        layer(a, x, qw, sc, zp, y)
+    binding.poll_status()
+    assert types[0] == FULL
+    assert PROGRAMMATIC in types[1:]                      # only the first call behind the writer is held back
 
 
 @pytest.mark.parametrize("widths,K,M,G", [((4096, 2304), 5248, 4, 128), ((2176, 4352), 8192, 8, 64)])
