@@ -5,6 +5,8 @@
 #include <cstring>
 #include <mutex>
 
+#include <cuda.h>
+
 #include "common.cuh"
 
 namespace awq {
@@ -74,12 +76,32 @@ int note_cuda(cudaError_t e) {
     return AWQ_ERR_CUDA;
 }
 
+// A thread that has not used the GPU has no context until the runtime makes one current, which a kernel launch does; tensor maps are
+// encoded by the driver in front of it, and that fails without one.
+int bind_context(int dev) {
+    typedef CUresult (*GetCurrentFn)(CUcontext*);
+    static const GetCurrentFn get_current = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPoint("cuCtxGetCurrent", &p, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            (void)cudaGetLastError();
+            p = nullptr;
+        }
+        return reinterpret_cast<GetCurrentFn>(p);
+    }();
+    CUcontext current = nullptr;
+    if (!get_current || (get_current(&current) == CUDA_SUCCESS && current)) return AWQ_OK;
+    return note_cuda(cudaSetDevice(dev));
+}
+
 // Per-device set-up on first use: compute capability and the status word's device address.
 int device_state(DeviceState** out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return note_cuda(e);
     if (dev < 0 || dev >= kMaxDevices) return AWQ_ERR_WRONG_DEVICE;
+    if (int rc = bind_context(dev)) return rc;
     std::lock_guard<std::mutex> lock(g_mutex);
     DeviceState& d = g_dev[dev];
     if (d.cc_major < 0) {

@@ -116,3 +116,35 @@ def test_several_matrices_up_to_8_tokens_need_no_workspace(widths, K, M, G):
         for plain, scaled in got[i]:
             assert all(torch.equal(y, w) for y, w in zip(plain, want[i]))
             assert all(torch.equal(y, w) for y, w in zip(scaled, want_scaled[i]))
+
+
+def test_calls_from_a_thread_that_has_not_used_the_gpu():
+    """Tensor maps are encoded by the driver in the thread's context, which nothing but the call itself has made current."""
+    import torch
+    from paper_2306_00978_b200 import binding
+    N, K, G = 1024, 1024, 128
+    L, n = binding.lib(), 3
+    operands = [(M, *_operands(N, K, M, G)) for M in (1, 16, 100, 300)]
+    for M, x, qw, sc, zp, y in operands:
+        binding.linear(x, qw, sc, zp, N, K, G, out=y)
+    W, X = (torch.randn((N, K), device="cuda") * 0.02).half(), torch.randn((96, K), device="cuda").half()
+    stat = X.float().abs().mean(dim=0)
+    alphas = [0.0, 0.5, 1.0]
+    want, best = binding.search_alpha(W, stat, X, G, alphas)
+    need = L.awq_search_scratch_bytes(96, N, K, G)
+    scratch = torch.empty(need, dtype=torch.uint8, device="cuda")
+    outs = [torch.empty_like(o[-1]) for o in operands]
+    a, losses, index = (ctypes.c_float * n)(*alphas), (ctypes.c_float * n)(), ctypes.c_int(-1)
+    torch.cuda.synchronize()
+    calls = [lambda o=o, y=y: L.awq_linear(*(t.data_ptr() for t in o[1:5]), y.data_ptr(), o[0], N, K, G, None) for o, y in zip(operands, outs)]
+    calls.append(lambda: L.awq_search_alpha(W.data_ptr(), stat.data_ptr(), X.data_ptr(), 96, N, K, G, a, n, losses, ctypes.byref(index),
+                                            scratch.data_ptr(), need, None))
+    status = []
+    for call in calls:
+        thread = threading.Thread(target=lambda: status.append(call()))
+        thread.start()
+        thread.join()
+    binding.poll_status()
+    assert status == [0] * len(calls)
+    assert all(torch.equal(y, o[-1]) for y, o in zip(outs, operands))
+    assert list(losses) == want and index.value == best
