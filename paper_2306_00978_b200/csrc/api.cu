@@ -355,8 +355,9 @@ int awq_set_workspace(void* dev_ptr, size_t bytes) {
     return AWQ_OK;
 }
 
-int awq_linear_path(const void* x, const void* qweight, const void* scales, const void* zeros,
-                    void* y, int M, int N, int K, int group, int path, void* stream) {
+// behind_writer: the caller has just enqueued a kernel that writes these packed arrays
+static int linear_path(const void* x, const void* qweight, const void* scales, const void* zeros,
+                       void* y, int M, int N, int K, int group, int path, void* stream, bool behind_writer) {
     if (int rc = check_shape(N, K, group)) return rc;
     group = stored_group(group);
     if (M < 1 || (long long)M * K > (1LL << 40) || (long long)M * N > (1LL << 40)) return AWQ_ERR_BAD_SHAPE;
@@ -392,7 +393,7 @@ int awq_linear_path(const void* x, const void* qweight, const void* scales, cons
     }
     if (path == AWQ_PATH_GEMV_MID && M > 8 && gemm_stream_applies(M, N, K, group)) path = AWQ_PATH_GEMM_SKINNY;
     const cudaStream_t st = (cudaStream_t)stream;
-    const LaunchOrder order = launch_order(d, stream);
+    const LaunchOrder order = launch_order(d, stream, behind_writer);
     if (path == AWQ_PATH_GEMV_MID) {
         if (!gemv_mid_applies(M, N, K, group, d->sms)) return AWQ_ERR_BAD_SHAPE;
         void* ws = nullptr;
@@ -446,6 +447,11 @@ int awq_linear_path(const void* x, const void* qweight, const void* scales, cons
     }
     return note_cuda(order.launched(launch_gemm(x, qweight, scales, zeros, y, M, N, K, group, path != AWQ_PATH_GEMM_1SM,
                                                 ws, ws_bytes, d->status_word, order.serialize, st)));
+}
+
+int awq_linear_path(const void* x, const void* qweight, const void* scales, const void* zeros,
+                    void* y, int M, int N, int K, int group, int path, void* stream) {
+    return linear_path(x, qweight, scales, zeros, y, M, N, K, group, path, stream, false);
 }
 
 int awq_linear_gemv_static(const void* x, const void* qweight, const void* scales, const void* zeros,
@@ -663,7 +669,7 @@ int awq_linear_int3(const void* x, const void* qweight3, const void* scales, con
     // every other kernel reads the 4-bit layout: expand first (one more launch), then the plain call
     if (!qweight_scratch) return AWQ_ERR_NULL_POINTER;
     if (int rc = awq_unpack_int3(qweight3, qweight_scratch, N, K, stream)) return rc;
-    return awq_linear(x, qweight_scratch, scales, zeros, y, M, N, K, group, stream);
+    return linear_path(x, qweight_scratch, scales, zeros, y, M, N, K, group, AWQ_PATH_AUTO, stream, true);
 }
 
 int awq_inverse_channel_scale(const float* act_mean_abs, float alpha, float* inv_s, int K, void* stream) {

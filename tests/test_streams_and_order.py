@@ -79,6 +79,41 @@ def test_a_call_on_another_stream_does_not_release_the_reader(M):
     assert PROGRAMMATIC in types[1:]                      # only the first call behind the writer is held back
 
 
+@pytest.mark.parametrize("M", [16, 300])
+def test_int3_expansion_and_its_reader_beside_another_thread(M):
+    import torch
+    from paper_2306_00978_b200 import binding
+    N, K, G, calls = 2048, 2048, 128, 300
+    L = binding.lib()
+    x, qw3, sc, zp, y = _operands(N, K, M, G, bits=3)
+    ox, oqw, osc, ozp, oy = _operands(N, K, M, G)
+    scratch = torch.empty(N * K // 2, dtype=torch.uint8, device="cuda")
+    a, b, stop = torch.cuda.Stream(), torch.cuda.Stream(), threading.Event()
+    binding.linear(ox, oqw, osc, ozp, N, K, G, out=oy)
+    torch.cuda.synchronize()
+
+    def others():
+        while not stop.is_set():
+            for _ in range(32):
+                assert L.awq_linear(ox.data_ptr(), oqw.data_ptr(), osc.data_ptr(), ozp.data_ptr(), oy.data_ptr(), M, N, K, G, b.cuda_stream) == 0
+            b.synchronize()
+
+    thread = threading.Thread(target=others)
+    thread.start()
+    try:
+        with _captured_edges(a) as types:
+            for _ in range(calls):
+                assert L.awq_linear_int3(x.data_ptr(), qw3.data_ptr(), sc.data_ptr(), zp.data_ptr(), y.data_ptr(), scratch.data_ptr(),
+                                         M, N, K, G, a.cuda_stream) == 0
+    finally:
+        stop.set()
+        thread.join()
+    binding.poll_status()
+    per_call = (len(types) + 1) // calls                  # the expansion, the layer's kernel, and the one that adds parts if there is one
+    assert per_call * calls == len(types) + 1 and per_call >= 2
+    assert [types[i * per_call] for i in range(calls)] == [FULL] * calls
+
+
 @pytest.mark.parametrize("widths,K,M,G", [((4096, 2304), 5248, 4, 128), ((2176, 4352), 8192, 8, 64)])
 def test_several_matrices_up_to_8_tokens_need_no_workspace(widths, K, M, G):
     """Long rows, many output rows: one launch of the band kernel, bit for bit what it gives each matrix alone, and nothing that two
