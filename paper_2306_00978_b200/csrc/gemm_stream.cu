@@ -127,28 +127,6 @@ __device__ __forceinline__ StTile st_tile(const StCut& c, int tile) {
 __device__ __forceinline__ size_t st_slot(const StCut& c, int slot, int rank) {
     return (size_t)(slot * 2 + rank) * (size_t)(c.rows * 128);
 }
-__device__ __forceinline__ uint32_t st_ctarank() {
-    uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r;
-}
-__device__ __forceinline__ uint32_t st_cluster_id() {
-    uint32_t r; asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r)); return r;
-}
-__device__ __forceinline__ uint32_t st_map_to_rank(uint32_t addr, uint32_t rank) {
-    uint32_t r; asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank)); return r;
-}
-__device__ __forceinline__ void st_arrive_cluster(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-// (what is handed over in front of it is the barriers' initialisation, which has a fence of its own)
-__device__ __forceinline__ void st_cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
-__device__ __forceinline__ void st_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ void st_umma(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
 // arrives on the barrier at this offset in both blocks of the pair when the products issued so far are done
 __device__ __forceinline__ void st_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
@@ -238,8 +216,8 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
 
     // (the shuffle tells the compiler that all lanes of a warp take the same role: addresses stay in uniform registers)
     const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    const uint32_t rank = st_ctarank();
-    const int pair = (int)st_cluster_id();
+    const uint32_t rank = cluster_ctarank();
+    const int pair = (int)cluster_id_x();
     const int nks = cut.nks, half_rows = cut.bn >> 1;
     const StRange range = st_range(cut, pair);
 
@@ -268,11 +246,11 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
     }
     if (warp == 0 || warp == 2) {
         asm volatile("bar.arrive 2, %0;" ::"r"(Cfg::kThreads) : "memory");
-        st_cluster_arrive();
+        cluster_arrive_start();
     } else {
         named_barrier_sync(2, Cfg::kThreads);
-        st_cluster_arrive();
-        st_cluster_wait();                   // both blocks' barriers exist before anyone arrives remotely
+        cluster_arrive_start();
+        cluster_wait();                   // both blocks' barriers exist before anyone arrives remotely
         tc_fence_after();
     }
     constexpr uint32_t tmem_base = 0;        // all 512 columns are this block's
@@ -360,7 +338,7 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
                     for (int h = h0; h < h1; ++h)
 #pragma unroll
                         for (int k = 0; k < kBK / 16; ++k)       // A: +8 columns, B: +32 bytes per K = 16 step
-                            st_umma(d_tmem, a_tmem + (uint32_t)(32 * h + 8 * k), bdesc + (uint64_t)(h * kb_step) + (uint64_t)(2 * k),
+                            umma_pair_f16_a_tmem(d_tmem, a_tmem + (uint32_t)(32 * h + 8 * k), bdesc + (uint64_t)(h * kb_step) + (uint64_t)(2 * k),
                                     idesc, (!start || h != h0 || k != 0) ? 1u : 0u);
                 };
                 if (EXACT) {
@@ -396,6 +374,9 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
                 if (++slot == (uint32_t)SL) { slot = 0; slot_phase ^= 1u; }
                 if (++ks == nks) ks = 0;
             }
+            // the epilogues' last arrivals, the other block's among them, are waited for here (see cluster_sync_end)
+            for (uint32_t b = 0; b < NACC && mbar_wait_warp(acc_empty(acc), acc_phase ^ 1u, ctl); ++b)
+                if (++acc == NACC) { acc = 0; acc_phase ^= 1u; }
         }
     } else if (warp >= 8 && warp < 24) {
         // ------------------------------------------------------------ dequantizers
@@ -405,7 +386,7 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
         const int band = 2 * quad + hsel;                // bands 0..7 <-> TMEM lanes 16 * band .. +15
         const int g = lane >> 2;
         const uint32_t taddr_band = tmem_base + ((uint32_t)(quad * 32 + hsel * 16) << 16) + (uint32_t)Cfg::kA0;
-        const uint32_t leader_a_full0 = st_map_to_rank(a_full(0), 0);
+        const uint32_t leader_a_full0 = map_to_rank(a_full(0), 0);
         const unsigned char* w_lane = base_ptr + Cfg::kXBytes + band * (kStTiles * 512) + lane * 16;
         // x's channels are brought into A's order in shared memory, 16 of a token (32 bytes) per thread and pass
         constexpr int kThreadsPerKb = 4 * Cfg::kHalf, kKbPerPass = 256 / kThreadsPerKb < kStTiles ? 256 / kThreadsPerKb : kStTiles;
@@ -494,7 +475,7 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
             tmem_st_wait();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) st_arrive_cluster(leader_a_full0 + 8u * slot);
+            if (lane == 0) mbar_arrive_cluster(leader_a_full0 + 8u * slot);
             stage += 2;
             if (stage >= (uint32_t)S) { stage -= S; phase ^= 1u; }
             old += 2;
@@ -510,7 +491,7 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
         asm volatile("griddepcontrol.wait;" ::: "memory");
         const int quad = warp & 3, thalf = warp >= 24 ? 1 : 0;
         const uint32_t taddr0 = tmem_base + ((uint32_t)(quad * 32) << 16);
-        const uint32_t leader_acc_empty0 = st_map_to_rank(acc_empty(0), 0);
+        const uint32_t leader_acc_empty0 = map_to_rank(acc_empty(0), 0);
         const unsigned char* sc_lane = base_ptr + Cfg::kParOff + (2 * quad + (lane >> 4)) * (GPS * 32) + (lane & 15) * 2;
         uint32_t acc = 0, acc_phase = 0, stage = 0, phase = 0;
         bool ok = true;
@@ -550,7 +531,7 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
                         tmem_ld_wait(r0, r1);
                         tc_fence_before();
                         __syncwarp();
-                        if (lane == 0) st_arrive_cluster(leader_acc_empty0 + 8u * acc);
+                        if (lane == 0) mbar_arrive_cluster(leader_acc_empty0 + 8u * acc);
 #pragma unroll
                         for (int i = 0; i < TH; i += 2) fma_pair(v[i], v[i + 1], d[q], r0[i], r0[i + 1]);
 #pragma unroll
@@ -602,7 +583,7 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
                         // the accumulator is in registers: the next part's products may overwrite it
                         tc_fence_before();
                         __syncwarp();
-                        if (lane == 0) st_arrive_cluster(leader_acc_empty0 + 8u * acc);
+                        if (lane == 0) mbar_arrive_cluster(leader_acc_empty0 + 8u * acc);
                     }
                     if (whole) {
                         float v[32];
@@ -621,11 +602,10 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
     }
 
     __syncwarp();
-    if (warp == 0 || warp == 2) st_cluster_wait();
+    if (warp == 0 || warp == 2) cluster_wait();
     tc_fence_before();
     __syncthreads();
-    st_cluster_arrive();
-    st_cluster_wait();                       // nothing of the pair still refers to this block
+    cluster_sync_end(*ctl.abort != 0u);      // nothing of the pair still refers to this block
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");

@@ -69,29 +69,6 @@ template <int BN> struct PairCfg {
 };
 
 // ---------------------------------------------------------------- cluster-scope PTX wrappers
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-    uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r;
-}
-__device__ __forceinline__ uint32_t cluster_id_x() {
-    uint32_t r; asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r)); return r;
-}
-__device__ __forceinline__ uint32_t num_clusters_x() {
-    uint32_t r; asm volatile("mov.u32 %0, %%nclusterid.x;" : "=r"(r)); return r;
-}
-// address of the same shared-memory location in block `rank` of the cluster
-__device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
-    uint32_t r; asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank)); return r;
-}
-// Arrival on a barrier of another block of the cluster.  What is handed over lives in tensor
-// memory or was written by the copy engine, and tcgen05.fence::before_thread_sync orders it, so
-// the default release at block scope is enough; a cluster-scope release costs about a thousand
-// cycles per arrival here.
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-// (what is handed over in front of it is the barriers' initialisation, which has a fence of its own)
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // x tile copy whose bytes are counted on a barrier of the pair's leader
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1,
                                                  uint32_t leader_bar) {
@@ -99,15 +76,6 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes "
         "[%0], [%1, {%2, %3}], [%4];"
         ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(leader_bar) : "memory");
-}
-// D (both blocks' tensor memory) += A (tensor memory, 128 lanes per block) * B (both blocks' smem)
-__device__ __forceinline__ void umma_pair_f16_a_tmem(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
-                                                     uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
 // arrives on ONE barrier (a shared::cluster address) when the pair's MMAs issued so far are done
 __device__ __forceinline__ void umma_pair_commit(uint32_t cluster_bar) {
@@ -221,7 +189,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
         }
         __syncwarp();
         asm volatile("bar.arrive 1, %0;" ::"r"(Cfg::kThreads) : "memory");
-        cluster_arrive();
+        cluster_arrive_start();
     } else {
         if (warp == 1) {
             asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -230,7 +198,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
             tc_fence_before();
         }
         named_barrier_sync(1, Cfg::kThreads);
-        cluster_arrive();
+        cluster_arrive_start();
         cluster_wait();                      // both blocks' barriers exist before anyone arrives remotely
         tc_fence_after();
     }
@@ -338,6 +306,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
                 __syncwarp();
                 if (++acc == NACC) { acc = 0; acc_phase ^= 1u; }
             }
+            // the epilogues' last arrivals, the other block's among them, are waited for here (see cluster_sync_end)
+            for (uint32_t b = 0; b < NACC && mbar_wait_warp(acc_empty(acc), acc_phase ^ 1u, ctl); ++b)
+                if (++acc == NACC) { acc = 0; acc_phase ^= 1u; }
         }
     } else if (warp >= 8 && warp < Cfg::kEpilogueWarp1) {
         // -------------------------------------------------------------- dequantizers
@@ -541,8 +512,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
     if (warp == 0) cluster_wait();
     tc_fence_before();
     __syncthreads();
-    cluster_arrive();
-    cluster_wait();                          // nothing of the pair still refers to this block
+    cluster_sync_end(*ctl.abort != 0u);      // nothing of the pair still refers to this block
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;"

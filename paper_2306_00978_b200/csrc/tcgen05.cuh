@@ -70,6 +70,50 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
+// ------------------------------------------------------------------ pairs of blocks (clusters of two)
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+    uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r;
+}
+__device__ __forceinline__ uint32_t cluster_id_x() {
+    uint32_t r; asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r)); return r;
+}
+__device__ __forceinline__ uint32_t num_clusters_x() {
+    uint32_t r; asm volatile("mov.u32 %0, %%nclusterid.x;" : "=r"(r)); return r;
+}
+// address of the same shared-memory location in block `rank` of the cluster
+__device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
+    uint32_t r; asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank)); return r;
+}
+// Arrival on a barrier of another block of the cluster.  What is handed over lives in tensor memory or was written by the copy
+// engine, and tcgen05.fence::before_thread_sync orders it; or (x in the stream kernel) it lies in the arriving block's own shared
+// memory, fenced to the asynchronous proxy, and only that block's half of the products reads it.  So the default release at
+// block scope is used; a cluster-scope release costs about a thousand cycles per arrival here.
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+// Between the blocks of a cluster.  At the start of a kernel nothing is handed over but the barriers' initialisation, which has a
+// fence of its own, so the arrival may be relaxed.
+__device__ __forceinline__ void cluster_arrive_start() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// In front of a block's end, which gives its shared memory away: no arrival of the other block may still be on the way there.
+// Either every remote arrival has been waited for by then (the warp that issues the products waits for the last ones too), or the
+// block is giving up and the barrier releases what is under way.  (Releasing always made the launches 0.4 us longer: the
+// epilogue's stores to global memory are under way as well.)
+__device__ __forceinline__ void cluster_sync_end(bool gave_up) {
+    if (gave_up) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    else asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    cluster_wait();
+}
+// D (both blocks' tensor memory) += A (tensor memory, 128 lanes per block) * B (both blocks' smem)
+__device__ __forceinline__ void umma_pair_f16_a_tmem(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
+                                                     uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of 128 bytes,
 // 8-row atoms 1024 bytes apart.
 __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
