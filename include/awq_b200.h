@@ -310,10 +310,11 @@ int awq_static_scratch_fill(int value, void* stream);
  * the paper does not name its norm: the mean squared difference has the same minimizer as any other
  * monotone function of the Frobenius norm).  The quantizer and the layer are the library's own
  * kernels, so the search scores exactly what deployment runs; the fp16 reference product W X is a
- * dense GEMM kernel of this library with fp32 accumulation and output.  Grid points are evaluated several at a
- * time, as many as 384 MB of x / s, packed arrays and y hold (above 64 tokens their products are one launch of the
- * SM-pair kernel).  Nothing is allocated: all intermediate arrays live in `scratch`.  The paper uses 20 grid points over [0, 1]; the grid is the
- * caller's.
+ * dense GEMM kernel of this library with fp32 accumulation and output.  Nothing is allocated: all intermediate
+ * arrays live in `scratch`.  Grid points are evaluated together, as many as it holds (384 MB at most; above 64 tokens
+ * their products are one launch of the SM-pair kernel): awq_search_scratch_bytes is what one grid point at a time
+ * needs, awq_search_scratch_bytes_points what `points` of them can use.  The paper uses 20 grid points over [0, 1]; the
+ * grid is the caller's.
  * W: in, fp16 [N][K] (device).  act_mean_abs: in, fp32 [K] (device).  X: in, fp16 [M][K] calibration
  * activations (device), M >= 1.  alphas: in, HOST array of n_alphas <= 64 values in [0, 1].
  * losses: out, HOST array of n_alphas floats.  best_index: out, HOST, index of the first least loss
@@ -325,6 +326,7 @@ int awq_static_scratch_fill(int value, void* stream);
  * scratch that is too small.
  */
 size_t awq_search_scratch_bytes(int M, int N, int K, int group);
+size_t awq_search_scratch_bytes_points(int M, int N, int K, int group, int points);
 int awq_search_alpha(const void* W, const float* act_mean_abs, const void* X, int M, int N, int K, int group,
                      const float* alphas, int n_alphas, float* losses, int* best_index,
                      void* scratch, size_t scratch_bytes, void* stream);

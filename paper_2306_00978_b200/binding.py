@@ -17,12 +17,14 @@ LIB_PATH = os.path.join(_HERE, "libawq_b200.so")
 
 PATH_AUTO, PATH_GEMV, PATH_GEMM, PATH_GEMV_SPLITK, PATH_GEMM_1SM, PATH_GEMV_MID, PATH_GEMM_SKINNY = 0, 1, 2, 3, 4, 5, 6
 
+MAX_SEARCH_ALPHAS = 64
+
 EXPORTS = (
     "awq_qweight_bytes", "awq_scales_bytes", "awq_zeros_bytes", "awq_quantize_pack",
     "awq_channel_scale", "awq_linear", "awq_linear_path", "awq_workspace_bytes",
     "awq_set_workspace", "awq_unpack_canonical", "awq_poll_status", "awq_status_string",
     "awq_last_cuda_error", "awq_layout_version", "awq_launch_count", "awq_linear_gemv_static",
-    "awq_linear_multi", "awq_search_scratch_bytes", "awq_search_alpha",
+    "awq_linear_multi", "awq_search_scratch_bytes", "awq_search_scratch_bytes_points", "awq_search_alpha",
     "awq_quantize_pack_ex", "awq_search_clip", "awq_static_scratch_fill",
     "awq_set_wait_limit_us", "awq_test_stall_next_gemv",
     "awq_linear_scaled", "awq_linear_multi_scaled", "awq_linear_scaled_needs_scratch",
@@ -76,6 +78,7 @@ def lib() -> ctypes.CDLL:
     L.awq_linear_scaled_needs_scratch.restype, L.awq_linear_scaled_needs_scratch.argtypes = i, [i, i, i, i]
     L.awq_linear_multi.restype, L.awq_linear_multi.argtypes = i, [vp, vp, i, i, i, i, vp]
     L.awq_search_scratch_bytes.restype, L.awq_search_scratch_bytes.argtypes = sz, [i, i, i, i]
+    L.awq_search_scratch_bytes_points.restype, L.awq_search_scratch_bytes_points.argtypes = sz, [i, i, i, i, i]
     L.awq_search_alpha.restype, L.awq_search_alpha.argtypes = i, [vp, vp, vp, i, i, i, i, vp, i, vp, vp, vp, sz, vp]
     L.awq_workspace_bytes.restype, L.awq_workspace_bytes.argtypes = sz, [i, i, i, i]
     L.awq_set_workspace.restype, L.awq_set_workspace.argtypes = i, [vp, sz]
@@ -358,14 +361,24 @@ def search_alpha(W: torch.Tensor, act_mean_abs: torch.Tensor, X: torch.Tensor, g
     need = int(lib().awq_search_scratch_bytes(M, N, K, int(group)))
     if need == 0:
         raise AwqError(f"shape N={N}, K={K}, group={group} is not accepted")
-    scratch = torch.empty(need, dtype=torch.uint8, device=W.device)
     ensure_workspace(workspace_bytes(M, N, K, group))
+    # room for all grid points at once; where memory is short for fewer, down to one at a time
+    points = max(1, min(n, MAX_SEARCH_ALPHAS))
+    while True:
+        size = max(need, int(lib().awq_search_scratch_bytes_points(M, N, K, int(group), points)))
+        try:
+            scratch = torch.empty(size, dtype=torch.uint8, device=W.device)
+            break
+        except torch.OutOfMemoryError:
+            if points == 1:
+                raise
+            points //= 2
     a = (ctypes.c_float * n)(*[float(v) for v in alphas])
     losses = (ctypes.c_float * n)()
     best = ctypes.c_int(0)
     rc = lib().awq_search_alpha(_dev(W, torch.float16, "W"), _dev(act_mean_abs, torch.float32, "act_mean_abs"),
                                 _dev(X, torch.float16, "X"), M, N, K, int(group), a, n, losses,
-                                ctypes.byref(best), scratch.data_ptr(), need, _stream())
+                                ctypes.byref(best), scratch.data_ptr(), size, _stream())
     _check(rc, "awq_search_alpha")
     return [float(v) for v in losses], int(best.value)
 

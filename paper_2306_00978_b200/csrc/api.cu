@@ -679,7 +679,12 @@ int awq_inverse_channel_scale(const float* act_mean_abs, float alpha, float* inv
 
 size_t awq_search_scratch_bytes(int M, int N, int K, int group) {
     if (check_shape(N, K, group) != AWQ_OK || M < 1 || group > 128) return 0;
-    return search_plan(nullptr, M, N, K, group).total;
+    return search_plan(nullptr, 0, M, N, K, group, 1).total;
+}
+
+size_t awq_search_scratch_bytes_points(int M, int N, int K, int group, int points) {
+    if (check_shape(N, K, group) != AWQ_OK || M < 1 || group > 128 || points < 1 || points > kMaxSearchAlphas) return 0;
+    return search_plan(nullptr, SIZE_MAX, M, N, K, group, points).total;
 }
 
 int awq_search_alpha(const void* W, const float* act_mean_abs, const void* X, int M, int N, int K, int group,
@@ -692,7 +697,7 @@ int awq_search_alpha(const void* W, const float* act_mean_abs, const void* X, in
     if (n_alphas < 1 || n_alphas > kMaxSearchAlphas) return AWQ_ERR_BAD_ARGUMENT;
     for (int i = 0; i < n_alphas; ++i)
         if (!(alphas[i] >= 0.0f && alphas[i] <= 1.0f)) return AWQ_ERR_BAD_ARGUMENT;
-    const SearchPlan p = search_plan(scratch, M, N, K, group);
+    const SearchPlan p = search_plan(scratch, scratch_bytes, M, N, K, group, n_alphas);
     if (scratch_bytes < p.total) return AWQ_ERR_BAD_ARGUMENT;
     if (!aligned16(W) || !aligned16(X) || (reinterpret_cast<uintptr_t>(scratch) & 255u) != 0) return AWQ_ERR_MISALIGNED;
     if (reinterpret_cast<uintptr_t>(act_mean_abs) & 3u) return AWQ_ERR_MISALIGNED;
@@ -707,17 +712,16 @@ int awq_search_alpha(const void* W, const float* act_mean_abs, const void* X, in
         ws_bytes = d->workspace_bytes;
     }
     if (int rc = note_cuda(launch_reference_product(W, X, p.yref, M, N, K, d->status_word, st))) return rc;
-    if (int rc = note_cuda(launch_channel_scales(act_mean_abs, alphas, n_alphas, p.s, K, st))) return rc;
     const int batches = (n_alphas + p.batch - 1) / p.batch, most = (n_alphas + batches - 1) / batches;
     for (int i0 = 0; i0 < n_alphas; i0 += most) {
         const int b = n_alphas - i0 < most ? n_alphas - i0 : most;
-        const float* s = p.s + (size_t)i0 * K;
-        if (int rc = note_cuda(launch_quantize_pack_many(reinterpret_cast<const __half*>(W), s, b, group,
+        if (int rc = note_cuda(launch_channel_scales(act_mean_abs, alphas + i0, b, p.s, K, st))) return rc;
+        if (int rc = note_cuda(launch_quantize_pack_many(reinterpret_cast<const __half*>(W), p.s, b, group,
                                                          reinterpret_cast<uint32_t*>(p.qweight), reinterpret_cast<__half*>(p.scales),
                                                          p.zeros, N, K, st)))
             return rc;
         // (the plainly ordered division stands between this writer and its readers)
-        if (int rc = note_cuda(launch_divide_by_scale(X, s, b, p.xs, M, p.rows, K, st))) return rc;
+        if (int rc = note_cuda(launch_divide_by_scale(X, p.s, b, p.xs, M, p.rows, K, st))) return rc;
         // all products at once where the layer's kernel rounds (q - z) * Delta to fp16 too (above 64 tokens)
         bool launched = false;
         if (M > 64)
@@ -729,11 +733,10 @@ int awq_search_alpha(const void* W, const float* act_mean_abs, const void* X, in
             if (int rc = awq_linear(p.xs + (size_t)i * p.rows * K, p.qweight + (size_t)i * N * K / 2, p.scales + i * groups * N * 2,
                                     p.zeros + i * groups * N / 2, p.yq + (size_t)i * p.rows * N, M, N, K, group, stream))
                 return rc;
-        if (int rc = note_cuda(launch_squared_difference(p.yq, p.yref, b, M, p.rows, N, search_partials(p, i0), st))) return rc;
+        if (int rc = note_cuda(launch_squared_difference(p.yq, p.yref, b, M, p.rows, N, p.partials, st))) return rc;
+        if (int rc = note_cuda(launch_losses(p.partials, b, (size_t)M * N, p.losses + i0, st))) return rc;
     }
-    float* dev_losses = p.losses;
-    if (int rc = note_cuda(launch_losses(p.partials, n_alphas, (size_t)M * N, dev_losses, st))) return rc;
-    if (int rc = note_cuda(cudaMemcpyAsync(losses, dev_losses, (size_t)n_alphas * sizeof(float),
+    if (int rc = note_cuda(cudaMemcpyAsync(losses, p.losses, (size_t)n_alphas * sizeof(float),
                                            cudaMemcpyDeviceToHost, st)))
         return rc;
     if (int rc = note_cuda(cudaStreamSynchronize(st))) return rc;

@@ -152,7 +152,7 @@ cudaError_t launch_gemm_stream(const void* x, const GemvMatrix* mats, int count,
 // Scratch of a search: `batch` grid points at a time, each with `rows` >= M rows of x / s and y and packed arrays of its own.
 struct SearchPlan {
     int batch, rows;
-    float* s;                                // [kMaxSearchAlphas][K]
+    float* s;                                // [batch][K]
     __half* xs;
     unsigned char* qweight;
     unsigned char* scales;
@@ -163,7 +163,7 @@ struct SearchPlan {
     float* losses;
     size_t total;
 };
-SearchPlan search_plan(void* scratch, int M, int N, int K, int group);
+SearchPlan search_plan(void* scratch, size_t scratch_bytes, int M, int N, int K, int group, int points);
 cudaError_t launch_reference_product(const void* W, const void* X, float* yref, int M, int N, int K,
                                      unsigned int* status_word, cudaStream_t st);
 // xs[i] = fp16_rne(fp32(X) / s[i]) for `count` scale arrays, `rows` rows apart
@@ -171,11 +171,10 @@ cudaError_t launch_divide_by_scale(const void* X, const float* s, int count, voi
 // xs = fp16_rne(fp32(X) * inv_s); inverse_scale: inv_s = fp32(1 / s), correctly rounded
 cudaError_t launch_multiply_by_inverse(const void* X, const float* inv_s, void* xs, int M, int K, cudaStream_t st);
 cudaError_t launch_inverse_scale(const float* s, float* inv_s, int K, cudaStream_t st);
-// partial sums of (yq[i] - yref)^2 for `count` arrays (search_partials(plan, first) is where the first one's go), then the means
+// partial sums of (yq[i] - yref)^2 for `count` arrays, then the means
 cudaError_t launch_squared_difference(const void* yq, const float* yref, int count, int M, int rows, int N, double* partials,
                                       cudaStream_t st);
 cudaError_t launch_losses(const double* partials, int count, size_t n, float* losses, cudaStream_t st);
-double* search_partials(const SearchPlan& p, int first);
 // s[i] of n alphas (a HOST array); W quantized with each of `count` scale arrays, packed arrays end to end
 cudaError_t launch_channel_scales(const float* a, const float* alphas, int n, float* s, int K, cudaStream_t st);
 cudaError_t launch_quantize_pack_many(const __half* W, const float* s, int count, int group, uint32_t* qweight, __half* scales,

@@ -508,14 +508,14 @@ cudaError_t launch_gemm(const void* x, const void* qweight, const void* scales, 
 #undef AWQ_GEMM_CASE
 }
 
-// `count` products with x [rows] x K, N channels and y [rows] x N each (M of the rows are used; rows a multiple of 32, N of
-// 256), all arrays end to end, in one launch of the SM-pair kernel.  *launched is false where it cannot run.
+// `count` products with x [rows] x K, N channels and y [rows] x N each (M of the rows are used; rows a multiple of 32 where
+// there are several products, N of 256), all arrays end to end, in one launch of the SM-pair kernel.  *launched is false where it cannot run.
 cudaError_t launch_gemm_blocks(const void* x, const void* qweight, const void* scales, const void* zeros, void* y, int count,
                                int M, int rows, int N, int K, int group, void* workspace, size_t workspace_bytes,
                                unsigned int* status_word, int sms, cudaStream_t st, bool* launched) {
     EncodeTiledFn enc = encode_fn();
     *launched = false;
-    if (!enc || N % 256 != 0 || rows % 32 != 0) return cudaSuccess;
+    if (!enc || N % 256 != 0 || (count > 1 && rows % 32 != 0)) return cudaSuccess;
     const cuuint32_t estr[2] = {1, 1};
     CUtensorMap wmap, ymap;
     const cuuint64_t wdims[2] = {(cuuint64_t)K * 2, (cuuint64_t)count * (N / 16)}, wstrides[1] = {(cuuint64_t)K * 8};

@@ -104,27 +104,23 @@ sqdiff_final_kernel(const double* __restrict__ partials, int blocks, double inv_
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// Grid points evaluated together: as many as 384 MB of scratch hold (twenty of 4096 -> 4096 with 512 tokens), at most kMaxSearchAlphas.
-int search_rows(int M) { return (M + 31) / 32 * 32; }
-size_t search_point_bytes(int M, int N, int K, int group) {
-    return (size_t)search_rows(M) * K * 2 + (size_t)N * K / 2 + (size_t)(K / group) * N * 5 / 2 + (size_t)search_rows(M) * N * 2;
-}
-SearchPlan carve(void* base, int M, int N, int K, int group) {
+// Scratch of `batch` grid points at a time.  One needs no more than its own arrays, in rows as they come; several are stacked, each
+// product's rows padded to what one store of the SM-pair kernel covers.
+SearchPlan carve(void* base, int M, int N, int K, int group, int batch) {
     SearchPlan r;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t o = off; off += align256(bytes); return static_cast<unsigned char*>(base) + o; };
-    const size_t fit = ((size_t)384 << 20) / search_point_bytes(M, N, K, group);
-    r.batch = fit < 1 ? 1 : fit > (size_t)kMaxSearchAlphas ? kMaxSearchAlphas : (int)fit;
-    r.rows = search_rows(M);
+    r.batch = batch;
+    r.rows = batch > 1 ? (M + 31) / 32 * 32 : M;
     const size_t b = (size_t)r.batch;
-    r.s = reinterpret_cast<float*>(take((size_t)kMaxSearchAlphas * K * 4));
+    r.s = reinterpret_cast<float*>(take(b * K * 4));
     r.xs = reinterpret_cast<__half*>(take(b * r.rows * K * 2));
     r.qweight = take(b * N * K / 2);
     r.scales = take(b * (K / group) * N * 2);
     r.zeros = take(b * (K / group) * N / 2);
     r.yq = reinterpret_cast<__half*>(take(b * r.rows * N * 2));
     r.yref = reinterpret_cast<float*>(take((size_t)M * N * 4));
-    r.partials = reinterpret_cast<double*>(take((size_t)kMaxSearchAlphas * kLossBlocks * 8));
+    r.partials = reinterpret_cast<double*>(take(b * kLossBlocks * 8));
     r.losses = reinterpret_cast<float*>(take((size_t)kMaxSearchAlphas * 4));
     r.total = off;
     return r;
@@ -238,7 +234,15 @@ reference_product_kernel(const __grid_constant__ CUtensorMap w_map, const __grid
 
 }  // namespace
 
-SearchPlan search_plan(void* scratch, int M, int N, int K, int group) { return carve(scratch, M, N, K, group); }
+// Grid points evaluated together: those asked for, as many as 384 MB hold beside the reference product (twenty of 4096 -> 4096 with
+// 512 tokens), and as many as the scratch at hand holds; at least one.
+SearchPlan search_plan(void* scratch, size_t scratch_bytes, int M, int N, int K, int group, int points) {
+    const size_t most = ((size_t)384 << 20) + (size_t)M * N * 4;
+    int batch = 1;
+    while (batch < points && carve(nullptr, M, N, K, group, batch + 1).total <= most) ++batch;
+    while (batch > 1 && carve(nullptr, M, N, K, group, batch).total > scratch_bytes) --batch;
+    return carve(scratch, M, N, K, group, batch);
+}
 
 // y_ref[m][n] = sum_k X[m][k] W[n][k], fp32 [M][N] row-major.
 cudaError_t launch_reference_product(const void* W, const void* X, float* yref, int M, int N, int K, unsigned int* status_word,
@@ -298,6 +302,4 @@ cudaError_t launch_losses(const double* partials, int count, size_t n, float* lo
     count_launch();
     return cudaGetLastError();
 }
-double* search_partials(const SearchPlan& p, int first) { return p.partials + (size_t)first * kLossBlocks; }
-
 }  // namespace awq
