@@ -77,11 +77,10 @@ typedef enum AwqPath {
                                    prefill kernels (M <= 8: the band or split-K kernel) */
     AWQ_PATH_GEMV = 1,          /* fused dequant matrix-vector kernel, M <= 16: band kernel when
                                    M <= 8 and N/16 is not much below the SM count, else split-K */
-    AWQ_PATH_GEMM = 2,          /* tcgen05 tensor-core kernels, any M >= 1: at 65 .. 256 tokens on few
-                                   tiles or long rows the stream kernel (with a workspace), else
-                                   pairs of SMs (cta_group::2, 256 channels x 64 .. 256 tokens per
-                                   tile) when M > 64 (M >= 32 from N = 16384; up to 128 tokens not on
-                                   few channels with long rows), else one SM per tile */
+    AWQ_PATH_GEMM = 2,          /* tcgen05 prefill kernels, any M >= 1: pairs of SMs
+                                   (cta_group::2, 256 channels x 64 .. 256 tokens per tile) when
+                                   M > 64 (M >= 32 from N = 16384; up to 128 tokens not on few
+                                   channels with long rows), else one SM per tile */
     AWQ_PATH_GEMV_SPLITK = 3,   /* the split-K matrix-vector kernel, M <= 16 */
     AWQ_PATH_GEMM_1SM = 4,      /* the tensor-core kernel with one SM per tile, any M >= 1 */
     AWQ_PATH_GEMV_MID = 5,      /* M <= 8: the chunked matrix-vector kernel: work units of 16 bands

@@ -387,7 +387,7 @@ static int linear_path(const void* x, const void* qweight, const void* scales, c
         std::lock_guard<std::mutex> lock(g_mutex);
         if (d->workspace_bytes >= gemv_mid_workspace_bytes(M, N, K)) path = AWQ_PATH_GEMV_MID;
     }
-    if (path == AWQ_PATH_GEMM) {
+    if (automatic && path == AWQ_PATH_GEMM) {          // (asked for by name it is the prefill kernels)
         const AwqLinearProblem one = {qweight, scales, zeros, y, N};
         if (stream_beats_prefill(d, &one, 1, M, K, group)) path = AWQ_PATH_GEMM_SKINNY;
     }

@@ -28,8 +28,12 @@ def test_linear(N, K, M, G):
     case = Case(6200 + N + K + M + G, N, K, M, G, 0.5)
     packed = oracle_packed_to_cuda(case)
     y = binding.linear(to_cuda(case.x), *packed, N, K, G)
+    n0 = binding.launch_count()
     again = binding.linear(to_cuda(case.x), *packed, N, K, G)
+    launches = binding.launch_count() - n0
     binding.poll_status()
+    if M > 64:
+        assert launches == 2                  # the prefill kernels are one launch
     y = y.cpu().numpy()
     assert np.array_equal(y.view(np.uint16), again.cpu().numpy().view(np.uint16))
     if M <= 32:
@@ -56,6 +60,25 @@ def test_several_matrices_and_the_folded_scale(widths, K, M, G):
     for c, y, ys in zip(cases, plain, scaled):
         assert_parity(y.cpu().numpy(), orc.linear(x, orc.dequantize(c.codes, c.zeros, c.scales, G)), f"N={c.N} of {widths}")
         assert np.array_equal(y.cpu().numpy().view(np.uint16), ys.cpu().numpy().view(np.uint16))
+
+
+@pytest.mark.parametrize("N,K,M,G", [(4096, 4096, 100, 128), (1152, 8192, 130, 64), (640, 8192, 256, 128)])
+def test_prefill_kernels_by_name_where_the_automatic_path_is_this_one(N, K, M, G):
+    """AWQ_PATH_GEMM is the prefill kernels whatever awq_linear takes, and a name for this kernel ends at 64 tokens."""
+    from paper_2306_00978_b200 import binding
+    case = Case(6950 + N + K + M + G, N, K, M, G, 0.5)
+    x, packed = to_cuda(case.x), oracle_packed_to_cuda(case)
+    got = []
+    for path in (binding.PATH_AUTO, binding.PATH_GEMM):
+        binding.linear(x, *packed, N, K, G, path=path)
+        n0 = binding.launch_count()
+        y = binding.linear(x, *packed, N, K, G, path=path)
+        got.append(binding.launch_count() - n0)
+        assert_parity(y.cpu().numpy(), case.y_ref(), f"path {path}, N={N} K={K} M={M} G={G}")
+    binding.poll_status()
+    assert got == [2, 1]
+    with pytest.raises(binding.AwqError):
+        binding.linear(x, *packed, N, K, G, path=binding.PATH_GEMM_SKINNY)
 
 
 def test_one_matrix_scaled_above_64_tokens_is_the_plain_call():
