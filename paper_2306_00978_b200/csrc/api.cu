@@ -378,6 +378,7 @@ static int linear_path(const void* x, const void* qweight, const void* scales, c
     }
     DeviceState* d;
     if (int rc = device_state(&d)) return rc;
+    const int without_stream = path;
     if (automatic && stream_kernel_preferred(M, N, K, group, d->sms)) {
         const size_t need = gemm_stream_workspace_bytes(M, d->sms);
         std::lock_guard<std::mutex> lock(g_mutex);
@@ -414,8 +415,10 @@ static int linear_path(const void* x, const void* qweight, const void* scales, c
             ws = d->workspace;
         }
         const GemvMatrix one = {qweight, scales, zeros, y, N};
-        return note_cuda(order.launched(launch_gemm_stream(x, &one, 1, M, K, group, nullptr, ws, d->status_word,
-                                                           d->sms, order.serialize, st)));
+        const cudaError_t e = order.launched(launch_gemm_stream(x, &one, 1, M, K, group, nullptr, ws, d->status_word,
+                                                                d->sms, order.serialize, st));
+        if (!automatic || e != cudaErrorNotSupported) return note_cuda(e);
+        path = without_stream;               // no pair of SMs to be had (a partition of the device): nothing was launched
     }
     if (path == AWQ_PATH_GEMV && gemv_uses_band_kernel(M, N, d->sms)) {
         const GemvMatrix one = {qweight, scales, zeros, y, N};
@@ -497,7 +500,7 @@ int awq_static_scratch_fill(int value, void* stream) {
     return note_cuda(cudaMemsetAsync(scratch, value & 0xFF, kCounterBytes, (cudaStream_t)stream));
 }
 
-// All matrices in one launch of the stream kernel, if the workspace holds their partial sums.
+// All matrices in one launch of the stream kernel, if the workspace holds their partial sums and the kernel can run.
 static int linear_multi_stream(DeviceState* d, const void* x, const float* inv_s, const AwqLinearProblem* problems,
                                int count, int M, int K, int group, void* stream, bool* launched) {
     const size_t need = gemm_stream_workspace_bytes(M, d->sms);
@@ -510,10 +513,12 @@ static int linear_multi_stream(DeviceState* d, const void* x, const float* inv_s
     GemvMatrix mats[kMaxMulti];
     for (int i = 0; i < count; ++i)
         mats[i] = GemvMatrix{problems[i].qweight, problems[i].scales, problems[i].zeros, problems[i].y, problems[i].N};
-    *launched = true;
     const LaunchOrder order = launch_order(d, stream);
-    return note_cuda(order.launched(launch_gemm_stream(x, mats, count, M, K, group, inv_s, ws, d->status_word, d->sms,
-                                                       order.serialize, (cudaStream_t)stream)));
+    const cudaError_t e = order.launched(launch_gemm_stream(x, mats, count, M, K, group, inv_s, ws, d->status_word, d->sms,
+                                                            order.serialize, (cudaStream_t)stream));
+    if (e == cudaErrorNotSupported) return AWQ_OK;           // as in linear_path
+    *launched = true;
+    return note_cuda(e);
 }
 
 int awq_linear_multi(const void* x, const AwqLinearProblem* problems, int count,

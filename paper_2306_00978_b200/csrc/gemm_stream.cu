@@ -673,7 +673,7 @@ int st_tile_tokens(int M) {                              // tokens per tile: a m
     return ((M + tiles - 1) / tiles + 15) / 16 * 16;
 }
 
-// pairs that can be resident at once on the current device (0 if the query fails); cached
+// pairs that can be resident at once on the current device (0 if the query fails); cached once there is one
 template <int G, int BN, bool XS>
 cudaError_t st_resident_pairs(int sms, int* out) {
     static std::mutex mutex;
@@ -703,7 +703,7 @@ cudaError_t st_resident_pairs(int sms, int* out) {
             n = 0;
         }
         pairs[dev] = n < sms / 2 ? n : sms / 2;          // (what the workspace is sized for)
-        done[dev] = true;
+        done[dev] = n > 0;
     }
     *out = pairs[dev];
     return cudaSuccess;
@@ -715,7 +715,7 @@ cudaError_t st_launch(const CUtensorMap& xmap, const StMats& mats, const float* 
     int resident = 0;
     cudaError_t e = st_resident_pairs<G, BN, XS>(sms, &resident);
     if (e != cudaSuccess) return e;
-    if (resident < 1) return cudaErrorNotSupported;
+    if (resident < 1) return cudaErrorNotSupported;          // the caller's cue to take another kernel
     cut.pairs = cut.total < resident ? cut.total : resident;
     cut.share = cut.total / cut.pairs;
     cut.longer = cut.total % cut.pairs;

@@ -524,7 +524,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constan
 // stream-K's part of the workspace: a flag per pair in its head, one fp32 tile per pair behind that
 size_t streamk_bytes(int bn, int pairs) { return kCounterBytes + (size_t)pairs * 256 * bn * sizeof(float); }
 
-// pairs that can be resident at once on the current device (0 if the query fails); cached
+// pairs that can be resident at once on the current device (0 if the query fails); cached once there is one
 template <int G, int BN>
 int resident_pairs(int sms, cudaError_t* err) {
     static bool done[64] = {};
@@ -551,7 +551,7 @@ int resident_pairs(int sms, cudaError_t* err) {
             n = 0;
         }
         pairs[dev & 63] = n;
-        done[dev & 63] = true;
+        done[dev & 63] = n > 0;
     }
     return pairs[dev & 63];
 }
