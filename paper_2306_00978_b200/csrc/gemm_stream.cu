@@ -719,8 +719,8 @@ cudaError_t st_launch(const CUtensorMap& xmap, const StMats& mats, const float* 
     cut.pairs = cut.total < resident ? cut.total : resident;
     cut.share = cut.total / cut.pairs;
     cut.longer = cut.total % cut.pairs;
-    // no tile is cut where every range starts at a tile
-    const bool second = cut.longer != 0 || cut.share % cut.nks != 0;
+    // no tile is cut where every range starts at a tile, as all do where a tile is one stage
+    const bool second = cut.nks > 1 && (cut.longer != 0 || cut.share % cut.nks != 0);
     float* partial = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + kCounterBytes);
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
