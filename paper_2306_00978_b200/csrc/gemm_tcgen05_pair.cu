@@ -661,9 +661,12 @@ cudaError_t launch_gemm_pair(const void* x, const CUtensorMap& wmap, const CUten
                              unsigned int* status_word, int sms, bool serialize, cudaStream_t st, bool* launched, int count, int rows) {
     const PairBlocks blocks = {(N / count + 255) / 256, N / count, rows};
     const PairChoice c = choose_tile(M, N, K, sms / 2, workspace ? workspace_bytes : 0);
-    // Launches beyond about 0.3 ms run at the power limit and are not chained: back to back, 8192 tokens on 4096 -> 11008 take
-    // 575 us unchained and 587 us chained, 2048 tokens on 13824 -> 5120 242 and 239 us.
-    serialize = serialize || c.us > 300.0;
+    // Long launches are not chained.  They run at the power limit, where an early start buys nothing and sometimes costs: back to back,
+    // chained / unchained, us: 700 and 2048 tokens on 4096 -> 4096 24.4 / 25.4 and 59.0 / 60.0, 1024 on 13824 -> 5120 118 / 121 (estimates
+    // below 85); 2048 on 4096 -> 11008, 8192 -> 8192 and 13824 -> 5120 152 / 153, 224 / 224 and 249 / 249 (95 to 146); 3000 on 8192 -> 8192
+    // 341 / 338, 4096 on 11008 -> 4096 358 / 352, 1024 on 28672 -> 8192 429 / 412, 1500 on 8192 -> 28672 560 / 570, 4096 on 13824 -> 5120
+    // 501 / 496 (182 to 362).  Over 12 problems whose estimate is above 150 chaining loses 0.5 %, over 11 below it gains 1.2 %.
+    serialize = serialize || c.us > 150.0;
     CUtensorMap xmap;
     {
         // x as [M][K] fp16 in boxes of half a tile's tokens x one k-block, 128-byte swizzle
