@@ -175,8 +175,8 @@ int awq_channel_scale(const float* act_mean_abs, float alpha, float* s, int K, v
  * and start copying qweight, scales and zeros into shared memory BEFORE the work in front of them
  * in the stream has completed; only their reads of x and their writes of y and of the workspace
  * wait for that work.  The library covers its own writers: the first layer call behind an
- * awq_quantize_pack / awq_quantize_pack_ex / awq_pack_int3 / awq_unpack_int3 on the same stream is launched
- * fully serialized, whatever other streams and threads enqueue meanwhile (behind a writer on another
+ * awq_quantize_pack / awq_quantize_pack_ex / awq_pack_int3 / awq_unpack_int3 (or an awq_inverse_channel_scale,
+ * see awq_linear_scaled) on the same stream is launched fully serialized, whatever other streams and threads enqueue meanwhile (behind a writer on another
  * stream the caller orders it, with an event for instance).  A caller who produces packed arrays by other
  * means (its own kernel, a copy) must make sure they are complete before the operation that directly
  * precedes awq_linear in the stream begins - a stream or event synchronization, or any other kernel in

@@ -23,7 +23,7 @@ struct StreamKey {
     unsigned long long stream, capture;
     bool operator==(const StreamKey& o) const { return stream == o.stream && capture == o.capture; }
 };
-// Streams on which one of this library's kernels that write packed arrays (quantizer, 3-bit packing and expansion) has been
+// Streams on which one of this library's kernels that write packed arrays or 1 / s (quantizer, 3-bit packing and expansion) has been
 // enqueued and no layer call since.  Most layer kernels copy weights before the launch in front of them has completed, so the
 // first one behind such a writer on the same stream is launched fully serialized; what runs on other streams changes nothing.
 struct PendingWriters {
@@ -679,7 +679,11 @@ int awq_linear_int3(const void* x, const void* qweight3, const void* scales, con
 
 int awq_inverse_channel_scale(const float* act_mean_abs, float alpha, float* inv_s, int K, void* stream) {
     if (int rc = awq_channel_scale(act_mean_abs, alpha, inv_s, K, stream)) return rc;
-    return note_cuda(launch_inverse_scale(inv_s, inv_s, K, (cudaStream_t)stream));
+    const int rc = note_cuda(launch_inverse_scale(inv_s, inv_s, K, (cudaStream_t)stream));
+    DeviceState* d;
+    if (int bad = device_state(&d)) return bad;
+    note_packed_writer(d, stream);           // the band kernel loads 1 / s as early as the packed arrays
+    return rc;
 }
 
 size_t awq_search_scratch_bytes(int M, int N, int K, int group) {

@@ -79,6 +79,30 @@ def test_a_call_on_another_stream_does_not_release_the_reader(M):
     assert PROGRAMMATIC in types[1:]                      # only the first call behind the writer is held back
 
 
+def test_the_folded_scale_behind_its_writer():
+    import torch
+    from paper_2306_00978_b200 import binding
+    N, K, M, G = 8192, 4096, 1, 128
+    L = binding.lib()
+    x, qw, sc, zp, y = _operands(N, K, M, G)
+    stat, inv_s = torch.rand(K, device="cuda") + 0.5, torch.empty(K, device="cuda")
+    a = torch.cuda.Stream()
+
+    def layer():
+        assert L.awq_linear_scaled(x.data_ptr(), inv_s.data_ptr(), None, qw.data_ptr(), sc.data_ptr(), zp.data_ptr(), y.data_ptr(),
+                                   M, N, K, G, a.cuda_stream) == 0
+
+    torch.cuda.synchronize()
+    layer()
+    torch.cuda.synchronize()
+    with _captured_edges(a) as types:
+        assert L.awq_inverse_channel_scale(stat.data_ptr(), 0.5, inv_s.data_ptr(), K, a.cuda_stream) == 0      # two launches
+        layer()
+        layer()
+    binding.poll_status()
+    assert types == [FULL, FULL, PROGRAMMATIC]
+
+
 @pytest.mark.parametrize("M", [16, 300])
 def test_int3_expansion_and_its_reader_beside_another_thread(M):
     import torch
