@@ -166,10 +166,11 @@ int awq_channel_scale(const float* act_mean_abs, float alpha, float* s, int K, v
  * (q - z) * Delta once to fp16 and accumulates in fp32 in tensor memory.  Results are
  * bit-reproducible.
  * Workspace.  The split-K matrix-vector kernel (small N, M <= 16) needs the registered workspace;
- * the chunked matrix-vector and the stream kernel (partial sums per part of K, added in ascending order by
+ * the chunked matrix-vector and the stream kernel (partial sums per part of K, added in a fixed order by
  * a second small kernel) and the prefill kernels' split-K / stream-K use it when it holds awq_workspace_bytes,
  * else awq_linear falls back to a kernel that needs none.  Calls that use the workspace must not
- * overlap on the GPU (issue them on one stream).
+ * overlap on the GPU (issue them on one stream): with one registered that is any call for which awq_workspace_bytes
+ * is not 0 and that the band kernel does not serve, so calls of 9 tokens and more in particular.
  * Stream order.  x and y follow plain stream order.  The packed arrays are treated as constants
  * of the layer: the band, chunked, stream and SM-pair kernels are launched with programmatic stream serialization
  * and start copying qweight, scales and zeros into shared memory BEFORE the work in front of them
@@ -336,7 +337,8 @@ int awq_search_alpha(const void* W, const float* act_mean_abs, const void* X, in
  * decide which kernel awq_linear takes:
  *  - the chunked matrix-vector kernel (AWQ_PATH_GEMV_MID, up to 8 tokens) keeps one fp32 [M][N] array of partial
  *    sums per chunk of K there, the stream kernel (AWQ_PATH_GEMM_SKINNY, and up to 256 tokens) the
- *    parts of the tiles that two or more SM pairs share; a second small kernel adds them in ascending order.  Without a workspace of this size awq_linear takes the band
+ *    parts of the tiles that two or more SM pairs share; a second small kernel adds them, chunks in ascending order, parts
+ *    neighbour by neighbour, the same way in every call.  Without a workspace of this size awq_linear takes the band
  *    matrix-vector kernel (M <= 8) or the prefill kernels instead (same result within the
  *    tolerance, slower);
  *  - the one-SM prefill kernel (M <= 128) splits each tile's K loop over several SMs (up to 16

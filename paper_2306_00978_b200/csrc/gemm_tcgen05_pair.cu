@@ -640,7 +640,7 @@ PairChoice choose_tile(int M, int N, int K, int pairs, size_t workspace_bytes) {
 
 }  // namespace
 
-// Above 64 tokens always; below, on wide matrices when the chunked kernel does not serve the call.
+// Above 64 tokens always; below, on wide matrices when the stream kernel does not serve the call.
 bool gemm_pair_applies(int M, int N) { return M > 64 || (M >= 32 && N >= 16384); }
 
 // workspace with which the pair kernel balances its tiles over all SM pairs (stream-K)

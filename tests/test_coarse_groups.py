@@ -113,7 +113,7 @@ def test_quantize_pack_coarse_groups_bit_exact(N, K, G, alpha, bits, symmetric, 
     (768, 4096, 40, 512), (512, 1024, 100, 256), (512, 2048, 300, 1024),
 ])
 def test_layer_on_coarse_groups(N, K, M, G):
-    """The kernels that awq_linear takes at these sizes (band matrix-vector, chunked tensor-core, SM-pair
+    """The kernels that awq_linear takes at these sizes (band matrix-vector, stream, SM-pair
     prefill) and the split-K matrix-vector kernel on arrays quantized with a coarse group, quantized on the
     GPU and by the oracle."""
     import torch

@@ -43,9 +43,9 @@ def _check(buf, nbytes, what):
     (512, 1408, 9, 128, 3),       # split-K matrix-vector kernel
     (1024, 1408, 7, 128, 5),      # chunked matrix-vector kernel
     (640, 2304, 8, 64, 5),
-    (1024, 1408, 13, 128, 5),     # above 8 tokens the chunked tensor-core kernel
+    (1024, 1408, 13, 128, 5),     # above 8 tokens the stream kernel
     (768, 2304, 24, 64, 5),
-    (1024, 1408, 33, 128, 6),     # chunked tensor-core kernel
+    (1024, 1408, 33, 128, 6),     # stream kernel
     (256, 640, 17, 64, 6),
     (384, 640, 100, 64, 4),       # one-SM prefill kernel, ragged token tile
     (512, 1024, 300, 128, 2),     # SM-pair prefill kernel, ragged token tile
@@ -100,8 +100,8 @@ def test_quantizer_outputs_stay_inside_their_arrays(N, K, G, bits):
 
 
 def test_workspace_is_not_overrun():
-    """The kernels that use the workspace (split-K, chunked matrix-vector, chunked tensor-core, the
-    prefill kernels' split-K / stream-K) with a workspace of exactly awq_workspace_bytes."""
+    """The kernels that use the workspace (split-K, chunked matrix-vector, stream, the prefill kernels'
+    split-K / stream-K) with a workspace of exactly awq_workspace_bytes."""
     import torch
     from paper_2306_00978_b200 import binding
     L = binding.lib()
@@ -111,7 +111,7 @@ def test_workspace_is_not_overrun():
     try:
         for (N, K, M, G, path) in ((512, 1408, 9, 128, 3), (2432, 4096, 8, 128, 5), (2432, 4096, 13, 128, 5), (1024, 1408, 24, 128, 5),
                                    (4096, 4096, 32, 128, 6), (1024, 1408, 64, 64, 6), (384, 4096, 100, 128, 4),
-                                   (512, 4096, 300, 128, 2)):
+                                   (512, 4096, 300, 128, 2), (2048, 8192, 128, 128, 0), (640, 8192, 250, 64, 0)):
             case = Case(7900 + N + K + M, N, K, M, G, 0.5)
             qw, sc, zp = oracle_packed_to_cuda(case)
             x = to_cuda(case.x)

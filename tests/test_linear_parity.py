@@ -197,7 +197,7 @@ def test_quantize_then_linear_back_to_back_on_one_stream():
 
 
 def test_auto_dispatch_between_9_and_16_tokens():
-    """awq_linear with 9..16 tokens: the chunked tensor-core kernel when a workspace is registered
+    """awq_linear with 9..16 tokens: the stream kernel when a workspace is registered
     (the binding registers one), the prefill kernel otherwise.  Each result is bit-equal to its
     forced path (AWQ_PATH_GEMV_MID is that kernel too above 8 tokens)."""
     import torch
@@ -209,7 +209,7 @@ def test_auto_dispatch_between_9_and_16_tokens():
         x = to_cuda(case.x)
         auto = binding.linear(x, qw, sc, zp, case.N, case.K, case.group)
         assert torch.equal(auto, binding.linear(x, qw, sc, zp, case.N, case.K, case.group, path=binding.PATH_GEMV_MID))
-        assert_parity(auto.cpu().numpy(), case.y_ref(), f"auto M=12, chunked tensor-core kernel, K={K}")
+        assert_parity(auto.cpu().numpy(), case.y_ref(), f"auto M=12, stream kernel, K={K}")
     # a large matrix (random packed arrays: only the choice of kernel is checked here; parity at
     # this size is covered by the 70B sweep)
     N, K, G, M = 16384, 8192, 128, 12
@@ -289,55 +289,53 @@ def test_missing_workspace_is_reported():
 
 
 @pytest.mark.parametrize("N,K,M,G", [
-    (512, 1024, 9, 128),      # one chunk
-    (1024, 1408, 16, 128),    # 16-token tile, ragged last chunk
-    (768, 4096, 17, 64),      # 32-token tile, several chunks
-    (512, 2304, 32, 128),     # full 32-token tile, ragged last chunk
+    (512, 1024, 9, 128),      # two tiles of four stages, a stage per pair
+    (1024, 1408, 16, 128),    # full 16-token tile, a last stage of 128 channels
+    (768, 4096, 17, 64),      # 32-token tile, sixteen parts
+    (512, 2304, 32, 128),     # full 32-token tile
     (640, 2048, 24, 64),      # an odd number of slabs
-    (2432, 4096, 13, 128),    # more units than blocks
-    (128, 8192, 10, 128),     # one slab, many chunks
-    (4224, 1152, 9, 128),     # units crossing from one chunk to the next inside a block
+    (2432, 4096, 13, 128),    # ranges of two and three stages that cross from one tile to the next
+    (128, 8192, 10, 128),     # half a tile in 32 parts
+    (4224, 1152, 9, 128),     # 85 stages for 74 pairs
 ])
-def test_chunked_matrix_vector_kernel(N, K, M, G):
-    """AWQ_PATH_GEMV_MID above 8 tokens, where it runs the chunked tensor-core kernel (below:
+def test_stream_kernel_as_the_chunked_path_above_8_tokens(N, K, M, G):
+    """AWQ_PATH_GEMV_MID above 8 tokens, where it runs the stream kernel (below:
     test_chunked_matrix_vector_kernel_up_to_8_tokens).  Parity with the oracle and bit-reproducibility."""
     from paper_2306_00978_b200 import binding
     case = Case(600 + N + K + M + G, N, K, M, G, 0.5)
     y = _run(case, binding.PATH_GEMV_MID)
-    assert_parity(y, case.y_ref(), f"chunked N={N} K={K} M={M} G={G}")
+    assert_parity(y, case.y_ref(), f"path {binding.PATH_GEMV_MID} N={N} K={K} M={M} G={G}")
     y2 = _run(case, binding.PATH_GEMV_MID)
     assert np.array_equal(y.view(np.uint16), y2.view(np.uint16))
 
 
 @pytest.mark.parametrize("N,K,M,G,alpha", [
-    (128, 128, 17, 128, 0.5),     # one slab, one stage
+    (128, 128, 17, 128, 0.5),     # half a tile of half a stage
     (256, 256, 20, 128, 0.5),
-    (512, 1024, 17, 128, 0.0),    # 16-token tile does not fit: 32-token tile
-    (1024, 1408, 33, 128, 0.5),   # 64-token tile; 11 stages per unit: the warps' stage parity crosses units
-    (768, 4096, 64, 64, 1.0),     # full 64-token tile, group 64, four chunks
+    (512, 1024, 17, 128, 0.0),    # 32-token tile
+    (1024, 1408, 33, 128, 0.5),   # 48-token tile, a last stage of 128 channels
+    (768, 4096, 64, 64, 1.0),     # full 64-token tile, group 64, sixteen parts
     (1280, 2048, 9, 128, 0.5),    # 16-token tile
     (2048, 5120, 48, 64, 0.5),
-    (4096, 4096, 32, 128, 0.5),   # more units than blocks: ranges that cross from one chunk to the next
-    (19072, 384, 25, 128, 0.5),   # 149 slabs, one short chunk of 3 stages per unit
-    (128, 8192, 40, 128, 0.5),    # one slab, many chunks
+    (4096, 4096, 32, 128, 0.5),   # ranges of three and four stages that cross from one tile to the next
+    (19072, 384, 25, 128, 0.5),   # 75 tiles of two stages for 74 pairs, an odd slab
+    (128, 8192, 40, 128, 0.5),    # half a tile in 32 parts
     (256, 640, 1, 64, 0.5),       # a single token
 ])
-def test_chunked_tensor_core_kernel(N, K, M, G, alpha):
-    """AWQ_PATH_GEMM_SKINNY: units of 128 channels x a chunk of K on tcgen05, the chunk's slice of x
-    resident in shared memory; partial sums per chunk, added by a second kernel.  Parity with the
-    oracle and bit-reproducibility."""
+def test_stream_kernel_by_name(N, K, M, G, alpha):
+    """AWQ_PATH_GEMM_SKINNY: tiles of 256 channels on tcgen05, their K loops cut into one range per pair of SMs; the parts of
+    cut tiles, added by a second kernel.  Parity with the oracle and bit-reproducibility."""
     from paper_2306_00978_b200 import binding
     case = Case(900 + N + K + M + G, N, K, M, G, alpha)
     y = _run(case, binding.PATH_GEMM_SKINNY)
-    assert_parity(y, case.y_ref(), f"chunked tensor-core N={N} K={K} M={M} G={G}")
+    assert_parity(y, case.y_ref(), f"stream kernel N={N} K={K} M={M} G={G}")
     y2 = _run(case, binding.PATH_GEMM_SKINNY)
     assert np.array_equal(y.view(np.uint16), y2.view(np.uint16))
 
 
 def test_auto_dispatch_between_17_and_64_tokens():
-    """awq_linear with 17..64 tokens and a registered workspace: the chunked tensor-core kernel
-    (AWQ_PATH_GEMV_MID is that kernel too above 8 tokens); above 64 tokens the prefill kernels.
-    Each result is bit-equal to its forced path."""
+    """awq_linear with 17..64 tokens and a registered workspace: the stream kernel (AWQ_PATH_GEMV_MID is that kernel too above 8
+    tokens); above 64 tokens on short rows the prefill kernels.  Each result is bit-equal to its forced path."""
     import torch
     from paper_2306_00978_b200 import binding
     for (N, K, M, want) in ((1024, 1408, 20, binding.PATH_GEMM_SKINNY), (1024, 1408, 64, binding.PATH_GEMM_SKINNY),

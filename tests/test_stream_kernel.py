@@ -6,7 +6,7 @@ import pytest
 
 from oracle import awq_oracle as orc
 from paper_2306_00978_b200 import synth
-from tests.test_chunked_tensor_core import unrounded_bound
+from tests.test_stream_kernel_to_64_tokens import unrounded_bound
 from tests.util import Case, assert_parity, oracle_packed_to_cuda, to_cuda
 
 pytestmark = pytest.mark.gpu

@@ -1,5 +1,5 @@
-"""The chunked tensor-core kernel (awq_linear with 9 .. 64 tokens, and fewer where the output rows are few):
-token tiles, groups, ragged chunks and several matrices in one launch, against the fp64 oracle."""
+"""The stream kernel (awq_linear with 9 .. 64 tokens, and fewer where the output rows are few): token tiles, groups, short last
+stages, tiles in few and in many parts, several matrices in one launch, against the fp64 oracle."""
 import numpy as np
 import pytest
 
@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 def unrounded_bound(x, W):
     """Up to 32 tokens nothing is rounded before the output: the products (q - z) * x are exact in the
-    tensor core, their sums, the multiplications by Delta and the sums over groups and chunks are fp32.
+    tensor core, their sums, the multiplications by Delta and the sums over groups and parts are fp32.
     At most K + 64 roundings of 2^-24 act on partial results bounded by sum |W||x|; the fp16 output adds
     2^-11 of the value (or 2^-25 in its subnormal range)."""
     a = np.abs(x.astype(np.float64)) @ np.abs(W).T
@@ -21,14 +21,14 @@ def unrounded_bound(x, W):
 
 
 @pytest.mark.parametrize("N,K,M,G", [
-    (128, 128, 1, 64), (128, 128, 9, 128),        # one slab, half a stage; few rows: also below 9 tokens
-    (256, 384, 16, 128),                           # last stage of the chunk holds one pair of k-blocks
-    (384, 2176, 17, 64),                           # past one chunk of 16 groups, 32-token tile
-    (1152, 4224, 32, 128),                         # several chunks, the last one short
-    (128, 9088, 8, 128),                           # one slab, many chunks
-    (19072, 640, 12, 64),                          # more units than blocks, ranges that cross chunks
+    (128, 128, 1, 64), (128, 128, 9, 128),        # half a tile of half a stage; few rows: also below 9 tokens
+    (256, 384, 16, 128),                           # two parts, the second of half a stage
+    (384, 2176, 17, 64),                           # an odd slab, nine parts, 32-token tile
+    (1152, 4224, 32, 128),                         # ranges of one and two stages, nine to seventeen parts
+    (128, 9088, 8, 128),                           # half a tile in 36 parts
+    (19072, 640, 12, 64),                          # 75 tiles of three stages for 74 pairs: ranges of three and four stages
     (2048, 5120, 31, 256),                         # a group stored per 128 columns
-    (512, 1152, 33, 64), (1280, 3200, 64, 128),    # 64-token tile
+    (512, 1152, 33, 64), (1280, 3200, 64, 128),    # 48 and 64 tokens a tile
 ])
 def test_linear(N, K, M, G):
     from paper_2306_00978_b200 import binding
@@ -47,12 +47,12 @@ def test_linear(N, K, M, G):
 
 
 @pytest.mark.parametrize("widths,K,M,G", [
-    ((256, 128, 384), 1408, 10, 128),              # three matrices, slabs end to end
+    ((256, 128, 384), 1408, 10, 128),              # three matrices, slabs end to end, two of them odd
     ((1024, 1024), 4096, 32, 64),
     ((512, 128, 128, 896), 2688, 48, 128),
 ])
 def test_several_matrices_and_the_folded_scale(widths, K, M, G):
-    """One launch (and the kernel that adds the chunks) serves all matrices; the scaled call gives bit for
+    """One launch (and the kernel that adds the parts) serves all matrices; the scaled call gives bit for
     bit what the plain one gives on x' = fp16(x * inv_s)."""
     from paper_2306_00978_b200 import binding
     cases = [Case(8100 + i, n, K, M, G, 0.5) for i, n in enumerate(widths)]
@@ -72,9 +72,9 @@ def test_several_matrices_and_the_folded_scale(widths, K, M, G):
 
 
 @pytest.mark.parametrize("N,K,M", [
-    (8192, 4096, 24),              # one unit per block, and a ring of five stages that wraps inside it
+    (8192, 4096, 24),              # ranges of six and seven stages, fewer than the ring's
     (8192, 4096, 32),
-    (22016, 4096, 32),             # three units per block, some in two chunks, six stages
+    (22016, 4096, 32),             # eighteen and nineteen stages: the ring wraps twice
 ])
 def test_back_to_back_calls_on_new_operands(N, K, M):
     """Operands made on the device, two calls on them with nothing in between: equal bit for bit, and every
