@@ -226,7 +226,10 @@ def workspace_bytes(M: int, N: int, K: int, group: int) -> int:
 def linear(x: torch.Tensor, qweight: torch.Tensor, scales: torch.Tensor, zeros: torch.Tensor,
            N: int, K: int, group: int, out: Optional[torch.Tensor] = None,
            path: int = PATH_AUTO) -> torch.Tensor:
-    """awq_linear / awq_linear_path: y = x . dequant(Wq)^T, x fp16 [M][K] already divided by s."""
+    """awq_linear / awq_linear_path: y = x . dequant(Wq)^T, x fp16 [M][K] already divided by s.
+
+    Calls that use the device's one workspace (all of 9 tokens and more may) must not overlap on the GPU: issue
+    them on one stream."""
     if _native is not None:                                   # the ordinary call; None: something is out of the ordinary
         y = _native.linear(x, qweight, scales, zeros, N, K, group, out, path)
         if y is not None:
