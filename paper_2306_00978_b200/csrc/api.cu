@@ -234,7 +234,7 @@ int awq_quantize_pack_ex(const void* W, const float* act_mean_abs, float alpha, 
     const int rc = note_cuda(launch_quantize_pack(reinterpret_cast<const __half*>(W), act_mean_abs, alpha, group, bits,
                                                   symmetric != 0, clip_ratio, reinterpret_cast<uint32_t*>(qweight),
                                                   reinterpret_cast<__half*>(scales),
-                                                  reinterpret_cast<uint8_t*>(zeros), N, K, (cudaStream_t)stream));
+                                                  reinterpret_cast<uint8_t*>(zeros), N, K, d->sms, (cudaStream_t)stream));
     note_packed_writer(d, stream);
     return rc;
 }
@@ -727,7 +727,7 @@ int awq_search_alpha(const void* W, const float* act_mean_abs, const void* X, in
         if (int rc = note_cuda(launch_channel_scales(act_mean_abs, alphas + i0, b, p.s, K, st))) return rc;
         if (int rc = note_cuda(launch_quantize_pack_many(reinterpret_cast<const __half*>(W), p.s, b, group,
                                                          reinterpret_cast<uint32_t*>(p.qweight), reinterpret_cast<__half*>(p.scales),
-                                                         p.zeros, N, K, st)))
+                                                         p.zeros, N, K, d->sms, st)))
             return rc;
         // (the plainly ordered division stands between this writer and its readers)
         if (int rc = note_cuda(launch_divide_by_scale(X, p.s, b, p.xs, M, p.rows, K, st))) return rc;

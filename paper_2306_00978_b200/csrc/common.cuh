@@ -30,7 +30,7 @@ cudaError_t launch_channel_scale(const float* a, float alpha, float* s, int K, c
 // bits: 4 or 3 (3-bit codes in the 4-bit fields); clip: optional per-group range ratios [N][K/group]
 cudaError_t launch_quantize_pack(const __half* W, const float* a, float alpha, int group, int bits,
                                  bool symmetric, const float* clip, uint32_t* qweight, __half* scales, uint8_t* zeros,
-                                 int N, int K, cudaStream_t st);
+                                 int N, int K, int sms, cudaStream_t st);
 constexpr int kMaxClipRatios = 32;
 constexpr int kMaxSearchAlphas = 64;
 // ratios: HOST array of n_ratios <= kMaxClipRatios values; clip: device out, fp32 [N][K/group]
@@ -178,7 +178,7 @@ cudaError_t launch_losses(const double* partials, int count, size_t n, float* lo
 // s[i] of n alphas (a HOST array); W quantized with each of `count` scale arrays, packed arrays end to end
 cudaError_t launch_channel_scales(const float* a, const float* alphas, int n, float* s, int K, cudaStream_t st);
 cudaError_t launch_quantize_pack_many(const __half* W, const float* s, int count, int group, uint32_t* qweight, __half* scales,
-                                      uint8_t* zeros, int N, int K, cudaStream_t st);
+                                      uint8_t* zeros, int N, int K, int sms, cudaStream_t st);
 // `count` products of the same shape in one launch (gemm_tcgen05.cu)
 cudaError_t launch_gemm_blocks(const void* x, const void* qweight, const void* scales, const void* zeros, void* y, int count,
                                int M, int rows, int N, int K, int group, void* workspace, size_t workspace_bytes,

@@ -1,13 +1,12 @@
 // Offline step of the layer: channel scale (Eq. 5), fold into W (Eq. 3), group-wise
 // asymmetric 4-bit round-to-nearest (Eq. 2) and the packed tile layout (Sec. 4.2).
 //
-// HBM-bound: 2 bytes read and ~0.52 bytes written per weight.  One warp owns a band of 16
-// rows x 128 columns; lane (g, t) loads rows g and g+8, columns 16j+4t..+3 (j = 0..3) of both
-// 64-column tiles (sixteen 8-byte loads in flight per thread; the four lanes of a row read 32
-// contiguous bytes), which is exactly the data of the two 16-byte packed pieces it writes, so
-// no shared-memory transpose is needed.  Every
+// 2 bytes read and ~0.52 bytes written per weight; the issue of instructions sets the time.  One warp takes a band of 16
+// rows x 128 columns; lane (g, t) holds rows g and g+8, columns 16j+4t..+3 (j = 0..3) of both 64-column
+// blocks, which is exactly the data of the two 16-byte packed pieces it writes.  Every
 // rounding point is an explicit IEEE operation (no contraction); the per-weight division is
 // replaced by a multiplication only where that provably rounds to the same integer.
+#include <mutex>
 #include <type_traits>
 
 #include "common.cuh"
@@ -39,12 +38,6 @@ __global__ void channel_scales_kernel(const float* __restrict__ a, const __grid_
     if (k < K) s[(size_t)i * K + k] = channel_scale_one(mode == kAlphaZero ? 1.0f : a[k], alphas.v[i], mode);
 }
 
-__device__ __forceinline__ uint2 ldg_stream(const uint2* p) {
-    uint2 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
-    return v;
-}
-
 // Delta (fp16) and zero point of a group from its min and max; `top` is the largest code
 // (15 for 4-bit, 7 for 3-bit grids).
 __device__ __forceinline__ void group_params(float mn, float mx, float top, __half& d16, float& d, float& z) {
@@ -65,261 +58,326 @@ __device__ __forceinline__ uint32_t code_of(float w, float d, float rd, float z,
     if (!(fabsf(t - r) < 0.499f && fabsf(t) < 1024.0f)) r = rintf(__fdiv_rn(w, d));
     return (uint32_t)fminf(fmaxf(__fadd_rn(r, z), 0.0f), top);
 }
-// four codes (exact small integers held in floats) as four nibbles: q0 + 16 q1 + 256 q2 + 4096 q3 is
-// exact in fp32, so three FFMAs and one conversion replace four conversions and the shifts and ORs
-__device__ __forceinline__ uint32_t pack4(float q0, float q1, float q2, float q3) {
-    return (uint32_t)fmaf(q3, 4096.0f, fmaf(q2, 256.0f, fmaf(q1, 16.0f, q0)));
-}
-
-// grid = (K/128, N/32), block = 128: warp w takes band w % 2 of the block's 32 rows and block w / 2 of
-// the 128 columns, a lane 2 rows x 16 columns - exactly the data of the 16-byte packed piece it writes.
-// The products w' = w * s stay in registers (32), formed once (64 registers, 32 warps per SM).  For
-// G = 128 the two warps that share a group exchange their min / max through shared memory.  The
-// division w' / Delta is done only where it can matter: w' * (1 / Delta) rounds to the same integer
-// unless it lies within the group's own error bound of a half-integer; that test is taken per
-// packed word and row (the largest distance of the word's products from their rounded values), so
-// there is no branch per element, and a word that fails is redone element by element with the
-// division (code_of).  Rounding is by adding 1.5 * 2^23 (the zero point rides in the subtraction
-// that follows), group min / max take three-input min / max instructions, clamping to [0, top] is
-// compiled in only for the warps one of whose groups can leave the range, the nibbles of four codes
-// are assembled by FFMA and converted once.
-// What bounds it (measured on 4096 -> 11008, 113.6 MB): a block loads, computes and stores in
-// phases, and the blocks of an SM run in step, so the loads overlap the arithmetic only as far as
-// the blocks drift apart.  With 512-thread blocks (two per SM) 45.4 us, whatever the instruction
-// count (a form with a third more instructions and half the warps: 45 us; a third fewer
-// integer-pipe instructions: 44.3 us); 256-thread blocks 41.6 us, 128-thread blocks 37.9 us, 64-thread
-// blocks 41.0 us (the 128 channel scales are then formed per 64 threads).  A persistent form whose
-// producer warp keeps six 32 KB tiles in flight by tensor-map copies for sixteen quantizing warps
-// measured 58 us: the arithmetic needs the 32 warps.  The same 128-thread blocks made persistent
-// (eight per SM, each walking the tiles): 44.0 us - blocks that never leave stay in step.
 __device__ __forceinline__ float min3(float a, float b, float c) {
     float d; asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c)); return d;
 }
 __device__ __forceinline__ float max3(float a, float b, float c) {
     float d; asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c)); return d;
 }
-// code (still a float) = clamp(rne(w * rd) + z): zc = 1.5 * 2^23 - z, so that (w * rd + 1.5 * 2^23) - zc
-// is the rounded product plus the zero point, exactly (the product enters the sum unrounded, by a
-// fused multiply-add: 4 instead of 5 instructions per weight, 38.0 -> 35.7 us on 4096 -> 11008)
-// `dev` receives |t - rne(t)|, the distance that decides whether the product may stand for the
-// quotient; CLAMP = false where the group's smallest and largest element are known to stay in range.
-template <bool CLAMP>
-__device__ __forceinline__ float level_fast2(float w, float rd, float zc, float top, float& dev) {
-    // one rounding to the integer grid (the product is not rounded first), and the distance of the
-    // exact product from that integer, by one fused multiply-add each
-    const float u = __fmaf_rn(w, rd, 12582912.0f);
-    const float r = __fsub_rn(u, 12582912.0f);
-    dev = fabsf(__fmaf_rn(w, rd, -r));
-    const float q = __fsub_rn(u, zc);
-    return CLAMP ? fminf(fmaxf(q, 0.0f), top) : q;
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {      // a NaN stays
+    float d; asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c)); return d;
 }
 
-// One warp per band (16 rows) and 64-column block.  A thread block covers one group of columns (two
-// groups for G = 64) so that the group's min / max meet in shared memory: 2 bands x 2 blocks up to
-// G = 128, 1 band x G / 64 blocks above.  Scales and zero points are stored per 128 columns for
-// G > 128 (each group's entry G / 128 times), so that the layer kernels need no variant for them.
+// Two floats in a register pair; fma, add and sub round each half as the scalar instructions do.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 d; asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi)); return d;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c)); return d;
+}
+// (nothing may be added to a packed product: about one such sum in 10^5 came out as if the two instructions were fused)
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 d; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+    f32x2 d; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d;
+}
+
+
+// One warp per band (16 rows) and 128 columns.  A thread block covers a group's columns (two groups for G = 64); up to
+// G = 128 its warps take bands of their own and never meet, above the warps of a band exchange their min / max through shared memory.
+// Scales and zero points are stored per 128 columns for G > 128 (each group's entry G / 128 times), so that the
+// layer kernels need no variant for them.
 template <int G> struct QCfg {
-    static constexpr int kBlocks = G < 128 ? 2 : G / 64;            // 64-column blocks per thread block
-    static constexpr int kBands = kBlocks <= 4 ? 4 / kBlocks : 1;   // bands per thread block
-    static constexpr int kThreads = kBlocks * kBands * 32;
+    static constexpr int kCols = G < 128 ? 128 : G;                 // columns per thread block
+    static constexpr int kColWarps = kCols / 128;
+    static constexpr int kBands = kColWarps <= 4 ? 4 / kColWarps : 1;
+    static constexpr int kWarps = kColWarps * kBands, kThreads = kWarps * 32;
+    static constexpr int kSets = G == 64 ? 4 : 2;                   // (row, group) pairs of a lane
     static constexpr int kStored = G < 128 ? G : 128;               // columns per stored scale / zero point
+    static constexpr int kBlocks = 16 / kWarps;                     // thread blocks per SM: 128 registers per thread
+};
+// A warp's tile of W in shared memory: 16 rows of 256 bytes, 32 bytes apart so that the eight-byte loads of four rows meet all banks.
+constexpr int kQRowBytes = 256 + 32, kQTileBytes = 16 * kQRowBytes, kQStages = 2;
+
+// What a launch covers: items of (array part, column block, band step) in that order; blocks take equal contiguous ranges.
+struct QuantizeCut {
+    int N, K;
+    int col_blocks, band_steps;              // column blocks of kCols, steps of kBands bands
+    int items, share, longer;                // all items; items / blocks, items % blocks
+    int arrays, per_part;                    // scale arrays (1 unless the scale search), arrays per part
 };
 
-// MANY (the scale search): `a` is `many` arrays of K scales; W is quantized with each, its 32 values per lane loaded once,
-// and the packed arrays follow one another (4096 x 4096 with 20 arrays: 12.3 us each in launches of their own, ~9 us here; with
-// four blocks per SM, which nothing spills in, the whole search takes 538 us, with five 545, with six 556).
+// Group-wise round-to-nearest and the packed layout.  Lane (g, t) of a warp holds rows g and g + 8, columns 16j + 4t .. +3 of both
+// 64-column blocks, which is the data of the two packed pieces that it writes; the products w' = w * s stay in registers (64),
+// formed once.  The division w' / Delta is done only where it can matter: w' * (1 / Delta) rounds to the same integer unless it
+// lies within the group's own error bound of a half-integer; the largest such distance of a packed word decides, and a
+// word that fails is redone element by element with the division (code_of).  Rounding is by adding 1.5 * 2^23;
+// clamping to [0, top] is compiled in only for the warps one of whose groups can leave the range.
+// What bounds it is issue: per scheduler and cycle count, a packed multiply-add takes 2 cycles for two weights, a three-input
+// min / max and a conversion fp16 -> fp32 2, a conversion to an integer 8.  So the four nibbles' sum ends in 2^23 + the
+// nibbles, which is read as bits (no conversion), all fp32 steps are packed in pairs of columns, and a lane has 64 weights, so that the
+// three IEEE divisions of a group's parameters, formed once per row by different lanes of the four that share it, weigh little.
+// W comes through shared memory, each warp's next tiles by asynchronous copies while it works on the one before.
+// 4096 -> 11008 (113.6 MB), calls among others: 31.3 us with 32 weights per lane, scalar steps and four conversions per packed word pair,
+// 29.2 us so; 20 arrays on 4096 x 4096 157 -> 133 us.  16 warps per SM issue in 60 % of the cycles (fma pipe 47 %, alu 43 %): the
+// warps' own dependencies are what is left.  Blocks per SM 3 / 4 / 5: 150 / 137 / 146 us (five spill); W widened once per item in
+// shared memory: 144 us (spills); a third tile in flight: 12 % slower; columns before bands in the order of items: 5 % slower.
+// MANY (the scale search): `a` is `arrays` arrays of K scales; W is quantized with each and the packed arrays follow one another.
 template <int G, int BITS, bool CLIP, bool SYM, bool MANY = false>
-__global__ void __launch_bounds__(QCfg<G>::kThreads, (MANY ? 512 : 1024) / QCfg<G>::kThreads)
+__global__ void __launch_bounds__(QCfg<G>::kThreads, QCfg<G>::kBlocks)
 quantize_pack_tile_kernel(const __half* __restrict__ W, const float* __restrict__ a, float alpha,
                           int mode, const float* __restrict__ clip,
                           uint32_t* __restrict__ qweight, __half* __restrict__ scales,
-                          uint8_t* __restrict__ zeros, int N, int K, int many) {
+                          uint8_t* __restrict__ zeros, const __grid_constant__ QuantizeCut cut) {
+    using Cfg = QCfg<G>;
     constexpr float top = (float)((1 << BITS) - 1);       // largest code
-    constexpr int kQBands = QCfg<G>::kBands, kQBlocks = QCfg<G>::kBlocks, kQThreads = QCfg<G>::kThreads;
-    __shared__ __align__(16) float s_sm[kQBlocks * 64];
-    __shared__ float2 s_mm[kQBlocks][kQBands * 16];        // G >= 128: [64-column block][row] (min, max)
-    const int kblk = blockIdx.x;
+    constexpr int kSets = Cfg::kSets, kColWarps = Cfg::kColWarps;
+    extern __shared__ __align__(16) unsigned char q_smem[];
+    __shared__ float2 s_mm[kColWarps > 1 ? 2 : 1][kColWarps][Cfg::kBands * 16];   // G > 128: [step parity][column warp][row] (min, max)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int bw = warp % kQBands, ti = warp / kQBands;
+    const int bw = warp % Cfg::kBands, cw = warp / Cfg::kBands;
     const int g = lane >> 2, t = lane & 3;
-    const int n0 = (blockIdx.y * kQBands + bw) * 16 + g;   // this lane's upper row; lower = n0 + 8
-    const int kbase = kblk * (kQBlocks * 64);
+    const int K = cut.K, bands = cut.N / 16;
+    unsigned char* tiles = q_smem + warp * (kQStages * kQTileBytes);
+    float* s_sm = reinterpret_cast<float*>(q_smem + Cfg::kWarps * (kQStages * kQTileBytes));   // [arrays of the part][kCols]
 
-    uint2 raw[2][4];                                       // [row h][word j] = columns 16j + 4t .. +3 of the block
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            raw[h][j] = ldg_stream(reinterpret_cast<const uint2*>(
-                W + (size_t)(n0 + 8 * h) * K + kbase + ti * 64 + 16 * j + 4 * t));
-    static_assert(!MANY || kQBlocks * 64 == kQThreads, "one scale per thread");
-    float s_next = 0.0f;
-    if (MANY) s_next = a[kbase + (int)threadIdx.x];
-    for (int rest = MANY ? many : 1; rest > 0; --rest) {
-    if (MANY) {
-        s_sm[threadIdx.x] = s_next;
-        a += K;
-        if (rest > 1) s_next = a[kbase + (int)threadIdx.x];
-    } else {
-        for (int i = threadIdx.x; i < kQBlocks * 64; i += kQThreads) {
-            const int k = kbase + i;
-            s_sm[i] = channel_scale_one(mode == kAlphaZero ? 1.0f : a[k], alpha, mode);
-        }
-    }
-    __syncthreads();
+    const int block = (int)blockIdx.x;
+    const int first = block * cut.share + min(block, cut.longer), last = first + cut.share + (block < cut.longer ? 1 : 0);
+    const int per_part_items = cut.col_blocks * cut.band_steps;
 
-    // w' = fp32(w) * s  (Eq. 3), once, and the min / max of this lane's 16 columns of each row
-    float wp[2][4][4];
-    float mn[2], mx[2];
+    // this warp's tile of an item, eight 16-byte pieces per lane
+    auto fetch = [&](int item) {
+        if (item < last) {
+            const int in_part = item % per_part_items, cb = in_part / cut.band_steps, band = (in_part - cb * cut.band_steps) * Cfg::kBands + bw;
+            const __half* src = W + (size_t)(band * 16 + (lane >> 4)) * K + cb * Cfg::kCols + cw * 128 + (lane & 15) * 8;
+            const uint32_t dst = (uint32_t)__cvta_generic_to_shared(tiles + (item % kQStages) * kQTileBytes + (lane >> 4) * kQRowBytes + (lane & 15) * 16);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) { mn[h] = INFINITY; mx[h] = -INFINITY; }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const float4 s4 = *reinterpret_cast<const float4*>(&s_sm[ti * 64 + 16 * j + 4 * t]);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const float2 f01 = __half22float2(*reinterpret_cast<const __half2*>(&raw[h][j].x));
-            const float2 f23 = __half22float2(*reinterpret_cast<const __half2*>(&raw[h][j].y));
-            wp[h][j][0] = __fmul_rn(f01.x, s4.x);
-            wp[h][j][1] = __fmul_rn(f01.y, s4.y);
-            wp[h][j][2] = __fmul_rn(f23.x, s4.z);
-            wp[h][j][3] = __fmul_rn(f23.y, s4.w);
-            mn[h] = min3(mn[h], wp[h][j][0], wp[h][j][1]);
-            mn[h] = min3(mn[h], wp[h][j][2], wp[h][j][3]);
-            mx[h] = max3(mx[h], wp[h][j][0], wp[h][j][1]);
-            mx[h] = max3(mx[h], wp[h][j][2], wp[h][j][3]);
+            for (int i = 0; i < 8; ++i)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * 2 * kQRowBytes), "l"(src + (size_t)(2 * i) * K) : "memory");
         }
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int off = 1; off <= 2; off <<= 1) {
-            mn[h] = fminf(mn[h], __shfl_xor_sync(0xFFFFFFFFu, mn[h], off));
-            mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xFFFFFFFFu, mx[h], off));
-        }
-    if (G >= 128) {
-        // the group spans all 64-column blocks of the thread block: the others' min / max through shared memory
-        if (t == 0) {
-            s_mm[ti][bw * 16 + g] = make_float2(mn[0], mx[0]);
-            s_mm[ti][bw * 16 + g + 8] = make_float2(mn[1], mx[1]);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int o = 1; o < kQBlocks; ++o) {
-                const float2 v = s_mm[(ti + o) % kQBlocks][bw * 16 + g + 8 * h];
-                mn[h] = fminf(mn[h], v.x);
-                mx[h] = fmaxf(mx[h], v.y);
-            }
-    }
-    float wabs[2];                                          // largest |w'| of each group (before clipping)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) wabs[h] = fmaxf(fabsf(mn[h]), fabsf(mx[h]));
-    const int gi = (G == 64) ? kblk * 2 + ti : kblk;
-    const int ng = K / G;
-    if (CLIP) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const float r = __ldg(clip + (size_t)(n0 + 8 * h) * ng + gi);
-            mn[h] = __fmul_rn(mn[h], r);
-            mx[h] = __fmul_rn(mx[h], r);
-        }
-    }
-    // Delta, the zero point and 1 / Delta cost three IEEE divisions: each of a row's four lanes needs both rows', so even lanes
-    // form the upper row's and odd ones the lower row's, and they exchange them (4096 -> 11008: 32.9 -> 31.2 us).
-    const bool low = (t & 1) != 0;
-    float d[2], z[2], rd[2], thr[2], zc[2];
-    {
-        const float mn1 = low ? mn[1] : mn[0], mx1 = low ? mx[1] : mx[0], wabs1 = low ? wabs[1] : wabs[0];
-        __half h16;
-        float d1, z1;
-        if (SYM) {
-            constexpr float half_levels = (float)(1 << (BITS - 1));
-            const float d32 = __fdiv_rn(fmaxf(fabsf(mn1), fabsf(mx1)), half_levels);
-            h16 = __float2half_rn(d32);
-            const unsigned short bits = __half_as_ushort(h16);
-            if ((bits & 0x7FFFu) == 0u || (bits & 0x7C00u) == 0x7C00u) h16 = __ushort_as_half(0x3C00u);
-            d1 = __half2float(h16);
-            z1 = half_levels;
-        } else {
-            group_params(mn1, mx1, top, h16, d1, z1);
-        }
-        const float rd1 = __frcp_rn(d1);
-        // |w * rd - w / d| <= 1.8e-7 |w / d| (three roundings); the group's largest |w / d|
-        // bounds it for every element; quotients beyond 1024 always take the division
-        const float tmax = __fmul_rn(wabs1, rd1);
-        const float thr1 = tmax < 1024.0f ? 0.5f - fmaf(tmax, 4e-7f, 1e-6f) : -1.0f;
-        const float d2 = __shfl_xor_sync(0xFFFFFFFFu, d1, 1), z2 = __shfl_xor_sync(0xFFFFFFFFu, z1, 1);
-        const float rd2 = __shfl_xor_sync(0xFFFFFFFFu, rd1, 1), thr2 = __shfl_xor_sync(0xFFFFFFFFu, thr1, 1);
-        d[0] = low ? d2 : d1; d[1] = low ? d1 : d2;
-        z[0] = low ? z2 : z1; z[1] = low ? z1 : z2;
-        rd[0] = low ? rd2 : rd1; rd[1] = low ? rd1 : rd2;
-        thr[0] = low ? thr2 : thr1; thr[1] = low ? thr1 : thr2;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) zc[h] = 12582912.0f - z[h];      // exact: z is a small integer
-    }
-    // Clamping to [0, top] can only matter where the group's smallest or largest element leaves the
-    // range (the level is monotone in w'): rare without clipping - rne(max / Delta) + rne(-min / Delta)
-    // exceeds top only when both quotients sit on a tie - so the warp takes the clamped code only if one
-    // of its lanes needs it.
-    bool need_clamp = CLIP || SYM;
-    if (!need_clamp) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float dummy;
-            const float qlo = level_fast2<false>(mn[h], rd[h], zc[h], top, dummy);
-            const float qhi = level_fast2<false>(mx[h], rd[h], zc[h], top, dummy);
-            need_clamp = need_clamp || !(qlo >= 0.0f && qhi <= top);
-        }
-        need_clamp = __any_sync(0xFFFFFFFFu, need_clamp);
-    }
-    uint32_t words[4];
-    auto quantize_words = [&](auto clamp_tag) {
-        constexpr bool CL = decltype(clamp_tag)::value;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            float qu[4], ql[4], du[4], dl[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                qu[e] = level_fast2<CL>(wp[0][j][e], rd[0], zc[0], top, du[e]);
-                ql[e] = level_fast2<CL>(wp[1][j][e], rd[1], zc[1], top, dl[e]);
-            }
-            // the word's largest distance from the rounded value, per row, decides
-            const float dmu = max3(max3(du[0], du[1], du[2]), du[3], 0.0f);
-            const float dml = max3(max3(dl[0], dl[1], dl[2]), dl[3], 0.0f);
-            const bool bad = !(dmu < thr[0]) || !(dml < thr[1]);
-            // nibbles 0 .. 3 = (g,c) (g+8,c) (g,c+2) (g+8,c+2), nibbles 4 .. 7 the same for c+1, c+3
-            words[j] = pack4(qu[0], ql[0], qu[2], ql[2]) | (pack4(qu[1], ql[1], qu[3], ql[3]) << 16);
-            if (bad)                                               // rare: the word again, element by element
-                words[j] = (code_of(wp[0][j][0], d[0], rd[0], z[0], top) << 0) | (code_of(wp[0][j][1], d[0], rd[0], z[0], top) << 16) |
-                           (code_of(wp[1][j][0], d[1], rd[1], z[1], top) << 4) | (code_of(wp[1][j][1], d[1], rd[1], z[1], top) << 20) |
-                           (code_of(wp[0][j][2], d[0], rd[0], z[0], top) << 8) | (code_of(wp[0][j][3], d[0], rd[0], z[0], top) << 24) |
-                           (code_of(wp[1][j][2], d[1], rd[1], z[1], top) << 12) | (code_of(wp[1][j][3], d[1], rd[1], z[1], top) << 28);
-        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    if (need_clamp) quantize_words(std::true_type{}); else quantize_words(std::false_type{});
-    // band-major: block (band, k-tile) is 512 bytes, a band's blocks are contiguous along K
-    const size_t band = (size_t)blockIdx.y * kQBands + bw;
-    const size_t block = band * (K / 64) + (size_t)kblk * kQBlocks + ti;
-    uint4* dst = reinterpret_cast<uint4*>(qweight) + block * 32 + lane;
-    *dst = make_uint4(words[0], words[1], words[2], words[3]);
-    if (t == 0 && (G == 64 || (ti & 1) == 0)) {
-        // scales: [band][stored group][16]; zero bytes: [band pair][stored group][16], 8 per band; a
-        // stored group is the group itself up to 128 columns, else each of its runs of 128 columns
-        const size_t nsg = K / QCfg<G>::kStored;
-        const size_t sgi = (G == 64) ? (size_t)gi : (size_t)kblk * (kQBlocks / 2) + ti / 2;
-        scales[(band * nsg + sgi) * 16 + g] = __float2half_rn(d[0]);         // exact: Delta is an fp16 value
-        scales[(band * nsg + sgi) * 16 + g + 8] = __float2half_rn(d[1]);
-        zeros[((band >> 1) * nsg + sgi) * 16 + (band & 1) * 8 + g] =
-            (uint8_t)((uint32_t)z[0] | ((uint32_t)z[1] << 4));
-    }
-    if (MANY) {
-        qweight += (size_t)N * K / 8;
-        scales += (size_t)N * (K / QCfg<G>::kStored);
-        zeros += (size_t)N * (K / QCfg<G>::kStored) / 2;
-        __syncthreads();                                     // s_sm and s_mm have been read
-    }
+    fetch(first);
+    fetch(first + 1);
+
+    const f32x2 big2 = pack2(12582912.0f, 12582912.0f), c16 = pack2(16.0f, 16.0f);
+    int columns = -1;                                      // (part, column block) whose scales are in shared memory
+    for (int item = first; item < last; ++item) {
+        const int part = MANY ? item / per_part_items : 0, in_part = item - part * per_part_items;
+        const int cb = in_part / cut.band_steps, band = (in_part - cb * cut.band_steps) * Cfg::kBands + bw;
+        const int kbase = cb * Cfg::kCols, array0 = part * cut.per_part, arrays = MANY ? min(cut.per_part, cut.arrays - array0) : 1;
+        if (part * cut.col_blocks + cb != columns) {
+            columns = part * cut.col_blocks + cb;
+            __syncthreads();                               // the scales before have been read
+            if (MANY) {
+                for (int i = threadIdx.x; i < arrays * Cfg::kCols; i += Cfg::kThreads)
+                    s_sm[i] = a[(size_t)(array0 + i / Cfg::kCols) * K + kbase + i % Cfg::kCols];
+            } else {
+                for (int i = threadIdx.x; i < Cfg::kCols; i += Cfg::kThreads)
+                    s_sm[i] = channel_scale_one(mode == kAlphaZero ? 1.0f : a[kbase + i], alpha, mode);
+            }
+            __syncthreads();
+        }
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        const unsigned char* tile = tiles + (item % kQStages) * kQTileBytes + g * kQRowBytes + t * 8;
+        // Where this lane's outputs go: packed blocks [band][k-tile][512 bytes], scales [band][stored group][16], zero bytes
+        // [band pair][stored group][16], 8 per band; a stored group is the group itself up to 128 columns, else each of its runs of 128.
+        const size_t nsg = (size_t)(K / Cfg::kStored), q_step = (size_t)bands * K * 2, d_step = (size_t)bands * nsg * 16;
+        const int sg0 = G == 64 ? cb * 2 : cb * kColWarps + cw;
+        const int own = t % kSets, own_row = own & 1, own_ti = own >> 1;       // the (row, group) whose parameters this lane forms
+        uint32_t* q_out = qweight + (MANY ? array0 * q_step : 0) + ((size_t)band * (K / 64) + (size_t)(kbase / 64 + cw * 2)) * 128 + lane * 4;
+        __half* d_out = scales + (MANY ? array0 * d_step : 0) + ((size_t)band * nsg + sg0 + own_ti) * 16 + g + 8 * own_row;
+        uint8_t* z_out = zeros + (MANY ? array0 * (d_step / 2) : 0) + ((size_t)(band >> 1) * nsg + sg0) * 16 + (band & 1) * 8 + g;
+        for (int ai = 0; ai < arrays; ++ai) {
+            // w' = fp32(w) * s  (Eq. 3), once, and the min / max of this lane's columns of each (row, group)
+            f32x2 wp[2][2][4][2];                          // [row h][64-column block][word j][columns 4t, 4t+1 | 4t+2, 4t+3]
+            float mn[kSets], mx[kSets];
+#pragma unroll
+            for (int q = 0; q < kSets; ++q) { mn[q] = INFINITY; mx[q] = -INFINITY; }
+            const float* sc = s_sm + ai * Cfg::kCols + cw * 128 + 4 * t;
+#pragma unroll
+            for (int ti = 0; ti < 2; ++ti)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float4 s4 = *reinterpret_cast<const float4*>(sc + ti * 64 + 16 * j);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint2 raw = *reinterpret_cast<const uint2*>(tile + h * 8 * kQRowBytes + ti * 128 + j * 32);
+                        const float2 f01 = __half22float2(*reinterpret_cast<const __half2*>(&raw.x));
+                        const float2 f23 = __half22float2(*reinterpret_cast<const __half2*>(&raw.y));
+                        const f32x2 w01 = mul2(pack2(f01.x, f01.y), pack2(s4.x, s4.y)), w23 = mul2(pack2(f23.x, f23.y), pack2(s4.z, s4.w));
+                        wp[h][ti][j][0] = w01;
+                        wp[h][ti][j][1] = w23;
+                        float w0, w1, w2, w3;
+                        unpack2(w01, w0, w1);
+                        unpack2(w23, w2, w3);
+                        const int q = G == 64 ? 2 * ti + h : h;
+                        mn[q] = min3(mn[q], w0, w1);
+                        mn[q] = min3(mn[q], w2, w3);
+                        mx[q] = max3(mx[q], w0, w1);
+                        mx[q] = max3(mx[q], w2, w3);
+                    }
+                }
+            if (ai + 1 == arrays) {                        // the tile is in registers: its place takes the one after the next
+                __syncwarp();
+                fetch(item + 2);
+            }
+// a row's four lanes meet; lane t ends with set t % kSets: of two (sets of) sets it hands on the one that it does not keep
+            auto halve = [&](float keep, float give, int off, bool least) {
+                const float v = __shfl_xor_sync(0xFFFFFFFFu, give, off);
+                return least ? fminf(keep, v) : fmaxf(keep, v);
+            };
+            const bool odd = (t & 1) != 0, high = (t & 2) != 0;
+            float mn1 = halve(odd ? mn[1] : mn[0], odd ? mn[0] : mn[1], 1, true), mx1 = halve(odd ? mx[1] : mx[0], odd ? mx[0] : mx[1], 1, false);
+            if constexpr (kSets == 4) {
+                const float mn2 = halve(odd ? mn[3] : mn[2], odd ? mn[2] : mn[3], 1, true), mx2 = halve(odd ? mx[3] : mx[2], odd ? mx[2] : mx[3], 1, false);
+                mn1 = halve(high ? mn2 : mn1, high ? mn1 : mn2, 2, true);
+                mx1 = halve(high ? mx2 : mx1, high ? mx1 : mx2, 2, false);
+            } else {
+                mn1 = halve(mn1, mn1, 2, true);
+                mx1 = halve(mx1, mx1, 2, false);
+            }
+            if (kColWarps > 1) {
+                // the group spans the block's column warps: the others' min / max through shared memory
+                float2(*mm)[Cfg::kBands * 16] = s_mm[kColWarps > 1 ? item & 1 : 0];
+                if (t < 2) mm[cw][bw * 16 + g + 8 * t] = make_float2(mn1, mx1);
+                __syncthreads();
+#pragma unroll
+                for (int o = 0; o < kColWarps; ++o) {
+                    const float2 v = mm[o][bw * 16 + g + 8 * own_row];
+                    mn1 = fminf(mn1, v.x);
+                    mx1 = fmaxf(mx1, v.y);
+                }
+            }
+            // Delta, the zero point and 1 / Delta cost three IEEE divisions: once per row and group, then handed on
+            const float wabs = fmaxf(fabsf(mn1), fabsf(mx1));      // largest |w'| of the group (before clipping)
+            if (CLIP) {
+                const int gi = G == 64 ? cb * 2 + own_ti : cb;
+                const float r = __ldg(clip + (size_t)(band * 16 + g + 8 * own_row) * (K / G) + gi);
+                mn1 = __fmul_rn(mn1, r);
+                mx1 = __fmul_rn(mx1, r);
+            }
+            __half h16;
+            float d1, z1;
+            if (SYM) {
+                constexpr float half_levels = (float)(1 << (BITS - 1));
+                const float d32 = __fdiv_rn(fmaxf(fabsf(mn1), fabsf(mx1)), half_levels);
+                h16 = __float2half_rn(d32);
+                const unsigned short bits = __half_as_ushort(h16);
+                if ((bits & 0x7FFFu) == 0u || (bits & 0x7C00u) == 0x7C00u) h16 = __ushort_as_half(0x3C00u);
+                d1 = __half2float(h16);
+                z1 = half_levels;
+            } else {
+                group_params(mn1, mx1, top, h16, d1, z1);
+            }
+            const float rd1 = __frcp_rn(d1);
+            // |w * rd - w / d| <= 1.8e-7 |w / d| (three roundings); the group's largest |w / d|
+            // bounds it for every element; quotients beyond 1024 always take the division
+            const float tmax = __fmul_rn(wabs, rd1);
+            const float thr1 = tmax < 1024.0f ? 0.5f - fmaf(tmax, 4e-7f, 1e-6f) : -1.0f;
+            // Clamping to [0, top] can only matter where the group's smallest or largest element leaves the
+            // range (the level is monotone in w'): rare without clipping - rne(max / Delta) + rne(-min / Delta)
+            // exceeds top only when both quotients sit on a tie - so the warp takes the clamped code only if one
+            // of its lanes needs it.
+            bool need_clamp = CLIP || SYM;
+            if (!need_clamp) {
+                const float zc = 12582912.0f - z1;               // exact: z is a small integer
+                const float qlo = __fsub_rn(__fmaf_rn(mn1, rd1, 12582912.0f), zc), qhi = __fsub_rn(__fmaf_rn(mx1, rd1, 12582912.0f), zc);
+                need_clamp = __any_sync(0xFFFFFFFFu, !(qlo >= 0.0f && qhi <= top));
+            }
+            if (t < kSets) *d_out = h16;
+            float z[2], d[2], rd[2], thr = 0.0f;
+#pragma unroll
+            for (int ti = 0; ti < 2; ++ti) {
+                if (ti == 0 || G == 64) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int from = (lane & ~3) + (G == 64 ? 2 * ti + h : h);
+                        d[h] = __shfl_sync(0xFFFFFFFFu, d1, from);
+                        z[h] = __shfl_sync(0xFFFFFFFFu, z1, from);
+                        rd[h] = __shfl_sync(0xFFFFFFFFu, rd1, from);
+                        const float th = __shfl_sync(0xFFFFFFFFu, thr1, from);
+                        thr = h == 0 ? th : fminf(thr, th);
+                    }
+                    if (t == 0)                                  // z + 2^23: z in the low bits
+                        z_out[ti * 16] = (uint8_t)((__float_as_uint(z[0] + 8388608.0f) & 15u) | ((__float_as_uint(z[1] + 8388608.0f) & 15u) << 4));
+                }
+                const f32x2 rdu = pack2(rd[0], rd[0]), rdl = pack2(rd[1], rd[1]);
+                uint32_t words[4];
+                float dev[4];
+                auto quantize_words = [&](auto clamp_tag) {
+                    constexpr bool CL = decltype(clamp_tag)::value;
+                    // 2^23 + the zero points' own word: the codes are integer + zero point, nibbles (row g, g + 8, g, g + 8)
+                    const float zz = fmaf(z[1], 4112.0f, fmaf(z[0], 257.0f, 8388608.0f));
+                    const f32x2 zz2 = pack2(zz, zz);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        // minus the integer nearest to the product w' / Delta (ties to even), and the product's distance from it
+                        f32x2 nu[2], nl[2], du[2], dl[2];
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            nu[e] = sub2(big2, fma2(wp[0][ti][j][e], rdu, big2));
+                            nl[e] = sub2(big2, fma2(wp[1][ti][j][e], rdl, big2));
+                            du[e] = fma2(wp[0][ti][j][e], rdu, nu[e]);
+                            dl[e] = fma2(wp[1][ti][j][e], rdl, nl[e]);
+                        }
+                        float x[8];
+                        unpack2(du[0], x[0], x[1]);
+                        unpack2(du[1], x[2], x[3]);
+                        unpack2(dl[0], x[4], x[5]);
+                        unpack2(dl[1], x[6], x[7]);
+                        dev[j] = max3_nan(max3_nan(max3_nan(fabsf(x[0]), fabsf(x[1]), fabsf(x[2])), fabsf(x[3]), fabsf(x[4])),
+                                          max3_nan(fabsf(x[5]), fabsf(x[6]), fabsf(x[7])), 0.0f);
+                        // nibbles 0 .. 3 = (g,c) (g+8,c) (g,c+2) (g+8,c+2), nibbles 4 .. 7 the same for c+1, c+3: each half's sum
+                        // stays within 2^23 .. 2^23 + 65535, exactly, and is read as bits
+                        f32x2 sum;
+                        if (CL) {
+                            auto clamp2 = [&](f32x2 n, float zp) {
+                                float q0, q1;
+                                unpack2(sub2(pack2(zp, zp), n), q0, q1);
+                                return pack2(fminf(fmaxf(q0, 0.0f), top), fminf(fmaxf(q1, 0.0f), top));
+                            };
+                            sum = fma2(fma2(clamp2(nl[1], z[1]), c16, clamp2(nu[1], z[0])), c16, clamp2(nl[0], z[1]));
+                            sum = add2(fma2(sum, c16, clamp2(nu[0], z[0])), pack2(8388608.0f, 8388608.0f));
+                        } else {
+                            sum = sub2(zz2, fma2(fma2(fma2(nl[1], c16, nu[1]), c16, nl[0]), c16, nu[0]));
+                        }
+                        float lo, hi;
+                        unpack2(sum, lo, hi);
+                        words[j] = __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x5410);
+                    }
+                };
+                if (need_clamp) quantize_words(std::true_type{}); else quantize_words(std::false_type{});
+                if (!(max3_nan(dev[0], dev[1], max3_nan(dev[2], dev[3], 0.0f)) < thr)) {       // rare: a word again, element by element
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        if (dev[j] < thr) continue;
+                        uint32_t word = 0;
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) {
+                                float w0, w1;
+                                unpack2(wp[h][ti][j][e], w0, w1);
+                                word |= (code_of(w0, d[h], rd[h], z[h], top) | (code_of(w1, d[h], rd[h], z[h], top) << 16)) << (4 * h + 8 * e);
+                            }
+                        words[j] = word;
+                    }
+                }
+                // band-major: block (band, k-tile) is 512 bytes, a band's blocks are contiguous along K
+                *reinterpret_cast<uint4*>(q_out + ti * 128) = make_uint4(words[0], words[1], words[2], words[3]);
+            }
+            if (MANY) { q_out += q_step; d_out += d_step; z_out += d_step / 2; }
+        }
     }
 }
 
@@ -347,27 +405,10 @@ struct ClipGrid {
     float minus_zero;                                       // -0.0f, see mul2
 };
 
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
-    f32x2 d; asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi)); return d;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 d; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c)); return d;
-}
 // The rounded product, as a * b + (-0.0) with the zero in a kernel argument: with mul.rn.f32x2 and an
 // add.rn.f32x2 behind it about one group in 10^5 came out with another ratio than the definition, as if the
 // two had been fused (the scalar forms with explicit rounding did not); like this all agree.
 __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b, f32x2 minus_zero) { return fma2(a, b, minus_zero); }
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 d; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d;
-}
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
-    f32x2 d; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d;
-}
-
 // the error of one (row, ratio) as it is defined; wg = its w'
 template <int G>
 __device__ __noinline__ float clip_error_by_division(const float* wg, float d, float z, float top) {
@@ -537,25 +578,68 @@ cudaError_t launch_channel_scales(const float* a, const float* alphas, int n, fl
     return cudaGetLastError();
 }
 
-cudaError_t launch_quantize_pack_many(const __half* W, const float* s, int count, int group, uint32_t* qweight, __half* scales,
-                                      uint8_t* zeros, int N, int K, cudaStream_t st) {
-    if (group == 64)
-        quantize_pack_tile_kernel<64, 4, false, false, true><<<dim3(K / 128, N / (16 * QCfg<64>::kBands)), QCfg<64>::kThreads, 0, st>>>(
-            W, s, 1.0f, kAlphaOne, nullptr, qweight, scales, zeros, N, K, count);
-    else
-        quantize_pack_tile_kernel<128, 4, false, false, true><<<dim3(K / 128, N / (16 * QCfg<128>::kBands)), QCfg<128>::kThreads, 0, st>>>(
-            W, s, 1.0f, kAlphaOne, nullptr, qweight, scales, zeros, N, K, count);
+// Blocks take equal ranges of items.  The scale search's arrays are divided into parts where that evens out the ranges:
+// (4096 x 4096: 2048 items of 20 arrays for 592 blocks would be 4 against 3.46 on average).
+template <int G, int BITS, bool CLIP, bool SYM, bool MANY = false>
+static cudaError_t launch_quantize(const __half* W, const float* a, float alpha, int mode, const float* clip, uint32_t* qweight,
+                                   __half* scales, uint8_t* zeros, int N, int K, int arrays, int sms, cudaStream_t st) {
+    using Cfg = QCfg<G>;
+    static std::mutex mutex;
+    static bool done[64] = {};
+    auto* kernel = quantize_pack_tile_kernel<G, BITS, CLIP, SYM, MANY>;
+    constexpr int tiles = Cfg::kWarps * kQStages * kQTileBytes, most = tiles + (MANY ? kMaxSearchAlphas : 1) * Cfg::kCols * 4;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    {
+        std::lock_guard<std::mutex> lock(mutex);
+        if (!done[dev & 63]) {
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+            if (e != cudaSuccess) return e;
+            done[dev & 63] = true;
+        }
+    }
+    QuantizeCut cut = {};
+    cut.N = N;
+    cut.K = K;
+    cut.col_blocks = K / Cfg::kCols;
+    cut.band_steps = N / 16 / Cfg::kBands;             // (N is a multiple of 128)
+    cut.arrays = arrays;
+    const int resident = sms * Cfg::kBlocks;
+    const long long tiles_all = (long long)cut.col_blocks * cut.band_steps;
+    int parts = 1;
+    if (MANY) {
+        double least = 0.0;
+        for (int p = 1; p <= 4 && p <= arrays; ++p) {
+            const int per = (arrays + p - 1) / p, real = (arrays + per - 1) / per;
+            const double rounds = (double)((tiles_all * real + resident - 1) / resident) * (per + 0.5);    // (an item's own start: half an array)
+            if (p == 1 || rounds < least) { least = rounds; parts = real; }
+        }
+    }
+    cut.per_part = (arrays + parts - 1) / parts;
+    const long long items = tiles_all * parts;
+    if (items > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
+    cut.items = (int)items;
+    const int blocks = items < resident ? (int)items : resident;
+    cut.share = cut.items / blocks;
+    cut.longer = cut.items % blocks;
+    kernel<<<blocks, Cfg::kThreads, tiles + cut.per_part * Cfg::kCols * 4, st>>>(W, a, alpha, mode, clip, qweight, scales, zeros, cut);
     count_launch();
     return cudaGetLastError();
 }
 
+cudaError_t launch_quantize_pack_many(const __half* W, const float* s, int count, int group, uint32_t* qweight, __half* scales,
+                                      uint8_t* zeros, int N, int K, int sms, cudaStream_t st) {
+    return group == 64 ? launch_quantize<64, 4, false, false, true>(W, s, 1.0f, kAlphaOne, nullptr, qweight, scales, zeros, N, K, count, sms, st)
+                       : launch_quantize<128, 4, false, false, true>(W, s, 1.0f, kAlphaOne, nullptr, qweight, scales, zeros, N, K, count, sms, st);
+}
+
 cudaError_t launch_quantize_pack(const __half* W, const float* a, float alpha, int group, int bits,
                                  bool symmetric, const float* clip, uint32_t* qweight, __half* scales, uint8_t* zeros,
-                                 int N, int K, cudaStream_t st) {
+                                 int N, int K, int sms, cudaStream_t st) {
     const int mode = (int)alpha_mode(alpha);
-#define AWQ_QP_LAUNCH(GG, BB, CC, SS)                                                                           \
-    quantize_pack_tile_kernel<GG, BB, CC, SS><<<dim3(K / (QCfg<GG>::kBlocks * 64), N / (16 * QCfg<GG>::kBands)), \
-                                                QCfg<GG>::kThreads, 0, st>>>(W, a, alpha, mode, clip, qweight, scales, zeros, N, K, 1)
+#define AWQ_QP_LAUNCH(GG, BB, CC, SS) \
+    return launch_quantize<GG, BB, CC, SS>(W, a, alpha, mode, clip, qweight, scales, zeros, N, K, 1, sms, st)
 #define AWQ_QP_PICK2(GG, SS)                                             \
     do {                                                                 \
         if (bits == 4 && !clip) AWQ_QP_LAUNCH(GG, 4, false, SS);         \
@@ -577,8 +661,7 @@ cudaError_t launch_quantize_pack(const __half* W, const float* a, float alpha, i
 #undef AWQ_QP_PICK
 #undef AWQ_QP_PICK2
 #undef AWQ_QP_LAUNCH
-    count_launch();
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
 }
 
 template <int G>
