@@ -386,29 +386,29 @@ quantize_pack_tile_kernel(const __half* __restrict__ W, const float* __restrict_
 // error is written to clip[n][group].  The choice decides integer codes downstream, so the error
 // is defined operation by operation: dequant = (q - z) * Delta (one fp32 multiply), e = dequant -
 // w', err += e * e in fp32 over ascending k (no contraction), a NaN error counts as +inf.
-// grid = (K / G, N / 64), block = 128: one group of columns of 64 rows.  Its w' stay in shared memory, and
-// a thread takes one (row, two ratios) item at a time and walks the group's elements
-// in order, both ratios in one packed fp32 instruction each (multiply, add and fused multiply-add on two
-// floats round each half as the scalar ones do).  As in the quantizer the quotient's rounded value comes
-// from w' * (1 / Delta) by one fused multiply-add, and the largest distance of a product from its integer
-// decides per (row, ratio) whether that was safe; if not (about 0.05 % of them) the item is redone with
-// the division.  Arithmetic bounds it: 6 packed instructions, two moves and 5 min / max per element and
-// ratio pair, ~5.6 us per ratio on 4096 -> 4096 and ~15 us for the rest.  4096 -> 4096 with 20 ratios 306 us
-// with a scalar division per element and ratio (a row's 2048 columns per 256 threads); packed with the
-// pairs (w', w') kept in shared memory, 11 warps per SM, 153 us; w' kept once, 20 warps, 117 us; with four
-// times four elements unrolled 112 us (192 or 256 threads: 119, 113 us); with the products kept from
-// contraction (mul2) 126 us.
-constexpr int kClipRows = 64, kClipThreads = 128;
+// grid = (K / G, N / 64), block = 256: one group of columns of 64 rows, its w' in shared memory; a thread takes one (row, two
+// ratios) item at a time.
+// First an estimate of every (row, ratio)'s error, in steps of Delta and in no particular order: t = w' / Delta by
+// w' * (1 / Delta), its nearest integer, clamped, f = t - that, S = sum of f * f, two elements per packed fp32 instruction
+// (4 of these, 4 min / max per pair of elements).  The estimate's root is within
+//     margin = 1e-5 sqrt(S) Delta + 6e-6 (T + 2) Delta,    T = max|w'| / Delta,
+// of the root of the error as it is defined: 1 / Delta is rounded once, f once, and where the product's nearest integer is not the
+// quotient's both lie half a step away, so |f| is off by less than 2^-21.6 (T + 1); the defined dequant and difference are each
+// rounded once, 2^-22.4 (T + 2) of a step; over 128 elements the norms differ by sqrt(128) times the sum of both, < 5.5e-6 (T + 2); the
+// two sums' own roundings are 130 and 70 times 2^-24 of the errors, half of that of the roots.  A ratio whose
+// estimate less its margin is above another's plus its margin is not the best.  Where more than one ratio is left (1 % of the rows),
+// those are evaluated as defined, in order, the quotient's integer by w' * (1 / Delta) where the largest distance of a product from
+// its integer shows that this is safe and by division elsewhere.  Not-a-number and overflow leave a ratio to be evaluated.
+// A packed fp32 instruction takes two issue slots, so a pair of elements and a ratio take 12 (12.3 measured on registers alone);
+// here they take 15.  4096 -> 4096 with 20 ratios: 94 us, of which 18 are loads, parameters and the choice (every ratio
+// evaluated as defined, 9 packed or min / max instructions per pair: 125 us).  128, 192, 320 threads: 103, 101, 96 us; one ratio at a
+// time 95, four 99; clamping by the saturation of a scalar multiply-add 91 to 99, at a wider margin.
+constexpr int kClipRows = 64, kClipThreads = 256;
 struct ClipGrid {
     float r[kMaxClipRatios];
     int n;
-    float minus_zero;                                       // -0.0f, see mul2
 };
 
-// The rounded product, as a * b + (-0.0) with the zero in a kernel argument: with mul.rn.f32x2 and an
-// add.rn.f32x2 behind it about one group in 10^5 came out with another ratio than the definition, as if the
-// two had been fused (the scalar forms with explicit rounding did not); like this all agree.
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b, f32x2 minus_zero) { return fma2(a, b, minus_zero); }
 // the error of one (row, ratio) as it is defined; wg = its w'
 template <int G>
 __device__ __noinline__ float clip_error_by_division(const float* wg, float d, float z, float top) {
@@ -421,6 +421,23 @@ __device__ __noinline__ float clip_error_by_division(const float* wg, float d, f
     }
     return err;
 }
+// the same without a division per element, where that gives the same integers
+template <int G>
+__device__ __noinline__ float clip_error(const float* wg, float tmax, float d, float rd, float z, float top) {
+    // |w rd - fl(w / d)| <= 2^-23 |w / d| (1 / d and the quotient are rounded once each); the distance
+    // itself is off by at most 2^-26, the threshold by 2^-25
+    const float thr = tmax < 1024.0f ? 0.5f - fmaf(tmax, 1.25e-7f, 6e-8f) : -1.0f;
+    float err = 0.0f, dev = 0.0f;
+#pragma unroll 8
+    for (int k = 0; k < G; ++k) {
+        const float w = wg[k];
+        const float n = __fsub_rn(12582912.0f, __fmaf_rn(w, rd, 12582912.0f));     // minus the product's integer
+        dev = max3_nan(dev, fabsf(__fmaf_rn(w, rd, n)), 0.0f);
+        const float e = __fadd_rn(__fmul_rn(fminf(fmaxf(n, z - top), z), d), w);    // minus the difference: its square is the same
+        err = __fadd_rn(err, __fmul_rn(e, e));
+    }
+    return dev < thr ? err : clip_error_by_division<G>(wg, d, z, top);
+}
 
 template <int G>
 struct ClipSmem {
@@ -428,6 +445,8 @@ struct ClipSmem {
     float w[kClipRows * kRowFloats];
     float err[kClipRows * (kMaxClipRatios + 1)];
     float2 mm[kClipRows];
+    int least[kClipRows];                                   // least estimate plus margin (a float that is not negative)
+    int left[kClipRows];                                    // ratios that may be the best
     float s[G];
 };
 
@@ -472,59 +491,95 @@ clip_search_kernel(const __half* __restrict__ W, const float* __restrict__ a, fl
             mn = fminf(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, off));
             mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
         }
-        if (p == 0) sm.mm[row] = make_float2(mn, mx);
+        if (p == 0) { sm.mm[row] = make_float2(mn, mx); sm.least[row] = 0x7F800000; sm.left[row] = 0; }
     }
     __syncthreads();
-    const int nr = ratios.n, np = (nr + 1) / 2;
+    const int nr = ratios.n;
+    // Delta, zero point, 1 / Delta and max|w'| / Delta of a (row, ratio)
+    auto params = [&](const float2& mm, float r, float& d, float& z, float& rd, float& tmax) {
+        __half d16;
+        group_params(__fmul_rn(mm.x, r), __fmul_rn(mm.y, r), top, d16, d, z);
+        rd = __frcp_rn(d);
+        tmax = __fmul_rn(fmaxf(fabsf(mm.x), fabsf(mm.y)), rd);
+    };
+    const int np = (nr + 1) / 2;
     for (int item = tid; item < kClipRows * np; item += kClipThreads) {
-        const int row = item / np, i0 = 2 * (item - row * np), i1 = min(i0 + 1, nr - 1);
-        const float2 mm = sm.mm[row];
-        float d[2], z[2], rd[2], thr[2];
+        const int row = item / np, i0 = 2 * (item - row * np);
+        const f32x2 big = pack2(12582912.0f, 12582912.0f);
+        float d[2], tmax[2], lo[2], hi[2];
+        f32x2 rd2[2], sum[2];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            const float r = ratios.r[j ? i1 : i0];
-            __half d16;
-            group_params(__fmul_rn(mm.x, r), __fmul_rn(mm.y, r), top, d16, d[j], z[j]);
-            rd[j] = __frcp_rn(d[j]);
-            // |w rd - fl(w / d)| <= 2^-23 |w / d| (1 / d and the quotient are rounded once each); the distance
-            // itself is off by at most 2^-26, the threshold by 2^-25
-            const float tmax = __fmul_rn(fmaxf(fabsf(mm.x), fabsf(mm.y)), rd[j]);
-            thr[j] = tmax < 1024.0f ? 0.5f - fmaf(tmax, 1.25e-7f, 6e-8f) : -1.0f;
+            float z, rd;
+            params(sm.mm[row], ratios.r[min(i0 + j, nr - 1)], d[j], z, rd, tmax[j]);
+            rd2[j] = pack2(rd, rd);
+            sum[j] = pack2(0.0f, 0.0f);
+            lo[j] = 12582912.0f - z;
+            hi[j] = lo[j] + top;
         }
-        const f32x2 rd2 = pack2(rd[0], rd[1]), d2 = pack2(d[0], d[1]), big = pack2(12582912.0f, 12582912.0f);
-        const f32x2 mz = pack2(ratios.minus_zero, ratios.minus_zero);
-        const float lo0 = z[0] - top, lo1 = z[1] - top, hi0 = z[0], hi1 = z[1];
         const float* wg = sm.w + row * kRowFloats;
-        f32x2 err = pack2(0.0f, 0.0f);
-        float dm0 = 0.0f, dm1 = 0.0f;
-#pragma unroll 4
-        for (int k = 0; k < G; k += 4) {
-            const float4 w4 = *reinterpret_cast<const float4*>(wg + k);
-            const float we[4] = {w4.x, w4.y, w4.z, w4.w};
-            float da[4], db[4];
+        constexpr int E = 4;                                     // pairs of elements at a time
+#pragma unroll 2
+        for (int k = 0; k < G; k += 2 * E) {
+            f32x2 w[E], u[2][E];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const f32x2 w = pack2(we[e], we[e]);
-                const f32x2 u = fma2(w, rd2, big);               // rounded to an integer in the sum
-                const f32x2 nr2 = sub2(big, u);                  // minus that integer
-                unpack2(fma2(w, rd2, nr2), da[e], db[e]);        // its distance from the product
-                float q0, q1;
-                unpack2(nr2, q0, q1);
-                q0 = fminf(fmaxf(q0, lo0), hi0);                 // z - q
-                q1 = fminf(fmaxf(q1, lo1), hi1);
-                const f32x2 dif = add2(mul2(pack2(q0, q1), d2, mz), w);  // minus the difference: its square is the same
-                err = add2(err, mul2(dif, dif, mz));
+            for (int e = 0; e < E; e += 2) {
+                const float4 w4 = *reinterpret_cast<const float4*>(wg + k + 2 * e);
+                w[e] = pack2(w4.x, w4.y);
+                w[e + 1] = pack2(w4.z, w4.w);
             }
-            dm0 = max3(max3(dm0, fabsf(da[0]), fabsf(da[1])), fabsf(da[2]), fabsf(da[3]));
-            dm1 = max3(max3(dm1, fabsf(db[0]), fabsf(db[1])), fabsf(db[2]), fabsf(db[3]));
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) u[j][e] = fma2(w[e], rd2[j], big);       // rounded to an integer in the sum
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    float u0, u1;
+                    unpack2(u[j][e], u0, u1);
+                    u[j][e] = pack2(fminf(fmaxf(u0, lo[j]), hi[j]), fminf(fmaxf(u1, lo[j]), hi[j]));
+                }
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) u[j][e] = fma2(w[e], rd2[j], sub2(big, u[j][e]));
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) sum[j] = fma2(u[j][e], u[j][e], sum[j]);
         }
-        float e0, e1;
-        unpack2(err, e0, e1);
-        if (!(dm0 < thr[0])) e0 = clip_error_by_division<G>(wg, d[0], z[0], top);
-        if (!(dm1 < thr[1])) e1 = clip_error_by_division<G>(wg, d[1], z[1], top);
-        float* out = sm.err + row * (kMaxClipRatios + 1);
-        out[i0] = (e0 != e0) ? INFINITY : e0;
-        if (i1 > i0) out[i1] = (e1 != e1) ? INFINITY : e1;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            if (i0 + j >= nr) break;
+            float s0, s1;
+            unpack2(sum[j], s0, s1);
+            const float root = sqrtf(s0 + s1) * d[j], margin = fmaf(1e-5f, root, 6e-6f * (tmax[j] + 2.0f) * d[j]);
+            const bool sure = tmax[j] < 1024.0f && root + margin < INFINITY;
+            sm.err[row * (kMaxClipRatios + 1) + i0 + j] = sure ? root - margin : -INFINITY;
+            if (sure) atomicMin(&sm.least[row], __float_as_int(root + margin));
+        }
+    }
+    __syncthreads();
+    for (int item = tid; item < kClipRows * nr; item += kClipThreads) {
+        const int row = item / nr, i = item - row * nr;
+        if (sm.err[row * (kMaxClipRatios + 1) + i] <= __int_as_float(sm.least[row])) atomicAdd(&sm.left[row], 1);
+    }
+    __syncthreads();
+    for (int item = tid; item < kClipRows * nr; item += kClipThreads) {
+        const int row = item / nr, i = item - row * nr;
+        float* e = sm.err + row * (kMaxClipRatios + 1) + i;
+        float err = INFINITY;
+        if (*e <= __int_as_float(sm.least[row])) {
+            err = 0.0f;                                     // the only one left
+            if (sm.left[row] > 1) {
+                float d, z, rd, tmax;
+                params(sm.mm[row], ratios.r[i], d, z, rd, tmax);
+                err = clip_error<G>(sm.w + row * kRowFloats, tmax, d, rd, z, top);
+                if (err != err) err = INFINITY;
+            }
+        }
+        *e = err;
     }
     __syncthreads();
     if (tid < kClipRows) {
@@ -687,7 +742,6 @@ cudaError_t launch_clip_search(const __half* W, const float* a, float alpha, int
                                cudaStream_t st) {
     ClipGrid grid_r;
     grid_r.n = n_ratios;
-    grid_r.minus_zero = -0.0f;
     for (int i = 0; i < kMaxClipRatios; ++i) grid_r.r[i] = i < n_ratios ? ratios[i] : 1.0f;
     const int mode = (int)alpha_mode(alpha);
     const float top = (float)((1 << bits) - 1);
