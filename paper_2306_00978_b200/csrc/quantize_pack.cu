@@ -35,6 +35,7 @@ struct Alphas {
 };
 __global__ void channel_scales_kernel(const float* __restrict__ a, const __grid_constant__ Alphas alphas, float* __restrict__ s, int K) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y, mode = alphas.mode[i];
+    start_behind_predecessor();
     if (k < K) s[(size_t)i * K + k] = channel_scale_one(mode == kAlphaZero ? 1.0f : a[k], alphas.v[i], mode);
 }
 
@@ -149,6 +150,7 @@ quantize_pack_tile_kernel(const __half* __restrict__ W, const float* __restrict_
     unsigned char* tiles = q_smem + warp * (kQStages * kQTileBytes);
     float* s_sm = reinterpret_cast<float*>(q_smem + Cfg::kWarps * (kQStages * kQTileBytes));   // [arrays of the part][kCols]
 
+    start_behind_predecessor();
     const int block = (int)blockIdx.x;
     const int first = block * cut.share + min(block, cut.longer), last = first + cut.share + (block < cut.longer ? 1 : 0);
     const int per_part_items = cut.col_blocks * cut.band_steps;
@@ -460,6 +462,7 @@ clip_search_kernel(const __half* __restrict__ W, const float* __restrict__ a, fl
     constexpr int kPieces = G / 8, kRowFloats = ClipSmem<G>::kRowFloats;
     const int n0 = blockIdx.y * kClipRows, k0 = blockIdx.x * G;
     const int tid = threadIdx.x;
+    start_behind_predecessor();
 
     for (int i = tid; i < G; i += kClipThreads) sm.s[i] = channel_scale_one(mode == kAlphaZero ? 1.0f : a[k0 + i], alpha, mode);
     __syncthreads();
@@ -628,7 +631,8 @@ cudaError_t launch_channel_scale(const float* a, float alpha, float* s, int K, c
 cudaError_t launch_channel_scales(const float* a, const float* alphas, int n, float* s, int K, cudaStream_t st) {
     Alphas list = {};
     for (int i = 0; i < n; ++i) { list.v[i] = alphas[i]; list.mode[i] = (int)alpha_mode(alphas[i]); }
-    channel_scales_kernel<<<dim3((K + 255) / 256, n), 256, 0, st>>>(a, list, s, K);
+    const cudaError_t e = launch_behind(channel_scales_kernel, dim3((K + 255) / 256, n), 256, 0, st, a, list, s, K);
+    if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
 }
@@ -678,7 +682,8 @@ static cudaError_t launch_quantize(const __half* W, const float* a, float alpha,
     const int blocks = items < resident ? (int)items : resident;
     cut.share = cut.items / blocks;
     cut.longer = cut.items % blocks;
-    kernel<<<blocks, Cfg::kThreads, tiles + cut.per_part * Cfg::kCols * 4, st>>>(W, a, alpha, mode, clip, qweight, scales, zeros, cut);
+    e = launch_behind(kernel, blocks, Cfg::kThreads, (size_t)(tiles + cut.per_part * Cfg::kCols * 4), st, W, a, alpha, mode, clip, qweight, scales, zeros, cut);
+    if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
 }
@@ -731,8 +736,8 @@ static cudaError_t launch_clip(const __half* W, const float* a, float alpha, int
         if (e != cudaSuccess) return e;
         done[dev & 63] = true;
     }
-    clip_search_kernel<G><<<dim3(K / G, N / kClipRows), kClipThreads, sizeof(ClipSmem<G>), st>>>(
-        W, a, alpha, mode, ratios, top, clip, N, K, aligned);
+    e = launch_behind(clip_search_kernel<G>, dim3(K / G, N / kClipRows), kClipThreads, sizeof(ClipSmem<G>), st, W, a, alpha, mode, ratios, top, clip, N, K, aligned);
+    if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
 }

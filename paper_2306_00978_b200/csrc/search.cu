@@ -96,6 +96,7 @@ sqdiff_partial_kernel(const __half* __restrict__ yq, const float* __restrict__ y
 }
 __global__ void __launch_bounds__(256)
 sqdiff_final_kernel(const double* __restrict__ partials, int blocks, double inv_count, float* __restrict__ out) {
+    start_behind_predecessor();
     double t = 0.0;
     for (int i = threadIdx.x; i < blocks; i += 256) t += partials[(size_t)blockIdx.x * blocks + i];
     const double sum = block_sum(t);
@@ -298,7 +299,8 @@ cudaError_t launch_squared_difference(const void* yq, const float* yref, int cou
     return cudaGetLastError();
 }
 cudaError_t launch_losses(const double* partials, int count, size_t n, float* losses, cudaStream_t st) {
-    sqdiff_final_kernel<<<(unsigned)count, 256, 0, st>>>(partials, kLossBlocks, 1.0 / (double)n, losses);
+    const cudaError_t e = launch_behind(sqdiff_final_kernel, (unsigned)count, 256, 0, st, partials, kLossBlocks, 1.0 / (double)n, losses);
+    if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
 }
