@@ -45,7 +45,7 @@ def _native_command() -> list:
     libs = os.path.join(os.path.dirname(torch.__file__), "lib")
     return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-o", NATIVE_PATH,
             os.path.join(CSRC, "native_calls.cpp"), f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
-            *[f"-isystem{i}" for i in includes], f"-L{libs}", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10",
+            *[f"-isystem{i}" for i in includes], f"-L{libs}", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-lc10",
             "-lc10_cuda"]
 
 

