@@ -8,7 +8,7 @@
 // that a cut divides leaves its parts' fp32 sums in the workspace, and a second, small kernel adds them in a fixed order:
 // deterministic, no counters, nobody waits for another pair.
 //   * a stage is 8 bands x 256 input channels of packed weights (16 KB), its scales and zero points, and the block's half
-//     of x (128-byte swizzle), one tensor-map copy each, up to eight stages ahead;
+//     of x (128-byte swizzle), one tensor-map copy each, up to six stages ahead;
 //   * sixteen dequantizer warps, each owning a band and every second stage; a slot of A in tensor memory is a stage;
 //   * one warp issues the products, four (16 tokens) or eight epilogue warps drain them.
 // A is stored in the 16x128b form (17 cycles per 16 x 32 columns; 16x256b, which is the packed piece as it is, takes 33, and
@@ -33,6 +33,8 @@
 //   warp number through a shuffle and tensor memory at column 0, so that a product's operands are formed in uniform
 //     registers (46 -> 32 cycles a product)                                            31 / 8
 //   64 registers, so that a block of the second kernel fits beside the first's         30 / 6.4
+//   (another machine: 30.5 / 5.85) a stage freed by its products, the scales read before, not by the epilogue behind them   29.2 / 5.72
+//   three stages of weights ahead at the start (kStAhead), six in all                  28.7 / 5.67
 // Adding the parts inside this kernel cost more: by the last pair to arrive 9.5 us, by all of a tile's pairs 9.6 us,
 // through distributed shared memory of clusters of 4 or 8 blocks (whole tiles only; 33 and 15 clusters fit) 7.0 us.
 #include "tcgen05.cuh"
@@ -48,6 +50,10 @@ constexpr int kStWBytes = kStTiles * kTileBytes;         // 8 bands x 4 k-blocks
 constexpr int kStInvBytes = kStStageK * 4;               // the stage's 1 / s
 constexpr int kStZeroBytes = 256, kStScaleBytes = 1024;  // zero points [4 band pairs][groups][16], scales [8 bands][groups][16]
 constexpr int kStMaxSmem = 226 * 1024 - 64;              // dynamic part: a few static bytes, and a block of the second kernel, come on top
+// Stages of weights that may be under way before the first has landed.  With the whole ring asked for at once x, which may be asked for
+// only after the launch in front, arrives behind it: 11008 -> 4096 at 16 / 32 tokens 10.2 / 11.6 us against 9.2 / 10.5, 4096 -> 12288 at 16
+// 10.7 against 9.6 (two: 9.5, but 4096 -> 22016 15.7 against 15.0; six stages in all instead of eight are as fast in the long run and faster here).
+constexpr int kStAhead = 3;
 constexpr int kStMaxThreads = 1024;                      // what registers are kept free for: the second kernel's block
 
 // BN: tokens per tile at most (N of the products is a multiple of 16 up to that)
@@ -61,7 +67,7 @@ template <int BN, bool XS> struct StCfg {
     static constexpr int kOutBytes = kExact ? 0 : 8 * 2048;
     static constexpr int kFixed = 1024 /*align*/ + 512 /*barriers*/ + kOutBytes;
     static constexpr int kFit = (kStMaxSmem - kFixed) / kStageBytes;
-    static constexpr int kStages = kFit < 8 ? kFit : 8;
+    static constexpr int kStages = kFit < 6 ? kFit : 6;
     // tensor memory: accumulators (EXACT: of pairs of groups), then 128 columns of A per slot
     static constexpr uint32_t kAccCols = kExact ? 2 * BN : BN;
     static constexpr uint32_t kNumAcc = BN == 16 ? 4 : BN <= 64 ? 2 : 1;
@@ -230,7 +236,7 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
             s_abort = 0u;
             for (uint32_t s = 0; s < (uint32_t)S; ++s) {
                 mbar_init(w_full(s), 1); mbar_init(x_full(s), 1);
-                mbar_init(empty(s), EXACT ? 4 * Cfg::kEpilogue : 1);      // EXACT: the epilogue has read the scales, after the products; else: the products
+                mbar_init(empty(s), EXACT ? 1 + 4 * Cfg::kEpilogue : 1);  // the products, and (EXACT) the epilogue has read the scales
             }
             for (uint32_t s = 0; s < (uint32_t)SL; ++s) { mbar_init(a_full(s), 16); mbar_init(a_empty(s), 1); }
             for (uint32_t b = 0; b < NACC; ++b) { mbar_init(acc_full(b), 1); mbar_init(acc_empty(b), 8 * Cfg::kEpilogue); }
@@ -269,6 +275,7 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
         StTile at = st_tile(cut, tile);
         bool ok = true;
         for (int n = 0; n < range.count; ++n) {
+            if (n >= kStAhead && n < S && !mbar_wait_warp(w_full((uint32_t)(n - kStAhead)), 0u, ctl)) { ok = false; break; }
             if (!mbar_wait_warp(empty(stage), phase ^ 1u, ctl)) { ok = false; break; }
             if (lead) {
                 mbar_arrive_expect_tx(w_full(stage), kStWBytes + GPS * (64 + 256));
@@ -356,7 +363,7 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
                             products(d_tmem + (uint32_t)BN, (q + 1) * KPG, (q + 2) * KPG, true);
                             // The slot before the last pair's sums: what the epilogue waits for comes last,
                             // so that no arrival is outstanding when the block exits.
-                            if (q + 2 >= GPS) st_commit(a_empty(slot));
+                            if (q + 2 >= GPS) { st_commit(a_empty(slot)); st_commit(empty(stage)); }
                             st_commit(acc_full(acc));
                         }
                         __syncwarp();
@@ -521,6 +528,8 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
 #pragma unroll
                     for (int q = 0; q < GPS; ++q)
                         d[q] = __half2float(*reinterpret_cast<const __half*>(sc_lane + x_off(stage) + q * 32));
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(empty(stage));    // (with the products' commit it frees the stage)
 #pragma unroll
                     for (int q = 0; q < GPS; q += 2) {
                         ok = __all_sync(0xFFFFFFFFu, mbar_wait(acc_full(acc), acc_phase, ctl));
@@ -540,8 +549,6 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
                         for (int i = 0; i < TH; i += 2) fma_pair(v[i], v[i + 1], d[q + 1], r1[i], r1[i + 1]);
                         if (++acc == NACC) { acc = 0; acc_phase ^= 1u; }
                     }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(empty(stage));    // its products are done and its scales have been read
                     if (++stage == (uint32_t)S) { stage = 0; phase ^= 1u; }
                 }
                 if (!ok) break;
