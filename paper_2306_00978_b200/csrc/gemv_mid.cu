@@ -46,6 +46,7 @@ constexpr int kMidSmem = 220 * 1024;
 constexpr int kMidChunkTiles = 16;                       // k-tiles (64 columns) per chunk: 16, or 8 where that fills the SMs better
 constexpr int kMidStageTiles = 4;                        // k-tiles per stage and band
 constexpr int kMidStageBytes = kMidMathWarps * kMidStageTiles * 512;
+constexpr int kMidAhead = 2;                            // stages under way before the first has landed
 constexpr int kMidStages = 4;
 
 // the same product starting a new accumulation (C = 0)
@@ -146,6 +147,10 @@ gemv_mid_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant
             tma_load_2d(pdst + (uint32_t)lay.z_in_par, &z_map, (kt0 / TPG) * 16, bg * (kMidMathWarps / 2),
                         bars + 128u + 8u * pb);
             for (int j = 0; j < nt; j += kMidStageTiles) {
+                // At the start two stages are under way until the first has landed: with the whole ring asked for at once x, which may be asked
+                // for only after the launch in front, arrives behind it (8192 -> 8192 at 8 tokens 11.7 us, with one, two, three stages
+                // 11.0, 11.0, 11.3; 13824 -> 5120 at 4 12.4, with 11.4, 11.9, 12.2; 28672 -> 8192 at 8 30.1, with 30.7, 30.1, 30.1).
+                if (issued >= kMidAhead && issued < S && !mbar_wait(bars + 8u * (uint32_t)(issued - kMidAhead), 0u, ctl)) { ok = false; break; }
                 if (!mbar_wait_relaxed(bars + 64u + 8u * stage, phase ^ 1u, ctl)) { ok = false; break; }
                 mbar_arrive_expect_tx(bars + 8u * stage, kMidStageBytes);
                 // 16 bands x 4 k-tiles at (64-bit element kt * 64 of the band's run, first band)
