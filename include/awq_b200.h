@@ -70,8 +70,9 @@ typedef enum AwqStatus {
 typedef enum AwqPath {
     AWQ_PATH_AUTO = 0,          /* what awq_linear does.  M <= 8: the matrix-vector kernels, and where
                                    K > 4096 from 3 tokens (N * K >= 2^26; from 2 where K >= 12288) or 5
-                                   tokens (N * K >= 2^25) the chunked one; M <= 64: the stream
-                                   kernel (below 9 tokens only where N/16 is well below the SM
+                                   tokens (N * K >= 2^25) the chunked one, or the stream kernel (K >=
+                                   5/4 N and N * K <= 2^28); M <= 64: the stream
+                                   kernel (below 9 tokens else only where N/16 is well below the SM
                                    count), up to 256 where its estimate is the best - these if a
                                    workspace of awq_workspace_bytes is registered; else the tensor-core
                                    prefill kernels (M <= 8: the band or split-K kernel) */
@@ -85,7 +86,8 @@ typedef enum AwqPath {
     AWQ_PATH_GEMM_1SM = 4,      /* the tensor-core kernel with one SM per tile, any M >= 1 */
     AWQ_PATH_GEMV_MID = 5,      /* M <= 8: the chunked matrix-vector kernel: work units of 16 bands
                                    x 1024 input channels, the unit's slice of x in shared memory, one
-                                   band per warp; 9 <= M <= 32: the stream kernel; needs a
+                                   band per warp; 9 <= M <= 32, and where awq_linear takes it
+                                   below: the stream kernel; needs a
                                    workspace of awq_workspace_bytes (fp32 partial sums per chunk of K) */
     AWQ_PATH_GEMM_SKINNY = 6    /* the stream kernel, M <= 64, N a multiple of 128: pairs of SMs
                                    (cta_group::2, 256 channels x up to 128 tokens per tile), the tiles' K

@@ -262,22 +262,36 @@ int awq_search_clip(const void* W, const float* act_mean_abs, float alpha, int g
                                         ratios, n_ratios, clip_ratio, N, K, (cudaStream_t)stream));
 }
 
-// Where the chunked matrix-vector kernel beats the band kernel, up to 8 tokens.
-// With one token fragment its time does not depend on M (32 us on the 70B shapes for 1 .. 8 tokens),
-// while the band kernel's grows with the tokens that travel through its stages.  Chunked / band, us:
-//   8192 -> 28672   3 tokens 31.3 / 34.5   5: 31.9 / 38.9   8: 32.5 / 49.1
-//   8192 -> 16384   3: 19.1 / 20.4   4: 19.2 / 20.7   8: 19.5 / 29.2
-//   8192 -> 8192    3: 13.0 / 13.0   4: 12.8 / 13.4   8: 13.2 / 18.7
-//   13824 -> 5120   3: 14.7 / 16.3   4: 14.8 / 17.5   8: 15.0 / 24.1
-//   5120 -> 13824   3: 13.6 / 13.4   4: 13.6 / 13.8   5: 13.7 / 15.1
-//   11008 -> 4096   4: 12.9 / 11.3   5: 13.1 / 12.9   6: 13.3 / 14.8   8: 13.1 / 16.1
-// With 4096 input channels the band kernel keeps x in registers and wins up to 8 tokens
+// Up to 8 tokens: where kernels that share their partial sums through the workspace beat the band kernel.  Their time hardly depends
+// on M, while the band kernel's grows with the tokens that travel through its stages.  Chunked / band, us (one machine):
+//   8192 -> 28672   3 tokens 27.4 / 31.5   5: 27.7 / 36.7   8: 28.3 / 46.6
+//   8192 -> 16384   3: 17.1 / 18.5   4: 17.1 / 18.7   8: 17.3 / 27.5
+//   8192 -> 8192    3: 10.9 / 11.3   4: 10.9 / 11.5   8: 11.0 / 17.2
+//   13824 -> 5120   3: 11.8 / 14.1   4: 11.8 / 15.1   8: 12.1 / 21.2
+//   5120 -> 13824   3: 11.1 / 11.9   4: 11.1 / 12.3   5: 11.2 / 13.8
+//   11008 -> 4096   4: 10.4 / 9.8   5: 10.6 / 11.5   6: 10.6 / 13.1   8: 10.6 / 14.0
+// With 4096 input channels the band kernel keeps x in registers and beats the chunked one up to 8 tokens
 // (4096 -> 11008 at 8 tokens: 11.7 / 9.8; 4096 -> 4096: 6.5 / 6.9).
+// (The stream kernel would win from 5 tokens on shorter rows too, 5120 -> 5120 at 8 tokens 6.6 / 10.2; the calls that the band kernel
+// serves touch no workspace and may run on several streams at once, so the line stays.)
 static bool mid_kernel_preferred(int M, int N, int K) {
     const long long nk = (long long)N * K;
     if (M < 2) return false;
-    if (M == 2) return K >= 12288 && nk >= (1LL << 26);   // 13824 -> 5120: 13.6 / 14.2 us, 28672 -> 8192: 32.3 / 33.5 us
+    if (M == 2) return K >= 12288 && nk >= (1LL << 26);   // 13824 -> 5120: 11.6 / 12.9 us, 28672 -> 8192: 29.1 / 30.9 us
     return M <= 8 && K > 4096 && nk >= (M <= 4 ? (1LL << 26) : (1LL << 25));
+}
+
+// Of those calls the stream kernel takes the ones with rows of at least 5/4 of the outputs and up to 2^28 weights: its ranges are equal
+// whatever the sizes, while the chunked kernel's blocks cross from one slice of x to the next and end on whole units.  Stream / chunked,
+// us, 3 and 8 tokens, groups of 128:
+//   11008 -> 4096  8.9 / 10.5   9.1 / 10.6      13824 -> 5120  11.4 / 11.8   11.5 / 12.1     28672 -> 8192  28.1 / 29.5   28.3 / 30.3
+//   10240 -> 8192  12.7 / 13.6   12.6 / 13.8    13824 -> 11008  19.6 / 21.6   19.7 / 22.2    65536 -> 512  10.0 / 11.8   9.8 / 12.0
+//   12288 -> 8192  14.2 / 14.2   14.3 / 14.6    16384 -> 6144  14.2 / 14.6   14.3 / 14.9
+// and beyond the lines: 9216 -> 8192 11.7 / 11.2   11.7 / 11.4, 8192 -> 8192 10.8 / 10.9   10.9 / 11.0, 8192 -> 28672 28.7 / 27.4   29.4 / 28.3,
+// 18944 -> 14336 31.9 / 31.2   32.2 / 32.2, 28672 -> 11008 at 2 tokens 37.0 / 36.0, 28672 -> 22016 66.6 / 61.7   67.8 / 64.4.
+// (Groups of 64 the same way: 28672 -> 8192 32.9 / 32.9   33.1 / 33.7, 11008 -> 4096 9.8 / 11.4   10.1 / 11.6.)
+static bool stream_beats_chunked(int M, int N, int K, int group) {
+    return mid_kernel_preferred(M, N, K) && 4LL * K >= 5LL * N && (long long)N * K <= (1LL << 28) && gemm_stream_applies(M, N, K, group);
 }
 
 // Where the stream kernel runs up to 64 tokens: from 9, and below where the output rows are too few for the band kernel
@@ -337,7 +351,8 @@ size_t awq_workspace_bytes(int M, int N, int K, int group) {
     }
     size_t gemm = gemm_workspace_bytes(M, N, sms);
     const size_t mid = (M <= 8 && gemv_mid_applies(M, N, K, group, sms)) ? gemv_mid_workspace_bytes(M, N, K) : 0;
-    const size_t parts = stream_kernel_preferred(M, N, K, group, sms) ? gemm_stream_workspace_bytes(M, sms) : 0;
+    const size_t parts = stream_kernel_preferred(M, N, K, group, sms) || stream_beats_chunked(M, N, K, group)
+                             ? gemm_stream_workspace_bytes(M, sms) : 0;
     if (parts > gemm) gemm = parts;
     if (M > 16) return gemm;
     size_t gemv = gemv_workspace_bytes(M);         // required by the split-K matrix-vector kernel
@@ -384,7 +399,8 @@ static int linear_path(const void* x, const void* qweight, const void* scales, c
     }
     DeviceState* d;
     if (int rc = device_state(&d)) return rc;
-    const int without_stream = path;
+    int without_stream = path;               // taken where the stream kernel cannot be launched
+    bool may_fall_back = automatic;
     if (automatic && stream_kernel_preferred(M, N, K, group, d->sms)) {
         const size_t need = gemm_stream_workspace_bytes(M, d->sms);
         std::lock_guard<std::mutex> lock(g_mutex);
@@ -399,19 +415,16 @@ static int linear_path(const void* x, const void* qweight, const void* scales, c
         if (stream_beats_prefill(d, &one, 1, M, K, group)) path = AWQ_PATH_GEMM_SKINNY;
     }
     if (path == AWQ_PATH_GEMV_MID && M > 8 && gemm_stream_applies(M, N, K, group)) path = AWQ_PATH_GEMM_SKINNY;
+    if (path == AWQ_PATH_GEMV_MID && stream_beats_chunked(M, N, K, group) && gemv_mid_applies(M, N, K, group, d->sms)) {
+        std::lock_guard<std::mutex> lock(g_mutex);
+        if (d->workspace_bytes >= gemm_stream_workspace_bytes(M, d->sms) && d->workspace_bytes >= gemv_mid_workspace_bytes(M, N, K)) {
+            path = AWQ_PATH_GEMM_SKINNY;
+            without_stream = AWQ_PATH_GEMV_MID;
+            may_fall_back = true;
+        }
+    }
     const cudaStream_t st = (cudaStream_t)stream;
     const LaunchOrder order = launch_order(d, stream, behind_writer);
-    if (path == AWQ_PATH_GEMV_MID) {
-        if (!gemv_mid_applies(M, N, K, group, d->sms)) return AWQ_ERR_BAD_SHAPE;
-        void* ws = nullptr;
-        {
-            std::lock_guard<std::mutex> lock(g_mutex);
-            if (d->workspace_bytes < gemv_mid_workspace_bytes(M, N, K)) return AWQ_ERR_NO_WORKSPACE;
-            ws = d->workspace;
-        }
-        return note_cuda(order.launched(launch_gemv_mid(x, qweight, scales, zeros, y, M, N, K, group, ws, d->status_word, d->sms,
-                                                        order.serialize, st)));
-    }
     if (path == AWQ_PATH_GEMM_SKINNY) {
         const size_t need = gemm_stream_workspace_bytes(M, d->sms);
         void* ws = nullptr;
@@ -423,8 +436,19 @@ static int linear_path(const void* x, const void* qweight, const void* scales, c
         const GemvMatrix one = {qweight, scales, zeros, y, N};
         const cudaError_t e = order.launched(launch_gemm_stream(x, &one, 1, M, K, group, nullptr, ws, d->status_word,
                                                                 d->sms, order.serialize, st));
-        if (!automatic || e != cudaErrorNotSupported) return note_cuda(e);
+        if (!may_fall_back || e != cudaErrorNotSupported) return note_cuda(e);
         path = without_stream;               // no pair of SMs to be had (a partition of the device): nothing was launched
+    }
+    if (path == AWQ_PATH_GEMV_MID) {
+        if (!gemv_mid_applies(M, N, K, group, d->sms)) return AWQ_ERR_BAD_SHAPE;
+        void* ws = nullptr;
+        {
+            std::lock_guard<std::mutex> lock(g_mutex);
+            if (d->workspace_bytes < gemv_mid_workspace_bytes(M, N, K)) return AWQ_ERR_NO_WORKSPACE;
+            ws = d->workspace;
+        }
+        return note_cuda(order.launched(launch_gemv_mid(x, qweight, scales, zeros, y, M, N, K, group, ws, d->status_word, d->sms,
+                                                        order.serialize, st)));
     }
     if (path == AWQ_PATH_GEMV && gemv_uses_band_kernel(M, N, d->sms)) {
         const GemvMatrix one = {qweight, scales, zeros, y, N};
