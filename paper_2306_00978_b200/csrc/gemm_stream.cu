@@ -20,11 +20,11 @@
 // Up to 32 tokens (EXACT) A is the integer q - z, every group has an accumulator of its own and the epilogue adds Delta times it
 // in fp32: nothing is rounded before the output (a 2-norm error of 2.1e-4); above A is fp16 (q - z) * Delta (2.8e-4).
 //
-// What bounds it: a stage takes 1190 / 1410 / 1760 cycles at 16 / 32 / 64 tokens (one tile per pair, 16 to 49 stages of cold
-// weights; 700 at the HBM rate), of which the products' and the dequantizers' own cycles, counted in a copy of the kernel at
-// 16 tokens, account for about 880 each; where the rest goes is not known.  Above 64 tokens x through L2 (32 KB a stage and SM at
-// 128 tokens, half of a tile's, beside 16 KB of weights) comes on top, on short launches their start (~3 us until the first
-// products are drained) and the second kernel (~1.5 us).
+// What bounds it: a stage takes 970 / 1130 / 1410 cycles at 16 / 32 / 64 tokens (18944 channels, one tile per pair, the slope of chained
+// calls with cold weights between 4096 and 12288 input channels; 1010 / 1140 / 1410 while a stage was freed by the epilogue behind its
+// products; 700 at the HBM rate), of which the products' and the dequantizers' own cycles, counted in a copy of the kernel at 16
+// tokens, are about 880 each.  Above 64 tokens x through L2 (32 KB a stage and SM at 128 tokens, half of a tile's, beside 16 KB of
+// weights) comes on top, on short launches their start (~3 us until the first products are drained) and the second kernel (~1.5 us).
 // What it took, 28672 -> 8192 / 4096 -> 4096 at 16 tokens, us (one machine, cold weights; 30.5 to 33.2 and 6 to 6.4 by now on others):
 //   one SM per 128 channels, chunks of K with x resident, whole units per block       37.6 / 7.9
 //   pairs, even ranges; parts added by the last pair to arrive                         45 / 10

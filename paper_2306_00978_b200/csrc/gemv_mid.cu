@@ -46,7 +46,7 @@ constexpr int kMidSmem = 220 * 1024;
 constexpr int kMidChunkTiles = 16;                       // k-tiles (64 columns) per chunk: 16, or 8 where that fills the SMs better
 constexpr int kMidStageTiles = 4;                        // k-tiles per stage and band
 constexpr int kMidStageBytes = kMidMathWarps * kMidStageTiles * 512;
-constexpr int kMidAhead = 2;                            // stages under way before the first has landed
+constexpr int kMidAhead = 2;                             // stages under way before the first has landed
 constexpr int kMidStages = 4;
 
 // the same product starting a new accumulation (C = 0)
