@@ -259,8 +259,8 @@ int awq_linear_scaled_needs_scratch(int M, int N, int K, int group);
  *  scales and zeros are unchanged.
  * awq_linear_int3: the layer on that storage.  Where the band matrix-vector kernel serves the call
  * (M <= 8 and N / 16 not far below the SM count) it streams the 3-bit array itself, 25 % fewer
- * weight bytes than the 4-bit layout; other shapes (split-K and tensor-core kernels read the
- * 4-bit layout) are first expanded into qweight_scratch (device, awq_qweight_bytes(N, K) bytes,
+ * weight bytes than the 4-bit layout; so does the stream kernel up to 64 tokens, where awq_linear takes it.  Other shapes (split-K
+ * and prefill kernels read the 4-bit layout) are first expanded into qweight_scratch (device, awq_qweight_bytes(N, K) bytes,
  * caller-owned; may be NULL when the band kernel applies, else AWQ_ERR_NULL_POINTER) and run as
  * awq_linear.  Results equal awq_linear on the expanded array bit for bit where the same kernel runs.
  */

@@ -168,7 +168,7 @@ size_t gemm_stream_workspace_bytes(int M, int sms);
 double gemm_stream_estimate(int M, int slabs, int K, int sms);     // us, above 64 tokens; slabs of 256 channels, all matrices'
 cudaError_t launch_gemm_stream(const void* x, const GemvMatrix* mats, int count, int M, int K, int group,
                                const float* inv_s, void* workspace, unsigned int* status_word, int sms,
-                               bool serialize, cudaStream_t st);
+                               bool serialize, cudaStream_t st, int bits = 4);
 
 // scale search (search.cu)
 // Scratch of a search: `batch` grid points at a time, each with `rows` >= M rows of x / s and y and packed arrays of its own.

@@ -46,7 +46,8 @@ namespace {
 // warps: 0 weight copies, 1 products (leader), 2 x copies, 4-7 and 24-27 epilogue, 8-23 dequantizers
 constexpr int kStTiles = 4;                              // k-blocks per stage
 constexpr int kStStageK = kStTiles * kBK;                // 256 input channels
-constexpr int kStWBytes = kStTiles * kTileBytes;         // 8 bands x 4 k-blocks x 512 bytes
+constexpr int kStBlockBytes = 512;                       // 16 rows x 64 columns (384 in the 3-bit storage)
+constexpr int kStWBytes = 8 * kStTiles * kStBlockBytes;  // 8 bands x 4 k-blocks
 constexpr int kStInvBytes = kStStageK * 4;               // the stage's 1 / s
 constexpr int kStZeroBytes = 256, kStScaleBytes = 1024;  // zero points [4 band pairs][groups][16], scales [8 bands][groups][16]
 constexpr int kStMaxSmem = 226 * 1024 - 64;              // dynamic part: a few static bytes, and a block of the second kernel, come on top
@@ -191,7 +192,17 @@ __device__ __forceinline__ void drain(uint32_t bar, uint32_t parity, const WaitC
     while (!mbar_try_wait(bar, parity) && global_ns() - t0 < drain_limit_ns(ctl)) {}
 }
 
-template <int G, int BN, bool XS>
+// A lane's piece of one block.  3-bit storage: three words, whose nibbles' top bits are the fourth's (the readers mask them out).
+template <int TB> __device__ __forceinline__ uint4 st_piece(const unsigned char* p) {
+    if constexpr (TB == kStBlockBytes) return *reinterpret_cast<const uint4*>(p);
+    const uint32_t* u = reinterpret_cast<const uint32_t*>(p);
+    return make_uint4(u[0], u[1], u[2], ((u[0] >> 3) & 0x11111111u) | ((u[1] >> 2) & 0x22222222u) | ((u[2] >> 1) & 0x44444444u));
+}
+
+// TB: bytes of a packed block (16 rows x 64 columns): 512 for 4-bit codes, 384 for the 3-bit storage, whose fourth word costs five
+// instructions per piece and the others none (their masks leave out a nibble's top bit): 8192 -> 28672 at 16 / 32 / 64 tokens 33.9 / 39.0 /
+// 44.1 us plainly ordered, 4-bit codes in chained launches 30.3 / 35.0 / 42.7.
+template <int G, int BN, bool XS, int TB = kStBlockBytes>
 __global__ void __launch_bounds__(kStMaxThreads, 1)
 gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ inv_s, float* partial, unsigned int* status_word, const __grid_constant__ CUtensorMap x_map,
                    const __grid_constant__ StMats mats) {
@@ -200,6 +211,7 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
     constexpr int S = Cfg::kStages, SL = Cfg::kSlots;
     constexpr int KPG = G / kBK;                         // k-blocks per group
     constexpr int GPS = kStTiles / KPG;                  // groups per stage
+    constexpr int kBlockK = TB / 8, kWBytes = 8 * kStTiles * TB;  // a block's 64-bit elements per band, a stage's weights
     constexpr uint32_t NACC = Cfg::kNumAcc;
     static_assert(8 * (3 * S + 2 * SL + 2 * (int)NACC) <= 512, "barriers");
     extern __shared__ unsigned char smem_dyn[];
@@ -278,9 +290,9 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
             if (n >= kStAhead && n < S && !mbar_wait_warp(w_full((uint32_t)(n - kStAhead)), 0u, ctl)) { ok = false; break; }
             if (!mbar_wait_warp(empty(stage), phase ^ 1u, ctl)) { ok = false; break; }
             if (lead) {
-                mbar_arrive_expect_tx(w_full(stage), kStWBytes + GPS * (64 + 256));
-                // 8 bands x 4 k-blocks (256 64-bit elements); past the last band or k-block zeros are filled in
-                tma_load_2d(base + w_off(stage), &mats.w[at.mi], ks * kStStageK, at.slab * 16 + (int)rank * 8, w_full(stage));
+                mbar_arrive_expect_tx(w_full(stage), kWBytes + GPS * (64 + 256));
+                // 8 bands x 4 k-blocks (256 or 192 64-bit elements); past the last band or k-block zeros are filled in
+                tma_load_2d(base + w_off(stage), &mats.w[at.mi], ks * kStTiles * kBlockK, at.slab * 16 + (int)rank * 8, w_full(stage));
                 tma_load_2d(base + x_off(stage) + Cfg::kZeroOff, &mats.z[at.mi], ks * GPS * 16, at.slab * 8 + (int)rank * 4, w_full(stage));
                 tma_load_2d(base + x_off(stage) + Cfg::kParOff, &mats.sc[at.mi], ks * GPS * 16, at.slab * 16 + (int)rank * 8, w_full(stage));
             }
@@ -396,7 +408,7 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
         const int g = lane >> 2;
         const uint32_t taddr_band = tmem_base + ((uint32_t)(quad * 32 + hsel * 16) << 16) + (uint32_t)Cfg::kA0;
         const uint32_t leader_a_full0 = map_to_rank(a_full(0), 0);
-        const unsigned char* w_lane = base_ptr + Cfg::kXBytes + band * (kStTiles * 512) + lane * 16;
+        const unsigned char* w_lane = base_ptr + Cfg::kXBytes + band * (kStTiles * TB) + lane * (TB / 32);
         // x's channels are brought into A's order in shared memory, 16 of a token (32 bytes) per thread and pass
         constexpr int kThreadsPerKb = 4 * Cfg::kHalf, kKbPerPass = 256 / kThreadsPerKb < kStTiles ? 256 / kThreadsPerKb : kStTiles;
         const int t256 = (wi & 7) * 32 + lane, xkb = t256 / kThreadsPerKb, xm = (t256 >> 2) % Cfg::kHalf, xj = t256 & 3;
@@ -418,7 +430,7 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
             bool ok = mbar_wait(w_full(stage), phase, ctl);
             uint4 pk[kStTiles];
 #pragma unroll
-            for (int h = 0; h < kStTiles; ++h) pk[h] = *reinterpret_cast<const uint4*>(w_lane + so + h * 512);
+            for (int h = 0; h < kStTiles; ++h) pk[h] = st_piece<TB>(w_lane + so + h * TB);
             ok = mbar_wait(old_bar0 + 8u * old, old_phase, ctl) && ok;
             tc_fence_after();
             uint32_t zc[GPS], du[GPS], dl[GPS];
@@ -442,10 +454,11 @@ gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ 
                 for (int jw = 0; jw < 4; ++jw) {
                     constexpr uint32_t kSixteenth = 0x2C002C00u;
                     const uint32_t w = wds[jw], w8 = w >> 8;
-                    v[4 * jw + 0] = hsub2_u32(code_pair(w, kLowCodes), zlo);                  // q - z, exactly
-                    v[4 * jw + 1] = hfma2_u32(code_pair(w, kHighCodes), kSixteenth, zhi);
-                    v[4 * jw + 2] = hsub2_u32(code_pair(w8, kLowCodes), zlo);
-                    v[4 * jw + 3] = hfma2_u32(code_pair(w8, kHighCodes), kSixteenth, zhi);
+                    constexpr uint32_t kLow = TB == kStBlockBytes ? kLowCodes : kLowCodes & 0x77777777u, kHigh = TB == kStBlockBytes ? kHighCodes : kHighCodes & 0x77777777u;
+                    v[4 * jw + 0] = hsub2_u32(code_pair(w, kLow), zlo);                  // q - z, exactly
+                    v[4 * jw + 1] = hfma2_u32(code_pair(w, kHigh), kSixteenth, zhi);
+                    v[4 * jw + 2] = hsub2_u32(code_pair(w8, kLow), zlo);
+                    v[4 * jw + 3] = hfma2_u32(code_pair(w8, kHigh), kSixteenth, zhi);
                     if (EXACT) continue;
                     v[4 * jw + 0] = hmul2_u32(v[4 * jw + 0], d_up);
                     v[4 * jw + 1] = hmul2_u32(v[4 * jw + 1], d_lo);
@@ -683,7 +696,7 @@ int st_tile_tokens(int M) {                              // tokens per tile: a m
 }
 
 // pairs that can be resident at once on the current device (0 if the query fails); cached once there is one
-template <int G, int BN, bool XS>
+template <int G, int BN, bool XS, int TB>
 cudaError_t st_resident_pairs(int sms, int* out) {
     static std::mutex mutex;
     static bool done[64] = {};
@@ -695,7 +708,7 @@ cudaError_t st_resident_pairs(int sms, int* out) {
     dev &= 63;
     std::lock_guard<std::mutex> lock(mutex);
     if (!done[dev]) {
-        e = cudaFuncSetAttribute(gemm_stream_kernel<G, BN, XS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes);
+        e = cudaFuncSetAttribute(gemm_stream_kernel<G, BN, XS, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes);
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
@@ -707,7 +720,7 @@ cudaError_t st_resident_pairs(int sms, int* out) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, gemm_stream_kernel<G, BN, XS>, &cfg) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveClusters(&n, gemm_stream_kernel<G, BN, XS, TB>, &cfg) != cudaSuccess) {
             (void)cudaGetLastError();
             n = 0;
         }
@@ -718,11 +731,11 @@ cudaError_t st_resident_pairs(int sms, int* out) {
     return cudaSuccess;
 }
 
-template <int G, int BN, bool XS>
+template <int G, int BN, bool XS, int TB = kStBlockBytes>
 cudaError_t st_launch(const CUtensorMap& xmap, const StMats& mats, const float* inv_s, StCut cut,
                       void* workspace, unsigned int* status_word, int sms, bool serialize, cudaStream_t st) {
     int resident = 0;
-    cudaError_t e = st_resident_pairs<G, BN, XS>(sms, &resident);
+    cudaError_t e = st_resident_pairs<G, BN, XS, TB>(sms, &resident);
     if (e != cudaSuccess) return e;
     if (resident < 1) return cudaErrorNotSupported;          // the caller's cue to take another kernel
     cut.pairs = cut.total < resident ? cut.total : resident;
@@ -743,7 +756,7 @@ cudaError_t st_launch(const CUtensorMap& xmap, const StMats& mats, const float* 
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = serialize ? 1 : 2;
-    e = cudaLaunchKernelEx(&cfg, gemm_stream_kernel<G, BN, XS>, cut, inv_s, partial, status_word, xmap, mats);
+    e = cudaLaunchKernelEx(&cfg, gemm_stream_kernel<G, BN, XS, TB>, cut, inv_s, partial, status_word, xmap, mats);
     if (e != cudaSuccess) return e;
     count_launch();
     if (!second) return cudaGetLastError();
@@ -755,7 +768,7 @@ cudaError_t st_launch(const CUtensorMap& xmap, const StMats& mats, const float* 
     cfg.blockDim = dim3(128);
     cfg.dynamicSmemBytes = 0;
     cfg.attrs = attr + 1;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = TB == kStBlockBytes ? 1 : 0;
     auto* reduce = per == 1 ? stream_reduce_kernel<1> : per == 2 ? stream_reduce_kernel<2> : stream_reduce_kernel<4>;
     e = cudaLaunchKernelEx(&cfg, reduce, cut, (const float*)partial);
     if (e != cudaSuccess) return e;
@@ -787,7 +800,7 @@ double gemm_stream_estimate(int M, int slabs, int K, int sms) {
 
 cudaError_t launch_gemm_stream(const void* x, const GemvMatrix* mats, int count, int M, int K, int group,
                                const float* inv_s, void* workspace, unsigned int* status_word, int sms,
-                               bool serialize, cudaStream_t st) {
+                               bool serialize, cudaStream_t st, int bits) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
     StCut cut = {};
@@ -817,9 +830,10 @@ cudaError_t launch_gemm_stream(const void* x, const GemvMatrix* mats, int count,
         const GemvMatrix& m = mats[i < count ? i : 0];
         if (i < count) {
             slabs += (m.n + 255) / 256;
-            // packed weights: one row of K * 8 bytes per band, as 64-bit elements; boxes of 8 bands x 4 k-blocks
-            const cuuint64_t wdims[2] = {(cuuint64_t)K, (cuuint64_t)(m.n / 16)}, wstr[1] = {(cuuint64_t)K * 8};
-            const cuuint32_t wbox[2] = {(cuuint32_t)kStStageK, 8}, estr[2] = {1, 1};
+            // packed weights: one row of K * 8 (3-bit storage: K * 6) bytes per band, as 64-bit elements; boxes of 8 bands x 4 k-blocks
+            const int per_block = bits * 16;             // 64-bit elements of a band's k-block
+            const cuuint64_t wdims[2] = {(cuuint64_t)(K / kBK) * per_block, (cuuint64_t)(m.n / 16)}, wstr[1] = {wdims[0] * 8};
+            const cuuint32_t wbox[2] = {(cuuint32_t)(kStTiles * per_block), 8}, estr[2] = {1, 1};
             if (enc(&sm.w[i], CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, const_cast<void*>(m.qweight), wdims, wstr, wbox, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -846,6 +860,13 @@ cudaError_t launch_gemm_stream(const void* x, const GemvMatrix* mats, int count,
     if ((long long)slabs * cut.m_tiles * cut.nks > (1LL << 22)) return cudaErrorInvalidValue;
     cut.tiles = slabs * cut.m_tiles;
     cut.total = cut.tiles * cut.nks;
+    if (bits == 3) {                                     // (up to 64 tokens, nothing folded in)
+        if (inv_s || cls > 64) return cudaErrorInvalidValue;
+#define AWQ_ST_LAUNCH3(GG, BNN) return st_launch<GG, BNN, false, 384>(xmap, sm, inv_s, cut, workspace, status_word, sms, true, st)
+        if (group == 128) { if (cls == 16) AWQ_ST_LAUNCH3(128, 16); if (cls == 32) AWQ_ST_LAUNCH3(128, 32); AWQ_ST_LAUNCH3(128, 64); }
+        if (cls == 16) AWQ_ST_LAUNCH3(64, 16); if (cls == 32) AWQ_ST_LAUNCH3(64, 32); AWQ_ST_LAUNCH3(64, 64);
+#undef AWQ_ST_LAUNCH3
+    }
 #define AWQ_ST_LAUNCH(GG, BNN)                                                                                             \
     return inv_s ? st_launch<GG, BNN, true>(xmap, sm, inv_s, cut, workspace, status_word, sms, serialize, st)       \
                  : st_launch<GG, BNN, false>(xmap, sm, inv_s, cut, workspace, status_word, sms, serialize, st)
