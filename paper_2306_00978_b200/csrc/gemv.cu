@@ -142,6 +142,10 @@ __device__ __forceinline__ void tile_sums_of_x(const __half* __restrict__ x, flo
 }
 
 // =========================================================================== band kernel
+// With x in shared memory a block asks for three stages of weights and for the others of the ring as those land: asked for at once, they queue
+// in front of x and of other blocks' first stages (8192 -> 8192 at one token 9.27 -> 9.05 us, 8192 -> 28672 25.0 -> 24.8, 5120 -> 5120 at two
+// 6.53 -> 6.43; with two stages 8.83, 24.6 and 6.34, but 11008 -> 4096 at one 7.10 -> 7.18).
+constexpr int kBandAhead = 3;
 constexpr int kBandThreads = kMathThreads + 96;        // + weight-copy warp + flush warp + x-copy warp
 
 // Stage layout of the band kernel, fixed at compile time by TPW (k-tiles per math warp and
@@ -414,6 +418,7 @@ gemv_band_kernel(const BandProblems probs, const __half* __restrict__ x, int M, 
         // ------------------------------------------------------------- weight-copy warp
         // lane 0 posts the stage's byte count (x included); lanes 0, 1, 2 each issue one bulk copy
         uint32_t stage = 0, phase = 0;
+        int ahead = 0;                                     // stages asked for (XSM)
         const uint64_t once = l2_policy_evict_first();     // every packed byte is read exactly once
         for (int task = b0; task < b1; ++task) {
             const BandRef br = band_ref(probs, task);
@@ -425,6 +430,8 @@ gemv_band_kernel(const BandProblems probs, const __half* __restrict__ x, int M, 
                 const uint32_t dst = sbase + stage * (uint32_t)lay.stage_bytes;
                 const uint32_t bar = bars + 8u * stage;
                 if (lane == 0) {
+                    if (XSM && ahead >= kBandAhead && ahead < S) mbar_wait_relaxed(bars + 8u * (uint32_t)(ahead - kBandAhead), 0u, ctl);
+                    ++ahead;
                     mbar_wait_relaxed(bars + 64u + 8u * stage, phase ^ 1u, ctl);
                     mbar_arrive_expect_tx(bar, (uint32_t)(nt * TB + ngr * 48 + ((XREG || XSM) ? 0 : M * nt * 128)));
                 }
