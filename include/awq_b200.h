@@ -180,7 +180,8 @@ int awq_channel_scale(const float* act_mean_abs, float alpha, float* s, int K, v
  * wait for that work.  The library covers its own writers: the first layer call behind an
  * awq_quantize_pack / awq_quantize_pack_ex / awq_pack_int3 / awq_unpack_int3 (or an awq_inverse_channel_scale,
  * see awq_linear_scaled) on the same stream is launched fully serialized, whatever other streams and threads enqueue meanwhile (behind a writer on another
- * stream the caller orders it, with an event for instance).  A caller who produces packed arrays by other
+ * stream the caller orders it, with an event for instance; in a stream capture, where the event alone would not do,
+ * every layer call on another stream than such a writer's is launched fully serialized).  A caller who produces packed arrays by other
  * means (its own kernel, a copy) must make sure they are complete before the operation that directly
  * precedes awq_linear in the stream begins - a stream or event synchronization, or any other kernel in
  * between that does not itself signal programmatic launch completion early, is enough.

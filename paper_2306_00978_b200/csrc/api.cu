@@ -26,27 +26,51 @@ struct StreamKey {
 // Streams on which one of this library's kernels that write packed arrays or 1 / s (quantizer, 3-bit packing and expansion) has been
 // enqueued and no layer call since.  Most layer kernels copy weights before the launch in front of them has completed, so the
 // first one behind such a writer on the same stream is launched fully serialized; what runs on other streams changes nothing.
+// Between streams an event waits for the writer's end - but not inside a capture: there a launch joined behind a writer by an event gets
+// a programmatic edge to it like one on its own stream (read from captured graphs), at any time up to the capture's end and also where a
+// call on the writer's stream has waited.  So a capture's entries stay, `taken` by their own stream's reader, and calls on the
+// capture's other streams are serialized.
 struct PendingWriters {
     static constexpr int kMost = 64;
-    struct Entry { StreamKey key; unsigned long long serial; };
+    struct Entry { StreamKey key; unsigned long long serial; bool taken; };
     Entry list[kMost];
     int count = 0;
     unsigned long long serial = 0;         // of the last writer
+    unsigned long long forgotten = 0;      // the largest of the captures whose entries made room for others: up to it every captured launch is serialized
     bool overflow = false;                 // more streams than fit: every launch is serialized until the device has been waited for
 
     void add(const StreamKey& key) {
-        ++serial;
-        for (int i = 0; i < count; ++i)
+        const Entry entry = {key, ++serial, false};
+        int room = -1;
+        for (int i = 0; i < count; ++i) {
             // a stream is in one capture at a time: a writer in an earlier one can have no reader any more
-            if (list[i].key.stream == key.stream && (list[i].key.capture != 0) == (key.capture != 0)) { list[i] = {key, serial}; return; }
-        if (count < kMost) list[count++] = {key, serial}; else overflow = true;
+            if (list[i].key.stream == key.stream && (list[i].key.capture != 0) == (key.capture != 0)) { list[i] = entry; return; }
+            if (list[i].taken && (room < 0 || list[i].serial < list[room].serial)) room = i;
+        }
+        if (count < kMost) {
+            list[count++] = entry;
+        } else if (room >= 0) {
+            if (list[room].key.capture > forgotten) forgotten = list[room].key.capture;
+            list[room] = entry;
+        } else {
+            overflow = true;
+        }
     }
     unsigned long long pending(const StreamKey& key) const {         // the writer's serial, 0: none
-        for (int i = 0; i < count; ++i) if (list[i].key == key) return list[i].serial;
+        for (int i = 0; i < count; ++i) if (list[i].key == key && !list[i].taken) return list[i].serial;
         return 0;
     }
+    bool elsewhere_in_capture(const StreamKey& key) const {
+        if (key.capture == 0) return false;
+        for (int i = 0; i < count; ++i) if (list[i].key.capture == key.capture && list[i].key.stream != key.stream) return true;
+        return key.capture <= forgotten;
+    }
     void remove(const StreamKey& key, unsigned long long upto) {
-        for (int i = 0; i < count; ++i) if (list[i].key == key && list[i].serial <= upto) { list[i] = list[--count]; return; }
+        for (int i = 0; i < count; ++i)
+            if (list[i].key == key && list[i].serial <= upto) {
+                if (key.capture != 0) list[i].taken = true; else list[i] = list[--count];
+                return;
+            }
     }
     void completed(unsigned long long upto) {                        // all work enqueued before this serial's writer, and it, has ended
         for (int i = 0; i < count;) if (list[i].key.capture == 0 && list[i].serial <= upto) list[i] = list[--count]; else ++i;
@@ -172,7 +196,7 @@ LaunchOrder launch_order(DeviceState* d, void* stream, bool behind_writer = fals
     o.key = stream_key((cudaStream_t)stream);
     std::lock_guard<std::mutex> lock(g_mutex);
     o.writer = d->writers.pending(o.key);
-    if (o.writer != 0) o.serialize = true;
+    if (o.writer != 0 || d->writers.elsewhere_in_capture(o.key)) o.serialize = true;
     return o;
 }
 

@@ -42,6 +42,24 @@ def _captured_edges(stream):
     assert rt.cudaGraphDestroy(graph) == 0
 
 
+@contextlib.contextmanager
+def _capture(rt, stream):
+    """Captures what is enqueued on `stream` and the streams joined to it; yields a list that holds the graph's edges (from, to, type)
+    afterwards."""
+    ptr, size, edges = ctypes.c_void_p, ctypes.c_size_t, []
+    graph, n = ptr(), size()
+    assert rt.cudaStreamBeginCapture(stream, 2) == 0
+    try:
+        yield edges
+    finally:
+        assert rt.cudaStreamEndCapture(stream, ctypes.byref(graph)) == 0
+    assert rt.cudaGraphGetEdges_v2(graph, None, None, None, ctypes.byref(n)) == 0
+    begin, end, data = (ptr * n.value)(), (ptr * n.value)(), (_EdgeData * n.value)()
+    assert rt.cudaGraphGetEdges_v2(graph, begin, end, data, ctypes.byref(n)) == 0
+    edges += [(b, e, d.type) for b, e, d in zip(begin, end, data)]
+    assert rt.cudaGraphDestroy(graph) == 0
+
+
 def _operands(N, K, M, G, bits=4):
     import torch
     torch.manual_seed(N + K + M)
@@ -77,6 +95,59 @@ def test_a_call_on_another_stream_does_not_release_the_reader(M):
     binding.poll_status()
     assert types[0] == FULL
     assert PROGRAMMATIC in types[1:]                      # only the first call behind the writer is held back
+
+
+@pytest.mark.parametrize("M,others", [(1, 0), (5, 0), (16, 0), (300, 0), (1, 70)])
+def test_a_captured_call_joined_behind_a_writer_on_another_stream(M, others):
+    """The quantizer on a second stream of the capture; a call there that waits for it, and one joined behind the quantizer itself by an
+    event, with `others` captures of a writer and its reader begun and ended in between (more than are remembered)."""
+    import torch
+    from paper_2306_00978_b200 import binding
+    rt = ctypes.CDLL("libcudart.so.12")
+    ptr = ctypes.c_void_p
+    N, K, G = (8192, 4096, 128) if M != 5 else (8192, 8320, 128)
+    L = binding.lib()
+    x, qw, sc, zp, y = _operands(N, K, M, G)
+    W = torch.zeros((N, K), dtype=torch.float16, device="cuda")
+    binding.linear(x, qw, sc, zp, N, K, G, out=y)
+    torch.cuda.synchronize()
+    events, streams = [ptr() for _ in range(3)], [ptr() for _ in range(2 + others)]
+    for e in events:
+        assert rt.cudaEventCreateWithFlags(ctypes.byref(e), 2) == 0       # without timing
+    for s in streams:
+        assert rt.cudaStreamCreateWithFlags(ctypes.byref(s), 1) == 0      # non-blocking
+    a, b = streams[:2]
+
+    def quantize(stream):
+        assert L.awq_quantize_pack(W.data_ptr(), None, 0.0, G, qw.data_ptr(), sc.data_ptr(), zp.data_ptr(), N, K, stream) == 0
+
+    def layer(stream):
+        assert L.awq_linear(x.data_ptr(), qw.data_ptr(), sc.data_ptr(), zp.data_ptr(), y.data_ptr(), M, N, K, G, stream) == 0
+
+    def record(event, stream, waits):
+        assert rt.cudaEventRecord(event, stream) == 0 and rt.cudaStreamWaitEvent(waits, event, 0) == 0
+
+    with _capture(rt, a) as edges:
+        record(events[0], a, b)
+        quantize(b)
+        assert rt.cudaEventRecord(events[1], b) == 0
+        layer(b)
+        for s in streams[2:]:
+            with _capture(rt, s):
+                quantize(s)
+                layer(s)
+        assert rt.cudaStreamWaitEvent(a, events[1], 0) == 0
+        layer(a)
+        layer(a)
+        record(events[2], b, a)
+    for s in streams:
+        assert rt.cudaStreamDestroy(s) == 0
+    for e in events:
+        assert rt.cudaEventDestroy(e) == 0
+    binding.poll_status()
+    roots = {f for f, _, _ in edges} - {t for _, t, _ in edges}
+    assert len(roots) == 1                                # the quantizer
+    assert [kind for f, _, kind in edges if f in roots] == [FULL, FULL]
 
 
 def test_the_folded_scale_behind_its_writer():
