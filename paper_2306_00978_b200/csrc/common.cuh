@@ -116,6 +116,8 @@ inline UnitStarts unit_starts(int units, int per_chunk, int blocks) {
 // Kernels that touch memory only after everything in front of them has completed, launched with programmatic stream serialization:
 // their blocks are set up while the kernel in front drains (two calls of the quantizer one behind the other: 28.7 -> 26.4 us each).
 // The launch behind them is let go after the wait, not before: it may rely on what lies in front of this kernel.
+// What they read may be written by a kernel of this kind in front while they are resident: read through L2 (__ldcg, asynchronous
+// copies), never as read-only data (__ldg, const __restrict__).
 __device__ __forceinline__ void start_behind_predecessor() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -33,10 +33,10 @@ struct Alphas {
     float v[kMaxSearchAlphas];
     int mode[kMaxSearchAlphas];
 };
-__global__ void channel_scales_kernel(const float* __restrict__ a, const __grid_constant__ Alphas alphas, float* __restrict__ s, int K) {
+__global__ void channel_scales_kernel(const float* a, const __grid_constant__ Alphas alphas, float* __restrict__ s, int K) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y, mode = alphas.mode[i];
     start_behind_predecessor();
-    if (k < K) s[(size_t)i * K + k] = channel_scale_one(mode == kAlphaZero ? 1.0f : a[k], alphas.v[i], mode);
+    if (k < K) s[(size_t)i * K + k] = channel_scale_one(mode == kAlphaZero ? 1.0f : __ldcg(a + k), alphas.v[i], mode);
 }
 
 // Delta (fp16) and zero point of a group from its min and max; `top` is the largest code
@@ -134,8 +134,8 @@ struct QuantizeCut {
 // MANY (the scale search): `a` is `arrays` arrays of K scales; W is quantized with each and the packed arrays follow one another.
 template <int G, int BITS, bool CLIP, bool SYM, bool MANY = false>
 __global__ void __launch_bounds__(QCfg<G>::kThreads, QCfg<G>::kBlocks)
-quantize_pack_tile_kernel(const __half* __restrict__ W, const float* __restrict__ a, float alpha,
-                          int mode, const float* __restrict__ clip,
+quantize_pack_tile_kernel(const __half* W, const float* a, float alpha,
+                          int mode, const float* clip,
                           uint32_t* __restrict__ qweight, __half* __restrict__ scales,
                           uint8_t* __restrict__ zeros, const __grid_constant__ QuantizeCut cut) {
     using Cfg = QCfg<G>;
@@ -181,10 +181,10 @@ quantize_pack_tile_kernel(const __half* __restrict__ W, const float* __restrict_
             __syncthreads();                               // the scales before have been read
             if (MANY) {
                 for (int i = threadIdx.x; i < arrays * Cfg::kCols; i += Cfg::kThreads)
-                    s_sm[i] = a[(size_t)(array0 + i / Cfg::kCols) * K + kbase + i % Cfg::kCols];
+                    s_sm[i] = __ldcg(a + (size_t)(array0 + i / Cfg::kCols) * K + kbase + i % Cfg::kCols);
             } else {
                 for (int i = threadIdx.x; i < Cfg::kCols; i += Cfg::kThreads)
-                    s_sm[i] = channel_scale_one(mode == kAlphaZero ? 1.0f : a[kbase + i], alpha, mode);
+                    s_sm[i] = channel_scale_one(mode == kAlphaZero ? 1.0f : __ldcg(a + kbase + i), alpha, mode);
             }
             __syncthreads();
         }
@@ -264,7 +264,7 @@ quantize_pack_tile_kernel(const __half* __restrict__ W, const float* __restrict_
             const float wabs = fmaxf(fabsf(mn1), fabsf(mx1));      // largest |w'| of the group (before clipping)
             if (CLIP) {
                 const int gi = G == 64 ? cb * 2 + own_ti : cb;
-                const float r = __ldg(clip + (size_t)(band * 16 + g + 8 * own_row) * (K / G) + gi);
+                const float r = __ldcg(clip + (size_t)(band * 16 + g + 8 * own_row) * (K / G) + gi);
                 mn1 = __fmul_rn(mn1, r);
                 mx1 = __fmul_rn(mx1, r);
             }
@@ -454,7 +454,7 @@ struct ClipSmem {
 
 template <int G>
 __global__ void __launch_bounds__(kClipThreads)
-clip_search_kernel(const __half* __restrict__ W, const float* __restrict__ a, float alpha, int mode,
+clip_search_kernel(const __half* W, const float* a, float alpha, int mode,
                    const __grid_constant__ ClipGrid ratios, float top, float* __restrict__ clip, int N, int K,
                    bool aligned) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -464,7 +464,7 @@ clip_search_kernel(const __half* __restrict__ W, const float* __restrict__ a, fl
     const int tid = threadIdx.x;
     start_behind_predecessor();
 
-    for (int i = tid; i < G; i += kClipThreads) sm.s[i] = channel_scale_one(mode == kAlphaZero ? 1.0f : a[k0 + i], alpha, mode);
+    for (int i = tid; i < G; i += kClipThreads) sm.s[i] = channel_scale_one(mode == kAlphaZero ? 1.0f : __ldcg(a + k0 + i), alpha, mode);
     __syncthreads();
     // w' = w * s (Eq. 3), eight columns of a row per thread; the row's min / max over its kPieces lanes
 #pragma unroll 4
@@ -473,10 +473,10 @@ clip_search_kernel(const __half* __restrict__ W, const float* __restrict__ a, fl
         const __half* src = W + (size_t)(n0 + row) * K + k0 + p * 8;
         __half h[8];
         if (aligned) {
-            *reinterpret_cast<uint4*>(h) = __ldg(reinterpret_cast<const uint4*>(src));
+            *reinterpret_cast<uint4*>(h) = __ldcg(reinterpret_cast<const uint4*>(src));
         } else {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) h[e] = src[e];
+            for (int e = 0; e < 8; ++e) h[e] = __ldcg(src + e);
         }
         float mn = INFINITY, mx = -INFINITY;
         float* dst = sm.w + row * kRowFloats + p * 8;

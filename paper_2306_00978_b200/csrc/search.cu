@@ -95,10 +95,10 @@ sqdiff_partial_kernel(const __half* __restrict__ yq, const float* __restrict__ y
     if (threadIdx.x == 0) partials[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = sum;
 }
 __global__ void __launch_bounds__(256)
-sqdiff_final_kernel(const double* __restrict__ partials, int blocks, double inv_count, float* __restrict__ out) {
+sqdiff_final_kernel(const double* partials, int blocks, double inv_count, float* __restrict__ out) {
     start_behind_predecessor();
     double t = 0.0;
-    for (int i = threadIdx.x; i < blocks; i += 256) t += partials[(size_t)blockIdx.x * blocks + i];
+    for (int i = threadIdx.x; i < blocks; i += 256) t += __ldcg(partials + (size_t)blockIdx.x * blocks + i);
     const double sum = block_sum(t);
     if (threadIdx.x == 0) out[blockIdx.x] = (float)(sum * inv_count);
 }
