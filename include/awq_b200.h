@@ -86,8 +86,7 @@ typedef enum AwqPath {
     AWQ_PATH_GEMM_1SM = 4,      /* the tensor-core kernel with one SM per tile, any M >= 1 */
     AWQ_PATH_GEMV_MID = 5,      /* M <= 8: the chunked matrix-vector kernel: work units of 16 bands
                                    x 1024 input channels, the unit's slice of x in shared memory, one
-                                   band per warp; 9 <= M <= 32, and where awq_linear takes it
-                                   below: the stream kernel; needs a
+                                   band per warp; 9 <= M <= 32: the stream kernel; needs a
                                    workspace of awq_workspace_bytes (fp32 partial sums per chunk of K) */
     AWQ_PATH_GEMM_SKINNY = 6    /* the stream kernel, M <= 64, N a multiple of 128: pairs of SMs
                                    (cta_group::2, 256 channels x up to 128 tokens per tile), the tiles' K

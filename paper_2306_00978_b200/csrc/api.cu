@@ -423,8 +423,7 @@ static int linear_path(const void* x, const void* qweight, const void* scales, c
     }
     DeviceState* d;
     if (int rc = device_state(&d)) return rc;
-    int without_stream = path;               // taken where the stream kernel cannot be launched
-    bool may_fall_back = automatic;
+    int without_stream = path;               // (automatic) taken where the stream kernel cannot be launched
     if (automatic && stream_kernel_preferred(M, N, K, group, d->sms)) {
         const size_t need = gemm_stream_workspace_bytes(M, d->sms);
         std::lock_guard<std::mutex> lock(g_mutex);
@@ -432,21 +431,16 @@ static int linear_path(const void* x, const void* qweight, const void* scales, c
     }
     if (automatic && path == AWQ_PATH_GEMV && mid_kernel_preferred(M, N, K) && gemv_mid_applies(M, N, K, group, d->sms)) {
         std::lock_guard<std::mutex> lock(g_mutex);
-        if (d->workspace_bytes >= gemv_mid_workspace_bytes(M, N, K)) path = AWQ_PATH_GEMV_MID;
+        if (d->workspace_bytes >= gemv_mid_workspace_bytes(M, N, K)) {
+            path = without_stream = AWQ_PATH_GEMV_MID;
+            if (stream_beats_chunked(M, N, K, group) && d->workspace_bytes >= gemm_stream_workspace_bytes(M, d->sms)) path = AWQ_PATH_GEMM_SKINNY;
+        }
     }
     if (automatic && path == AWQ_PATH_GEMM) {          // (asked for by name it is the prefill kernels)
         const AwqLinearProblem one = {qweight, scales, zeros, y, N};
         if (stream_beats_prefill(d, &one, 1, M, K, group)) path = AWQ_PATH_GEMM_SKINNY;
     }
     if (path == AWQ_PATH_GEMV_MID && M > 8 && gemm_stream_applies(M, N, K, group)) path = AWQ_PATH_GEMM_SKINNY;
-    if (path == AWQ_PATH_GEMV_MID && stream_beats_chunked(M, N, K, group) && gemv_mid_applies(M, N, K, group, d->sms)) {
-        std::lock_guard<std::mutex> lock(g_mutex);
-        if (d->workspace_bytes >= gemm_stream_workspace_bytes(M, d->sms) && d->workspace_bytes >= gemv_mid_workspace_bytes(M, N, K)) {
-            path = AWQ_PATH_GEMM_SKINNY;
-            without_stream = AWQ_PATH_GEMV_MID;
-            may_fall_back = true;
-        }
-    }
     const cudaStream_t st = (cudaStream_t)stream;
     const LaunchOrder order = launch_order(d, stream, behind_writer);
     if (path == AWQ_PATH_GEMM_SKINNY) {
@@ -460,7 +454,7 @@ static int linear_path(const void* x, const void* qweight, const void* scales, c
         const GemvMatrix one = {qweight, scales, zeros, y, N};
         const cudaError_t e = order.launched(launch_gemm_stream(x, &one, 1, M, K, group, nullptr, ws, d->status_word,
                                                                 d->sms, order.serialize, st));
-        if (!may_fall_back || e != cudaErrorNotSupported) return note_cuda(e);
+        if (!automatic || e != cudaErrorNotSupported) return note_cuda(e);
         path = without_stream;               // no pair of SMs to be had (a partition of the device): nothing was launched
     }
     if (path == AWQ_PATH_GEMV_MID) {

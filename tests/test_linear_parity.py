@@ -389,15 +389,15 @@ def test_chunked_matrix_vector_kernel_up_to_8_tokens(N, K, M, G):
     assert np.array_equal(y.view(np.uint16), y2.view(np.uint16))
 
 
-@pytest.mark.parametrize("N,K,M,mid", [
-    (5504, 12288, 2, True), (5504, 12160, 2, False),        # 2 tokens: rows of at least 12288
-    (8192, 8320, 3, True), (8192, 8064, 4, False),          # 3, 4 tokens: at least 2^26 weights
-    (4096, 8320, 5, True), (4096, 8064, 8, False),          # 5 .. 8 tokens: at least 2^25 weights
-    (16384, 4096, 8, False),                                # rows of at most 4096: the band kernel
+@pytest.mark.parametrize("N,K,M,kernel", [
+    (5504, 12288, 2, "stream"), (9856, 12288, 2, "chunked"), (5504, 12160, 2, "band"),       # 2 tokens: rows of at least 12288
+    (8192, 8320, 3, "chunked"), (8192, 8064, 4, "band"),                                     # 3, 4 tokens: at least 2^26 weights
+    (4096, 8320, 5, "stream"), (6784, 8320, 5, "chunked"), (4096, 8064, 8, "band"),          # 5 .. 8 tokens: at least 2^25 weights
+    (16384, 4096, 8, "band"),                                                                # rows of at most 4096: the band kernel
 ])
-def test_auto_dispatch_up_to_8_tokens(N, K, M, mid):
-    """awq_linear up to 8 tokens on many output rows: the chunked matrix-vector kernel on long rows, else the band
-    kernel, whose sums are formed in another order."""
+def test_auto_dispatch_up_to_8_tokens(N, K, M, kernel):
+    """awq_linear up to 8 tokens on many output rows: the chunked matrix-vector kernel on long rows, the stream kernel where they
+    are 5/4 of the outputs and more, else the band kernel; each forms its sums in another order."""
     import torch
     from paper_2306_00978_b200 import binding
     qw, sc, zp, x = _random_operands(N, K, M, 128, N + K + M)
@@ -405,5 +405,7 @@ def test_auto_dispatch_up_to_8_tokens(N, K, M, mid):
     chunked = binding.linear(x, qw, sc, zp, N, K, 128, path=binding.PATH_GEMV_MID)
     band = binding.linear(x, qw, sc, zp, N, K, 128, path=binding.PATH_GEMV)
     binding.poll_status()
-    assert not torch.equal(chunked, band)
-    assert torch.equal(auto, chunked if mid else band)
+    stream = binding.linear(x, qw, sc, zp, N, K, 128, path=binding.PATH_GEMM_SKINNY)
+    binding.poll_status()
+    forced = {"chunked": chunked, "band": band, "stream": stream}
+    assert [name for name, y in forced.items() if torch.equal(auto, y)] == [kernel]

@@ -48,6 +48,14 @@ if sys.argv[1] == "none":
         binding.poll_status()
         assert torch.equal(both[0], both[1]) and not both[2].any() and not both[3].any()
         assert_parity(both[0].cpu().numpy(), case.y_ref(), f"several, M={M}")
+    N, K, M = 4096, 8320, 5                  # few tokens on long rows: the chunked kernel and the one that adds its parts
+    qw = torch.randint(0, 256, (N * K // 2,), dtype=torch.uint8, device="cuda")
+    sc, zp = torch.rand((N // 16, K // G, 16), device="cuda").half(), torch.randint(0, 256, (N // 32, K // G, 16), dtype=torch.uint8, device="cuda")
+    long_x = torch.randn((M, K), device="cuda").half()
+    binding.linear(long_x, qw, sc, zp, N, K, G)
+    y, n = launches(lambda: binding.linear(long_x, qw, sc, zp, N, K, G))
+    assert n == 2 and torch.equal(y, binding.linear(long_x, qw, sc, zp, N, K, G, path=binding.PATH_GEMV_MID))
+    N, K = 512, 1024
     try:
         binding.linear(x[:16], *packed, N, K, G, path=binding.PATH_GEMM_SKINNY)
         raise SystemExit("a kernel asked for by name must not be replaced")
