@@ -768,7 +768,7 @@ cudaError_t st_launch(const CUtensorMap& xmap, const StMats& mats, const float* 
     cfg.blockDim = dim3(128);
     cfg.dynamicSmemBytes = 0;
     cfg.attrs = attr + 1;
-    cfg.numAttrs = TB == kStBlockBytes ? 1 : 0;
+    cfg.numAttrs = 1;
     auto* reduce = per == 1 ? stream_reduce_kernel<1> : per == 2 ? stream_reduce_kernel<2> : stream_reduce_kernel<4>;
     e = cudaLaunchKernelEx(&cfg, reduce, cut, (const float*)partial);
     if (e != cudaSuccess) return e;
@@ -862,7 +862,7 @@ cudaError_t launch_gemm_stream(const void* x, const GemvMatrix* mats, int count,
     cut.total = cut.tiles * cut.nks;
     if (bits == 3) {                                     // (up to 64 tokens, nothing folded in)
         if (inv_s || cls > 64) return cudaErrorInvalidValue;
-#define AWQ_ST_LAUNCH3(GG, BNN) return st_launch<GG, BNN, false, 384>(xmap, sm, inv_s, cut, workspace, status_word, sms, true, st)
+#define AWQ_ST_LAUNCH3(GG, BNN) return st_launch<GG, BNN, false, 384>(xmap, sm, inv_s, cut, workspace, status_word, sms, serialize, st)
         if (group == 128) { if (cls == 16) AWQ_ST_LAUNCH3(128, 16); if (cls == 32) AWQ_ST_LAUNCH3(128, 32); AWQ_ST_LAUNCH3(128, 64); }
         if (cls == 16) AWQ_ST_LAUNCH3(64, 16); if (cls == 32) AWQ_ST_LAUNCH3(64, 32); AWQ_ST_LAUNCH3(64, 64);
 #undef AWQ_ST_LAUNCH3

@@ -175,7 +175,9 @@ def test_the_folded_scale_behind_its_writer():
 
 
 @pytest.mark.parametrize("M", [16, 300])
-def test_int3_expansion_and_its_reader_beside_another_thread(M):
+def test_int3_calls_beside_another_thread(M):
+    """At 16 tokens the stream kernel reads the 3-bit storage, plainly ordered, and the kernel that adds its parts may be set up meanwhile; at
+    300 the storage is expanded, and expansion and reader are plainly ordered."""
     import torch
     from paper_2306_00978_b200 import binding
     N, K, G, calls = 2048, 2048, 128, 300
@@ -204,9 +206,10 @@ def test_int3_expansion_and_its_reader_beside_another_thread(M):
         stop.set()
         thread.join()
     binding.poll_status()
-    per_call = (len(types) + 1) // calls                  # the expansion, the layer's kernel, and the one that adds parts if there is one
+    per_call = (len(types) + 1) // calls                  # the expansion if there is one, the layer's kernel, and the one that adds parts if there is one
     assert per_call * calls == len(types) + 1 and per_call >= 2
-    assert [types[i * per_call] for i in range(calls)] == [FULL] * calls
+    assert types[per_call - 1::per_call] == [FULL] * (calls - 1)          # from call to call
+    assert types[::per_call] == [PROGRAMMATIC if M == 16 else FULL] * calls
 
 
 @pytest.mark.parametrize("widths,K,M,G", [((4096, 2304), 5248, 4, 128), ((2176, 4352), 8192, 8, 64)])
