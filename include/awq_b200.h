@@ -261,8 +261,8 @@ int awq_linear_scaled_needs_scratch(int M, int N, int K, int group);
  * (M <= 8 and N / 16 not far below the SM count) it streams the 3-bit array itself, 25 % fewer
  * weight bytes than the 4-bit layout; so does the stream kernel up to 64 tokens, where awq_linear takes it.  Other shapes (split-K
  * and prefill kernels read the 4-bit layout) are first expanded into qweight_scratch (device, awq_qweight_bytes(N, K) bytes,
- * caller-owned; may be NULL when the band kernel applies, else AWQ_ERR_NULL_POINTER) and run as
- * awq_linear.  Results equal awq_linear on the expanded array bit for bit where the same kernel runs.
+ * caller-owned; may be NULL where one of those two serves the call - the stream kernel needs a registered workspace of
+ * awq_workspace_bytes(M, N, K, group) - else AWQ_ERR_NULL_POINTER, and nothing is launched) and run as awq_linear.  Results equal awq_linear on the expanded array bit for bit where the same kernel runs.
  */
 size_t awq_qweight_bytes_int3(int N, int K);
 int awq_pack_int3(const void* qweight, void* qweight3, int N, int K, void* stream);

@@ -320,11 +320,12 @@ def linear_int3(x: torch.Tensor, qweight3: torch.Tensor, scales: torch.Tensor, z
     M = x.shape[0]
     y = out if out is not None else torch.empty((M, N), dtype=torch.float16, device=x.device)
     ensure_workspace(workspace_bytes(M, N, K, group))
-    if scratch is None:
+    args = (_dev(x, torch.float16, "x"), _dev(qweight3, torch.uint8, "qweight3"), _dev(scales, torch.float16, "scales"),
+            _dev(zeros, torch.uint8, "zeros"), _dev(y, torch.float16, "y"))
+    rc = lib().awq_linear_int3(*args, None if scratch is None else scratch.data_ptr(), M, N, K, int(group), _stream())
+    if rc == 1 and scratch is None:                           # (refused before anything was launched: it needs the expansion)
         scratch = torch.empty(N * K // 2, dtype=torch.uint8, device=x.device)
-    rc = lib().awq_linear_int3(_dev(x, torch.float16, "x"), _dev(qweight3, torch.uint8, "qweight3"),
-                               _dev(scales, torch.float16, "scales"), _dev(zeros, torch.uint8, "zeros"),
-                               _dev(y, torch.float16, "y"), scratch.data_ptr(), M, N, K, int(group), _stream())
+        rc = lib().awq_linear_int3(*args, scratch.data_ptr(), M, N, K, int(group), _stream())
     _check(rc, "awq_linear_int3")
     return y
 

@@ -719,7 +719,6 @@ int awq_linear_int3(const void* x, const void* qweight3, const void* scales, con
         return note_cuda(order.launched(launch_gemv_band(x, &one, 1, M, K, group, d->status_word, d->sms, order.serialize,
                                                          (cudaStream_t)stream, nullptr, 3)));
     }
-    if (!qweight_scratch) return AWQ_ERR_NULL_POINTER;
     // Up to 64 tokens, where awq_linear takes the stream kernel, that kernel reads the 3-bit storage as it is (expanding and then it / it
     // alone, us: 4096 -> 11008 at 16 / 64 tokens 17.2 / 21.2 against 12.7 / 16.5, 4096 -> 4096 at 16 11.3 against 9.4, 8192 -> 28672 at 16
     // 64.0 against 33.9).  Its launches are plainly ordered, as an expansion's and its reader's are, since the packed words
@@ -739,6 +738,7 @@ int awq_linear_int3(const void* x, const void* qweight3, const void* scales, con
         }
     }
     // every other kernel reads the 4-bit layout: expand first (one more launch), then the plain call
+    if (!qweight_scratch) return AWQ_ERR_NULL_POINTER;
     if (int rc = awq_unpack_int3(qweight3, qweight_scratch, N, K, stream)) return rc;
     return linear_path(x, qweight_scratch, scales, zeros, y, M, N, K, group, AWQ_PATH_AUTO, stream, true);
 }

@@ -135,7 +135,7 @@ PyObject* linear_int3(PyObject*, PyObject* const* a, Py_ssize_t n) {
     at::Tensor scratch;
     int rc = 1;
     void* stream = current_stream(c.dev);
-    for (int pass = c.M <= 8 ? 0 : 1; pass < 2 && rc == 1; ++pass) {
+    for (int pass = c.M <= 64 ? 0 : 1; pass < 2 && rc == 1; ++pass) {
         if (pass == 1) scratch = at::empty({(int64_t)c.N * c.K / 2}, c.qweight->options());
         void* s = pass == 1 ? scratch.mutable_data_ptr() : nullptr;
         Py_BEGIN_ALLOW_THREADS

@@ -28,6 +28,46 @@ def test_same_bits_as_on_the_expanded_array(N, K, M, G):
     scratch = torch.full((N * K // 2,), 0xA5, dtype=torch.uint8, device="cuda")
     want = binding.linear(x, qw, sc, zp, N, K, G)
     got = binding.linear_int3(x, qw3, sc, zp, N, K, G, scratch=scratch)
+    alone = binding.linear_int3(x, qw3, sc, zp, N, K, G)
     binding.poll_status()
-    assert torch.equal(got, want)
+    assert torch.equal(got, want) and torch.equal(alone, want)
     assert bool((scratch == 0xA5).all())                 # nothing was expanded
+
+
+def test_scratch_only_where_the_storage_is_expanded():
+    import numpy as np
+    import torch
+    from paper_2306_00978_b200 import binding
+    N, K, G = 2048, 2048, 128
+    L = binding.lib()
+    qw3 = torch.randint(0, 256, (N * K // 8 * 3,), dtype=torch.uint8, device="cuda")
+    sc, zp = torch.rand((N // 16, K // G, 16), device="cuda").half(), torch.zeros((N // 32, K // G, 16), dtype=torch.uint8, device="cuda")
+    scratch = torch.empty(N * K // 2, dtype=torch.uint8, device="cuda")
+
+    def call(M, given):
+        x, y = torch.ones((M, K), device="cuda").half(), torch.empty((M, N), dtype=torch.float16, device="cuda")
+        n0 = binding.launch_count()
+        rc = L.awq_linear_int3(x.data_ptr(), qw3.data_ptr(), sc.data_ptr(), zp.data_ptr(), y.data_ptr(),
+                               scratch.data_ptr() if given else None, M, N, K, G, torch.cuda.current_stream().cuda_stream)
+        assert rc == 0 or binding.launch_count() == n0
+        return rc
+
+    for M in (8, 9, 64, 65):
+        binding.ensure_workspace(binding.workspace_bytes(M, N, K, G))
+    ws = binding._workspace[torch.cuda.current_device()]
+    assert [call(M, False) for M in (8, 9, 64, 65)] == [0, 0, 0, 1]
+    for M, more in ((9, False), (64, False), (65, True)):
+        for group in (G, np.int64(G)):                       # the native call and the one through ctypes
+            x = torch.ones((M, K), device="cuda").half()
+            torch.cuda.synchronize()
+            torch.cuda.reset_peak_memory_stats()
+            before = torch.cuda.memory_allocated()
+            binding.linear_int3(x, qw3, sc, zp, N, K, group)
+            assert (torch.cuda.max_memory_allocated() - before >= N * K // 2) == more
+    binding.poll_status()
+    try:                                                     # without a workspace for its parts the stream kernel is not taken
+        assert L.awq_set_workspace(None, 0) == 0
+        assert call(9, False) == 1 and call(9, True) == 0
+        binding.poll_status()
+    finally:
+        assert L.awq_set_workspace(ws.data_ptr(), ws.numel()) == 0
