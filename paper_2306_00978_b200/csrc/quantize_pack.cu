@@ -6,6 +6,7 @@
 // blocks, which is exactly the data of the two 16-byte packed pieces it writes.  Every
 // rounding point is an explicit IEEE operation (no contraction); the per-weight division is
 // replaced by a multiplication only where that provably rounds to the same integer.
+#include <algorithm>
 #include <mutex>
 #include <type_traits>
 
@@ -664,13 +665,15 @@ static cudaError_t launch_quantize(const __half* W, const float* a, float alpha,
     cut.col_blocks = K / Cfg::kCols;
     cut.band_steps = N / 16 / Cfg::kBands;             // (N is a multiple of 128)
     cut.arrays = arrays;
-    const int resident = sms * Cfg::kBlocks;
+    // blocks that can be resident with `per` arrays of scales in shared memory: of 228 KB per SM, a block keeps 1.5 KB beside its dynamic part
+    auto resident_with = [&](int per) { return sms * std::min(Cfg::kBlocks, 228 * 1024 / (tiles + per * Cfg::kCols * 4 + 1536)); };
     const long long tiles_all = (long long)cut.col_blocks * cut.band_steps;
     int parts = 1;
     if (MANY) {
         double least = 0.0;
         for (int p = 1; p <= 4 && p <= arrays; ++p) {
             const int per = (arrays + p - 1) / p, real = (arrays + per - 1) / per;
+            const int resident = resident_with(per);
             const double rounds = (double)((tiles_all * real + resident - 1) / resident) * (per + 0.5);    // (an item's own start: half an array)
             if (p == 1 || rounds < least) { least = rounds; parts = real; }
         }
@@ -679,7 +682,7 @@ static cudaError_t launch_quantize(const __half* W, const float* a, float alpha,
     const long long items = tiles_all * parts;
     if (items > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
     cut.items = (int)items;
-    const int blocks = items < resident ? (int)items : resident;
+    const int resident = resident_with(cut.per_part), blocks = items < resident ? (int)items : resident;
     cut.share = cut.items / blocks;
     cut.longer = cut.items % blocks;
     e = launch_behind(kernel, blocks, Cfg::kThreads, (size_t)(tiles + cut.per_part * Cfg::kCols * 4), st, W, a, alpha, mode, clip, qweight, scales, zeros, cut);

@@ -95,6 +95,8 @@ def test_a_search_near_the_memory_limit(monkeypatch):
 @pytest.mark.parametrize("N,K,M,G,n", [
     (256, 128, 65, 64, 3),          # all points in one launch, one token past a tile
     (512, 1152, 97, 128, 64),       # the longest list, rows padded to 128
+    (1536, 2048, 24, 128, 64),      # the quantizer's blocks hold so many arrays of scales that three of them fit an SM
+    (2048, 2048, 24, 128, 64),      # and would, but parts of half the arrays fill the SMs better
     (384, 640, 200, 128, 5),        # an odd number of 128-channel slabs: one launch per point
     (512, 1024, 20, 64, 4),         # few tokens: the layer's own kernel per point
     (4096, 8192, 900, 128, 11),     # two batches, of six and five
