@@ -389,7 +389,7 @@ quantize_pack_tile_kernel(const __half* W, const float* a, float alpha,
 // error is written to clip[n][group].  The choice decides integer codes downstream, so the error
 // is defined operation by operation: dequant = (q - z) * Delta (one fp32 multiply), e = dequant -
 // w', err += e * e in fp32 over ascending k (no contraction), a NaN error counts as +inf.
-// grid = (K / G, N / 64), block = 256: one group of columns of 64 rows, its w' in shared memory; a thread takes one (row, two
+// grid = (K / G, N / 64), block = 256 or 128: one group of columns of 64 rows, its w' in shared memory; a thread takes one (row, J
 // ratios) item at a time.
 // First an estimate of every (row, ratio)'s error, in steps of Delta and in no particular order: t = w' / Delta by
 // w' * (1 / Delta), its nearest integer, clamped, f = t - that, S = sum of f * f, two elements per packed fp32 instruction
@@ -406,7 +406,7 @@ quantize_pack_tile_kernel(const __half* W, const float* a, float alpha,
 // here they take 15.  4096 -> 4096 with 20 ratios: 94 us, of which 18 are loads, parameters and the choice (every ratio
 // evaluated as defined, 9 packed or min / max instructions per pair: 125 us).  128, 192, 320 threads: 103, 101, 96 us; one ratio at a
 // time 95, four 99; clamping by the saturation of a scalar multiply-add 91 to 99, at a wider margin.
-constexpr int kClipRows = 64, kClipThreads = 256;
+constexpr int kClipRows = 64;
 struct ClipGrid {
     float r[kMaxClipRatios];
     int n;
@@ -453,8 +453,9 @@ struct ClipSmem {
     float s[G];
 };
 
-template <int G>
-__global__ void __launch_bounds__(kClipThreads)
+// THREADS per block, items of J ratios of a row
+template <int G, int J, int THREADS>
+__global__ void __launch_bounds__(THREADS)
 clip_search_kernel(const __half* W, const float* a, float alpha, int mode,
                    const __grid_constant__ ClipGrid ratios, float top, float* __restrict__ clip, int N, int K,
                    bool aligned) {
@@ -465,11 +466,11 @@ clip_search_kernel(const __half* W, const float* a, float alpha, int mode,
     const int tid = threadIdx.x;
     start_behind_predecessor();
 
-    for (int i = tid; i < G; i += kClipThreads) sm.s[i] = channel_scale_one(mode == kAlphaZero ? 1.0f : __ldcg(a + k0 + i), alpha, mode);
+    for (int i = tid; i < G; i += THREADS) sm.s[i] = channel_scale_one(mode == kAlphaZero ? 1.0f : __ldcg(a + k0 + i), alpha, mode);
     __syncthreads();
     // w' = w * s (Eq. 3), eight columns of a row per thread; the row's min / max over its kPieces lanes
 #pragma unroll 4
-    for (int i = tid; i < kClipRows * kPieces; i += kClipThreads) {
+    for (int i = tid; i < kClipRows * kPieces; i += THREADS) {
         const int row = i / kPieces, p = i % kPieces;
         const __half* src = W + (size_t)(n0 + row) * K + k0 + p * 8;
         __half h[8];
@@ -506,14 +507,14 @@ clip_search_kernel(const __half* W, const float* a, float alpha, int mode,
         rd = __frcp_rn(d);
         tmax = __fmul_rn(fmaxf(fabsf(mm.x), fabsf(mm.y)), rd);
     };
-    const int np = (nr + 1) / 2;
-    for (int item = tid; item < kClipRows * np; item += kClipThreads) {
-        const int row = item / np, i0 = 2 * (item - row * np);
+    const int np = (nr + J - 1) / J;
+    for (int item = tid; item < kClipRows * np; item += THREADS) {
+        const int row = item / np, i0 = J * (item - row * np);
         const f32x2 big = pack2(12582912.0f, 12582912.0f);
-        float d[2], tmax[2], lo[2], hi[2];
-        f32x2 rd2[2], sum[2];
+        float d[J], tmax[J], lo[J], hi[J];
+        f32x2 rd2[J], sum[J];
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
+        for (int j = 0; j < J; ++j) {
             float z, rd;
             params(sm.mm[row], ratios.r[min(i0 + j, nr - 1)], d[j], z, rd, tmax[j]);
             rd2[j] = pack2(rd, rd);
@@ -525,7 +526,7 @@ clip_search_kernel(const __half* W, const float* a, float alpha, int mode,
         constexpr int E = 4;                                     // pairs of elements at a time
 #pragma unroll 2
         for (int k = 0; k < G; k += 2 * E) {
-            f32x2 w[E], u[2][E];
+            f32x2 w[E], u[J][E];
 #pragma unroll
             for (int e = 0; e < E; e += 2) {
                 const float4 w4 = *reinterpret_cast<const float4*>(wg + k + 2 * e);
@@ -535,11 +536,11 @@ clip_search_kernel(const __half* W, const float* a, float alpha, int mode,
 #pragma unroll
             for (int e = 0; e < E; ++e)
 #pragma unroll
-                for (int j = 0; j < 2; ++j) u[j][e] = fma2(w[e], rd2[j], big);       // rounded to an integer in the sum
+                for (int j = 0; j < J; ++j) u[j][e] = fma2(w[e], rd2[j], big);       // rounded to an integer in the sum
 #pragma unroll
             for (int e = 0; e < E; ++e)
 #pragma unroll
-                for (int j = 0; j < 2; ++j) {
+                for (int j = 0; j < J; ++j) {
                     float u0, u1;
                     unpack2(u[j][e], u0, u1);
                     u[j][e] = pack2(fminf(fmaxf(u0, lo[j]), hi[j]), fminf(fmaxf(u1, lo[j]), hi[j]));
@@ -547,14 +548,14 @@ clip_search_kernel(const __half* W, const float* a, float alpha, int mode,
 #pragma unroll
             for (int e = 0; e < E; ++e)
 #pragma unroll
-                for (int j = 0; j < 2; ++j) u[j][e] = fma2(w[e], rd2[j], sub2(big, u[j][e]));
+                for (int j = 0; j < J; ++j) u[j][e] = fma2(w[e], rd2[j], sub2(big, u[j][e]));
 #pragma unroll
             for (int e = 0; e < E; ++e)
 #pragma unroll
-                for (int j = 0; j < 2; ++j) sum[j] = fma2(u[j][e], u[j][e], sum[j]);
+                for (int j = 0; j < J; ++j) sum[j] = fma2(u[j][e], u[j][e], sum[j]);
         }
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
+        for (int j = 0; j < J; ++j) {
             if (i0 + j >= nr) break;
             float s0, s1;
             unpack2(sum[j], s0, s1);
@@ -565,12 +566,12 @@ clip_search_kernel(const __half* W, const float* a, float alpha, int mode,
         }
     }
     __syncthreads();
-    for (int item = tid; item < kClipRows * nr; item += kClipThreads) {
+    for (int item = tid; item < kClipRows * nr; item += THREADS) {
         const int row = item / nr, i = item - row * nr;
         if (sm.err[row * (kMaxClipRatios + 1) + i] <= __int_as_float(sm.least[row])) atomicAdd(&sm.left[row], 1);
     }
     __syncthreads();
-    for (int item = tid; item < kClipRows * nr; item += kClipThreads) {
+    for (int item = tid; item < kClipRows * nr; item += THREADS) {
         const int row = item / nr, i = item - row * nr;
         float* e = sm.err + row * (kMaxClipRatios + 1) + i;
         float err = INFINITY;
@@ -727,7 +728,7 @@ cudaError_t launch_quantize_pack(const __half* W, const float* a, float alpha, i
     return cudaErrorInvalidValue;
 }
 
-template <int G>
+template <int G, int J, int THREADS>
 static cudaError_t launch_clip(const __half* W, const float* a, float alpha, int mode, const ClipGrid& ratios, float top,
                                float* clip, int N, int K, bool aligned, cudaStream_t st) {
     static bool done[64] = {};
@@ -735,11 +736,11 @@ static cudaError_t launch_clip(const __half* W, const float* a, float alpha, int
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (!done[dev & 63]) {
-        e = cudaFuncSetAttribute(clip_search_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClipSmem<G>));
+        e = cudaFuncSetAttribute(clip_search_kernel<G, J, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ClipSmem<G>));
         if (e != cudaSuccess) return e;
         done[dev & 63] = true;
     }
-    e = launch_behind(clip_search_kernel<G>, dim3(K / G, N / kClipRows), kClipThreads, sizeof(ClipSmem<G>), st, W, a, alpha, mode, ratios, top, clip, N, K, aligned);
+    e = launch_behind(clip_search_kernel<G, J, THREADS>, dim3(K / G, N / kClipRows), THREADS, sizeof(ClipSmem<G>), st, W, a, alpha, mode, ratios, top, clip, N, K, aligned);
     if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
@@ -754,8 +755,13 @@ cudaError_t launch_clip_search(const __half* W, const float* a, float alpha, int
     const int mode = (int)alpha_mode(alpha);
     const float top = (float)((1 << bits) - 1);
     const bool aligned = (reinterpret_cast<uintptr_t>(W) & 15u) == 0;   // rows are multiples of 256 bytes
-    return group == 128 ? launch_clip<128>(W, a, alpha, mode, grid_r, top, clip, N, K, aligned, st)
-                        : launch_clip<64>(W, a, alpha, mode, grid_r, top, clip, N, K, aligned, st);
+    // Groups of 64 and up to four ratios: smaller blocks, which the items of one or two ratios fill (11008 x 4096, us, against 256 threads and two
+    // ratios an item: 1 ratio 72.1 -> 59.9, 2: 76.1 -> 64.5, 3: 83.4 -> 73.9, 4: 85.7 -> 76.0; groups of 128, whose rows keep a thread busy for
+    // twice as long: 63.0 -> 75.3, 65.9 -> 80.3, 71.1 -> 86.8, 72.6 -> 87.7).
+    if (group == 64 && n_ratios <= 2) return launch_clip<64, 1, 128>(W, a, alpha, mode, grid_r, top, clip, N, K, aligned, st);
+    if (group == 64 && n_ratios <= 4) return launch_clip<64, 2, 128>(W, a, alpha, mode, grid_r, top, clip, N, K, aligned, st);
+    return group == 128 ? launch_clip<128, 2, 256>(W, a, alpha, mode, grid_r, top, clip, N, K, aligned, st)
+                        : launch_clip<64, 2, 256>(W, a, alpha, mode, grid_r, top, clip, N, K, aligned, st);
 }
 
 cudaError_t launch_unpack(const uint32_t* qweight, const __half* scales, const uint8_t* zeros,

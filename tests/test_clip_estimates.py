@@ -31,7 +31,8 @@ def _groups(N, K, G, seed):
 
 @pytest.mark.parametrize("N,K,G,bits", [(256, 1024, 128, 4), (256, 1024, 64, 3), (1024, 4096, 128, 3)])
 @pytest.mark.parametrize("ratios", [[1.0], [1.0, 0.9, 0.9, 1.0, 0.8, 0.8, 0.8], [1.0 - 0.5 * i / 32 for i in range(32)],
-                                    [1.0 - 1e-6 * i for i in range(9)], [0.5 + 0.05 * i for i in range(11)]], ids=len)
+                                    [1.0 - 1e-6 * i for i in range(9)], [0.5 + 0.05 * i for i in range(11)],
+                                    [0.9, 1.0], [0.7, 0.85, 0.85], [1.0, 1.0 - 1e-6, 0.8, 0.8], [0.6, 0.7, 0.8, 0.9, 1.0]], ids=len)
 @pytest.mark.parametrize("scaled", [False, True])
 def test_ratios_are_the_defined_ones(N, K, G, bits, ratios, scaled):
     from paper_2306_00978_b200 import binding
