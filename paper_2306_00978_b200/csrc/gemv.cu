@@ -142,9 +142,10 @@ __device__ __forceinline__ void tile_sums_of_x(const __half* __restrict__ x, flo
 }
 
 // =========================================================================== band kernel
-// With x in shared memory a block asks for three stages of weights and for the others of the ring as those land: asked for at once, they queue
-// in front of x and of other blocks' first stages (8192 -> 8192 at one token 9.27 -> 9.05 us, 8192 -> 28672 25.0 -> 24.8, 5120 -> 5120 at two
-// 6.53 -> 6.43; with two stages 8.83, 24.6 and 6.34, but 11008 -> 4096 at one 7.10 -> 7.18).
+// With x in shared memory and groups of 128 a block asks for three stages of weights and for the others of the ring as those land: asked for at
+// once, they queue in front of x and of other blocks' first stages (8192 -> 8192 at one token 9.39 -> 9.13 us, 8192 -> 16384 14.0 -> 13.8,
+// 5120 -> 5120 at two 6.77 -> 6.66; with two stages more, but 11008 -> 4096 at one token 1 % slower).  With groups of 64 it costs, why is not known
+// (8192 -> 8192 at one and two tokens 9.81 -> 9.88 and 10.28 -> 10.40, 5120 -> 13824 11.06 -> 11.14).
 constexpr int kBandAhead = 3;
 constexpr int kBandThreads = kMathThreads + 96;        // + weight-copy warp + flush warp + x-copy warp
 
@@ -430,7 +431,7 @@ gemv_band_kernel(const BandProblems probs, const __half* __restrict__ x, int M, 
                 const uint32_t dst = sbase + stage * (uint32_t)lay.stage_bytes;
                 const uint32_t bar = bars + 8u * stage;
                 if (lane == 0) {
-                    if (XSM && ahead >= kBandAhead && ahead < S) mbar_wait_relaxed(bars + 8u * (uint32_t)(ahead - kBandAhead), 0u, ctl);
+                    if (XSM && G == 128 && ahead >= kBandAhead && ahead < S) mbar_wait_relaxed(bars + 8u * (uint32_t)(ahead - kBandAhead), 0u, ctl);
                     ++ahead;
                     mbar_wait_relaxed(bars + 64u + 8u * stage, phase ^ 1u, ctl);
                     mbar_arrive_expect_tx(bar, (uint32_t)(nt * TB + ngr * 48 + ((XREG || XSM) ? 0 : M * nt * 128)));
