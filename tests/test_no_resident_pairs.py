@@ -55,6 +55,12 @@ if sys.argv[1] == "none":
     binding.linear(long_x, qw, sc, zp, N, K, G)
     y, n = launches(lambda: binding.linear(long_x, qw, sc, zp, N, K, G))
     assert n == 2 and torch.equal(y, binding.linear(long_x, qw, sc, zp, N, K, G, path=binding.PATH_GEMV_MID))
+    N, K, M = 2048, 1024, 16                 # 3-bit storage: expanded, and the prefill kernel behind it
+    qw3 = torch.randint(0, 256, (N * K // 8 * 3,), dtype=torch.uint8, device="cuda")
+    sc, zp = torch.rand((N // 16, K // G, 16), device="cuda").half(), torch.randint(0, 8, (N // 32, K // G, 16), dtype=torch.uint8, device="cuda")
+    some_x = torch.randn((M, K), device="cuda").half()
+    y, n = launches(lambda: binding.linear_int3(some_x, qw3, sc, zp, N, K, G))
+    assert n == 2 and torch.equal(y, binding.linear(some_x, binding.unpack_int3(qw3, N, K), sc, zp, N, K, G))
     N, K = 512, 1024
     try:
         binding.linear(x[:16], *packed, N, K, G, path=binding.PATH_GEMM_SKINNY)

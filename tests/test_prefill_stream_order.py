@@ -1,5 +1,5 @@
-"""The SM-pair prefill kernel copies packed weights before the work in front of it in the stream has completed: calls right
-behind the library's own writers, and chains of calls that read what the one before wrote, give what they give alone."""
+"""The SM-pair prefill kernel and the stream kernel copy packed weights before the work in front of them in the stream has completed:
+calls right behind the library's own writers, and chains of calls that read what the one before wrote, give what they give alone."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -9,6 +9,9 @@ pytestmark = pytest.mark.gpu
     (2048, 2048, 300, 4),       # 128-token tiles
     (1024, 4096, 1000, 4),      # 256-token tiles
     (4096, 4096, 700, 3),       # behind the kernel that expands the 3-bit storage
+    (4096, 4096, 16, 3),        # behind the kernel that packs it: the stream kernel reads it as it is
+    (2048, 4096, 48, 3),
+    (4096, 4096, 16, 4),        # behind the quantizer
 ])
 def test_calls_behind_the_writers_of_their_operands(N, K, M, bits):
     import torch

@@ -69,11 +69,14 @@ def _operands(N, K, M, G, bits=4):
     return torch.randn((M, K), device="cuda").half(), qw, sc, zp, torch.empty((M, N), dtype=torch.float16, device="cuda")
 
 
-@pytest.mark.parametrize("M", [1, 5, 16, 100, 300])      # band, chunked, stream and SM-pair kernel
-def test_a_call_on_another_stream_does_not_release_the_reader(M):
+@pytest.mark.parametrize("M,N,K", [
+    (1, 8192, 4096), (5, 8192, 8320), (5, 4096, 8320),                   # band, chunked and stream kernel
+    (16, 8192, 4096), (100, 8192, 4096), (300, 8192, 4096),              # stream and SM-pair kernel
+])
+def test_a_call_on_another_stream_does_not_release_the_reader(M, N, K):
     import torch
     from paper_2306_00978_b200 import binding
-    N, K, G = (8192, 4096, 128) if M != 5 else (4096, 8320, 128)
+    G = 128
     L = binding.lib()
     x, qw, sc, zp, y = _operands(N, K, M, G)
     other = _operands(N, K, M, G)
