@@ -720,9 +720,9 @@ int awq_linear_int3(const void* x, const void* qweight3, const void* scales, con
                                                          (cudaStream_t)stream, nullptr, 3)));
     }
     // Up to 64 tokens, where awq_linear takes the stream kernel, that kernel reads the 3-bit storage as it is (expanding and then it / it
-    // alone, us: 4096 -> 11008 at 16 / 64 tokens 17.2 / 21.2 against 12.7 / 16.5, 4096 -> 4096 at 16 11.3 against 9.4, 8192 -> 28672 at 16
-    // 64.0 against 33.9).  Its launches are plainly ordered, as an expansion's and its reader's are, since the packed words
-    // may come from any writer in front; that costs the 3 us by which awq_linear's launches on 4-bit words overlap.
+    // alone, us: 4096 -> 11008 at 16 / 64 tokens 16.6 / 20.3 against 11.3 / 14.9, 4096 -> 4096 at 16 10.6 against 8.1, 8192 -> 28672 at 16
+    // 62.1 against 32.1).  The stream kernel is plainly ordered here: an expansion waited for whatever wrote the 3-bit words in front of
+    // it, a caller's own kernel too, and such calls stay right.  That costs about 2 us against awq_linear's launches on 4-bit words.
     if (stream_kernel_preferred(M, N, K, group, d->sms)) {
         void* ws = nullptr;
         {

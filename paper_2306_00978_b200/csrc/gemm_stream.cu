@@ -200,8 +200,8 @@ template <int TB> __device__ __forceinline__ uint4 st_piece(const unsigned char*
 }
 
 // TB: bytes of a packed block (16 rows x 64 columns): 512 for 4-bit codes, 384 for the 3-bit storage, whose fourth word costs five
-// instructions per piece and the others none (their masks leave out a nibble's top bit): 8192 -> 28672 at 16 / 32 / 64 tokens 33.9 / 39.0 /
-// 44.1 us plainly ordered, 4-bit codes in chained launches 30.3 / 35.0 / 42.7.
+// instructions per piece and the others none (their masks leave out a nibble's top bit): 8192 -> 28672 at 16 / 32 / 64 tokens 32.1 / 36.7 /
+// 44.2 us plainly ordered, 4-bit codes in chained launches 30.6 / 35.7 / 45.5.
 template <int G, int BN, bool XS, int TB = kStBlockBytes>
 __global__ void __launch_bounds__(kStMaxThreads, 1)
 gemm_stream_kernel(const __grid_constant__ StCut cut, const float* __restrict__ inv_s, float* partial, unsigned int* status_word, const __grid_constant__ CUtensorMap x_map,

@@ -129,7 +129,7 @@ struct QuantizeCut {
 // three IEEE divisions of a group's parameters, formed once per row by different lanes of the four that share it, weigh little.
 // W comes through shared memory, each warp's next tiles by asynchronous copies while it works on the one before.
 // 4096 -> 11008 (113.6 MB), calls among others: 31.3 us with 32 weights per lane, scalar steps and four conversions per packed word pair,
-// 29.2 us so; 20 arrays on 4096 x 4096 157 -> 133 us.  16 warps per SM issue in 60 % of the cycles (fma pipe 47 %, alu 43 %): the
+// 29.2 us so, 27.3 with the launch set up behind the call in front (a single launch 32.2); 20 arrays on 4096 x 4096 157 -> 133 us.  16 warps per SM issue in 60 % of the cycles (fma pipe 47 %, alu 43 %): the
 // warps' own dependencies are what is left.  Blocks per SM 3 / 4 / 5: 150 / 137 / 146 us (five spill); W widened once per item in
 // shared memory: 144 us (spills); a third tile in flight: 12 % slower; columns before bands in the order of items: 5 % slower.
 // MANY (the scale search): `a` is `arrays` arrays of K scales; W is quantized with each and the packed arrays follow one another.
