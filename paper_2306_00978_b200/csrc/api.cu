@@ -191,7 +191,7 @@ LaunchOrder launch_order(DeviceState* d, void* stream, bool behind_writer = fals
     {
         std::lock_guard<std::mutex> lock(g_mutex);
         if (d->writers.overflow) o.serialize = true;
-        if (d->writers.count == 0) return o;
+        if (d->writers.count == 0 && d->writers.forgotten == 0) return o;
     }
     o.key = stream_key((cudaStream_t)stream);
     std::lock_guard<std::mutex> lock(g_mutex);
